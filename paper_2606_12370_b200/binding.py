@@ -1,12 +1,14 @@
 """ctypes binding of libbebop.so.  Same names as the C ABI (include/bebop.h).
 
 Argument marshalling only: tensors are torch CUDA tensors whose device pointers
-are handed to the library, outputs are allocated here when not supplied, and the
-call is enqueued on torch's current stream.  Nothing is computed in Python.
+are handed to the library, outputs are allocated when not supplied, and the
+call is enqueued on torch's current stream.  Nothing is computed here: the four
+calls go through the native marshaller csrc/bebop_host.cpp (_bebop_host.so, built
+beside the library), everything else through ctypes.
 """
 import ctypes as C
+import importlib
 import os
-from typing import Optional
 
 import torch
 
@@ -14,6 +16,7 @@ BEBOP_F32, BEBOP_BF16 = 0, 1
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libbebop.so")
 _lib = None
+_host = None
 
 
 class BebopError(RuntimeError):
@@ -74,27 +77,32 @@ def _check(code: int):
         raise BebopError(code, bebop_status_string(code))
 
 
-def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return BEBOP_F32
-    if t.dtype == torch.bfloat16:
-        return BEBOP_BF16
-    raise BebopError(3, "logits must be float32 or bfloat16")
+_HOST_CODES = {-8: (8, "tensors must live on a CUDA device (no CPU fallback)"),
+               -3: (3, "logits must be float32 or bfloat16")}
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+def _load_host():
+    """The native marshaller, bound to the library's entry points (never builds, never falls back)."""
+    global _host
+    lib = load_library()
+    try:
+        host = importlib.import_module("._bebop_host", __package__)
+    except ImportError as e:
+        raise ImportError("_bebop_host.so is missing or does not load: build it with "
+                          "`python -m paper_2606_12370_b200.build`") from e
+    host.init(*(C.cast(f, C.c_void_p).value for f in
+                (lib.bebop_verify, lib.bebop_tv, lib.bebop_tv_static, lib.bebop_greedy_verify, lib.bebop_workspace_bytes)))
+    _host = host
+    return host
 
 
-def _rows(t: torch.Tensor, ndim: int):
-    """(pointer, ld) of a [.., R, V] tensor whose rows are equally spaced."""
-    if not t.is_cuda:
-        raise BebopError(8, "tensors must live on a CUDA device (no CPU fallback)")
-    assert t.dim() == ndim and t.stride(-1) == 1, "vocabulary must be contiguous"
-    ld = t.stride(-2)
-    if ndim == 3 and t.shape[0] > 1:
-        assert t.stride(0) == t.shape[1] * ld, "rows of the batch must be equally spaced"
-    return C.c_void_p(t.data_ptr()), int(ld)
+def _result(r):
+    """The marshaller's answer: the outputs, or the code of what went wrong."""
+    if type(r) is not int:
+        return r
+    if r in _HOST_CODES:
+        raise BebopError(*_HOST_CODES[r])
+    _check(r)
 
 
 def bebop_debug_force_general_path(on) -> None:
@@ -138,113 +146,29 @@ def bebop_workspace_bytes(B: int, K: int, V: int, dt: int) -> int:
 POISON_OUTPUTS = False
 
 
-def _new(shape, dtype, dev):
-    if POISON_OUTPUTS:
-        return torch.full(shape if isinstance(shape, tuple) else (shape,), -77, dtype=dtype, device=dev)
-    return torch.empty(shape, dtype=dtype, device=dev)
-
-
-def _workspace(B, K, V, dt, device, workspace):
-    need = bebop_workspace_bytes(B, K, V, dt)
-    if workspace is None:
-        workspace = torch.zeros(max(need, 256), dtype=torch.uint8, device=device)
-    return workspace, workspace.numel() * workspace.element_size()
-
-
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
-
-
 def bebop_verify(target_logits, draft_logits, draft_tokens, u_accept, u_final, draft_len=None,
                  temperature=None, temperature_all=1.0, out=None, workspace=None,
                  want_tv=True, want_probs=True, want_status=True):
     """Chain rejection-sampling verification.  Returns a dict of CUDA tensors:
     accept_len [B] i32, out_tokens [B,K+1] i32, tv / p_draft / q_draft [B,K] f32,
     row_status [B] i32 (the optional ones are None when not requested)."""
-    lib = load_library()
-    B, K1, V = target_logits.shape
-    K = K1 - 1
-    dt = _dt(target_logits)
-    assert draft_logits.dtype == target_logits.dtype and tuple(draft_logits.shape) == (B, K, V)
-    dev = target_logits.device
-    tp, ldt = _rows(target_logits, 3)
-    dp, ldd = _rows(draft_logits, 3)
-    o = out or {}
-    def get(name, shape, dtype, want=True):
-        if name in o and o[name] is not None:
-            return o[name]
-        return _new(shape, dtype, dev) if want else None
-    res = dict(
-        accept_len=get("accept_len", (B,), torch.int32), out_tokens=get("out_tokens", (B, K + 1), torch.int32),
-        tv=get("tv", (B, K), torch.float32, want_tv), p_draft=get("p_draft", (B, K), torch.float32, want_probs),
-        q_draft=get("q_draft", (B, K), torch.float32, want_probs),
-        row_status=get("row_status", (B,), torch.int32, want_status))
-    ws, wsb = _workspace(B, K, V, dt, dev, workspace)
-    for t in (draft_tokens, u_accept, u_final):
-        assert t.is_cuda and t.is_contiguous()
-    assert draft_tokens.dtype == torch.int32 and u_accept.dtype == torch.float32 and u_final.dtype == torch.float32
-    if draft_len is not None:
-        assert draft_len.dtype == torch.int32 and draft_len.is_contiguous()
-    if temperature is not None:
-        assert temperature.dtype == torch.float32 and temperature.is_contiguous()
-    _check(lib.bebop_verify(tp, ldt, dp, ldd, _ptr(draft_tokens), _ptr(draft_len), _ptr(temperature),
-                            float(temperature_all), _ptr(u_accept), _ptr(u_final), B, K, V, dt,
-                            _ptr(res["accept_len"]), _ptr(res["out_tokens"]), _ptr(res["tv"]),
-                            _ptr(res["p_draft"]), _ptr(res["q_draft"]), _ptr(res["row_status"]),
-                            _ptr(ws), wsb, _stream()))
-    res["workspace"] = ws
-    return res
+    return _result((_host or _load_host()).verify(target_logits, draft_logits, draft_tokens, u_accept, u_final, draft_len, temperature,
+                                                  temperature_all, None if not out else out if isinstance(out, dict) else dict(out), workspace, want_tv, want_probs, want_status, POISON_OUTPUTS))
 
 
 def bebop_tv(target_logits, draft_logits, temperature=None, temperature_all=1.0, workspace=None,
              want_s_aux=True, want_status=True):
     """TV distance (and the auxiliary S) of N paired rows [N,V]."""
-    lib = load_library()
-    N, V = target_logits.shape
-    dt = _dt(target_logits)
-    assert draft_logits.dtype == target_logits.dtype and tuple(draft_logits.shape) == (N, V)
-    dev = target_logits.device
-    tp, ldt = _rows(target_logits, 2)
-    dp, ldd = _rows(draft_logits, 2)
-    tv = _new(N, torch.float32, dev)
-    s_aux = _new(N, torch.float32, dev) if want_s_aux else None
-    st = _new(N, torch.int32, dev) if want_status else None
-    ws, wsb = _workspace(N, 1, V, dt, dev, workspace)
-    _check(lib.bebop_tv(tp, ldt, dp, ldd, _ptr(temperature), float(temperature_all), N, V, dt,
-                        _ptr(tv), _ptr(s_aux), _ptr(st), _ptr(ws), wsb, _stream()))
-    return dict(tv=tv, s_aux=s_aux, row_status=st)
+    return _result((_host or _load_host()).tv(target_logits, draft_logits, temperature, temperature_all, workspace, want_s_aux, want_status,
+                                              POISON_OUTPUTS))
 
 
 def bebop_tv_static(target_logits, draft_logits, temperature=None, temperature_all=1.0, want_s_aux=True):
     """bebop_tv with the library's built-in scratch instead of a workspace (no allocation in the call)."""
-    lib = load_library()
-    N, V = target_logits.shape
-    dt = _dt(target_logits)
-    assert draft_logits.dtype == target_logits.dtype and tuple(draft_logits.shape) == (N, V)
-    dev = target_logits.device
-    tp, ldt = _rows(target_logits, 2)
-    dp, ldd = _rows(draft_logits, 2)
-    tv = _new(N, torch.float32, dev)
-    s_aux = _new(N, torch.float32, dev) if want_s_aux else None
-    st = _new(N, torch.int32, dev)
-    _check(lib.bebop_tv_static(tp, ldt, dp, ldd, _ptr(temperature), float(temperature_all), N, V, dt,
-                               _ptr(tv), _ptr(s_aux), _ptr(st), _stream()))
-    return dict(tv=tv, s_aux=s_aux, row_status=st)
+    return _result((_host or _load_host()).tv(target_logits, draft_logits, temperature, temperature_all, False, want_s_aux, True,
+                                              POISON_OUTPUTS))
 
 
 def bebop_greedy_verify(target_logits, draft_tokens, draft_len=None, workspace=None):
     """Greedy-draft mode: accept while x_k equals the target argmax."""
-    lib = load_library()
-    B, K1, V = target_logits.shape
-    K = K1 - 1
-    dt = _dt(target_logits)
-    dev = target_logits.device
-    tp, ldt = _rows(target_logits, 3)
-    assert draft_tokens.dtype == torch.int32 and draft_tokens.is_contiguous() and draft_tokens.is_cuda
-    acc = _new(B, torch.int32, dev)
-    out = _new((B, K + 1), torch.int32, dev)
-    st = _new(B, torch.int32, dev)
-    ws, wsb = _workspace(B, K, V, dt, dev, workspace)
-    _check(lib.bebop_greedy_verify(tp, ldt, _ptr(draft_tokens), _ptr(draft_len), B, K, V, dt,
-                                   _ptr(acc), _ptr(out), _ptr(st), _ptr(ws), wsb, _stream()))
-    return dict(accept_len=acc, out_tokens=out, row_status=st)
+    return _result((_host or _load_host()).greedy_verify(target_logits, draft_tokens, draft_len, workspace, POISON_OUTPUTS))

@@ -1,11 +1,14 @@
-"""Compile the CUDA library (sm_100a) in-tree: paper_2606_12370_b200/libbebop.so."""
+"""Compile the CUDA library (sm_100a) and the binding's native marshaller in-tree: paper_2606_12370_b200/libbebop.so
+and paper_2606_12370_b200/_bebop_host.so."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbebop.so")
+HOST = os.path.join(HERE, "_bebop_host.so")
 SOURCES = ["bebop_api.cu", "bebop_general.cu", "bebop_redraw.cu", "bebop_pipe.cu", "bebop_fuse.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -18,19 +21,41 @@ def _deps():
     return out
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and all(os.path.getmtime(LIB) >= os.path.getmtime(d) for d in _deps()):
-        return LIB
-    tmp = LIB + ".tmp.%d" % os.getpid()
-    extra = os.environ.get("BEBOP_NVCC_EXTRA", "").split()
-    cmd = [NVCC] + FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + \
-        [os.path.join(CSRC, s) for s in SOURCES]
-    r = subprocess.run(cmd, capture_output=True, text=True)
+def _run(cmd, out, verbose):
+    """Run a compiler that writes `out` (under another name until it is complete)."""
+    tmp = out + ".tmp.%d" % os.getpid()
+    r = subprocess.run(cmd + ["-o", tmp], capture_output=True, text=True)
     if verbose or r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
     if r.returncode != 0:
-        raise RuntimeError("nvcc failed")
-    os.replace(tmp, LIB)
+        raise RuntimeError("%s failed" % cmd[0])
+    os.replace(tmp, out)
+
+
+def _fresh(out, deps):
+    return os.path.exists(out) and all(os.path.getmtime(out) >= os.path.getmtime(d) for d in deps)
+
+
+def build_host(force: bool = False, verbose: bool = False) -> str:
+    """The native marshaller: a CPython module against torch's headers and libraries."""
+    src = os.path.join(CSRC, "bebop_host.cpp")
+    if force or not _fresh(HOST, [src, os.path.join(os.path.dirname(HERE), "include", "bebop.h")]):
+        import torch
+        root = os.path.dirname(torch.__file__)
+        inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+        _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] +
+             ["-I" + d for d in inc] + [src, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"],
+             HOST, verbose)
+    return HOST
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    build_host(force, verbose)
+    if not force and _fresh(LIB, _deps()):
+        return LIB
+    extra = os.environ.get("BEBOP_NVCC_EXTRA", "").split()
+    _run([NVCC] + FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + [os.path.join(CSRC, s) for s in SOURCES], LIB, verbose)
     return LIB
 
 
