@@ -48,7 +48,7 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-KERNEL_NAME = {1: "general kernels", 2: "k_pipe", 3: "k_fuse"}      # by bebop_debug_last_kernel()
+KERNEL_NAME = {1: "general kernels", 2: "k_pipe", 3: "k_fuse or k_seq"}      # by bebop_debug_last_kernel()
 
 
 def ncu_traffic(kernel):

@@ -163,14 +163,15 @@ bebop_status_t bebop_greedy_verify(
  * Test and measurement hooks (no counterpart in the paper).  They set process-wide switches that every later
  * call in the process sees: not thread-safe, and not meant for code that serves requests.
  * bebop_debug_force_general_path(mode) chooses the kernels behind bebop_verify, bebop_tv and bebop_greedy_verify:
- * 0 (the default) the faster, by measurement, of the fused and the pipelined kernel for the shape, and the
- * split-row general kernels for shapes neither takes; 1 the general kernels always; 2 never the fused kernel;
- * 3 the fused kernel wherever it applies (the greedy mode has no fused form).  All give the same results up to
- * the documented tolerances.  bebop_debug_last_kernel() says what the last of these calls ran: 1 the general kernels,
- * 2 the pipelined kernel, 3 the fused kernel (0: no call yet).
+ * 0 (the default) the fastest, by measurement, of the sequence, the fused and the pipelined kernel for the shape, and the
+ * split-row general kernels for shapes none of them takes; 1 the general kernels always; 2 the pipelined kernel
+ * wherever it applies; 3 the fused kernel wherever it applies (the greedy mode has no fused form); 4 the sequence kernel
+ * wherever it applies.  All give the same results up to the documented tolerances.  bebop_debug_last_kernel() says
+ * what the last of these calls ran: 1 the general kernels, 2 the pipelined kernel, 3 a kernel that reads every logit
+ * once, the fused or the sequence kernel (0: no call yet).
  * bebop_debug_fallback_offset returns the byte offset, inside the workspace of this
- * shape, of an int32 that after a bebop_verify call holds the number of sequences
- * whose draw was re-done by the fp64 kernels.
+ * shape, of an int32 that after a bebop_verify call through the pipelined or the fused kernel holds the number of
+ * sequences whose draw was re-done by the fp64 kernels.
  * bebop_debug_set_timing_events(start, stop): two cudaEvent_t handles that the next
  * bebop_verify calls record around the main (pipelined or fused) kernel, on the caller's stream (NULL,
  * NULL switches it off).

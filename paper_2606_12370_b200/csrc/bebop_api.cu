@@ -9,9 +9,10 @@ namespace {
 
 // Test hook: route bebop_verify through the general (split-row) path even where the fused
 // kernel applies, so that both paths are covered by the parity tests.
-int g_last_kernel = 0;   // what the last call ran: 1 general kernels, 2 pipelined kernel, 3 fused kernel
-int g_path = 0;   // 0: the faster of the fused and the pipelined kernel where they apply, else the general kernels;
-                  // 1: general kernels only; 2: never the fused kernel; 3: the fused kernel wherever it applies
+int g_last_kernel = 0;   // what the last call ran: 1 general kernels, 2 pipelined kernel, 3 a kernel that reads every logit once
+                         // (fused or sequence kernel)
+int g_path = 0;   // 0: the fastest for the shape; 1: general kernels only; 2: never a one-read kernel; 3: the fused kernel wherever
+                  // it applies; 4: the sequence kernel wherever it applies
 
 int g_expire_wait = 0;   // test hook: which device-side wait the next call lets give up at once
 float g_draw_kappa = -1.f;   // test hook: factor of the fast draw's error bound (negative: the built-in value)
@@ -113,7 +114,11 @@ bebop_status_t bebop_verify(const void* target_logits, int64_t ld_target, const 
     cudaError_t e = cudaSuccess;
     bool launched = false;
     g_last_kernel = 1;
-    if ((g_path == 3 || (g_path == 0 && fuse_preferred(a, false))) && fuse_supported(a)) {
+    if ((g_path == 4 && seq_supported(a, false)) || (g_path == 0 && seq_preferred(a, false))) {
+        e = seq_verify(a, draft_tokens, u_accept, u_final, o, stream, &launched);
+        if (launched) g_last_kernel = 3;
+    }
+    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, false))) && fuse_supported(a)) {
         e = fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
         if (launched) g_last_kernel = 3;
     }
@@ -146,7 +151,11 @@ bebop_status_t bebop_tv(const void* target_logits, int64_t ld_target, const void
     bool launched = false;
     VerifyOut o{nullptr, nullptr, tv, nullptr, nullptr, row_status};
     g_last_kernel = 1;
-    if ((g_path == 3 || (g_path == 0 && fuse_preferred(a, true))) && fuse_supported(a)) {
+    if ((g_path == 4 && seq_supported(a, true)) || (g_path == 0 && seq_preferred(a, true))) {
+        e = seq_verify(a, nullptr, nullptr, nullptr, o, stream, &launched, true, s_aux);
+        if (launched) g_last_kernel = 3;
+    }
+    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, true))) && fuse_supported(a)) {
         e = fuse_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
         if (launched) g_last_kernel = 3;
     }
@@ -179,7 +188,11 @@ bebop_status_t bebop_greedy_verify(const void* target_logits, int64_t ld_target,
     cudaError_t e = cudaSuccess;
     bool launched = false;
     g_last_kernel = 1;
-    if (g_path != 1 && pipe_supported(a)) {
+    if (g_path == 4 || (g_path == 0 && seq_greedy_preferred(a))) {
+        e = seq_greedy(a, draft_tokens, accept_len, out_tokens, row_status, stream, &launched);
+        if (launched) g_last_kernel = 3;
+    }
+    if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
         e = pipe_greedy(a, p, draft_tokens, accept_len, out_tokens, row_status, static_cast<char*>(workspace), stream, &launched);
         if (launched) g_last_kernel = 2;
     }

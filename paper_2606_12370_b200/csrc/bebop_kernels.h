@@ -73,6 +73,16 @@ cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
 
+// Sequence kernel (bebop_seq.cu): a thread-block cluster per sequence (row pair), its logits in the cluster's shared memory;
+// one launch, no workspace; same contract.
+bool seq_supported(const RowArgs& a, bool tv_only);
+bool seq_preferred(const RowArgs& a, bool tv_only);
+bool seq_greedy_preferred(const RowArgs& a);
+cudaError_t seq_verify(const RowArgs& a, const int32_t* draft_tokens, const float* u_accept, const float* u_final, VerifyOut o,
+                       cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
+cudaError_t seq_greedy(const RowArgs& a, const int32_t* draft_tokens, int32_t* accept_len, int32_t* out_tokens,
+                       int32_t* row_status, cudaStream_t stream, bool* launched);
+
 // The greedy mode through the pipelined kernel: one sweep over the target rows (maximum and lowest index per
 // slice), then a small kernel that merges the slices and runs the argmax match.
 cudaError_t pipe_greedy(const RowArgs& a, const Plan& p, const int32_t* draft_tokens, int32_t* accept_len,
