@@ -100,9 +100,12 @@ __device__ __forceinline__ bool t_tail(int m) { return (m >> 26) & 1; }
 // that the slice holds a NaN or +inf; the other bits are those of a float u that bounds the slice's sum of e^2
 // (around the slice's exponent) from above: e <= 1, so a chunk's is at most its sum of e.
 struct __align__(16) Rec { double s; int ecode; int flags; };
-__device__ __forceinline__ int rec_e(const Rec& r) { return (r.ecode - 1) >> 1; }
+// (an exponent is stored as e + 2^24, far from zero and from the ends of the integers; 1: the slice holds nothing but -inf)
+constexpr int kCodeBias = 1 << 24, kCodeEmpty = 1;
+__device__ __forceinline__ int rec_e(const Rec& r) { return r.ecode == kCodeEmpty ? E_EMPTY : r.ecode - kCodeBias; }
+__device__ __forceinline__ int rec_code(int e) { return e > E_EMPTY ? e + kCodeBias : kCodeEmpty; }
 __device__ __forceinline__ float rec_ub(const Rec& r) { return __int_as_float(r.flags & ~1); }
-__device__ __forceinline__ Rec no_rec() { Rec r; r.s = 0.0; r.ecode = 2 * E_EMPTY + 1; r.flags = 0; return r; }
+__device__ __forceinline__ Rec no_rec() { Rec r; r.s = 0.0; r.ecode = kCodeEmpty; r.flags = 0; return r; }
 struct __align__(16) Row { double inv_s; int e; int st; };            // a merged row: 1/S, exponent, status bits (| kRowValid)
 
 struct StreamArgs {
@@ -635,7 +638,7 @@ __device__ __noinline__ void stats_warp(const StreamArgs& a, SharedD<DT>& S, int
             const unsigned long long w0 = (unsigned long long)__double_as_longlong(nonzero_bits(row ? p1.s : p0.s));
             const float ub = (float)(row ? p1.ub : p0.ub) * 6.103515625e-05f;                // 2^-14; below 2^24 units: exact
             const unsigned ubits = ((unsigned)__float_as_int(ub) + 1u) & ~1u;                // (bit 0 is the flag)
-            const unsigned long long w1 = (unsigned long long)(unsigned)(2 * (row ? p1.em : p0.em) + 1)
+            const unsigned long long w1 = (unsigned long long)(unsigned)rec_code(row ? p1.em : p0.em)
                                         | ((unsigned long long)(ubits | ((row ? p1.bad : p0.bad) ? 1u : 0u)) << 32);
             const unsigned doit = (chunk == 0 && (row == 0 || two)) ? 1u : 0u;
             asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};\n\t}"
