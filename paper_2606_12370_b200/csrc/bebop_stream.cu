@@ -399,11 +399,13 @@ __device__ __noinline__ bool produce(const StreamArgs& a, Shared& S, uint32_t da
 // The end of the tasks, marked in as many descriptions as there are stats warps.  Nothing is in flight when this returns, also
 // when somebody has given up.
 __device__ __forceinline__ void produce_stop(const StreamArgs& a, Shared& S, const Producer& P) {
+    int u = max(P.u - NSTG, 0);
     if (!aborted(S) && mbar_wait<S_EMPTY>(S, smem_u32(&S.empty[P.st]), ((uint32_t)(P.u / NSTG) & 1u) ^ 1u)) {
         for (int i = 0; i < NSTAT; ++i) S.task[(P.n + i) % RT].meta = kStop;
         mbar_arrive(&S.full[P.st]);
+        u = max(P.u - NSTG + 1, 0);          // (the stage that the mark took had been read: its barrier is a turn further)
     }
-    for (int u = max(P.u - NSTG, 0); u < P.u; ++u)
+    for (; u < P.u; ++u)
         for (uint32_t i = 0; i < kWaitSpin && !mbar_try(smem_u32(&S.full[u % NSTG]), (uint32_t)(u / NSTG) & 1u); ++i) {}
 }
 
