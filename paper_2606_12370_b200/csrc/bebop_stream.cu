@@ -23,7 +23,7 @@
 // What CTAs pass to each other are words that are valid by themselves once non-zero (the memory is cleared by the kernel,
 // before the grid meets once), written and read by relaxed accesses: no fence on the streaming path.  Every wait is
 // bounded; one that gives up sets the wait flag and lets the CTA run out (status bit 32 of every row).  No cluster.
-// Tasks wait only for tasks of earlier rounds of the deal (a CTA's task n waits for the units of its task n - LAG - 1),
+// Tasks wait only for tasks of earlier rounds of the deal (a CTA's task n waits for the units of its task n - NSLOT),
 // so nothing can deadlock.
 #include <cooperative_groups.h>
 
@@ -42,10 +42,10 @@ constexpr int NSTG = 3;                       // stages of the ring of logits: o
 constexpr int STAGE = SV * 16;
 constexpr int RING = NSTG * STAGE;
 #ifndef BS_NSTAT
-#define BS_NSTAT 4
+#define BS_NSTAT 2
 #endif
 #ifndef BS_NF
-#define BS_NF 3
+#define BS_NF 1
 #endif
 #ifndef S_FULL
 #define S_FULL 32
@@ -79,7 +79,6 @@ template <int DT> struct Dims {
     static constexpr int TSLOT = 128 / (2 * NR);               // tasks a warp's 128 TMEM columns hold
     static constexpr int MSLOT = DT == 1 ? 1 : 0;              // further tasks held in shared memory
     static constexpr int NSLOT = TSLOT + MSLOT;
-    static constexpr int LAG = NSLOT - 1;                      // pass 2 of task m begins with the second row of task m + LAG
     static constexpr int MWARP = 32 * 2 * NR * 4;              // bytes of a warp's part of a task held in shared memory
     static constexpr int DATA = RING + MSLOT * CW * MWARP;
     static_assert(NSLOT == 3 || NSLOT == 4, "rings");
@@ -187,10 +186,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 // N consecutive 32-bit columns of this thread's TMEM lane
 template <int N> __device__ __forceinline__ void tmem_st(uint32_t t, const float* v);
-template <> __device__ __forceinline__ void tmem_st<16>(uint32_t t, const float* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-                 :: "r"(t), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
-                    "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]) : "memory");
+template <> __device__ __forceinline__ void tmem_st<4>(uint32_t t, const float* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" :: "r"(t), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
 }
 template <> __device__ __forceinline__ void tmem_st<8>(uint32_t t, const float* v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
@@ -462,139 +459,151 @@ template <> __device__ __forceinline__ float vecs_max<1>(const uint4* v) {
     return max_nan(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
 }
 
-// A consumer warp.  Step h = 2 n + row: pass 1 of its chunk of a row of task n, and half of pass 2 (two quarters, in front of the
-// stores of the two halves of the exponentials) of the task that was LAG and a half before: the second half
-// of task m's pass 2 runs with the first row of task m + LAG + 1, which takes m's place; a quarter is read before
-// what stands there is overwritten.  The warps do not wait for each other.
+// A consumer warp.  Step n: pass 1 of its chunk of both rows of task n and pass 2 of task n - NSLOT, whose place task n
+// takes: a vector's exponentials are read before those of the new task are put there.  Both rows and both passes in one
+// step: the chains of dependent instructions around the arithmetic (barrier, description, largest logit, sums) are
+// as long as the arithmetic itself and are met once per task.  The warps do not wait for each other.
 template <int DT, bool TVM>
 __device__ __forceinline__ void consumer(const StreamArgs& a, SharedD<DT>& S, uint32_t data, int tid) {
     using D = Dims<DT>;
-    constexpr int VEC = D::VEC, NR = D::NR, NQ = NR / 4, LAG = D::LAG, NSLOT = D::NSLOT, TSLOT = D::TSLOT;
+    constexpr int VEC = D::VEC, NR = D::NR, NSLOT = D::NSLOT, TSLOT = D::TSLOT;
     const int lane = tid & 31, w = tid >> 5;
     const bool one = lane == 0;
     // the warp's 128 columns of its quarter of the lanes
     const uint32_t tbase = S.tmem_base + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 128);
     const uint32_t mine = data + (w * CV + lane) * 16;
     const uint32_t msl = data + RING + w * D::MWARP + lane * 16;
-    const uint32_t full0 = smem_u32(S.full), empty0 = smem_u32(S.empty);
+    const uint32_t full0 = smem_u32(S.full), empty0 = smem_u32(S.empty), task0 = smem_u32(S.task);
     uint32_t st = 0, par = 0;                         // stage of the next row, parity of its turn
-    uint32_t h_end = 0x7fffff00u;                     // the first step without a row
-    int wslot = 0, rslot = 0;                         // places of task n and of the task in pass 2
-    float2 tm = make_float2(0.f, 0.f), sx = make_float2(0.f, 0.f);
+    int n_end = 0x7fffff00;                           // the first step without a task
+    int slot = 0;                                     // n % NSLOT
 #pragma unroll 1
-    for (uint32_t h = 0; h < h_end + (2 * LAG + 1); ++h) {
-        const uint32_t n = h >> 1, row = h & 1u;
-        const uint32_t g = h - (2 * LAG + 1), m = g >> 1, half = g & 1u;       // the half of pass 2
-        bool live = h < h_end;
-        const bool live2 = h >= 2 * LAG + 1;           // (g < h_end by the loop's bound)
-        uint4 x[4];
+    for (int n = 0; n < n_end + NSLOT; ++n) {
+        bool live = n < n_end;
+        const bool live2 = n >= NSLOT;
+        const int m = n - NSLOT;
+        uint4 xp[4], xq[4];
         float c = 0.f;
-        int meta = 0;
+        int meta = kStop;
         if (live) {
             if (!mbar_wait<S_FULL>(S, full0 + st * 8, par)) { if (one) give_up(a, S); return; }
-            const uint32_t pd = mine + st * STAGE;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) x[j] = lds16(pd + j * 512);
-            c = S.task[n % RT].c;
-            meta = S.task[n % RT].meta;
-            __syncwarp();
-            if (one) mbar_arrive(empty0 + st * 8);
-            if (++st == NSTG) { st = 0; par ^= 1u; }
+            const uint4 d = lds16(task0 + (n % RT) * 16);
+            c = __uint_as_float(d.x); meta = (int)d.y;
             if (t_kind(meta) == kStop) {
-                h_end = h; live = false;
+                n_end = n; live = false;
                 if (one) for (int i = 0; i < NSTAT; ++i) mbar_arrive(&S.pdone[(n + i) % R8]);       // every stats warp meets the end
+            } else {
+                const uint32_t s0 = st, p0 = mine + st * STAGE;
+                if (++st == NSTG) { st = 0; par ^= 1u; }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) xp[j] = lds16(p0 + j * 512);
+                if (!mbar_wait<S_FULL>(S, full0 + st * 8, par)) { if (one) give_up(a, S); return; }
+                const uint32_t p1 = mine + st * STAGE;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) xq[j] = lds16(p1 + j * 512);
+                __syncwarp();
+                if (one) { mbar_arrive(empty0 + s0 * 8); mbar_arrive(empty0 + st * 8); }
+                if (++st == NSTG) { st = 0; par ^= 1u; }
             }
         }
-        int meta2 = kStop;
-        float4 rho = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool two = false;                              // there is a quarter of pass 2 to do
-        if (live2) {
-            if (half == 0 && !mbar_wait<S_STAT>(S, smem_u32(&S.stats[m % R8]), (m / R8) & 1u)) { if (one) give_up(a, S); return; }
-            meta2 = S.task[m % RT].meta;
-            two = t_kind(meta2) == kPair && w * CV < t_nv(meta2);
-            if (two) rho = S.slot[rslot].rho[w];
-            tmem_wait_st();
-        }
-        const int left = live ? (row ? t_nv2(meta) : t_nv(meta)) - w * CV : 0;       // vectors from the chunk's first to the end of the slice
-        const bool keep = left > 0 && t_kind(meta) == kPair;     // (a bonus task's exponentials are summed and not kept)
-        QExp E;
-        E.e = E_EMPTY; E.ef = 0.f;
-        if (left > 0) {
-            if (left < CV || t_tail(meta)) {
+        const int left0 = live ? t_nv(meta) - w * CV : 0, left1 = live ? t_nv2(meta) - w * CV : 0;     // vectors from the chunk's first to the end of the slice
+        const bool any = left0 > 0;                              // (the second row is never the longer one)
+        const bool keep = any && t_kind(meta) == kPair;          // (a bonus task's exponentials are summed and not kept)
+        QExp Ep, Eq;
+        Ep.e = E_EMPTY; Ep.ef = 0.f; Eq.e = E_EMPTY; Eq.ef = 0.f;
+        if (any) {
+            if (left1 < CV || t_tail(meta)) {
                 // not a full chunk: vectors beyond the slice read as -inf, a row's ragged last vector loses the lanes beyond the vocabulary
+                const int lastn = a.r.V - (a.r.nvec - 1) * VEC;
+                const bool tp = t_tail(meta) && (t_kind(meta) == kPair || t_nv2(meta) == 0), tq = t_tail(meta);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int vi = j * 32 + lane;
-                    if (vi >= left) x[j] = neg_inf_vec<DT>();
-                    if (t_tail(meta) && vi == left - 1 && (row || t_kind(meta) == kPair || t_nv2(meta) == 0)) mask_tail<DT>(x[j], a.r.V - (a.r.nvec - 1) * VEC);
+                    if (vi >= left0) xp[j] = neg_inf_vec<DT>();
+                    if (vi >= left1) xq[j] = neg_inf_vec<DT>();
+                    if (tp && vi == left0 - 1) mask_tail<DT>(xp[j], lastn);
+                    if (tq && vi == left1 - 1) mask_tail<DT>(xq[j], lastn);
                 }
             }
-            E = chunk_exponent(vecs_max<DT>(x), c);
+            Ep = chunk_exponent(vecs_max<DT>(xp), c);
+            Eq = chunk_exponent(vecs_max<DT>(xq), c);
         }
-        const bool wt = D::MSLOT == 0 || wslot < TSLOT, rt = D::MSLOT == 0 || rslot < TSLOT;
-        float2 acc = make_float2(0.f, 0.f);
+        int meta2 = kStop, us2 = 0;
+        float4 rho = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool two = false;                              // there is pass 2 to do
+        if (live2) {
+            if (!mbar_wait<S_STAT>(S, smem_u32(&S.stats[m % R8]), (m / R8) & 1u)) { if (one) give_up(a, S); return; }
+            const uint4 d = lds16(task0 + (m % RT) * 16);
+            meta2 = (int)d.y; us2 = (int)d.z;
+            two = t_kind(meta2) == kPair && w * CV < t_nv(meta2);
+            if (two) rho = S.slot[slot].rho[w];
+            tmem_wait_st();
+        }
+        const bool tm_slot = D::MSLOT == 0 || slot < TSLOT;
+        const uint32_t tcol = tbase + slot * 2 * NR;
+        float2 ap = make_float2(0.f, 0.f), aq = ap, tm = ap, sx = ap;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const uint32_t col = (half * 2 + q) * NQ;
-            float p[NQ], r[NQ];
+        for (int j = 0; j < 4; ++j) {
+            float p[VEC], r[VEC], e[VEC], f[VEC];
             if (two) {
-                if (rt) {
-                    tmem_ld(tbase + rslot * 2 * NR + col, p);
-                    tmem_ld(tbase + rslot * 2 * NR + NR + col, r);
+                if (tm_slot) {
+                    tmem_ld(tcol + j * VEC, p);
+                    tmem_ld(tcol + NR + j * VEC, r);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < NQ / 4; ++i) {
-                        const float4 u = lds16f(msl + (col / 4 + i) * 512), v = lds16f(msl + D::MWARP / 2 + (col / 4 + i) * 512);
+                    for (int i = 0; i < VEC / 4; ++i) {
+                        const float4 u = lds16f(msl + (j * (VEC / 4) + i) * 512), v = lds16f(msl + D::MWARP / 2 + (j * (VEC / 4) + i) * 512);
                         p[4 * i] = u.x; p[4 * i + 1] = u.y; p[4 * i + 2] = u.z; p[4 * i + 3] = u.w;
                         r[4 * i] = v.x; r[4 * i + 1] = v.y; r[4 * i + 2] = v.z; r[4 * i + 3] = v.w;
                     }
                 }
             }
-            float e[NR / 2];
-            if (left > 0) {
-                exp_vec<DT>(x[2 * q], c, E.ef, e);
-                exp_vec<DT>(x[2 * q + 1], c, E.ef, e + VEC);
+            if (any) {
+                exp_vec<DT>(xp[j], c, Ep.ef, e);
+                exp_vec<DT>(xq[j], c, Eq.ef, f);
             }
             if (two) {
-                if (rt) tmem_wait_ld(p, r);
-                if (TVM) resid_aux_n<NQ>(p, r, rho.x, rho.y, &tm, &sx);
-                else resid_n<NQ, false>(p, r, rho.x, rho.y, &tm, nullptr);
+                if (tm_slot) tmem_wait_ld(p, r);
+                if (TVM) resid_aux_n<VEC>(p, r, rho.x, rho.y, &tm, &sx);
+                else resid_n<VEC, false>(p, r, rho.x, rho.y, &tm, nullptr);
             }
-            if (left > 0) {
-                acc = add_pairs(acc, e, NR / 2);
+            if (any) {
+                ap = add_pairs(ap, e, VEC);
+                aq = add_pairs(aq, f, VEC);
                 if (keep) {
-                    if (wt) tmem_st<NR / 2>(tbase + (wslot * 2 + row) * NR + q * (NR / 2), e);
-                    else {
+                    if (tm_slot) {
+                        tmem_st<VEC>(tcol + j * VEC, e);
+                        tmem_st<VEC>(tcol + NR + j * VEC, f);
+                    } else {
 #pragma unroll
-                        for (int i = 0; i < NR / 8; ++i) sts16(msl + row * (D::MWARP / 2) + (q * (NR / 8) + i) * 512, e + 4 * i);
+                        for (int i = 0; i < VEC / 4; ++i) {
+                            sts16(msl + (j * (VEC / 4) + i) * 512, e + 4 * i);
+                            sts16(msl + D::MWARP / 2 + (j * (VEC / 4) + i) * 512, f + 4 * i);
+                        }
                     }
                 }
             }
         }
-        if (live2 && half == 1u) {
-            if (t_kind(meta2) == kPair) {
-                const int64_t o = (int64_t)S.task[m % RT].us * CH + w;
-                if (TVM) {
-                    const float z = warp_sum2(tm.x + tm.y, sx.x + sx.y, lane >= 16) * (lane >= 16 ? rho.w : rho.z);
-                    if ((lane & 15) == 0) st_relaxed_f((lane ? a.ca : a.cm) + o, nonzero_f(z));
-                } else {
-                    const float z = warp_sum(tm.x + tm.y) * rho.z;
-                    if (one) st_relaxed_f(a.cm + o, nonzero_f(z));
-                }
-                tm = make_float2(0.f, 0.f); sx = make_float2(0.f, 0.f);
-            }
-            if (++rslot == NSLOT) rslot = 0;
-        }
         if (live) {
-            const int2 sum = left > 0 ? warp_sum_words(acc.x + acc.y) : make_int2(kNoSum0, kNoSum1);
+            const int2 s0 = warp_sum_words(ap.x + ap.y), s1 = warp_sum_words(aq.x + aq.y);
             if (one) {
-                S.slot[wslot].part[row][w] = make_int4(sum.x, sum.y, E.e, 0);
-                if (row) mbar_arrive(&S.pdone[n % R8]);
+                S.slot[slot].part[0][w] = make_int4(s0.x, s0.y, Ep.e, 0);
+                S.slot[slot].part[1][w] = make_int4(s1.x, s1.y, Eq.e, 0);
+                mbar_arrive(&S.pdone[n % R8]);
             }
-            if (row && ++wslot == NSLOT) wslot = 0;
         }
+        if (t_kind(meta2) == kPair) {
+            const int64_t o = (int64_t)us2 * CH + w;
+            if (TVM) {
+                const float z = warp_sum2(tm.x + tm.y, sx.x + sx.y, lane >= 16) * (lane >= 16 ? rho.w : rho.z);
+                if ((lane & 15) == 0) st_relaxed_f((lane ? a.ca : a.cm) + o, nonzero_f(z));
+            } else {
+                const float z = warp_sum(tm.x + tm.y) * rho.z;
+                if (one) st_relaxed_f(a.cm + o, nonzero_f(z));
+            }
+        }
+        if (++slot == NSLOT) slot = 0;
         __syncwarp();
-        if (aborted(S)) return;
     }
 }
 
