@@ -119,7 +119,7 @@ static inline FusePlan make_fuse_plan(int B, int K, int nvec, int ups) {
 
 // Workspace of the streaming kernel (bebop_stream.cu).  A unit is a row pair or a bonus row; a sequence owns `ups`
 // consecutive units (K + 1 for bebop_verify, 1 for bebop_tv); every unit is cut into T slices of kStreamWarps chunks.
-constexpr int kStreamWarps = 16, kStreamChunkVecs = 128;
+constexpr int kStreamWarps = 12, kStreamChunkVecs = 128;
 constexpr int kStreamSliceVecs = kStreamWarps * kStreamChunkVecs;
 constexpr int kStreamMaxSlices = 128;
 struct StreamPlan {

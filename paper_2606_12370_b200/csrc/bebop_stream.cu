@@ -37,8 +37,8 @@ constexpr int CW = kStreamWarps;              // consumer warps = chunks of a sl
 constexpr int CV = kStreamChunkVecs;          // vectors per chunk and row: four per lane
 constexpr int CH = CW;
 constexpr int SV = kStreamSliceVecs;          // vectors per slice, at most
-static_assert(CW == 16 && CV == 128 && SV == CH * CV, "slice size, chunks, TMEM columns per warp");
-constexpr int NSTG = 3;                       // stages of the ring of logits: one row of a slice each
+static_assert(CW == 12 && CH % 4 == 0 && CV == 128 && SV == CH * CV, "slice size, chunks, TMEM columns per warp");
+constexpr int NSTG = 6;                       // stages of the ring of logits: one row of a slice each
 constexpr int STAGE = SV * 16;
 constexpr int RING = NSTG * STAGE;
 #ifndef BS_NSTAT
@@ -75,12 +75,14 @@ constexpr int XV = 64;                        // vectors of an item of the re-dr
 
 template <int DT> struct Dims {
     static constexpr int VEC = Elem<DT>::VEC;
-    static constexpr int NR = 4 * VEC;                         // exponentials per thread and row
-    static constexpr int TSLOT = 128 / (2 * NR);               // tasks a warp's 128 TMEM columns hold
-    static constexpr int MSLOT = DT == 1 ? 1 : 0;              // further tasks held in shared memory
-    static constexpr int NSLOT = TSLOT + MSLOT;
-    static constexpr int MWARP = 32 * 2 * NR * 4;              // bytes of a warp's part of a task held in shared memory
-    static constexpr int DATA = RING + MSLOT * CW * MWARP;
+    static constexpr int TCOL = 2 * 4 * VEC;                   // TMEM columns of a task: per vector VEC of the target row, VEC of the draft row
+    static constexpr int WCOL = 160;                           // columns of a warp: three warps share a quarter of the lanes
+    // Tasks whose exponentials wait at a time.  bf16: two and a half of them in the warp's columns, the last two vectors of
+    // every third task in shared memory.
+    static constexpr int NSLOT = DT == 1 ? 3 : 4;
+    static constexpr int MWARP = NSLOT * TCOL > WCOL ? 2 * 32 * 2 * VEC * 4 : 0;      // bytes of a warp's part in shared memory
+    static constexpr int DATA = RING + CW * MWARP;
+    static_assert((NSLOT - 1) * TCOL + TCOL / (MWARP ? 2 : 1) <= WCOL && 3 * WCOL <= TCOLS, "columns");
     static_assert(NSLOT == 3 || NSLOT == 4, "rings");
 };
 
@@ -186,28 +188,30 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 // N consecutive 32-bit columns of this thread's TMEM lane
 template <int N> __device__ __forceinline__ void tmem_st(uint32_t t, const float* v);
-template <> __device__ __forceinline__ void tmem_st<4>(uint32_t t, const float* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" :: "r"(t), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+template <> __device__ __forceinline__ void tmem_st<16>(uint32_t t, const float* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 :: "r"(t), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+                    "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]) : "memory");
 }
 template <> __device__ __forceinline__ void tmem_st<8>(uint32_t t, const float* v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                  :: "r"(t), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
 }
 // (the registers hold the columns after tmem_wait_ld, through which they pass, so that no use is moved ahead of it)
+__device__ __forceinline__ void tmem_ld(uint32_t t, float (&v)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]) : "r"(t) : "memory");
+}
 __device__ __forceinline__ void tmem_ld(uint32_t t, float (&v)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
 }
-__device__ __forceinline__ void tmem_ld(uint32_t t, float (&v)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
-}
-__device__ __forceinline__ void pin(float (&v)[8]) {
-    asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]));
-}
-__device__ __forceinline__ void pin(float (&v)[4]) { asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3])); }
-template <int N> __device__ __forceinline__ void tmem_wait_ld(float (&p)[N], float (&q)[N]) {
+template <int N> __device__ __forceinline__ void tmem_wait_ld(float (&v)[N]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    pin(p); pin(q);
+#pragma unroll
+    for (int i = 0; i < N; i += 8)
+        asm volatile("" : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3]), "+f"(v[i + 4]), "+f"(v[i + 5]), "+f"(v[i + 6]), "+f"(v[i + 7]));
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -459,6 +463,75 @@ template <> __device__ __forceinline__ float vecs_max<1>(const uint4* v) {
     return max_nan(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
 }
 
+// Where a chunk's exponentials wait for pass 2: vector j's, target row then draft row, in TMEM columns; MIX: the last
+// two vectors' in shared memory.
+template <int DT, bool MIX> __device__ __forceinline__ void park(uint32_t tcol, uint32_t msl, int j, const float* v) {
+    constexpr int N = 2 * Elem<DT>::VEC;
+    if (MIX && j >= 2) {
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) sts16(msl + ((j - 2) * (N / 4) + i) * 512, v + 4 * i);
+    } else tmem_st<N>(tcol + j * N, v);
+}
+// (from TMEM: in the registers after tmem_wait_ld)
+template <int DT, bool MIX, int N> __device__ __forceinline__ void fetch(uint32_t tcol, uint32_t msl, int j, float (&v)[N]) {
+    if (MIX && j >= 2) {
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const float4 u = lds16f(msl + ((j - 2) * (N / 4) + i) * 512);
+            v[4 * i] = u.x; v[4 * i + 1] = u.y; v[4 * i + 2] = u.z; v[4 * i + 3] = u.w;
+        }
+    } else tmem_ld(tcol + j * N, v);
+}
+template <int N, bool TVM> __device__ __forceinline__ void resid(const float* p, const float* r, float4 rho, float2& tm, float2& sx) {
+    if (TVM) resid_aux_n<N>(p, r, rho.x, rho.y, &tm, &sx);
+    else resid_n<N, false>(p, r, rho.x, rho.y, &tm, nullptr);
+}
+// A full chunk of both rows (p0, p1: the lane's first vectors in the stages) and pass 2 of the task before in its place.
+// The logits are read twice from shared memory, for the largest and for the exponentials: kept in registers they
+// were spilled, and with all but 20 KB of the SM's memory taken as shared, spills go to L2.
+template <int DT, bool TVM, bool MIX>
+__device__ __forceinline__ void both_passes(uint32_t tcol, uint32_t msl, uint32_t p0, uint32_t p1, float c, float efp, float efq,
+                                            float4 rho, float2& ap, float2& aq, float2& tm, float2& sx) {
+    constexpr int VEC = Elem<DT>::VEC;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float v[2 * VEC], e[2 * VEC];
+        const uint4 x = lds16(p0 + j * 512), y = lds16(p1 + j * 512);
+        fetch<DT, MIX>(tcol, msl, j, v);
+        exp_vec<DT>(x, c, efp, e);
+        exp_vec<DT>(y, c, efq, e + VEC);
+        if (!(MIX && j >= 2)) tmem_wait_ld(v);
+        resid<VEC, TVM>(v, v + VEC, rho, tm, sx);
+        ap = add_pairs(ap, e, VEC);
+        aq = add_pairs(aq, e + VEC, VEC);
+        park<DT, MIX>(tcol, msl, j, e);
+    }
+}
+template <int DT, bool TVM>
+__device__ __forceinline__ void pass2(bool mix, uint32_t tcol, uint32_t msl, float4 rho, float2& tm, float2& sx) {
+    constexpr int VEC = Elem<DT>::VEC;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float v[2 * VEC];
+        if (mix && j >= 2) fetch<DT, true>(tcol, msl, j, v); else { fetch<DT, false>(tcol, msl, j, v); tmem_wait_ld(v); }
+        resid<VEC, TVM>(v, v + VEC, rho, tm, sx);
+    }
+}
+template <int DT>
+__device__ __forceinline__ void pass1(bool mix, bool keep, uint32_t tcol, uint32_t msl, const uint4* xp, const uint4* xq, float c, float efp, float efq,
+                                      float2& ap, float2& aq) {
+    constexpr int VEC = Elem<DT>::VEC;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float e[2 * VEC];
+        exp_vec<DT>(xp[j], c, efp, e);
+        exp_vec<DT>(xq[j], c, efq, e + VEC);
+        ap = add_pairs(ap, e, VEC);
+        aq = add_pairs(aq, e + VEC, VEC);
+        if (keep) { if (mix && j >= 2) park<DT, true>(tcol, msl, j, e); else park<DT, false>(tcol, msl, j, e); }
+    }
+}
+
 // A consumer warp.  Step n: pass 1 of its chunk of both rows of task n and pass 2 of task n - NSLOT, whose place task n
 // takes: a vector's exponentials are read before those of the new task are put there.  Both rows and both passes in one
 // step: the chains of dependent instructions around the arithmetic (barrier, description, largest logit, sums) are
@@ -466,11 +539,11 @@ template <> __device__ __forceinline__ float vecs_max<1>(const uint4* v) {
 template <int DT, bool TVM>
 __device__ __forceinline__ void consumer(const StreamArgs& a, SharedD<DT>& S, uint32_t data, int tid) {
     using D = Dims<DT>;
-    constexpr int VEC = D::VEC, NR = D::NR, NSLOT = D::NSLOT, TSLOT = D::TSLOT;
+    constexpr int VEC = D::VEC, NSLOT = D::NSLOT;
     const int lane = tid & 31, w = tid >> 5;
     const bool one = lane == 0;
-    // the warp's 128 columns of its quarter of the lanes
-    const uint32_t tbase = S.tmem_base + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 128);
+    // the warp's columns of its quarter of the lanes
+    const uint32_t tbase = S.tmem_base + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * D::WCOL);
     const uint32_t mine = data + (w * CV + lane) * 16;
     const uint32_t msl = data + RING + w * D::MWARP + lane * 16;
     const uint32_t full0 = smem_u32(S.full), empty0 = smem_u32(S.empty), task0 = smem_u32(S.task);
@@ -482,9 +555,9 @@ __device__ __forceinline__ void consumer(const StreamArgs& a, SharedD<DT>& S, ui
         bool live = n < n_end;
         const bool live2 = n >= NSLOT;
         const int m = n - NSLOT;
-        uint4 xp[4], xq[4];
         float c = 0.f;
         int meta = kStop;
+        uint32_t p0 = 0, p1 = 0, e0 = 0, e1 = 0;
         if (live) {
             if (!mbar_wait<S_FULL>(S, full0 + st * 8, par)) { if (one) give_up(a, S); return; }
             const uint4 d = lds16(task0 + (n % RT) * 16);
@@ -493,40 +566,12 @@ __device__ __forceinline__ void consumer(const StreamArgs& a, SharedD<DT>& S, ui
                 n_end = n; live = false;
                 if (one) for (int i = 0; i < NSTAT; ++i) mbar_arrive(&S.pdone[(n + i) % R8]);       // every stats warp meets the end
             } else {
-                const uint32_t s0 = st, p0 = mine + st * STAGE;
+                p0 = mine + st * STAGE; e0 = empty0 + st * 8;
                 if (++st == NSTG) { st = 0; par ^= 1u; }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) xp[j] = lds16(p0 + j * 512);
                 if (!mbar_wait<S_FULL>(S, full0 + st * 8, par)) { if (one) give_up(a, S); return; }
-                const uint32_t p1 = mine + st * STAGE;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) xq[j] = lds16(p1 + j * 512);
-                __syncwarp();
-                if (one) { mbar_arrive(empty0 + s0 * 8); mbar_arrive(empty0 + st * 8); }
+                p1 = mine + st * STAGE; e1 = empty0 + st * 8;
                 if (++st == NSTG) { st = 0; par ^= 1u; }
             }
-        }
-        const int left0 = live ? t_nv(meta) - w * CV : 0, left1 = live ? t_nv2(meta) - w * CV : 0;     // vectors from the chunk's first to the end of the slice
-        const bool any = left0 > 0;                              // (the second row is never the longer one)
-        const bool keep = any && t_kind(meta) == kPair;          // (a bonus task's exponentials are summed and not kept)
-        QExp Ep, Eq;
-        Ep.e = E_EMPTY; Ep.ef = 0.f; Eq.e = E_EMPTY; Eq.ef = 0.f;
-        if (any) {
-            if (left1 < CV || t_tail(meta)) {
-                // not a full chunk: vectors beyond the slice read as -inf, a row's ragged last vector loses the lanes beyond the vocabulary
-                const int lastn = a.r.V - (a.r.nvec - 1) * VEC;
-                const bool tp = t_tail(meta) && (t_kind(meta) == kPair || t_nv2(meta) == 0), tq = t_tail(meta);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int vi = j * 32 + lane;
-                    if (vi >= left0) xp[j] = neg_inf_vec<DT>();
-                    if (vi >= left1) xq[j] = neg_inf_vec<DT>();
-                    if (tp && vi == left0 - 1) mask_tail<DT>(xp[j], lastn);
-                    if (tq && vi == left1 - 1) mask_tail<DT>(xq[j], lastn);
-                }
-            }
-            Ep = chunk_exponent(vecs_max<DT>(xp), c);
-            Eq = chunk_exponent(vecs_max<DT>(xq), c);
         }
         int meta2 = kStop, us2 = 0;
         float4 rho = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -539,50 +584,50 @@ __device__ __forceinline__ void consumer(const StreamArgs& a, SharedD<DT>& S, ui
             if (two) rho = S.slot[slot].rho[w];
             tmem_wait_st();
         }
-        const bool tm_slot = D::MSLOT == 0 || slot < TSLOT;
-        const uint32_t tcol = tbase + slot * 2 * NR;
+        const int left0 = live ? t_nv(meta) - w * CV : 0, left1 = live ? t_nv2(meta) - w * CV : 0;     // vectors from the chunk's first to the end of the slice
+        const bool mix = D::MWARP != 0 && slot == NSLOT - 1;
+        const uint32_t tcol = tbase + slot * D::TCOL;
+        QExp Ep, Eq;
+        Ep.e = E_EMPTY; Ep.ef = 0.f; Eq.e = E_EMPTY; Eq.ef = 0.f;
         float2 ap = make_float2(0.f, 0.f), aq = ap, tm = ap, sx = ap;
+        if (two && left1 >= CV && t_kind(meta) == kPair && !t_tail(meta)) {
+            // the usual step, without a branch inside, so that the compiler deals the exponentials out among the rest
+            uint4 x[4], y[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float p[VEC], r[VEC], e[VEC], f[VEC];
-            if (two) {
-                if (tm_slot) {
-                    tmem_ld(tcol + j * VEC, p);
-                    tmem_ld(tcol + NR + j * VEC, r);
-                } else {
+            for (int j = 0; j < 4; ++j) x[j] = lds16(p0 + j * 512);
 #pragma unroll
-                    for (int i = 0; i < VEC / 4; ++i) {
-                        const float4 u = lds16f(msl + (j * (VEC / 4) + i) * 512), v = lds16f(msl + D::MWARP / 2 + (j * (VEC / 4) + i) * 512);
-                        p[4 * i] = u.x; p[4 * i + 1] = u.y; p[4 * i + 2] = u.z; p[4 * i + 3] = u.w;
-                        r[4 * i] = v.x; r[4 * i + 1] = v.y; r[4 * i + 2] = v.z; r[4 * i + 3] = v.w;
+            for (int j = 0; j < 4; ++j) y[j] = lds16(p1 + j * 512);
+            Ep = chunk_exponent(vecs_max<DT>(x), c);
+            Eq = chunk_exponent(vecs_max<DT>(y), c);
+            if (!mix) both_passes<DT, TVM, false>(tcol, msl, p0, p1, c, Ep.ef, Eq.ef, rho, ap, aq, tm, sx);
+            else both_passes<DT, TVM, true>(tcol, msl, p0, p1, c, Ep.ef, Eq.ef, rho, ap, aq, tm, sx);
+        } else {
+            if (two) pass2<DT, TVM>(mix, tcol, msl, rho, tm, sx);
+            if (left0 > 0) {                           // (the second row is never the longer one)
+                uint4 xp[4], xq[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { xp[j] = lds16(p0 + j * 512); xq[j] = lds16(p1 + j * 512); }
+                if (left1 < CV || t_tail(meta)) {
+                    // not a full chunk: vectors beyond the slice read as -inf, a row's ragged last vector loses the lanes beyond the vocabulary
+                    const int lastn = a.r.V - (a.r.nvec - 1) * VEC;
+                    const bool tp = t_tail(meta) && (t_kind(meta) == kPair || t_nv2(meta) == 0), tq = t_tail(meta);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int vi = j * 32 + lane;
+                        if (vi >= left0) xp[j] = neg_inf_vec<DT>();
+                        if (vi >= left1) xq[j] = neg_inf_vec<DT>();
+                        if (tp && vi == left0 - 1) mask_tail<DT>(xp[j], lastn);
+                        if (tq && vi == left1 - 1) mask_tail<DT>(xq[j], lastn);
                     }
                 }
+                Ep = chunk_exponent(vecs_max<DT>(xp), c);
+                Eq = chunk_exponent(vecs_max<DT>(xq), c);
+                pass1<DT>(mix, t_kind(meta) == kPair, tcol, msl, xp, xq, c, Ep.ef, Eq.ef, ap, aq);       // (a bonus task's exponentials are summed and not kept)
             }
-            if (any) {
-                exp_vec<DT>(xp[j], c, Ep.ef, e);
-                exp_vec<DT>(xq[j], c, Eq.ef, f);
-            }
-            if (two) {
-                if (tm_slot) tmem_wait_ld(p, r);
-                if (TVM) resid_aux_n<VEC>(p, r, rho.x, rho.y, &tm, &sx);
-                else resid_n<VEC, false>(p, r, rho.x, rho.y, &tm, nullptr);
-            }
-            if (any) {
-                ap = add_pairs(ap, e, VEC);
-                aq = add_pairs(aq, f, VEC);
-                if (keep) {
-                    if (tm_slot) {
-                        tmem_st<VEC>(tcol + j * VEC, e);
-                        tmem_st<VEC>(tcol + NR + j * VEC, f);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < VEC / 4; ++i) {
-                            sts16(msl + (j * (VEC / 4) + i) * 512, e + 4 * i);
-                            sts16(msl + D::MWARP / 2 + (j * (VEC / 4) + i) * 512, f + 4 * i);
-                        }
-                    }
-                }
-            }
+        }
+        if (live) {
+            __syncwarp();
+            if (one) { mbar_arrive(e0); mbar_arrive(e1); }
         }
         if (live) {
             const int2 s0 = warp_sum_words(ap.x + ap.y), s1 = warp_sum_words(aq.x + aq.y);
@@ -639,7 +684,8 @@ __device__ __noinline__ void stats_warp(const StreamArgs& a, SharedD<DT>& S, int
         if (t_kind(meta) == kStop) return;
         const bool pair = t_kind(meta) == kPair;
         Slot& sl = S.slot[n % Dims<DT>::NSLOT];
-        const int4 c = sl.part[row][chunk];
+        int4 c = sl.part[row][min(chunk, CH - 1)];
+        if (chunk >= CH) c = make_int4(kNoSum0, kNoSum1, E_EMPTY, 0);     // (lanes without a chunk)
         const long long ns = words_sum(c.x, c.y);
         const Part p0 = slice_part(ns, row ? E_EMPTY : c.z), p1 = slice_part(ns, row ? c.z : E_EMPTY);
         const bool two = t_nv2(meta) > 0;                   // a second record: the draft row's, or the bonus row's second slice's
@@ -658,7 +704,7 @@ __device__ __noinline__ void stats_warp(const StreamArgs& a, SharedD<DT>& S, int
         if (!pair) {
             const Part& p = row ? p1 : p0;
             const float m = c.z > E_EMPTY && !p.bad ? (float)ns * 9.094947017729282e-13f * pow2f(max(c.z - p.em, -127)) : 0.f;
-            if (row == 0 || two) st_relaxed_f(a.cm + (int64_t)(us + row) * CH + chunk, nonzero_f(m));
+            if (chunk < CH && (row == 0 || two)) st_relaxed_f(a.cm + (int64_t)(us + row) * CH + chunk, nonzero_f(m));
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.stats[n % R8]);
             __syncwarp();
@@ -670,7 +716,7 @@ __device__ __noinline__ void stats_warp(const StreamArgs& a, SharedD<DT>& S, int
         else { const Rows r = merge_rows_long(a, S, unit); rp = r.p; rq = r.q; }
         const Scale sc = scale_of(rp, rq);
         const int exq = __shfl_xor_sync(0xffffffffu, c.z, 16);
-        if (row == 0) sl.rho[chunk] = chunk_rho(sc, c.z, exq);
+        if (row == 0 && chunk < CH) sl.rho[chunk] = chunk_rho(sc, c.z, exq);
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.stats[n % R8]);
         if (lane < 2 && us == unit * a.T) {
