@@ -154,7 +154,8 @@ __device__ __forceinline__ double q_exp2(double t, const double* tab) {
     p = fma(f, p, 0.6931471805599453);                                  // ln2
     const double s = tab[n & 63];
     const double r = fma(s * f, p, s);
-    return t > -1000.0 ? __hiloint2double(__double2hiint(r) + ((n >> 6) << 20), __double2loint(r)) : 0.0;
+    const int keep = t > -1000.0 ? -1 : 0;                   // (a mask: as a choice of doubles it became a branch around all of the above)
+    return __hiloint2double((__double2hiint(r) + ((n >> 6) << 20)) & keep, __double2loint(r) & keep);
 }
 
 }  // namespace

@@ -14,14 +14,17 @@ struct alignas(16) FbRec {
     int kp;                             // 2 * draw row + (1 if the row is a residual of a target / draft pair)
     int ep, eq;                         // reference exponents of the target row and of the draft row
 };
-constexpr int kRedrawCut = 4;   // the fp64 re-draw cuts every row slice into so many work items
+// The fp64 re-draw cuts every row slice into so many work items: four, or eight where a row has few slices and four would
+// leave most SMs without one.
+constexpr int kRedrawCut = 4, kRedrawCutMax = 8;
+static inline int redraw_cut(int T) { return T <= 8 ? kRedrawCutMax : kRedrawCut; }
 constexpr size_t kRedrawTicketOffset = 192;   // unsigned: next work item of the fp64 re-draw (zeroed head of the workspace)
 constexpr size_t kFbCountOffset = 128;   // 8 bytes inside the zeroed head of the workspace: low int, sequences listed for the fp64
                                          // re-draw; high int, sequences whose draw is decided
 struct PipePlan {
     int T, slice_vecs;     // slices per row, vectors per slice (multiple of 16)
     size_t off_p1done, off_p2done, off_ddone, off_xdone, off_xsdone, off_fbrec, off_rowcnt, zero_bytes;
-    size_t off_xsum, off_xmass;   // fp64 re-draw: per listed sequence done counter; sums and masses per quarter slice
+    size_t off_xsum, off_xmass;   // fp64 re-draw: per listed sequence done counter; sums and masses per item
     size_t off_part, off_rstat, off_dpart, off_tvacc, off_sacc, off_sinfo, total;
 };
 
@@ -87,8 +90,8 @@ static inline PipePlan make_pipe_plan(int B, int K, int nvec, int dt, int slice_
     w.off_sacc = o;   o += align256(8 * (size_t)B * (K > 0 ? K : 1));
     w.off_sinfo = o;  o += align256(16 * (size_t)B);
     w.zero_bytes = o;
-    w.off_xsum = o;   o += align256(16 * (size_t)B * kRedrawCut * w.T);
-    w.off_xmass = o;  o += align256(8 * (size_t)B * kRedrawCut * w.T * 8);
+    w.off_xsum = o;   o += align256(16 * (size_t)B * redraw_cut(w.T) * w.T);
+    w.off_xmass = o;  o += align256(8 * (size_t)B * redraw_cut(w.T) * w.T);
     w.total = o;
     return w;
 }
@@ -111,8 +114,8 @@ static inline FusePlan make_fuse_plan(int B, int K, int nvec, int ups) {
     f.off_saux = o;   o += align256(8 * f.units * f.T);
     f.off_smass = o;  o += align256(8 * f.units * f.T);
     f.off_rows = o;   o += align256(32 * f.units);
-    f.off_xsum = o;   o += align256(16 * (size_t)B * kRedrawCut * wv.T);
-    f.off_xmass = o;  o += align256(8 * (size_t)B * kRedrawCut * wv.T * 8);
+    f.off_xsum = o;   o += align256(16 * (size_t)B * redraw_cut(wv.T) * wv.T);
+    f.off_xmass = o;  o += align256(8 * (size_t)B * redraw_cut(wv.T) * wv.T);
     f.total = o;
     return f;
 }

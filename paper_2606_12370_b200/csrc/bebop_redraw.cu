@@ -1,22 +1,29 @@
 // The fp64 re-draw of the sequences whose fast draw did not clear its error bound (its first kernel also turns
 // an expired device-side wait into a status bit), and the hook that times the main kernel.
-#include "bebop_pipe.cuh"
+#include "bebop_chunk.cuh"
 
 namespace bebop {
 
 namespace {
 
 // ------------------------------------------------------------------ fp64 re-draw of the listed sequences
-// One small kernel beside the pipelined kernel, for the few sequences whose fast draw did not clear its
-// error bound.  Every row is cut into XT = 4T quarter slices; the work items (listed sequence, quarter
-// slice) are taken from a counter by a grid that fits the device at once.  Everything is evaluated in double
+// One small kernel beside the pipelined and the fused kernel, for the few sequences whose fast draw did not clear its
+// error bound.  Every row is cut into nx items (a quarter or an eighth of a slice); the items (listed sequence,
+// place) are taken from a counter by a grid that fits the device at once.  Everything is evaluated in double
 // around the row exponents that phase A left (any common reference cancels in p = a / sum a).  An item is
-//   sum    exact normalisers: sum of exponentials of its quarter slice of the draw rows; then, once
-//          the sums of all quarter slices of the sequence are there (a counter per listed sequence),
-//   mass   residual mass of the quarter slice, one sum per warp (warp w owns the contiguous vectors
-//          [w*cw, (w+1)*cw)); the CTA that completes a sequence picks its token at once: quarter slice
-//          and warp chunk from the stored sums, then the few hundred tokens of that chunk are evaluated
-//          once more, one or two per thread, and scanned.
+//   sum    exact normalisers: the sum of exponentials of its vectors of the draw rows, which stay in shared
+//          memory; then, once the sums of all items of the sequence are there (a counter per listed sequence),
+//   mass   its residual mass; and once all masses are there,
+//   token  every CTA finds the item that owns the target, and the one that holds it goes on: the warp's chunk from
+//          the masses of its warps, the token from the exponentials.
+// What bounds it is a chain, met in full by the last listed sequence, when the main kernel has ended: the list, the
+// logits, two exchanges through L2 and the arithmetic of one thread.  So a thread's exponentials run side by side (as a
+// choice of doubles, the test for -inf had become a branch around each of them: 170 cycles apiece, one after the
+// other), and the token is found where the exponentials are, instead of by the last CTA to finish, which chose with one
+// thread and evaluated the chosen chunk again.  A call with re-drawn sequences (2 per cent of them) ends 5 to 8 us earlier:
+// 92.9 -> 84.4 us for 64 sequences of 32,000 bf16 logits, 212 -> 206 for 64 of 151,936.
+// A warp per 64 vectors instead of a CTA per item, 300 to 600 items a row, was slower (90 and 239 us): every warp then reads all
+// sums and masses, and all of them do the scans, in double, that one CTA's worth of warps does here.
 // The kernel is a programmatic dependent of the pipelined kernel that does NOT wait for that grid: its
 // CTAs move in as CTAs of the main kernel leave, and work through the list while it still grows (records
 // carry a mark; one word counts the listed sequences and the sequences whose draw is decided, which tells the
@@ -30,37 +37,14 @@ struct RedrawArgs {
     const FbRec* fb_list;    // records, valid once their b1 is non-zero
     int expect;              // sequences that get decided: the list is complete when the high half reaches it
     int* wait_failed;        // set by a device-side wait that gave up
-    double2* xsum;           // [B][XT] sums of exponentials (target row, draft row) per quarter slice
-    double* xmass;           // [B][XT][WW] residual mass per quarter slice and warp chunk
+    double2* xsum;           // [B][nx] sums of exponentials (target row, draft row) per item
+    double* xmass;           // [B][nx] residual mass per item
     int* xsdone;             // [B] per listed sequence: sum tasks finished
     int* xdone;              // [B] per listed sequence: mass tasks finished
     int expire;              // test hook: the wait for the list gives up at once
     unsigned* xticket;       // [1] next work item
-    int T, slice_vecs;
+    int nx, item_vecs;       // items per sequence, vectors of an item
 };
-
-// 2^t in double for t <= about 0: t = n/64 + f with |f| <= 1/128, 2^t = 2^(n >> 6) * tab[n & 63] * 2^f,
-// 2^f by its series to the fifth power (the next term is below 4e-17 of the result).  About a dozen
-// double-precision instructions, a third of the library routine; the result is within 2 ulp.
-// `tab` holds 2^(j/64), j = 0..63, in shared memory.  Arguments below -1000 (and -inf) give 0.
-constexpr int XTAB = 64;
-__device__ __forceinline__ void x_exp2_table(double* tab) {
-    if (threadIdx.x < XTAB) tab[threadIdx.x] = exp2((double)threadIdx.x * (1.0 / XTAB));
-}
-__device__ __forceinline__ double x_exp2(double t, const double* tab) {
-    const double magic = 6755399441055744.0;                 // 1.5 * 2^52: adding it rounds to an integer
-    const double tm = fma(t, (double)XTAB, magic);
-    const int n = __double2loint(tm);
-    const double f = fma(tm - magic, -1.0 / XTAB, t);         // exact
-    double p = fma(f, 0.0013333558146428443, 0.009618129107628477);     // ln2^5/120, ln2^4/24
-    p = fma(f, p, 0.05550410866482158);                                 // ln2^3/6
-    p = fma(f, p, 0.2402265069591007);                                  // ln2^2/2
-    p = fma(f, p, 0.6931471805599453);                                  // ln2
-    const double s = tab[n & (XTAB - 1)];
-    const double r = fma(s * f, p, s);
-    // branch-free: an argument of -inf runs through as NaN and is replaced here
-    return t > -1000.0 ? __hiloint2double(__double2hiint(r) + ((n >> 6) << 20), __double2loint(r)) : 0.0;
-}
 
 struct XRow {
     const char* prow; const char* qrow;
@@ -68,12 +52,11 @@ struct XRow {
     int b, k;
     bool pair;
 };
-__device__ __forceinline__ double x_resid(const XRow& d, float zp, float zq, const double* tab) {
-    // explicit roundings: a contracted p * ip - q would leave rounding dust when p == q
-    const double p = __dmul_rn(x_exp2(fma((double)zp, d.c, -d.ep), tab), d.ip);
-    if (!d.pair) return p;
-    const double q = __dmul_rn(x_exp2(fma((double)zq, d.c, -d.eq), tab), d.iq);
-    const double df = p - q;
+// explicit roundings: a contracted p * ip - q would leave rounding dust when p == q
+__device__ __forceinline__ double x_resid(const XRow& d, double ea, double eb, bool two) {
+    const double p = __dmul_rn(ea, d.ip);
+    if (!two) return p;
+    const double df = p - __dmul_rn(eb, d.iq);
     return df > 0.0 ? df : 0.0;
 }
 __device__ __forceinline__ void x_row(const RedrawArgs& a, int slot, XRow* d) {
@@ -99,7 +82,7 @@ __device__ __forceinline__ void x_load(const RedrawArgs& a, const XRow& d, int s
                                        float (*fq)[Elem<DT>::VEC]) {
     constexpr int VEC = Elem<DT>::VEC;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int qv = a.slice_vecs / kRedrawCut, cw = (qv + WW - 1) / WW;
+    const int qv = a.item_vecs, cw = (qv + WW - 1) / WW;
     const int v0 = s * qv, nv = max(min(qv, a.r.nvec - v0), 0);
 #pragma unroll
     for (int u = 0; u < XNU; ++u) {
@@ -112,32 +95,6 @@ __device__ __forceinline__ void x_load(const RedrawArgs& a, const XRow& d, int s
             if (d.pair) load_vec<DT>(d.qrow, v0 + vl, a.r.V, fq[u]);
         }
     }
-}
-
-struct PickShared {
-    double part[kRedrawCut * MAX_SLICES];     // slice masses of the sequence, later the warp masses of one slice
-    double redd[WW];
-    double base, target;
-    int last, sel, chunk, tok_first, tok_last;
-};
-
-// first entry with mass whose running sum reaches t (running sum starts at *C); by rounding none may:
-// then the last entry with mass.  Leaves in *C the sum before the chosen entry.
-__device__ __forceinline__ int pick_entry(const double* m, int n, double t, double* C) {
-    const double c0 = *C;
-    double run = c0;
-    int last = 0;
-    for (int i = 0; i < n; ++i) {
-        if (m[i] > 0.0) {
-            if (run + m[i] >= t) { *C = run; return i; }
-            last = i;
-        }
-        run += m[i];
-    }
-    run = c0;
-    for (int i = 0; i < last; ++i) run += m[i];
-    *C = run;
-    return last;
 }
 
 __device__ __forceinline__ unsigned long long x_ld_count(const unsigned long long* p) {
@@ -166,17 +123,16 @@ __device__ __forceinline__ int x_wait_slot(const RedrawArgs& a, int slot) {
 template <int DT>
 __global__ void __launch_bounds__(WT) k_redraw(const RedrawArgs a) {
     constexpr int VEC = Elem<DT>::VEC;
-    __shared__ PickShared S;
-    __shared__ double sh[2][WW];
-    __shared__ double tab[XTAB];
+    __shared__ double shs[2][WW], shm[WW];          // sums and masses of the warps' chunks
+    __shared__ double tab[64];
     __shared__ int go;
     __shared__ unsigned item_sh;
     extern __shared__ double xe[];       // [2][XNU * VEC][WT] exponentials of this item's elements (target row, draft row)
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    x_exp2_table(tab);
-    const int K = R.K, XT = kRedrawCut * a.T;
-    const int qv = a.slice_vecs / kRedrawCut, cw = (qv + WW - 1) / WW;
+    if (tid < 64) tab[tid] = g_pow2_64[tid];
+    const int K = R.K, XT = a.nx;
+    const int qv = a.item_vecs, cw = (qv + WW - 1) / WW;
     const long items_max = (long)R.B * XT;
     __syncthreads();
     // Work items are taken in order from a ticket counter, so the CTAs that are on the device work on the oldest
@@ -199,175 +155,135 @@ __global__ void __launch_bounds__(WT) k_redraw(const RedrawArgs a) {
         XRow d;
         x_row(a, slot, &d);
         const int b = d.b;
-        // ---- sum of exponentials of this quarter slice
+        const float uf = a.u_final[b];
+        // ---- sums of exponentials of this item
         {
             float fp[XNU][VEC], fq[XNU][VEC];
             x_load<DT>(a, d, s, fp, fq);
             double sa = 0.0, sb = 0.0;
 #pragma unroll
             for (int u = 0; u < XNU; ++u) {
+                if (32 * u >= cw) break;
 #pragma unroll
                 for (int i = 0; i < VEC; ++i) {
-                    const double ea = x_exp2(fma((double)fp[u][i], d.c, -d.ep), tab);
+                    const double ea = q_exp2(fma((double)fp[u][i], d.c, -d.ep), tab);
                     sa += ea;
+                    // kept for the masses and for the token, which then need neither the rows nor the exponentials again
+                    xe[(u * VEC + i) * WT + tid] = ea;
                     if (d.pair) {
-                        const double eb = x_exp2(fma((double)fq[u][i], d.c, -d.eq), tab);
+                        const double eb = q_exp2(fma((double)fq[u][i], d.c, -d.eq), tab);
                         sb += eb;
-                        // kept for the mass pass, which then needs neither the rows nor the exponentials again
-                        xe[(u * VEC + i) * WT + tid] = ea;
                         xe[((XNU + u) * VEC + i) * WT + tid] = eb;
                     }
                 }
             }
             sa = warp_sum(sa); sb = warp_sum(sb);
-            if (lane == 0) { sh[0][warp] = sa; sh[1][warp] = sb; }
+            if (lane == 0) { shs[0][warp] = sa; shs[1][warp] = sb; }
             __syncthreads();
             if (tid == 0) {
                 double ta = 0.0, tb = 0.0;
-                for (int w = 0; w < WW; ++w) { ta += sh[0][w]; tb += sh[1][w]; }
+                for (int w = 0; w < WW; ++w) { ta += shs[0][w]; tb += shs[1][w]; }
                 a.xsum[(int64_t)b * XT + s] = make_double2(ta, tb);
                 __threadfence();
                 atomicAdd(a.xsdone + slot, 1);
-                // ... and wait (bounded) for the other quarter slices of the sequence
+                // ... and wait (bounded) for the other items of the sequence
                 go = spin_ge(a.xsdone + slot, XT) ? 1 : 0;
             }
             __syncthreads();
-            const int ok = go;
-            __syncthreads();
-            if (!ok) {
-                if (tid == 0) { atomicExch(a.wait_failed, 1); if (a.o.row_status) atomicOr(a.o.row_status + b, ST_WAIT); }
-                continue;
-            }
         }
-        // exact normalisers: every warp adds the quarter-slice sums in the same order (lane t takes sums t,
+        bool ok = go != 0;
+        // exact normalisers: every warp adds the items' sums in the same order (lane t takes sums t,
         // t + 32, ...; the butterfly leaves the same bits in every lane), so every CTA gets the same value
         double Sa = 0.0, Sb = 0.0;
-        for (int t = lane; t < XT; t += 32) { const double2 x = __ldcg(a.xsum + (int64_t)b * XT + t); Sa += x.x; Sb += x.y; }
+        if (ok) for (int t = lane; t < XT; t += 32) { const double2 x = __ldcg(a.xsum + (int64_t)b * XT + t); Sa += x.x; Sb += x.y; }
         Sa = warp_sum(Sa); Sb = warp_sum(Sb);
         d.ip = 1.0 / Sa; d.iq = d.pair ? 1.0 / Sb : 0.0;
-        if (d.pair) {     // a bonus row needs no mass pass: its masses are sums of exponentials over Sa
+        if (ok && d.pair) {     // a bonus row needs no mass pass: its masses are sums of exponentials over Sa
             double m = 0.0;
 #pragma unroll
-            for (int j = 0; j < XNU * VEC; ++j) {
-                // as x_resid, from the stored exponentials (explicit roundings: see there)
-                const double p = __dmul_rn(xe[j * WT + tid], d.ip);
-                const double q = __dmul_rn(xe[(XNU * VEC + j) * WT + tid], d.iq);
-                const double df = p - q;
-                m += df > 0.0 ? df : 0.0;
+            for (int u = 0; u < XNU; ++u) {
+                if (32 * u >= cw) break;
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) m += x_resid(d, xe[(u * VEC + i) * WT + tid], xe[((XNU + u) * VEC + i) * WT + tid], true);
             }
             m = warp_sum(m);
-            if (lane == 0) a.xmass[((int64_t)b * XT + s) * WW + warp] = m;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();
-            S.last = atomicAdd(a.xdone + slot, 1) == XT - 1;
-        }
-        __syncthreads();
-        if (!S.last) continue;
-        __threadfence();
-
-        // ---- pick.  Stage 1: quarter slice from the slice masses.
-        bool zero_resid = false;
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int t = tid; t < XT; t += WT) {
-                double m = 0.0;
-                if (d.pair) { for (int w = 0; w < WW; ++w) m += __ldcg(a.xmass + ((int64_t)b * XT + t) * WW + w); }
-                else m = __ldcg(a.xsum + (int64_t)b * XT + t).x * d.ip;
-                S.part[t] = m;
-            }
+            if (lane == 0) shm[warp] = m;
             __syncthreads();
             if (tid == 0) {
-                double Z = 0.0;
-                for (int t = 0; t < XT; ++t) Z += S.part[t];
-                S.base = Z;
+                double t = 0.0;
+                for (int w = 0; w < WW; ++w) t += shm[w];
+                a.xmass[(int64_t)b * XT + s] = t;
+                __threadfence();
+                atomicAdd(a.xdone + slot, 1);
+                go = spin_ge(a.xdone + slot, XT) ? 1 : 0;
             }
             __syncthreads();
-            if (S.base > 0.0 || !d.pair) break;
-            // residual mass vanished at a rejected position: draw from p of that position
-            d.pair = false; zero_resid = true;
-            __syncthreads();
+            ok = go != 0;
         }
-        if (tid == 0) {
-            if (zero_resid && a.o.row_status) {
+        if (!ok) {
+            if (tid == 0) { atomicExch(a.wait_failed, 1); if (a.o.row_status) atomicOr(a.o.row_status + b, ST_WAIT); }
+            __syncthreads();
+            continue;
+        }
+        // ---- the item.  Every warp chooses, from the same numbers in the same order, and the CTA that holds the chosen item
+        // goes on.  (The last CTA to finish chose before, by one thread, and evaluated the chosen chunk again.)
+        bool two = d.pair, hit;
+        const int per = (XT + 31) / 32, t0 = min(lane * per, XT), t1 = min(t0 + per, XT);
+        auto mass = [&](int t) { return two ? __ldcg(a.xmass + (int64_t)b * XT + t) : __ldcg(a.xsum + (int64_t)b * XT + t).x * d.ip; };
+        double base, tot, t;
+        int ol;
+        for (;;) {
+            double mine = 0.0;
+            for (int i = t0; i < t1; ++i) mine += mass(i);
+            t = (double)uf * warp_sum(mine);
+            ol = pick_lane(mine, 0.0, t, &base, &tot, &hit);
+            if (ol >= 0 || !two) break;
+            two = false;                                // residual mass vanished at a rejected position: draw from p of that position
+        }
+        ol = max(ol, 0);
+        int qs = ol * per; double cb = base;
+        if (per > 1) {
+            const int src = pick_lane(lane < per && ol * per + lane < XT ? mass(ol * per + lane) : 0.0, base, t, &cb, &tot, &hit);
+            if (src >= 0) qs = ol * per + src;
+        }
+        if (qs == s) {
+            if (tid == 0 && two != d.pair && a.o.row_status) {
                 // the main kernel writes this row's status word once, with a plain store: add the bit only when
                 // that grid is through (rare, and then a wait of some microseconds at most)
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 atomicOr(a.o.row_status + b, ST_ZERO_RESID);
             }
-            const double t = (double)a.u_final[b] * S.base;
-            double C = 0.0;
-            S.sel = pick_entry(S.part, XT, t, &C);
-            S.target = t; S.base = C;
-        }
-        __syncthreads();
-        const int qs = S.sel;
-        // Stage 2: warp chunk inside the quarter slice (residual: stored; plain softmax row: evaluated now)
-        const int p0 = qs * qv, pn = max(min(qv, R.nvec - p0), 0);
-        double wm = 0.0;
-        if (!d.pair) {
+            // ---- the chunk, and the token in it: the first with mass whose running sum reaches the target; by rounding none
+            // may: then the last with mass
+            double c0;
+            const int wsel = max(pick_lane(lane < WW ? (two ? shm[lane] : shs[0][lane] * d.ip) : 0.0, cb, t, &c0, &tot, &hit), 0);
+            if (warp == wsel) {
+                int y = INT_MAX, last = -1;
+#pragma unroll 1
+                for (int u = 0; u < XNU; ++u) {
+                    const bool in = lane + 32 * u < cw && 32 * u < cw;
+                    double r[VEC], vs = 0.0;
 #pragma unroll
-            for (int u = 0; u < XNU; ++u) {
-                const int vl = warp * cw + lane + 32 * u;
-                if (lane + 32 * u < cw && vl < pn) {
-                    float f[VEC];
-                    load_vec<DT>(d.prow, p0 + vl, R.V, f);
+                    for (int i = 0; i < VEC; ++i) {
+                        r[i] = in ? x_resid(d, xe[(u * VEC + i) * WT + tid], xe[((XNU + u) * VEC + i) * WT + tid], two) : 0.0;
+                        vs += r[i];
+                    }
+                    double incl = vs;
 #pragma unroll
-                    for (int i = 0; i < VEC; ++i) wm += x_resid(d, f[i], 0.f, tab);
+                    for (int o = 1; o < 32; o <<= 1) { const double t2 = shfl_up_d(incl, o); if (lane >= o) incl += t2; }
+                    double C = c0 + (incl - vs);
+                    const int v = s * qv + warp * cw + lane + 32 * u;
+#pragma unroll
+                    for (int i = 0; i < VEC; ++i) {
+                        if (r[i] > 0.0) { last = v * VEC + i; if (y == INT_MAX && C + r[i] >= t) y = last; }
+                        C += r[i];
+                    }
+                    c0 += __shfl_sync(0xffffffffu, incl, 31);
                 }
-            }
-            wm = warp_sum(wm);
-        }
-        __syncthreads();                                   // S.part is about to be overwritten
-        if (lane == 0) S.part[warp] = d.pair ? __ldcg(a.xmass + ((int64_t)b * XT + qs) * WW + warp) : wm;
-        __syncthreads();
-        if (tid == 0) {
-            double C = S.base;
-            S.chunk = pick_entry(S.part, WW, S.target, &C);
-            S.base = C;
-            S.tok_first = 0x7fffffff; S.tok_last = -1;
-        }
-        __syncthreads();
-        // Stage 3: the tokens of the chunk, `per` consecutive tokens per thread, scanned in token order
-        const int e0 = (p0 + S.chunk * cw) * VEC;                                 // first token of the chunk
-        const int e1 = min(min((p0 + min((S.chunk + 1) * cw, pn)) * VEC, R.V), e0 + 4 * WT);
-        const int per = (max(e1 - e0, 0) + WT - 1) / WT;                          // <= 2 (cw <= 64 vectors of 8)
-        double r[4] = {0.0, 0.0, 0.0, 0.0};
-        double mine = 0.0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int v = e0 + tid * per + i;
-            if (i < per && v < e1) {
-                const float zp = load_one<DT>(d.prow, v);
-                const float zq = d.pair ? load_one<DT>(d.qrow, v) : 0.f;
-                r[i] = x_resid(d, zp, zq, tab);
-                mine += r[i];
+                y = __reduce_min_sync(0xffffffffu, y); last = __reduce_max_sync(0xffffffffu, last);
+                if (lane == 0) a.o.out_tokens[(int64_t)b * (K + 1) + d.k] = y != INT_MAX ? y : last;
             }
         }
-        double incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const double t2 = shfl_up_d(incl, o); if (lane >= o) incl += t2; }
-        if (lane == 31) S.redd[warp] = incl;
-        __syncthreads();
-        double C = S.base;
-        for (int w = 0; w < warp; ++w) C += S.redd[w];
-        C += incl - mine;
-        const double t = S.target;
-        // the first token with mass whose prefix sum reaches the target; by rounding none may: then the
-        // last token with mass
-        int y = -1, lastpos = -1;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (r[i] > 0.0) {
-                lastpos = e0 + tid * per + i;
-                if (y < 0 && C + r[i] >= t) y = lastpos;
-            }
-            C += r[i];
-        }
-        if (y >= 0) atomicMin(&S.tok_first, y);
-        if (lastpos >= 0) atomicMax(&S.tok_last, lastpos);
-        __syncthreads();
-        if (tid == 0) a.o.out_tokens[(int64_t)b * (K + 1) + d.k] = S.tok_first != 0x7fffffff ? S.tok_first : S.tok_last;
         __syncthreads();
     }
     // Every CTA waits here for the main grid, whatever the caller asked for: a dependent of a grid that lets its
@@ -422,12 +338,13 @@ cudaError_t redraw_launch(const RowArgs& a, const float* u_final, VerifyOut o, c
     ra.xsdone = reinterpret_cast<int*>(w + wp.off_xsdone);
     ra.xdone = reinterpret_cast<int*>(w + wp.off_xdone);
     ra.xticket = reinterpret_cast<unsigned*>(w + kRedrawTicketOffset);
-    ra.T = wp.T; ra.slice_vecs = wp.slice_vecs;
-    // CTAs of this grid wait for one another (the sums of a sequence come from kRedrawCut * T of them), so
+    const int cut = redraw_cut(wp.T);
+    ra.nx = cut * wp.T; ra.item_vecs = wp.slice_vecs / cut;
+    // CTAs of this grid wait for one another (the sums of a sequence come from nx of them), so
     // the grid is at most what fits the device at once; a CTA takes work items from a counter.
     const int cap = a.dt == 0 ? redraw_grid<0>() : redraw_grid<1>();
     if (cap < 1) return cudaErrorLaunchOutOfResources;
-    const long items_max = (long)a.B * kRedrawCut * wp.T;
+    const long items_max = (long)a.B * ra.nx;
     const int grid = (int)(items_max < cap ? items_max : cap);
     // scheduled as soon as the main kernel lets go of SMs; it does not wait for that grid as a whole
     cudaLaunchAttribute attr[1];
