@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbebop.so")
 HOST = os.path.join(HERE, "_bebop_host.so")
 SOURCES = ["bebop_api.cu", "bebop_general.cu", "bebop_redraw.cu", "bebop_pipe.cu", "bebop_fuse.cu",
-           "bebop_seq.cu", "bebop_stream.cu"]
+           "bebop_seq.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-shared"]

@@ -118,10 +118,6 @@ bebop_status_t bebop_verify(const void* target_logits, int64_t ld_target, const 
         e = seq_verify(a, draft_tokens, u_accept, u_final, o, stream, &launched);
         if (launched) g_last_kernel = 3;
     }
-    if (e == cudaSuccess && !launched && g_path == 5 && stream_supported(a)) {
-        e = stream_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
-        if (launched) g_last_kernel = 5;
-    }
     if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, false))) && fuse_supported(a)) {
         e = fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
         if (launched) g_last_kernel = 3;
@@ -158,10 +154,6 @@ bebop_status_t bebop_tv(const void* target_logits, int64_t ld_target, const void
     if ((g_path == 4 && seq_supported(a, true)) || (g_path == 0 && seq_preferred(a, true))) {
         e = seq_verify(a, nullptr, nullptr, nullptr, o, stream, &launched, true, s_aux);
         if (launched) g_last_kernel = 3;
-    }
-    if (e == cudaSuccess && !launched && g_path == 5 && stream_supported(a)) {
-        e = stream_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
-        if (launched) g_last_kernel = 5;
     }
     if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, true))) && fuse_supported(a)) {
         e = fuse_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);

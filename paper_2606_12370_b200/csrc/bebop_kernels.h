@@ -73,12 +73,6 @@ cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
 
-// Streaming kernel (bebop_stream.cu): every row read and exponentiated once, one launch; same contract as pipe_verify.
-bool stream_supported(const RowArgs& a);
-cudaError_t stream_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
-                          const float* u_accept, const float* u_final, VerifyOut o, char* ws,
-                          cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
-
 // Sequence kernel (bebop_seq.cu): a thread-block cluster per sequence (row pair), its logits in the cluster's shared memory;
 // one launch, no workspace; same contract.
 bool seq_supported(const RowArgs& a, bool tv_only);

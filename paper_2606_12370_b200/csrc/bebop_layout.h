@@ -120,36 +120,6 @@ static inline FusePlan make_fuse_plan(int B, int K, int nvec, int ups) {
     return f;
 }
 
-// Workspace of the streaming kernel (bebop_stream.cu).  A unit is a row pair or a bonus row; a sequence owns `ups`
-// consecutive units (K + 1 for bebop_verify, 1 for bebop_tv); every unit is cut into T slices of kStreamWarps chunks.
-constexpr int kStreamWarps = 12, kStreamChunkVecs = 128;
-constexpr int kStreamSliceVecs = kStreamWarps * kStreamChunkVecs;
-constexpr int kStreamMaxSlices = 128;
-struct StreamPlan {
-    int T, slice_vecs, nx;        // nx: items of the fp64 re-draw per sequence
-    // cleared per call: head (wait flag, counters of the re-draw), its list, slice records, merged rows, chunk masses
-    size_t off_fbrec, off_rec, off_rows, off_cm, off_ca, zero_bytes;
-    size_t off_xsum, off_xmass, total;
-};
-static inline StreamPlan make_stream_plan(int B, int nvec, int ups) {
-    StreamPlan f;
-    f.T = (nvec + kStreamSliceVecs - 1) / kStreamSliceVecs; if (f.T < 1) f.T = 1;
-    f.slice_vecs = ((nvec + f.T - 1) / f.T + kStreamChunkVecs - 1) / kStreamChunkVecs * kStreamChunkVecs;   // whole chunks
-    f.nx = (nvec + 63) / 64;
-    const size_t units = (size_t)B * (size_t)ups, chunks = (size_t)f.T * kStreamWarps;
-    size_t o = 256;
-    f.off_fbrec = o;  o += align256(16 * (size_t)B);
-    f.off_rec = o;    o += align256(32 * units * f.T);
-    f.off_rows = o;   o += align256(32 * units);
-    f.off_cm = o;     o += align256(4 * units * chunks);
-    f.off_ca = o;     if (ups == 1) o += align256(4 * units * chunks);
-    f.zero_bytes = o;
-    f.off_xsum = o;   if (ups > 1) o += align256(16 * (size_t)B * f.nx);
-    f.off_xmass = o;  if (ups > 1) o += align256(8 * (size_t)B * f.nx);
-    f.total = o;
-    return f;
-}
-
 static inline Plan make_plan(int B, int K, int V, int dt) {
     Plan p;
     p.B = B; p.K = K; p.V = V; p.dt = dt;
@@ -182,11 +152,7 @@ static inline Plan make_plan(int B, int K, int V, int dt) {
         const size_t wp = make_pipe_plan(B, K, p.nvec, dt).total, wf = make_fuse_plan(B, K, p.nvec, K + 1).total;
         p.off_pipe = o;
         p.off_fuse = o;
-        size_t m = wp > wf ? wp : wf;
-        // (bebop_tv of B rows: K = 1 and one unit per row)
-        const size_t w1 = make_stream_plan(B, p.nvec, K + 1).total, w2 = K == 1 ? make_stream_plan(B, p.nvec, 1).total : 0;
-        m = m > w1 ? m : w1; m = m > w2 ? m : w2;
-        o = align256(o + m);
+        o = align256(o + (wp > wf ? wp : wf));
     }
     p.total = o;
     return p;
