@@ -29,7 +29,7 @@
 //
 // Every wait is bounded; a wait that gives up sets the wait flag (status bit 32 of every row).
 // No multicast, no cluster: each CTA copies from this GPU's own memory.
-#include "bebop_pipe.cuh"
+#include "bebop_chunk.cuh"
 
 namespace bebop {
 
@@ -61,6 +61,7 @@ struct __align__(16) TaskDesc {
     float tau;        // temperature, and c = log2(e) / tau computed once per row
     float c;
     RowScale P, Q;
+    float2 rho;       // P2, D: S_p / S_q as two floats
     int need;         // P2: partials the sequence's second sweep delivers in all (the last one starts the draw's set-up)
     float bound;      // D: the error bound the draw must clear,
     double tt, base;  //    the target of the inverse CDF and the mass before the half slice in the stage
@@ -73,6 +74,7 @@ struct DrawTask {
     float bound, c;
     int b, k, owner, pair;
     RowScale P, Q;
+    float2 rho;
 };
 constexpr int kMbox = 16;                    // mailbox entries: more than the tasks a CTA can have unpublished
 static_assert(kMbox >= kBatch + NST + 1, "a run's tasks plus the ring may each complete a sequence before the producer looks");
@@ -97,24 +99,12 @@ struct PipeShared {
     float d1_sq[2 * MAX_SLICES];
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* b, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(b)), "r"(count) : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(b)) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect(unsigned long long* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(b)), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity) {
     const uint32_t addr = smem_u32(b);
-    for (uint32_t i = 0; i < kBarSpin; ++i) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
-        if (ok) return true;
-    }
+    for (uint32_t i = 0; i < kBarSpin; ++i) if (mbar_try(addr, parity)) return true;
     return false;
 }
 // contiguous copy global -> shared of this CTA; 16-byte aligned on both sides, size a multiple of 16
@@ -250,7 +240,7 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
             TaskDesc d;
             d.phase = 3; d.b = t.b; d.r = t.k; d.s = t.owner; d.flags = (t.pair ? 1 : 0) | 2;
             d.v0 = t.owner * sv2; d.nv = max(min(sv2, R.nvec - d.v0), 0);
-            d.tau = 1.f; d.c = t.c; d.P = t.P; d.Q = t.Q; d.need = 0;
+            d.tau = 1.f; d.c = t.c; d.P = t.P; d.Q = t.Q; d.rho = t.rho; d.need = 0;
             d.bound = t.bound; d.tt = t.tt; d.base = t.base;
             issue(d, row_ptr(R, t.b, t.k), t.pair ? row_ptr(R, t.b, K + 1 + t.k) : nullptr, pol_drop);
         }
@@ -310,7 +300,7 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
             // the row's numbers
             TaskDesc d;
             d.phase = ph; d.b = b; d.r = r; d.s = 0; d.v0 = 0; d.nv = 0; d.flags = 0; d.tau = 1.f; d.c = 0.f;
-            d.P = no_row(); d.Q = no_row();
+            d.P = no_row(); d.Q = no_row(); d.rho = make_float2(0.f, 0.f);
             d.need = 0; d.bound = 0.f; d.tt = 0.0; d.base = 0.0;
             const char* row0 = nullptr; const char* row1 = nullptr;
             bool skip = false;
@@ -346,7 +336,7 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
                 if (!skip) {
                     d.flags = (pair ? 1 : 0) | (drawrow ? 2 : 0);
                     d.P = row_scale(sp);
-                    if (pair) d.Q = row_scale(sq);
+                    if (pair) { d.Q = row_scale(sq); d.rho = row_rho(sp, sq); }
                     row0 = row_ptr(R, b, k);
                     if (pair) row1 = row_ptr(R, b, K + 1 + k);
                 }
@@ -489,6 +479,45 @@ __device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long
     asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
 }
 
+// the largest logit of N vectors (NaN if there is one); bf16: packed maxima, unpacked once
+template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* v) {
+    if (DT == 1) {
+        uint32_t a[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) a[j] = max_nan_bf16x2(max_nan_bf16x2(v[j].x, v[j].y), max_nan_bf16x2(v[j].z, v[j].w));
+#pragma unroll
+        for (int j = 1; j < N; ++j) a[0] = max_nan_bf16x2(a[0], a[j]);
+        return max_nan(__uint_as_float(a[0] << 16), __uint_as_float(a[0] & 0xffff0000u));
+    }
+    float m = vec_max<DT>(v[0]);
+#pragma unroll
+    for (int j = 1; j < N; ++j) m = max_nan(m, vec_max<DT>(v[j]));
+    return m;
+}
+// Residuals from the exponentials of a row pair: r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q as two floats
+// (equal rows give rho = 1 and r' = 0 exactly); as e_p <= 1, saturating to [0, 1] is taking the maximum with 0.  Two
+// instructions a token, where p, q, their difference and its maximum with 0 took four.
+template <int N> __device__ __forceinline__ void resid_n(const float* p, const float* q, float2 rho, float* r) {
+    const float2 nl = make_float2(-rho.y, -rho.y);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        const float2 t = __ffma2_rn(nl, make_float2(q[i], q[i + 1]), make_float2(p[i], p[i + 1]));
+        r[i] = fma_sat(-rho.x, q[i], t.x); r[i + 1] = fma_sat(-rho.x, q[i + 1], t.y);
+    }
+}
+// ... their sum, and the sum of e_q over the tokens with q <= p: the mask 1[d >= 0] serves both
+template <int N> __device__ __forceinline__ void resid_aux_n(const float* p, const float* q, float2 rho, float2* z, float2* x) {
+    const float2 nh = make_float2(-rho.x, -rho.x), nl = make_float2(-rho.y, -rho.y);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        const float2 q2 = make_float2(q[i], q[i + 1]);
+        const float2 d = __ffma2_rn(nh, q2, __ffma2_rn(nl, q2, make_float2(p[i], p[i + 1])));
+        const float2 mk = make_float2(d.x >= 0.f ? 1.f : 0.f, d.y >= 0.f ? 1.f : 0.f);
+        *z = __ffma2_rn(d, mk, *z);
+        *x = __ffma2_rn(q2, mk, *x);
+    }
+}
+
 // P1: softmax partial (E, S) of one slice of one row, from shared memory.
 template <int DT>
 __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const TaskDesc& d, const unsigned char* data,
@@ -496,7 +525,6 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
     constexpr int VEC = Elem<DT>::VEC, NV = PSLICE / PC;
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    TempScale ts; ts.hi = d.c;
     const int nv = d.nv;
     uint4 raw[NV];
     if (nv >= (NV - 1) * PC) {                   // the usual case: only a thread's last vector may lie beyond the slice
@@ -519,36 +547,23 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
             if (tid + u * PC < nv && gbase + VEC > R.V) mask_tail<DT>(raw[u], R.V - gbase);
         }
     }
-    float m = vec_max<DT>(raw[0]);
+    // one exponent per warp, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time, four running sums
+    const QExp E = chunk_exponent(vecs_max<DT, NV>(raw), d.c);
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
-    for (int u = 1; u < NV; ++u) m = max_nan(m, vec_max<DT>(raw[u]));
-    const bool bad = m != m || m == INFINITY;
-    int E = E_EMPTY;
-    float Ef = 0.f;
-    if (!bad && m != -INFINITY) E = ref_exponent(m, ts, &Ef);
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    if (E > E_EMPTY) {
+    for (int u = 0; u < NV; ++u) {
+        float e[VEC];
+        exp_vec<DT>(raw[u], d.c, E.ef, e);
 #pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            float f[VEC];
-            unpack<DT>(raw[u], f);
-#pragma unroll
-            for (int i = 0; i < VEC; i += 4) {
-                s0 += exp2_scaled(f[i], ts, Ef);
-                s1 += exp2_scaled(f[i + 1], ts, Ef);
-                s2 += exp2_scaled(f[i + 2], ts, Ef);
-                s3 += exp2_scaled(f[i + 3], ts, Ef);
-            }
+        for (int i = 0; i < VEC; i += 4) {
+            s0 = __fadd2_rn(s0, make_float2(e[i], e[i + 1]));
+            s1 = __fadd2_rn(s1, make_float2(e[i + 2], e[i + 3]));
         }
     }
-    // thread -> warp, exact power-of-two rescaling, sums in a fixed order
-    float st = (s0 + s1) + (s2 + s3);
-    const int Ew = redux_max(E);
-    st = E > E_EMPTY ? st * pow2f(max(E - Ew, -126)) : 0.f;
-    st = warp_sum(st);
-    const unsigned anybad = __ballot_sync(0xffffffffu, bad);
-    float mw = ord2f(redux_max(f2ord(bad ? -INFINITY : m)));
-    if (anybad) mw = __int_as_float(0x7fc00000);
+    const bool bad = E.e == E_BAD;
+    const int Ew = bad ? E_EMPTY : E.e;
+    const float st = Ew > E_EMPTY ? warp_sum((s0.x + s1.x) + (s0.y + s1.y)) : 0.f;
+    const float mw = bad ? __int_as_float(0x7fc00000) : 0.f;
     if (lane == 0) { S.wf[stage][0][warp] = st; S.wi[stage][warp] = Ew; S.wf[stage][1][warp] = mw; }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
@@ -630,8 +645,9 @@ __device__ __forceinline__ void pipe_p2(const PipeArgs& a, PipeShared& S, const 
             if (v < nv) { rp[u] = lds16(data + (size_t)v * 16); if (pair) rq[u] = lds16(qdata + (size_t)v * 16); }
         }
     }
-    TempScale c; c.hi = d.c;
     const RowScale SP = d.P, SQ = d.Q;
+    const float2 rho = d.rho;
+    const double ip = (double)SP.inv + (double)SP.inv_lo;
     if ((d.v0 + nv) * VEC > R.V) {
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
@@ -639,50 +655,54 @@ __device__ __forceinline__ void pipe_p2(const PipeArgs& a, PipeShared& S, const 
             if (tid + u * PC < nv && gbase + VEC > R.V) { mask_tail<DT>(rp[u], R.V - gbase); mask_tail<DT>(rq[u], R.V - gbase); }
         }
     }
-    float z0 = 0.f, z1 = 0.f, sqs = 0.f;
-    double zd = 0.0;
+    // residuals in units of 1 / S_p, which is applied to the warp's sums
+    float2 z2 = make_float2(0.f, 0.f), a2 = z2, b2 = z2;
+    float sqs = 0.f;
+    double z, zd = 0.0;
     if (TVO && a.sacc) {
         // bebop_tv with the auxiliary sum: TV and S = sum of q over the tokens with q <= p (Eq. tv_grad)
-        float sx = 0.f;
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            float fp[VEC], fq[VEC];
-            unpack<DT>(rp[u], fp);
-            unpack<DT>(rq[u], fq);
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                const float p = __fmul_rn(exp2_scaled(fp[i], c, SP.ef), SP.inv);
-                const float q = __fmul_rn(exp2_scaled(fq[i], c, SQ.ef), SQ.inv);
-                z0 += fmaxf(p - q, 0.f);
-                sx += q <= p ? q : 0.f;
-            }
+            float p[VEC], q[VEC];
+            exp_vec<DT>(rp[u], d.c, SP.ef, p);
+            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
+            resid_aux_n<VEC>(p, q, rho, &z2, &a2);
         }
-        zd = (double)warp_sum(sx);
+        z = (double)warp_sum(z2.x + z2.y) * ip;
+        zd = (double)warp_sum(a2.x + a2.y) * ((double)SQ.inv + (double)SQ.inv_lo);
     } else if (!draw) {
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            float r[8];
+            float p[VEC], q[VEC], r[VEC];
+            exp_vec<DT>(rp[u], d.c, SP.ef, p);
+            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
+            resid_n<VEC>(p, q, rho, r);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = 0.f;
-            residual_vec<DT, false>(rp[u], rq[u], c, SP, SQ, r, nullptr);
-            const float vs = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
-            if (u & 1) z1 += vs; else z0 += vs;
+            for (int i = 0; i < VEC; i += 4) {
+                z2 = __fadd2_rn(z2, make_float2(r[i], r[i + 1]));
+                a2 = __fadd2_rn(a2, make_float2(r[i + 2], r[i + 3]));
+            }
         }
+        z = (double)warp_sum((z2.x + a2.x) + (z2.y + a2.y)) * ip;
     } else {
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            float r[8];
+            float p[VEC], q[VEC], r[VEC];
+            exp_vec<DT>(rp[u], d.c, SP.ef, p);
+            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
+            resid_n<VEC>(p, q, rho, r);
+            zd += (double)sum_fixed<VEC>(r);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = 0.f;
-            residual_vec<DT, true>(rp[u], rq[u], c, SP, SQ, r, &sqs);
-            const float vs = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
-            z0 += vs;
-            zd += (double)vs;
+            for (int i = 0; i < VEC; i += 2) {
+                a2 = __ffma2_rn(make_float2(p[i], p[i + 1]), make_float2(p[i], p[i + 1]), a2);
+                b2 = __ffma2_rn(make_float2(q[i], q[i + 1]), make_float2(q[i], q[i + 1]), b2);
+            }
         }
+        zd = warp_sum(zd) * ip;
+        z = zd;
+        sqs = warp_sum((a2.x + a2.y) * (SP.inv * SP.inv) + (b2.x + b2.y) * (SQ.inv * SQ.inv));
     }
-    const float z = warp_sum(z0 + z1);
-    if (draw && !(TVO && a.sacc)) { zd = warp_sum(zd); sqs = warp_sum(sqs); }
-    if (lane == 0) { S.wf[stage][0][warp] = z; S.wd[stage][warp] = zd; S.wf[stage][1][warp] = sqs; }
+    if (lane == 0) { S.wf[stage][0][warp] = (float)z; S.wd[stage][warp] = zd; S.wf[stage][1][warp] = sqs; }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
 }
@@ -775,7 +795,7 @@ __device__ __noinline__ void draw_setup_warp(const PipeArgs& a, PipeShared& S, i
                 DrawTask t;
                 t.tt = Tt; t.base = base; t.bound = (float)draw_bound(sumsq, (double)a.kappa); t.c = __int_as_float(si.pad0);
                 t.b = b; t.k = k; t.owner = owner; t.pair = pair ? 1 : 0;
-                t.P = row_scale(sp); t.Q = pair ? row_scale(sq) : no_row();
+                t.P = row_scale(sp); t.Q = pair ? row_scale(sq) : no_row(); t.rho = pair ? row_rho(sp, sq) : make_float2(0.f, 0.f);
                 S.mbox[tail % kMbox] = t;
                 __threadfence_block();
                 *(volatile int*)&S.mb_tail = tail + 1;
@@ -801,27 +821,31 @@ __device__ __forceinline__ void pipe_d(const PipeArgs& a, PipeShared& PS, const 
     const unsigned char* qdata = data + STAGE_BYTES / 2;
     int found_y = -1, found_cert = 0;
     if (!(d.flags & 4)) {
-        TempScale c; c.hi = d.c;
-        const RowScale SP = d.P, SQ = d.Q;
+        const double ip = (double)d.P.inv + (double)d.P.inv_lo;
         const int v0 = d.v0, nv = d.nv;
-        // per-vector residual mass, same arithmetic as phase P2
+        // the vector's residuals, same arithmetic as phase P2
+        auto residuals = [&](const uint4& rp, const uint4& rq, float* r) {
+            float p[VEC], q[VEC];
+            exp_vec<DT>(rp, d.c, d.P.ef, p);
+            exp_vec<DT>(rq, d.c, d.Q.ef, q);
+            resid_n<VEC>(p, q, d.rho, r);
+        };
+        // residual mass per vector
         for (int v = tid; v < nv; v += PC) {
             uint4 rp = lds16(data + (size_t)v * 16), rq = neg_inf_vec<DT>();
             if (pair) rq = lds16(qdata + (size_t)v * 16);
             const int gbase = (v0 + v) * VEC;
             if (gbase + VEC > R.V) { mask_tail<DT>(rp, R.V - gbase); mask_tail<DT>(rq, R.V - gbase); }
-            float r[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = 0.f;
-            residual_vec<DT, true>(rp, rq, c, SP, SQ, r, nullptr);
-            vsum[v] = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
+            float r[VEC];
+            residuals(rp, rq, r);
+            vsum[v] = sum_fixed<VEC>(r);
         }
         consumers_meet(a.wait_failed, &PS.dsync, meet);
         // contiguous ranges of vectors per thread, inclusive scan over threads
         const int per = (nv + PC - 1) / PC;
         const int vb = min(tid * per, nv), ve = min(vb + per, nv);
         double mine = 0.0;
-        for (int v = vb; v < ve; ++v) mine += (double)vsum[v];
+        for (int v = vb; v < ve; ++v) mine += (double)vsum[v] * ip;
         double incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { double t2 = shfl_up_d(incl, o); if (lane >= o) incl += t2; }
@@ -836,21 +860,19 @@ __device__ __forceinline__ void pipe_d(const PipeArgs& a, PipeShared& PS, const 
         if (lower < Tt && Tt <= upper) {
             double C = lower;
             for (int v = vb; v < ve && found_y < 0; ++v) {
-                const double nxt = C + (double)vsum[v];
+                const double nxt = C + (double)vsum[v] * ip;
                 if (Tt <= nxt) {
                     uint4 rp = lds16(data + (size_t)v * 16), rq = neg_inf_vec<DT>();
                     if (pair) rq = lds16(qdata + (size_t)v * 16);
                     const int gbase = (v0 + v) * VEC;
                     if (gbase + VEC > R.V) { mask_tail<DT>(rp, R.V - gbase); mask_tail<DT>(rq, R.V - gbase); }
-                    float r[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) r[i] = 0.f;
-                    residual_vec<DT, true>(rp, rq, c, SP, SQ, r, nullptr);
+                    float r[VEC];
+                    residuals(rp, rq, r);
                     double Cw = C;
 #pragma unroll
                     for (int i = 0; i < VEC; ++i) {
                         if (found_y < 0) {
-                            const double r1 = (double)r[i];
+                            const double r1 = (double)r[i] * ip;
                             const double Cn = Cw + r1;
                             if (r1 > 0.0 && Cn >= Tt) { found_y = gbase + i; found_cert = (Tt - Cw > bound) && (Cn - Tt >= bound); }
                             Cw = Cn;

@@ -160,16 +160,6 @@ __device__ __forceinline__ TempScale temp_scale(float tau) {
     TempScale r; r.hi = kLog2e / (tau_ok(tau) ? tau : 1.f);
     return r;
 }
-__device__ __forceinline__ float exp2_scaled(float x, const TempScale& t, float Ef) {
-    return ex2f(fmaf(x, t.hi, -Ef));
-}
-// E = ceil(m * c) of a maximum m, as int and float: any integer near m * c serves as the reference, and
-// integer references make every merge of partial sums an exact power-of-two scaling.
-__device__ __forceinline__ int ref_exponent(float m, const TempScale& t, float* Ef) {
-    const float th = fminf(fmaxf(m * t.hi, -4.0e6f), 4.0e6f);
-    return ceil_alu(th, Ef);
-}
-
 struct DrawShared {
     double redd[WW];
     float redf[2][WW];
@@ -187,7 +177,7 @@ __device__ __forceinline__ const char* row_ptr(const RowArgs& R, int b, int r) {
                   : R.draft + ((int64_t)b * R.d_seq_rows + (r - K - 1)) * R.d_row_bytes;
 }
 
-// residuals of one vector pair: p = 2^(x*c - E_p) / S_p, q likewise
+// the scale of a row's exponentials: p = 2^(x c - E_p) / S_p
 struct RowScale { float ef, inv, inv_lo; };     // exponent E; 1/S = inv + inv_lo to about 2^-48
 __device__ __forceinline__ RowScale row_scale(const RowStat& s) {
     RowScale r; r.ef = (float)s.e; r.inv = (float)s.inv_s; r.inv_lo = (float)(s.inv_s - (double)r.inv);
@@ -195,27 +185,11 @@ __device__ __forceinline__ RowScale row_scale(const RowStat& s) {
 }
 __device__ __forceinline__ RowScale no_row() { RowScale r; r.ef = 0.f; r.inv = 0.f; r.inv_lo = 0.f; return r; }
 
-// FINE (the rows a token is drawn from): the normaliser enters as two floats, so that its rounding to fp32
-// is not an error common to all tokens of the row; what is left is one rounding per token.
-// A row that is not there (the draft row of a bonus task, vectors beyond the slice) is passed as -inf logits
-// with a zero normaliser: it gives q = 0 without a branch.
-template <int DT, bool FINE>
-__device__ __forceinline__ void residual_vec(const uint4& rp, const uint4& rq, const TempScale& c, const RowScale& P,
-                                             const RowScale& Q, float* r, float* sq) {
-    constexpr int VEC = Elem<DT>::VEC;
-    float fp[VEC], fq[VEC];
-    unpack<DT>(rp, fp);
-    unpack<DT>(rq, fq);
-#pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-        const float ap = exp2_scaled(fp[i], c, P.ef);
-        const float aq = exp2_scaled(fq[i], c, Q.ef);
-        // explicit roundings: a contracted p - a*inv would leave rounding dust when the rows are equal
-        const float p = FINE ? __fmaf_rn(ap, P.inv_lo, __fmul_rn(ap, P.inv)) : __fmul_rn(ap, P.inv);
-        const float q = FINE ? __fmaf_rn(aq, Q.inv_lo, __fmul_rn(aq, Q.inv)) : __fmul_rn(aq, Q.inv);
-        r[i] = fmaxf(p - q, 0.f);
-        if (sq) { *sq = fmaf(p, p, *sq); *sq = fmaf(q, q, *sq); }
-    }
+// S_p / S_q of a row pair as two floats
+__device__ __forceinline__ float2 row_rho(const RowStat& p, const RowStat& q) {
+    if (!(p.inv_s > 0.0)) return make_float2(0.f, 0.f);
+    const float ip = (float)p.inv_s, h = (float)q.inv_s / ip;
+    return make_float2(h, (float)fma(-(double)h, p.inv_s, q.inv_s) / ip);
 }
 
 }  // namespace

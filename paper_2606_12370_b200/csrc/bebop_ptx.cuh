@@ -1,5 +1,5 @@
 // Device helpers of the pipelined kernel: warp reductions through redux, order-preserving
-// float/int map, packed bf16 maximum, power-of-two construction, conversion-free ceil.
+// float/int map, packed bf16 maximum, power-of-two construction.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -53,19 +53,6 @@ template <int DT> __device__ __forceinline__ void mask_tail(uint4& v, int keep) 
         if (keep <= 6) v.w = (v.w & 0xffff0000u) | lo;
         if (keep <= 7) v.w = (v.w & 0x0000ffffu) | hi;
     }
-}
-
-
-
-// ceil(x) for |x| < 2^22 without the conversion pipe: returns the integer and, in *r, the same value as a float
-__device__ __forceinline__ int ceil_alu(float x, float* r) {
-    const float magic = 12582912.f;               // 1.5 * 2^23
-    float y = x + magic;                          // round to nearest integer
-    int i = __float_as_int(y) - 0x4B400000;
-    float f = y - magic;
-    if (f < x) { f += 1.f; i += 1; }
-    *r = f;
-    return i;
 }
 
 }  // namespace bebop
