@@ -397,8 +397,8 @@ __device__ __forceinline__ void f_producer(const FuseArgs& a, FShared& S, unsign
 }
 
 // ------------------------------------------------------------------ consumers
-// Reference exponent of a warp chunk from its maximum m: the integer nearest to m c (any integer near it serves),
-// found by adding 1.5 * 2^23.  The sum y = m c + 1.5 * 2^23 of a finite m with |m c| < 2^22 lies in [2^23, 2^24):
+// Reference exponent of a warp chunk from its maximum m: ceil(m c), so that every e = 2^(x c - E) is at most 1,
+// found by adding 1.5 * 2^23 with rounding upwards.  The sum y = m c + 1.5 * 2^23 of a finite m with |m c| < 2^22 lies in [2^23, 2^24):
 // a positive float whose bit pattern grows with its value, so the warp's maximum is one integer reduction, and
 // everything that is not the usual case -- NaN or +inf (bits above the range), -inf in every lane (negative),
 // huge logits -- shows as a result outside [kYLo, kYHi] and takes the slow way.
@@ -414,19 +414,22 @@ __device__ __noinline__ FExp warp_exponent_slow(float m, float c) {
     x.ef = 0.f; x.e = E_EMPTY;
     if (x.bad || mw == -INFINITY) return x;            // around 0 the chunk's -inf logits give e = 0
     const float th = fminf(fmaxf(mw * c, -4.0e6f), 4.0e6f);
-    const float y = th + kMagic;
+    const float y = __fadd_ru(th, kMagic);
     x.ef = y - kMagic;
     x.e = __float_as_int(y) - kMagicBits;
     return x;
 }
 __device__ __forceinline__ FExp warp_exponent(float m, float c) {
-    const int yi = redux_max(__float_as_int(fmaf(m, c, kMagic)));
+    const int yi = redux_max(__float_as_int(__fmaf_ru(m, c, kMagic)));
     if (yi < kYLo || yi > kYHi) return warp_exponent_slow(m, c);
     FExp x;
     x.e = yi - kMagicBits; x.ef = __int_as_float(yi) - kMagic; x.bad = 0;
     return x;
 }
 
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {      // min(max(a b + c, 0), 1), rounded once
+    float d; asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d;
+}
 // the exponentials of one vector around exponent Ef, two at a time
 template <int DT>
 __device__ __forceinline__ void exp_vec(const uint4& raw, float c, float Ef, float* e) {
@@ -449,19 +452,26 @@ template <int N> __device__ __forceinline__ float sum_fixed(const float* e) {
     return acc.x + acc.y;
 }
 // Residuals of N token pairs from their exponentials: d = e_p - rho e_q, rho as two floats, each product entering
-// one fused multiply-add (equal rows give rho = 1 and d = 0 exactly); r' = max(0, d) = d * [d >= 0].  Adds the sum of
-// the r' to *tm and, with AUX, the sum of e_q over the pairs with d >= 0 (q <= p) to *sx; with R, leaves the r'.
+// one fused multiply-add (equal rows give rho = 1 and d = 0 exactly); r' = max(0, d), which is d saturated to
+// [0, 1], as e_p <= 1.  Adds the sum of the r' to *tm; with R, leaves the r'; with AUX adds the sum of e_q over the
+// pairs with d >= 0 (q <= p) to *sx, and one mask [d >= 0] serves both sums.
 template <int N, bool AUX, bool R>
 __device__ __forceinline__ void resid_n(const float* ep, const float* eq, const FRho& rho, float2* tm, float2* sx, float* r) {
     const float2 nh = make_float2(-rho.h, -rho.h), nl = make_float2(-rho.l, -rho.l);
 #pragma unroll
     for (int i = 0; i < N; i += 2) {
         const float2 q2 = make_float2(eq[i], eq[i + 1]);
-        const float2 d = __ffma2_rn(nl, q2, __ffma2_rn(nh, q2, make_float2(ep[i], ep[i + 1])));
-        const float2 mk = make_float2(set_ge0(d.x), set_ge0(d.y));
-        if (R) { r[i] = d.x * mk.x; r[i + 1] = d.y * mk.y; }
-        *tm = __ffma2_rn(d, mk, *tm);
-        if (AUX) *sx = __ffma2_rn(q2, mk, *sx);
+        if (AUX) {
+            const float2 d = __ffma2_rn(nh, q2, __ffma2_rn(nl, q2, make_float2(ep[i], ep[i + 1])));
+            const float2 mk = make_float2(set_ge0(d.x), set_ge0(d.y));
+            *tm = __ffma2_rn(d, mk, *tm);
+            *sx = __ffma2_rn(q2, mk, *sx);
+        } else {
+            const float2 t = __ffma2_rn(nl, q2, make_float2(ep[i], ep[i + 1]));
+            const float2 d = make_float2(fma_sat(nh.x, eq[i], t.x), fma_sat(nh.x, eq[i + 1], t.y));
+            if (R) { r[i] = d.x; r[i + 1] = d.y; }
+            *tm = __fadd2_rn(*tm, d);
+        }
     }
 }
 
