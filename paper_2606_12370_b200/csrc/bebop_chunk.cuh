@@ -1,4 +1,4 @@
-// What the sequence kernel and the streaming kernel share: barriers and bulk copies, the exponentials of a chunk around an
+// What the kernels share: barriers and bulk copies, the exponentials of a chunk around an
 // integer exponent, fixed-point warp sums, owners of a target among the lanes of a warp, 2^t in double.
 #pragma once
 #include "bebop_pipe.cuh"
