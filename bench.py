@@ -402,7 +402,7 @@ def run_ours(args):
     kern_ms = sum(kern_ms) / len(kern_ms)
     clocks = sampler.summary(t0, t1)
     main_kernel = P.bebop_debug_last_kernel()           # what the timed calls ran: the library chooses by shape
-    launches_per_call = 6 if main_kernel == 1 else 2    # main kernel, fp64 re-draw kernel | 6 general kernels
+    launches_per_call = {1: 6, 2: 3}.get(main_kernel, 2)      # clearing, k_pipe, fp64 re-draw | 6 general kernels | main kernel, re-draw
 
     # median and best of single calls (an event pair around each call, so a little above the back-to-back mean)
     single = stats(per_call_ms(torch, [step], max(10, min(steps, 100)), barrier))
