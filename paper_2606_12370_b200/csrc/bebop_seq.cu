@@ -689,18 +689,6 @@ int sm_count() {
     if (dev >= 0 && dev < 64) cached[dev] = n;
     return n;
 }
-// The cluster size for a call: a share per CTA that lets two CTAs run on an SM (one's exchanges then overlap the other's
-// arithmetic, and a re-draw is spread over more SMs: 300 sequences of 12,000 bf16 logits, K = 3, take 51 instead of 60 us,
-// 48 of 32,000 20 instead of 33), as far as sixteen CTAs go; and more while SMs would idle and the CTAs have work.
-constexpr int kSeqShare = 112000;
-int seq_cluster_for(int B, int rows, int K, int nvec) {
-    int C = seq_cluster(rows, K, nvec);
-    if (!C) return 0;
-    while (C < kSeqMaxCluster && seq_plan(rows, K, nvec, C).bytes > kSeqShare) ++C;
-    const int sms = sm_count();
-    while (C < kSeqMaxCluster && (long long)B * (C + 1) <= sms && (long long)rows * nvec > (long long)C * 2048) ++C;
-    return C;
-}
 template <auto kernel> bool seq_ready() {
     static bool done[64] = {false};
     int dev = 0;
@@ -710,6 +698,54 @@ template <auto kernel> bool seq_ready() {
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { cudaGetLastError(); return false; }
     if (dev >= 0 && dev < 64) done[dev] = true;
     return true;
+}
+// The cluster size for a call: a share per CTA that lets two CTAs run on an SM (one's exchanges then overlap the other's
+// arithmetic, and a re-draw is spread over more SMs: 300 sequences of 12,000 bf16 logits, K = 3, take 51 instead of 60 us,
+// 48 of 32,000 20 instead of 33), as far as sixteen CTAs go; and more while SMs would idle and the CTAs have work.
+constexpr int kSeqShare = 112000;
+// How many clusters of C CTAs the device holds at a time, one CTA per SM or two (asked once per device; 0: not known).
+// A cluster stays inside one of the chip's GPCs, so large ones leave SMs over: of sixteen CTAs seven, of ten about twice as many.
+int seq_resident(int C, bool two) {
+    static int cached[64][2][kSeqMaxCluster + 1] = {{{0}}};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 0; }
+    int& n = cached[dev][two][C];
+    if (n) return n > 0 ? n : 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C); cfg.blockDim = dim3(kSeqThreads); cfg.dynamicSmemBytes = two ? kSeqShare : kSeqSmem;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int got = 0;
+    if (!seq_ready<k_seq<1, false>>() || cudaOccupancyMaxActiveClusters(&got, k_seq<1, false>, &cfg) != cudaSuccess) { cudaGetLastError(); got = 0; }
+    n = got > 0 ? got : -1;
+    return got > 0 ? got : 0;
+}
+int seq_cluster_for(int B, int rows, int K, int nvec, int dt) {
+    const int least = seq_cluster(rows, K, nvec);
+    int C = least;
+    if (!C) return 0;
+    while (C < kSeqMaxCluster && seq_plan(rows, K, nvec, C).bytes > kSeqShare) ++C;
+    const int sms = sm_count();
+    if (C > 8 && B > 1) {
+        // Clusters beyond the portable size leave SMs unused: the size whose waves are done first, a wave taken as 6 us and
+        // 0.08 us per KB of bf16 logits in a CTA's share, half of that for fp32 (half as much again where two CTAs share an SM).  24 ragged fp32 sequences of 49,999
+        // logits, K = 5: ten CTAs each instead of sixteen, 44 -> 33 us; 8 of 151,936 bf16, K = 3, 32 -> 20.
+        double best = 1e30;
+        for (int c = least; c <= kSeqMaxCluster; ++c) {
+            const int bytes = seq_plan(rows, K, nvec, c).bytes;
+            if (bytes == INT_MAX) continue;
+            const bool two = bytes <= kSeqShare;
+            const int n = seq_resident(c, two);
+            if (!n) continue;
+            const double t = (double)((B + n - 1) / n) * (6.0 + (two ? 0.12e-3 : 0.08e-3) * (dt == 0 ? 0.5 : 1.0) * bytes);
+            if (t < best) { best = t; C = c; }
+        }
+        return C;
+    }
+    while (C < kSeqMaxCluster && (long long)B * (C + 1) <= sms && (long long)rows * nvec > (long long)C * 2048) ++C;
+    return C;
 }
 template <typename K, typename A> cudaError_t seq_launch(K kernel, const A& args, int B, int C, int threads, int smem, cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
@@ -739,7 +775,8 @@ bool seq_supported(const RowArgs& a, bool tv_only) {
 // slower; bebop_tv 3,000 pairs of 12,000 67 against 88, but 1,024 of 32,000, two CTAs each, 65 against 58).  Larger clusters
 // leave SMs unused (seven clusters of sixteen run at a time) and run in waves without overlap: faster while the call
 // is a few waves (128 of 32,000 49 against 60; 48 of 65,536 42 against 55; 24 fp32 ragged ones of 49,999, K = 5, 36
-// against 54; one of 151,936 16 against 32), slower beyond (300 of 32,000 104 against 97; 16 of 151,936 46 against 41).
+// against 54; one of 151,936 16 against 32), slower beyond (300 of 32,000 104 against 97; 16 of 151,936 44 against 37); with nine CTAs, of which fifteen to thirty
+// clusters run at a time, somewhat longer (32 of 65,536 31 against 48, 40 35 against 38).
 bool seq_preferred(const RowArgs& a, bool tv_only) {
     const int rows = tv_only ? 2 : 2 * a.K + 1;
     int C = seq_cluster(rows, a.K, a.nvec);
@@ -749,6 +786,7 @@ bool seq_preferred(const RowArgs& a, bool tv_only) {
     if (C == 1) return true;
     if (C == 2) return logits <= (tv_only || a.dt == 0 ? 30e6 : 100e6);
     if (C <= 8) return logits <= (tv_only ? 15e6 : 30e6);
+    if (C == 9 && !tv_only) return logits <= 20e6;
     return logits <= (tv_only ? 6e6 : 14e6);
 }
 // Faster than the sweep of the pipelined kernel and its two companions up to about 100 MB of target logits (7 against 11 us
@@ -759,7 +797,7 @@ cudaError_t seq_verify(const RowArgs& a, const int32_t* draft_tokens, const floa
                        cudaStream_t stream, bool* launched, bool tv_only, float* s_aux) {
     *launched = false;
     const int rows = tv_only ? 2 : 2 * a.K + 1;
-    const int C = seq_cluster_for(a.B, rows, a.K, a.nvec);
+    const int C = seq_cluster_for(a.B, rows, a.K, a.nvec, a.dt);
     if (!C) return cudaSuccess;
     SeqArgs sa;
     sa.r = a; sa.draft_tokens = draft_tokens; sa.u_accept = u_accept; sa.u_final = u_final; sa.o = o; sa.s_aux = tv_only ? s_aux : nullptr;
