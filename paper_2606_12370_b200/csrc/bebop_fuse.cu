@@ -322,7 +322,10 @@ __device__ __forceinline__ FRho warp_rho(const FScale& sc, int ewp, int ewq) {
     if (ewp > E_EMPTY && ewq > E_EMPTY && sc.ep > E_EMPTY && sc.eq > E_EMPTY) k = (ewq - sc.eq) - (ewp - sc.ep);
     k = max(min(k, 126), -126);
     const float f = pow2f(k);
-    FRho r; r.h = sc.rho_h * f; r.l = sc.rho_l * f;
+    // Finite whatever the scales: where the target's chunk lies more than 2^100 below its row's largest logit and the draft's does
+    // not, rho runs past the largest float, and bebop_tv multiplies d = e_p - rho e_q by a mask (-inf * 0 was NaN, and the
+    // pair's TV 0).  At the bound d is below zero for every e_q that is not itself next to nothing, as it would be beyond.
+    FRho r; r.h = fminf(sc.rho_h * f, 1e38f); r.l = sc.rho_l * f;
     return r;
 }
 // the factor that turns the chunk's sum of r' (or of e) into probability mass: 2^(E_wp - E_rp) / S_p
