@@ -458,7 +458,8 @@ template <int N> __device__ __forceinline__ float sum_fixed(const float* e) {
 }
 // Residuals of N token pairs from their exponentials: d = e_p - rho e_q, rho as two floats, each product entering
 // one fused multiply-add (equal rows give rho = 1 and d = 0 exactly); r' = max(0, d), which is d saturated to
-// [0, 1], as e_p <= 1.  Adds the sum of the r' to *tm; with R, leaves the r'; with AUX adds the sum of e_q over the
+// [0, 1], as e_p <= 1.  The large product goes first: where q is close to p it leaves a small difference without rounding, and
+// the small product then decides its sign (the other way round it is lost in the rounding of e_p).  Adds the sum of the r' to *tm; with R, leaves the r'; with AUX adds the sum of e_q over the
 // pairs with d >= 0 (q <= p) to *sx, and one mask [d >= 0] serves both sums.
 template <int N, bool AUX, bool R>
 __device__ __forceinline__ void resid_n(const float* ep, const float* eq, const FRho& rho, float2* tm, float2* sx, float* r) {
@@ -467,13 +468,13 @@ __device__ __forceinline__ void resid_n(const float* ep, const float* eq, const 
     for (int i = 0; i < N; i += 2) {
         const float2 q2 = make_float2(eq[i], eq[i + 1]);
         if (AUX) {
-            const float2 d = __ffma2_rn(nh, q2, __ffma2_rn(nl, q2, make_float2(ep[i], ep[i + 1])));
+            const float2 d = __ffma2_rn(nl, q2, __ffma2_rn(nh, q2, make_float2(ep[i], ep[i + 1])));
             const float2 mk = make_float2(set_ge0(d.x), set_ge0(d.y));
             *tm = __ffma2_rn(d, mk, *tm);
             *sx = __ffma2_rn(q2, mk, *sx);
         } else {
-            const float2 t = __ffma2_rn(nl, q2, make_float2(ep[i], ep[i + 1]));
-            const float2 d = make_float2(fma_sat(nh.x, eq[i], t.x), fma_sat(nh.x, eq[i + 1], t.y));
+            const float2 t = __ffma2_rn(nh, q2, make_float2(ep[i], ep[i + 1]));
+            const float2 d = make_float2(fma_sat(nl.x, eq[i], t.x), fma_sat(nl.x, eq[i + 1], t.y));
             if (R) { r[i] = d.x; r[i + 1] = d.y; }
             *tm = __fadd2_rn(*tm, d);
         }

@@ -495,14 +495,15 @@ template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* 
     return m;
 }
 // Residuals from the exponentials of a row pair: r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q as two floats
-// (equal rows give rho = 1 and r' = 0 exactly); as e_p <= 1, saturating to [0, 1] is taking the maximum with 0.  Two
-// instructions a token, where p, q, their difference and its maximum with 0 took four.
+// (equal rows give rho = 1 and r' = 0 exactly); as e_p <= 1, saturating to [0, 1] is taking the maximum with 0.  The large
+// product goes first: where q is close to p it leaves a small difference without rounding, and the small product then
+// decides its sign.  Two instructions a token, where p, q, their difference and its maximum with 0 took four.
 template <int N> __device__ __forceinline__ void resid_n(const float* p, const float* q, float2 rho, float* r) {
-    const float2 nl = make_float2(-rho.y, -rho.y);
+    const float2 nh = make_float2(-rho.x, -rho.x);
 #pragma unroll
     for (int i = 0; i < N; i += 2) {
-        const float2 t = __ffma2_rn(nl, make_float2(q[i], q[i + 1]), make_float2(p[i], p[i + 1]));
-        r[i] = fma_sat(-rho.x, q[i], t.x); r[i + 1] = fma_sat(-rho.x, q[i + 1], t.y);
+        const float2 t = __ffma2_rn(nh, make_float2(q[i], q[i + 1]), make_float2(p[i], p[i + 1]));
+        r[i] = fma_sat(-rho.y, q[i], t.x); r[i + 1] = fma_sat(-rho.y, q[i + 1], t.y);
     }
 }
 // ... their sum, and the sum of e_q over the tokens with q <= p: the mask 1[d >= 0] serves both
@@ -511,7 +512,7 @@ template <int N> __device__ __forceinline__ void resid_aux_n(const float* p, con
 #pragma unroll
     for (int i = 0; i < N; i += 2) {
         const float2 q2 = make_float2(q[i], q[i + 1]);
-        const float2 d = __ffma2_rn(nh, q2, __ffma2_rn(nl, q2, make_float2(p[i], p[i + 1])));
+        const float2 d = __ffma2_rn(nl, q2, __ffma2_rn(nh, q2, make_float2(p[i], p[i + 1])));
         const float2 mk = make_float2(d.x >= 0.f ? 1.f : 0.f, d.y >= 0.f ? 1.f : 0.f);
         *z = __ffma2_rn(d, mk, *z);
         *x = __ffma2_rn(q2, mk, *x);

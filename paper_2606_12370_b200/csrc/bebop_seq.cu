@@ -96,12 +96,13 @@ __device__ __forceinline__ void chunk_vecs(const unsigned char* row, int c, bool
         for (int j = 0; j < QV; ++j) x[j] = slice_vec<DT>(row, vi + j * 32, nv, v0, V);
     }
 }
-// r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q as two floats (equal rows give rho = 1 and 0 exactly); as
-// e_p <= 1, saturating to [0, 1] is taking the maximum with 0
+// r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q as two floats (equal rows give rho = 1 and 0 exactly; the
+// large product first, so that the small one decides the sign where q is close to p); as e_p <= 1, saturating to [0, 1] is
+// taking the maximum with 0
 template <int DT>
 __device__ __forceinline__ void resid_vec(const float* ep, const float* eq, float2 rho, float* r) {
 #pragma unroll
-    for (int i = 0; i < Elem<DT>::VEC; ++i) r[i] = fma_sat(-rho.x, eq[i], fmaf(-rho.y, eq[i], ep[i]));
+    for (int i = 0; i < Elem<DT>::VEC; ++i) r[i] = fma_sat(-rho.y, eq[i], fmaf(-rho.x, eq[i], ep[i]));
 }
 // What the threads of a CTA share besides the tables of the plan.
 struct QShared {
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(kSeqThreads, 2) k_seq(const __grid_constant__ 
                     // q <= p: e_p - rho e_q >= 0; the sum S of Eq. tv_grad goes with the residuals
 #pragma unroll
                     for (int i = 0; i < VEC; ++i) {
-                        const float d = fmaf(-rh.x, q[i], fmaf(-rh.y, q[i], p[i]));
+                        const float d = fmaf(-rh.y, q[i], fmaf(-rh.x, q[i], p[i]));
                         r[i] = fmaxf(d, 0.f);
                         sx += d >= 0.f ? q[i] : 0.f;
                     }

@@ -210,3 +210,25 @@ def test_the_library_chooses_the_kernel_by_shape():
         assert P.bebop_debug_last_kernel() == want
     P.bebop_debug_force_general_path(0)
     torch.cuda.synchronize()
+
+
+# ------------------------------------------------------------- p and q that differ by less than a rounding
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("path", [2, 3, 4])
+def test_the_sign_of_p_minus_q_below_fp32_resolution(path, dtype):
+    """A flat target row and a draft row that differs from it in one token, by 1.2e-4 of that token's weight: every other token has
+    q = p (1 + 3e-8), more than p, so S = sum of q over q <= p is that one token's q = 1 / V.  Half an ulp of fp32 is 6e-8, so
+    the sign comes out only if the product of the low part of S_p / S_q is not rounded away (S was 1.0 then)."""
+    P.bebop_debug_force_general_path(path)
+    try:
+        N, V = 40, 4096
+        tgt = torch.zeros(N, V, dtype=torch.float32 if dtype == "f32" else torch.bfloat16, device=DEV)
+        drf = tgt.clone()
+        drf[torch.arange(N, device=DEV), torch.arange(N, device=DEV) * 97] = -1.220703125e-4
+        got = P.bebop_tv(tgt, drf)
+        ref = oracle.tv(tgt.float().cpu().numpy(), drf.float().cpu().numpy())
+        assert abs(ref["s_aux"][0] - 1.0 / V) < 1e-6
+        assert np.abs(to_np(got["s_aux"]) - ref["s_aux"]).max() <= 1e-6
+        assert np.abs(to_np(got["tv"]) - ref["tv"]).max() <= 1e-9      # TV is 3e-8: sums of 4,096 terms of fp32, about 1e-10 off
+    finally:
+        P.bebop_debug_force_general_path(0)
