@@ -48,7 +48,7 @@ __device__ __forceinline__ QExp chunk_exponent(float m, float c) {
     x.ef = 0.f; x.e = E_EMPTY;
     if (!(mw < INFINITY)) { x.e = E_BAD; return x; }
     if (mw == -INFINITY) return x;                    // around 0 the chunk's -inf logits give e = 0
-    const float y = __fadd_ru(fminf(fmaxf(mw * c, -4.0e6f), 4.0e6f), kMagic);
+    const float y = __fadd_ru(fminf(fmaxf(mw * c, -(float)kFarExp), (float)kFarExp), kMagic);      // (at either end: far_exponent)
     x.ef = y - kMagic; x.e = __float_as_int(y) - kMagicBits;
     return x;
 }

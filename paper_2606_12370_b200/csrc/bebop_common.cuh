@@ -49,6 +49,17 @@ template <> __device__ __forceinline__ void unpack<1>(const uint4& v, float* f) 
     f[6] = __uint_as_float(v.w << 16); f[7] = __uint_as_float(v.w & 0xffff0000u);
 }
 
+template <int DT> __device__ __forceinline__ uint4 pack(const float* f);
+template <> __device__ __forceinline__ uint4 pack<0>(const float* f) {
+    return make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+}
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    uint32_t r; asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo)); return r;
+}
+template <> __device__ __forceinline__ uint4 pack<1>(const float* f) {
+    return make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+}
+
 // A 16-byte vector of -inf logits (used for out-of-range loads).
 template <int DT> __device__ __forceinline__ uint4 neg_inf_vec() {
     if (DT == 0) return make_uint4(kNegInfBits, kNegInfBits, kNegInfBits, kNegInfBits);

@@ -15,6 +15,11 @@ constexpr int BEBOP_MAX_K_INT = 32;
 constexpr int MAX_SLICES = 64;
 constexpr int E_EMPTY = INT_MIN / 2;
 constexpr uint32_t kSpin = 1u << 22;
+// The integer reference exponents end at +-kFarExp (chunk_exponent): a row whose largest scaled logit lies beyond -- one that is
+// nothing but a mask of -1e9, or a temperature next to zero -- shows by a merged exponent at the end of the range, and
+// is marked ST_FAR.  That stops what would follow, as a fatal bit does; it never is part of the caller's row_status.
+constexpr int kFarExp = 4000000, ST_FAR = 64, ST_STOP = ST_FATAL | ST_FAR;
+__device__ __forceinline__ bool far_exponent(int e) { return e >= kFarExp || (e <= -kFarExp && e > E_EMPTY); }
 
 struct __align__(16) P1Part { double s; int e; float m; };             // per (row, slice); m = NaN marks a non-finite logit
 struct __align__(16) RowStat { double inv_s; int e; int st; };   // per row, after the merge: 1/S, exponent E, status bits | kRowValid
@@ -157,7 +162,7 @@ __device__ __forceinline__ double draw_bound(double sumsq, double kappa = kDrawK
 // is a sum of zero-mean terms of the size draw_bound() already allows per token.
 struct TempScale { float hi; };
 __device__ __forceinline__ TempScale temp_scale(float tau) {
-    TempScale r; r.hi = kLog2e / (tau_ok(tau) ? tau : 1.f);
+    TempScale r; r.hi = fminf(kLog2e / (tau_ok(tau) ? tau : 1.f), 3e38f);      // (finite: 0 * c is 0)
     return r;
 }
 struct DrawShared {

@@ -122,9 +122,47 @@ __device__ __forceinline__ void merge_cluster(const SeqArgs& a, const QRec* rrec
         const double s = warp_sum(r.s * f), ub = warp_sum(r.ub * f * f);
         if (lane == 0) {
             QStat x;
-            x.st = (bad & 2) ? ST_WAIT : ((bad & 1) || !(s == s)) ? ST_NONFINITE : Em == E_EMPTY ? ST_EMPTY : 0;
+            x.st = (bad & 2) ? ST_WAIT : ((bad & 1) || !(s == s)) ? ST_NONFINITE : Em == E_EMPTY ? ST_EMPTY : far_exponent(Em) ? ST_FAR : 0;
             x.inv_s = !x.st && s > 0.0 ? 1.0 / s : 0.0; x.e = Em; x.ub = ub * x.inv_s * x.inv_s; x.pad = 0.0;
             stat[i] = x;
+        }
+    }
+}
+
+// Rows marked ST_FAR are moved into the range of the reference exponents: every logit becomes x - m, m the row's maximum, in the
+// shared memory of all CTAs.  That is exact wherever it matters: a logit within a factor of two of m differs from it by a
+// number of the same type, and any other lies at least |m| / 2 below, 2^(-2e6) of the row's largest weight.  The
+// softmax does not change, and pass 1 runs again.  Ordinary calls only pay for the test of the statuses, which they make
+// anyway (one sequence of 151,936 bf16 logits 15.8 -> 16.1 us, the other calls measured alike); a call, never made, to a
+// function that evaluates such a sequence in double, or a flag of its own, cost 0.2 to 0.3 us in all of them.
+template <int DT>
+__device__ __forceinline__ void move_far_rows(const SeqArgs& a, unsigned char* smem, const QStat* stat, int* rmax, int rows, int nv, int v0, int rank) {
+    constexpr int VEC = Elem<DT>::VEC;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    cluster_sync();                                         // (every CTA has merged: the rows' records may be written again)
+#pragma unroll 1
+    for (int i = warp; i < rows; i += nw) {
+        if (stat[i].st != ST_FAR) continue;
+        const unsigned char* const row = smem + (size_t)i * a.p.sv * 16;
+        float m = -INFINITY;
+#pragma unroll 1
+        for (int v = lane; v < nv; v += 32) m = fmaxf(m, vec_max<DT>(slice_vec<DT>(row, v, nv, v0, a.r.V)));
+        const int om = redux_max(f2ord(m));
+        if (lane < a.p.C) st_remote(at_rank(rmax + rank * a.p.rows + i, lane), om);
+    }
+    cluster_sync();
+#pragma unroll 1
+    for (int i = warp; i < rows; i += nw) {
+        if (stat[i].st != ST_FAR) continue;
+        uint4* const row = reinterpret_cast<uint4*>(smem + (size_t)i * a.p.sv * 16);
+        const float m = ord2f(redux_max(lane < a.p.C ? rmax[lane * a.p.rows + i] : INT_MIN));
+#pragma unroll 1
+        for (int v = lane; v < nv; v += 32) {
+            float f[VEC];
+            unpack<DT>(row[v], f);
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) f[j] -= m;
+            row[v] = pack<DT>(f);
         }
     }
 }
@@ -152,7 +190,7 @@ __device__ __forceinline__ void accept_scan(const SeqArgs& a, QShared& S, const 
     if (!seq_st && badrows) seq_st = rs_first;
     double px = 0.0, qx = 0.0;
     bool acc = false;
-    if (active && !(seq_st & ST_FATAL) && lane < first_bad) {
+    if (active && !(seq_st & ST_STOP) && lane < first_bad) {
         const double cd = (double)ts.hi;
         px = exp2((double)zpx * cd - (double)sp.e) * sp.inv_s;
         qx = exp2((double)zqx * cd - (double)sq.e) * sq.inv_s;
@@ -160,9 +198,9 @@ __device__ __forceinline__ void accept_scan(const SeqArgs& a, QShared& S, const 
     }
     const unsigned rej = __ballot_sync(0xffffffffu, active && !acc);
     const int n = rej ? __ffs(rej) - 1 : L;
-    if (!(seq_st & ST_FATAL) && n == L) seq_st |= sb.st;              // bonus row, counted only now
+    if (!(seq_st & ST_STOP) && n == L) seq_st |= sb.st;               // bonus row, counted only now
     if (wait) seq_st = ST_WAIT;
-    const bool fatal = (seq_st & (ST_FATAL | ST_WAIT)) != 0;
+    const bool fatal = (seq_st & (ST_STOP | ST_WAIT)) != 0;
     const int nn = fatal ? 0 : n;
     if (write) {
         for (int q = lane; q <= K; q += 32)
@@ -402,65 +440,78 @@ __global__ void __launch_bounds__(kSeqThreads, 2) k_seq(const __grid_constant__ 
         if (tk >= 0 && tk < R.V) { zpx = load_one<DT>(row_ptr(R, b, lane), tk); zqx = load_one<DT>(row_ptr(R, b, R.K + 1 + lane), tk); }
     }
     const float uf = !TVM && warp == 0 ? a.u_final[b] : 0.f;
-    // ---- pass 1: a warp per (row, chunk)
-    for (int it = warp; it < rows * nch; it += nw) {
-        const int i = it / nch, ch = it - i * nch;
-        double s = 0.0;
-        int e = E_EMPTY;
-        if (ch * QCV < nv) {
-            if (!mbar_wait(&bar[i])) S.failed = 1;
-            uint4 x[QV];
-            chunk_vecs<DT>(row_of(i), ch, (ch + 1) * QCV <= nfull, nv, v0, R.V, x);
-            const QExp E = chunk_exponent(max_nan(max_nan(vec_max<DT>(x[0]), vec_max<DT>(x[1])), max_nan(vec_max<DT>(x[2]), vec_max<DT>(x[3]))), c);
-            float sum = 0.f;
+    // ---- pass 1: a warp per (row, chunk).  (Once more when the statuses say that rows lie beyond its range; what stands between
+    // here and pass 2 writes the same places again then.)
+    for (bool moved = false;; moved = true) {
+        for (int it = warp; it < rows * nch; it += nw) {
+            const int i = it / nch, ch = it - i * nch;
+            double s = 0.0;
+            int e = E_EMPTY;
+            if (ch * QCV < nv) {
+                if (!mbar_wait(&bar[i])) S.failed = 1;
+                uint4 x[QV];
+                chunk_vecs<DT>(row_of(i), ch, (ch + 1) * QCV <= nfull, nv, v0, R.V, x);
+                const QExp E = chunk_exponent(max_nan(max_nan(vec_max<DT>(x[0]), vec_max<DT>(x[1])), max_nan(vec_max<DT>(x[2]), vec_max<DT>(x[3]))), c);
+                float sum = 0.f;
 #pragma unroll
-            for (int j = 0; j < QV; ++j) { float f[VEC]; exp_vec<DT>(x[j], c, E.ef, f); sum += sum_fixed<VEC>(f); }
-            e = E.e;
-            s = e == E_BAD ? 0.0 : warp_sum_fixed(sum);
+                for (int j = 0; j < QV; ++j) { float f[VEC]; exp_vec<DT>(x[j], c, E.ef, f); sum += sum_fixed<VEC>(f); }
+                e = E.e;
+                s = e == E_BAD ? 0.0 : warp_sum_fixed(sum);
+            }
+            if (lane == 0) { psum[it] = s; pexp[it] = e; }
         }
-        if (lane == 0) { psum[it] = s; pexp[it] = e; }
-    }
-    cluster_wait();                                         // every CTA of the cluster has started
-    __syncthreads();
-    // ---- the CTA's sum of every row, sent to all CTAs
-    for (int i = warp; i < rows; i += nw) {
-        int em = E_EMPTY;
-        for (int k = lane; k < nch; k += 32) em = max(em, pexp[i * nch + k]);
-        em = redux_max(em);
-        const int bad = em == E_BAD;                        // (what the row's sum is then does not matter)
-        double s = 0.0, ub = 0.0;
-        for (int k = lane; k < nch; k += 32) {
-            const int e = pexp[i * nch + k];
-            const double f = e > E_EMPTY && e != E_BAD ? pow2d(max(e - em, -500)) : 0.0;
-            s += psum[i * nch + k] * f; ub += psum[i * nch + k] * f * f;        // (e <= 1: a chunk's sum of e^2 is at most its sum of e)
+        if (!moved) cluster_wait();                         // every CTA of the cluster has started
+        __syncthreads();
+        // ---- the CTA's sum of every row, sent to all CTAs
+        for (int i = warp; i < rows; i += nw) {
+            int em = E_EMPTY;
+            for (int k = lane; k < nch; k += 32) em = max(em, pexp[i * nch + k]);
+            em = redux_max(em);
+            const int bad = em == E_BAD;                        // (what the row's sum is then does not matter)
+            double s = 0.0, ub = 0.0;
+            for (int k = lane; k < nch; k += 32) {
+                const int e = pexp[i * nch + k];
+                const double f = e > E_EMPTY && e != E_BAD ? pow2d(max(e - em, -500)) : 0.0;
+                s += psum[i * nch + k] * f; ub += psum[i * nch + k] * f * f;        // (e <= 1: a chunk's sum of e^2 is at most its sum of e)
+            }
+            s = warp_sum(s); ub = warp_sum(ub);
+            if (lane < C) {
+                const uint32_t d = at_rank(rrec + rank * a.p.rows + i, lane);
+                st_remote(d, s); st_remote(d + 8, ub); st_remote(d + 16, em); st_remote(d + 20, bad | (S.failed ? 2 : 0));
+            }
         }
-        s = warp_sum(s); ub = warp_sum(ub);
-        if (lane < C) {
-            const uint32_t d = at_rank(rrec + rank * a.p.rows + i, lane);
-            st_remote(d, s); st_remote(d + 8, ub); st_remote(d + 16, em); st_remote(d + 20, bad | (S.failed ? 2 : 0));
+        cluster_sync();
+        merge_cluster(a, rrec, stat, rows);
+        __syncthreads();
+        // ---- the accept scan (bebop_tv: the pair's status)
+        if (TVM) {
+            if (tid == 0) { const int w = (stat[0].st | stat[1].st) & ST_WAIT; S.status = w ? w : !tau_ok(tau) ? ST_BAD_TEMP : (stat[0].st | stat[1].st); S.nn = -1; }
+        } else if (warp == aw) accept_scan(a, S, stat, b, L, tau, tk, u, zpx, zqx, rank == 0);
+        if (warp == 0) for (int k = lane; k < L; k += 32) {
+            const double r = stat[2 * k].inv_s > 0.0 ? stat[2 * k + 1].inv_s / stat[2 * k].inv_s : 0.0;
+            rho[k] = make_float2((float)r, (float)(r - (double)(float)r));
         }
+        __syncthreads();
+        if (__builtin_expect(!(S.status & (ST_STOP | ST_WAIT)), 1)) break;
+        if (moved || !(S.status & ST_FAR)) {                // (the same in every CTA: nothing more is sent)
+            if (TVM && rank == 0 && tid == 0) {
+                a.o.tv[b] = 0.f;
+                if (a.s_aux) a.s_aux[b] = 0.f;
+                if (a.o.row_status) a.o.row_status[b] = S.status;
+            }
+            return;
+        }
+        int* const rmax = reinterpret_cast<int*>(rmass);    // [C][rows held]
+        move_far_rows<DT>(a, smem, stat, rmax, rows, nv, v0, rank);
+        if (!TVM && warp == aw && lane < L)
+            for (int w = 0; w < 2; ++w) if (stat[2 * lane + w].st == ST_FAR) {
+                int om = INT_MIN;
+                for (int q = 0; q < C; ++q) om = max(om, rmax[q * a.p.rows + 2 * lane + w]);
+                if (w) zqx -= ord2f(om); else zpx -= ord2f(om);
+            }
+        __syncthreads();
     }
-    cluster_sync();
-    merge_cluster(a, rrec, stat, rows);
-    __syncthreads();
-    // ---- the accept scan (bebop_tv: the pair's status)
-    if (TVM) {
-        if (tid == 0) { const int w = (stat[0].st | stat[1].st) & ST_WAIT; S.status = w ? w : !tau_ok(tau) ? ST_BAD_TEMP : (stat[0].st | stat[1].st); S.nn = -1; }
-    } else if (warp == aw) accept_scan(a, S, stat, b, L, tau, tk, u, zpx, zqx, rank == 0);
-    if (warp == 0) for (int k = lane; k < L; k += 32) {
-        const double r = stat[2 * k].inv_s > 0.0 ? stat[2 * k + 1].inv_s / stat[2 * k].inv_s : 0.0;
-        rho[k] = make_float2((float)r, (float)(r - (double)(float)r));
-    }
-    __syncthreads();
     const int nn = S.nn;
-    if (S.status & (ST_FATAL | ST_WAIT)) {                  // (the same in every CTA: nothing more is sent)
-        if (TVM && rank == 0 && tid == 0) {
-            a.o.tv[b] = 0.f;
-            if (a.s_aux) a.s_aux[b] = 0.f;
-            if (a.o.row_status) a.o.row_status[b] = S.status;
-        }
-        return;
-    }
     // ---- pass 2: a warp per (row pair, chunk); without a TV output only the pair a token is drawn from
     const bool all = TVM || a.o.tv;
     const int k0 = all ? 0 : nn, pairs = all ? L : (nn < L ? 1 : 0);

@@ -1,6 +1,6 @@
 """Finite logits far from zero, through every kernel, against the oracle: masks of a large negative number on one side of a
-row pair.  Every case is well defined (the softmax subtracts the maximum), so no status bit and no tolerance is given
-away."""
+row pair, rows that hold nothing but such a mask, and temperatures that carry ordinary logits far out.  Every case is
+well defined (the softmax subtracts the maximum), so no status bit and no tolerance is given away."""
 import numpy as np
 import pytest
 import torch
@@ -61,3 +61,63 @@ def test_a_finite_mask_on_one_side(dtype, mask):
 def run_verify(x, **kw):
     return P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
                           temperature=x["temperature"], temperature_all=x["temperature_all"], **kw)
+
+
+FAR_PATHS = ("auto", "seq")
+
+
+def far_inputs(dtype, V):
+    """Ten sequences of two drafts, most with rows whose scaled logits lie beyond +-4e6."""
+    B, K = 10, 2
+    cfg = G.Config("far", B, K, V, dtype, 2.0, False, 0.5, 1.0, seed=V)
+    x = G.make_inputs(cfg, DEV, pad_ld=(-V) % 8)
+    t, d, low = x["target"], x["draft"], float(torch.finfo(TYPES[dtype]).min)
+    tau = torch.ones(B, device=DEV)
+    t[1, 0] = low                                            # a target row that is nothing but mask: p uniform
+    d[2, 1] = -1e9; t[2, 1] = -1e9                           # both rows of a position
+    t[3] = 1e9; d[3] = 1e9; t[3, :, : V // 2] = 1.1e9        # far up: p uniform over one half, q over all
+    tau[4] = 1e-6                                            # ordinary logits, carried out by the temperature
+    tau[5] = 1e-6; t[5] -= 20; d[5] -= 20
+    d[6] = t[6, :2]; t[6, 2] = -1e9                          # the bonus row alone
+    t[7, :, V // 3:] = low; d[7, :, V // 3:] = -1e9          # masks beside ordinary logits: nothing is far out
+    t[8, 1] = 3e38; t[8, 1, 5:] = -3e38; d[8, 1] = t[8, 1]   # both ends of the type
+    t[9, 0] = -1e9; t[9, 1, 3] = float("nan")                # a bad row behind a far one
+    x["temperature"] = tau
+    x["draft_tokens"] = d.float().argmax(-1).int().contiguous()
+    x["draft_tokens"][3, 0] = V - 1                          # p(x) = 0 there: rejected
+    x["u_accept"][6] = 0.5
+    return x
+
+
+@pytest.mark.parametrize("dtype,V", [("f32", 1024), ("bf16", 1024), ("bf16", 2051), ("f32", 30001), ("bf16", 65536)])
+@pytest.mark.parametrize("kappa", [-1.0, 1e9])               # (1e9: no fp32 draw clears its bound)
+def test_rows_far_from_zero(kernel_path, dtype, V, kappa):
+    if kernel_path not in FAR_PATHS:
+        pytest.skip("not through this kernel")
+    x = far_inputs(dtype, V)
+    ref = oracle_on(x)
+    P.bebop_debug_set_draw_kappa(kappa)
+    try:
+        got = run_verify(x)
+        bare = run_verify(x, want_tv=False, want_probs=False, want_status=False)
+    finally:
+        P.bebop_debug_set_draw_kappa(-1.0)
+    compare_verify(got, ref, dtype)
+    assert to_np(got["row_status"])[9] == 1 and (to_np(got["out_tokens"])[:9, 0] >= 0).all()
+    for k in ("accept_len", "out_tokens"):                   # the optional outputs change nothing
+        assert torch.equal(bare[k], got[k]), k
+    # the call after it, on the same workspace, with ordinary rows
+    y = G.make_inputs(x["cfg"], DEV, pad_ld=(-V) % 8)
+    compare_verify(run_verify(y, workspace=got["workspace"]), oracle_on(y), dtype)
+
+
+@pytest.mark.parametrize("dtype,V", [("f32", 1024), ("bf16", 2051), ("f32", 30001), ("bf16", 65536)])
+def test_tv_of_rows_far_from_zero(kernel_path, dtype, V):
+    if kernel_path not in FAR_PATHS:
+        pytest.skip("not through this kernel")
+    x = far_inputs(dtype, V)
+    n = x["target"].shape[0] * 2
+    tgt = torch.cat([x["target"][:, 0], x["target"][:, 1]])
+    drf = torch.cat([x["draft"][:, 0], x["draft"][:, 1]])
+    pad = lambda r: torch.cat([r, torch.zeros(n, (-V) % 8, dtype=r.dtype, device=DEV)], 1)[:, :V]
+    check_tv(pad(tgt), pad(drf), x["temperature"].repeat(2), dtype)
