@@ -64,26 +64,16 @@ inline int64_t row_distance(const at::Tensor& t, int64_t ndim) {
 }
 inline void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// New outputs, on the inputs' device: pieces of one block straight from the allocator.  One by one through the dispatcher
-// an output costs 1 us, and the smallest calls of bebop_tv and of the greedy mode, with three outputs each, were bound by
-// that (6.2 us a call; 5.5 with three blocks straight from the allocator).
+// New outputs, on the inputs' device, each with a storage of its own, straight from the allocator.  (As pieces of one block they
+// cost 0.45 us less apiece -- a greedy call of the smallest size 4.1 us instead of 5.0, bebop_verify without given buffers
+// 4.9 instead of 7.6 -- but then a resize_() of one runs into the next, saving one saves all, and holding one holds all.
+// Building the tensors by hand on the allocator's blocks is no faster than empty_cuda.)
 struct Maker {
     at::Device dev;
-    bool poison;                        // filled with a value no call leaves, one by one (tests)
-    int64_t bytes;                      // what all outputs of the call may need
-    at::Tensor block = {};
-    int64_t used = 0;
-    static constexpr int64_t kAlign = 256;
-    Maker(at::Device d, bool p, std::initializer_list<int64_t> words) : dev(d), poison(p), bytes(0) { for (int64_t w : words) bytes += (4 * w + kAlign - 1) / kAlign * kAlign; }
-    at::Tensor make(at::IntArrayRef shape, at::ScalarType type) {       // (int32 or float32)
+    bool poison;                        // filled with a value no call leaves (tests)
+    at::Tensor make(at::IntArrayRef shape, at::ScalarType type) const {       // (int32 or float32)
         if (poison) return at::full(shape, -77, at::TensorOptions().dtype(type).device(dev));
-        if (!block.defined()) block = at::Tensor(at::detail::empty_cuda({bytes}, at::kByte, dev, c10::nullopt));
-        auto t = at::detail::make_tensor<c10::TensorImpl>(c10::Storage(block.storage()), c10::DispatchKeySet(c10::DispatchKey::CUDA), c10::scalarTypeToTypeMeta(type));
-        c10::TensorImpl* const i = t.unsafeGetTensorImpl();
-        i->set_sizes_contiguous(shape);
-        i->set_storage_offset(used / 4);
-        used += (4 * t.numel() + kAlign - 1) / kAlign * kAlign;
-        return t;
+        return at::Tensor(at::detail::empty_cuda(shape, type, dev, c10::nullopt));
     }
 };
 // a result dictionary that owns what is put into it
@@ -102,7 +92,7 @@ struct Dict {
     PyObject* release() { PyObject* r = d; d = nullptr; return r; }
 };
 // the caller's buffer for an output, a new one, or none
-void* output(Dict& d, PyObject* out, PyObject* key, Maker& m, at::IntArrayRef shape, at::ScalarType type, bool want) {
+void* output(Dict& d, PyObject* out, PyObject* key, const Maker& m, at::IntArrayRef shape, at::ScalarType type, bool want) {
     if (given(out)) {
         PyObject* o = PyDict_GetItemWithError(out, key);
         if (!o && PyErr_Occurred()) throw Raised();
@@ -158,8 +148,7 @@ PyObject* py_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
         need(dr.scalar_type() == tg.scalar_type() && dr.dim() == 3 && dr.size(0) == B && dr.size(1) == K && dr.size(2) == V,
              "draft_logits must be [B, K, V] of the target's type");
         const int64_t ldt = row_distance(tg, 3), ldd = row_distance(dr, 3);
-        const int64_t b1 = B, bk = (int64_t)B * K;
-        Maker m(tg.device(), truth(a[13]), {b1, b1 + bk, bk, bk, bk, b1});
+        const Maker m{tg.device(), truth(a[13])};
         const bool want_tv = truth(a[10]), want_probs = truth(a[11]), want_status = truth(a[12]);
         Dict d;
         int32_t* acc = (int32_t*)output(d, a[8], k_accept_len, m, {B}, at::kInt, true);
@@ -199,7 +188,7 @@ PyObject* py_tv(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const bebop_dtype_t dt = dtype_of(tg);
         need(dr.scalar_type() == tg.scalar_type() && dr.dim() == 2 && dr.size(0) == N && dr.size(1) == V, "draft_logits must be as target_logits");
         const int64_t ldt = row_distance(tg, 2), ldd = row_distance(dr, 2);
-        Maker m(tg.device(), truth(a[7]), {N, N, N});
+        const Maker m{tg.device(), truth(a[7])};
         Dict d;
         float* tv = (float*)output(d, Py_None, k_tv, m, {N}, at::kFloat, true);
         float* sx = (float*)output(d, Py_None, k_s_aux, m, {N}, at::kFloat, truth(a[5]));
@@ -229,7 +218,7 @@ PyObject* py_greedy(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int64_t ldt = row_distance(tg, 3);
         const at::Tensor& tok = tensor(a[1]);
         need(tok.scalar_type() == at::kInt && tok.is_contiguous() && tok.is_cuda(), "draft_tokens must be contiguous int32 on the device");
-        Maker m(tg.device(), truth(a[4]), {B, (int64_t)B * (K + 1), B});
+        const Maker m{tg.device(), truth(a[4])};
         Dict d;
         int32_t* acc = (int32_t*)output(d, Py_None, k_accept_len, m, {B}, at::kInt, true);
         int32_t* out = (int32_t*)output(d, Py_None, k_out_tokens, m, {B, K + 1}, at::kInt, true);
