@@ -11,6 +11,7 @@
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/bebop.h"
@@ -133,7 +134,7 @@ template <typename F> PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
     catch (const Code& c) { return PyLong_FromLong(c.v); }
     catch (const Bad& b) { PyErr_SetString(PyExc_AssertionError, b.what); return nullptr; }
     catch (const Raised&) { return nullptr; }
-    catch (const std::exception& e) { PyErr_SetString(PyExc_RuntimeError, e.what()); return nullptr; }
+    catch (...) { torch::translate_exception_to_python(std::current_exception()); return nullptr; }      // torch's own types: OutOfMemoryError and the like
 }
 
 // target, draft, draft_tokens, u_accept, u_final, draft_len, temperature, temperature_all, out, workspace, want_tv,

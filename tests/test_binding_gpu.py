@@ -64,3 +64,24 @@ def test_new_outputs_given_outputs_and_none_agree(x):
     assert torch.equal(r["tv"], full["tv"]) and torch.equal(r["out_tokens"], full["out_tokens"])
     t = P.bebop_tv(x["target"][:, 0], x["draft"][:, 0], want_s_aux=False, want_status=False)
     assert t["s_aux"] is None and t["row_status"] is None and t["tv"].shape == (5,)
+
+
+# ------------------------------------------------------------------ exceptions
+def test_an_allocation_that_fails_raises_what_torch_raises(x):
+    """Programs catch torch.cuda.OutOfMemoryError to free memory and call again.  The allocator's limit for this process is set to
+    what it holds already (and put back)."""
+    torch.cuda.synchronize(); torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    hold = []
+    torch.cuda.set_per_process_memory_fraction(torch.cuda.memory_reserved() / total)
+    try:
+        for n in (1 << 21, 1 << 9):                          # what is free inside the blocks held
+            with pytest.raises(torch.cuda.OutOfMemoryError):
+                while True:
+                    hold.append(torch.empty(n, dtype=torch.uint8, device=DEV))
+        with pytest.raises(torch.cuda.OutOfMemoryError):
+            verify(x)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+        hold.clear()
+    assert verify(x)["accept_len"].shape == (5,)
