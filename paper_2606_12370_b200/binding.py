@@ -160,13 +160,13 @@ def bebop_tv(target_logits, draft_logits, temperature=None, temperature_all=1.0,
              want_s_aux=True, want_status=True):
     """TV distance (and the auxiliary S) of N paired rows [N,V]."""
     return _result((_host or _load_host()).tv(target_logits, draft_logits, temperature, temperature_all, workspace, want_s_aux, want_status,
-                                              POISON_OUTPUTS))
+                                              POISON_OUTPUTS, False))
 
 
 def bebop_tv_static(target_logits, draft_logits, temperature=None, temperature_all=1.0, want_s_aux=True):
     """bebop_tv with the library's built-in scratch instead of a workspace (no allocation in the call)."""
-    return _result((_host or _load_host()).tv(target_logits, draft_logits, temperature, temperature_all, False, want_s_aux, True,
-                                              POISON_OUTPUTS))
+    return _result((_host or _load_host()).tv(target_logits, draft_logits, temperature, temperature_all, None, want_s_aux, True,
+                                              POISON_OUTPUTS, True))
 
 
 def bebop_greedy_verify(target_logits, draft_tokens, draft_len=None, workspace=None):

@@ -30,6 +30,7 @@ PyObject *k_accept_len, *k_out_tokens, *k_tv, *k_p_draft, *k_q_draft, *k_row_sta
 struct Code { long v; };
 struct Bad { const char* what; };      // AssertionError
 struct Raised {};                      // a Python error is set
+struct Shape { const char* what; };    // ValueError
 constexpr long kNotCuda = -8, kBadDtype = -3;
 
 inline void need(bool ok, const char* what) { if (!ok) throw Bad{what}; }
@@ -37,6 +38,7 @@ inline const at::Tensor& tensor(PyObject* o) {
     if (!THPVariable_Check(o)) { PyErr_SetString(PyExc_TypeError, "a tensor is expected"); throw Raised(); }
     return THPVariable_Unpack(o);
 }
+inline void need_rank(const at::Tensor& t, int64_t n, const char* what) { if (t.dim() != n) throw Shape{what}; }
 inline bool given(PyObject* o) { return o != Py_None; }
 inline bool truth(PyObject* o) {
     if (o == Py_True) return true;
@@ -46,8 +48,11 @@ inline bool truth(PyObject* o) {
     return t != 0;
 }
 inline float number(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Raised();
+    if (PyFloat_CheckExact(o)) return (float)PyFloat_AS_DOUBLE(o);
+    PyObject* const f = PyNumber_Float(o);                  // what float() takes
+    if (!f) throw Raised();
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
     return (float)v;
 }
 inline bebop_dtype_t dtype_of(const at::Tensor& t) {
@@ -133,6 +138,7 @@ template <typename F> PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
     try { return f(); }
     catch (const Code& c) { return PyLong_FromLong(c.v); }
     catch (const Bad& b) { PyErr_SetString(PyExc_AssertionError, b.what); return nullptr; }
+    catch (const Shape& b) { PyErr_SetString(PyExc_ValueError, b.what); return nullptr; }
     catch (const Raised&) { return nullptr; }
     catch (...) { torch::translate_exception_to_python(std::current_exception()); return nullptr; }      // torch's own types: OutOfMemoryError and the like
 }
@@ -143,7 +149,7 @@ PyObject* py_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 14, [&]() -> PyObject* {
         const at::Tensor& tg = tensor(a[0]);
         const at::Tensor& dr = tensor(a[1]);
-        need(tg.dim() == 3, "target_logits must be [B, K+1, V]");
+        need_rank(tg, 3, "target_logits must be [B, K+1, V]");
         const int B = (int)tg.size(0), K = (int)tg.size(1) - 1, V = (int)tg.size(2);
         const bebop_dtype_t dt = dtype_of(tg);
         need(dr.scalar_type() == tg.scalar_type() && dr.dim() == 3 && dr.size(0) == B && dr.size(1) == K && dr.size(2) == V,
@@ -179,12 +185,12 @@ PyObject* py_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
-// target, draft, temperature, temperature_all, workspace (False: the built-in scratch), want_s_aux, want_status, poison
+// target, draft, temperature, temperature_all, workspace, want_s_aux, want_status, poison, whether the built-in scratch takes the workspace's place
 PyObject* py_tv(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    return guarded(n, 8, [&]() -> PyObject* {
+    return guarded(n, 9, [&]() -> PyObject* {
         const at::Tensor& tg = tensor(a[0]);
         const at::Tensor& dr = tensor(a[1]);
-        need(tg.dim() == 2, "target_logits must be [N, V]");
+        need_rank(tg, 2, "target_logits must be [N, V]");
         const int N = (int)tg.size(0), V = (int)tg.size(1);
         const bebop_dtype_t dt = dtype_of(tg);
         need(dr.scalar_type() == tg.scalar_type() && dr.dim() == 2 && dr.size(0) == N && dr.size(1) == V, "draft_logits must be as target_logits");
@@ -199,7 +205,7 @@ PyObject* py_tv(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const void* tp = tg.data_ptr();
         const void* dp = dr.data_ptr();
         void* const s = stream();
-        if (a[4] == Py_False) {
+        if (truth(a[8])) {
             call([&] { return f_tv_static(tp, ldt, dp, ldd, temp, tau, N, V, dt, tv, sx, st, s); });
         } else {
             const Space ws = workspace_of(a[4], N, 1, V, dt, m.dev);
@@ -213,7 +219,7 @@ PyObject* py_tv(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_greedy(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 5, [&]() -> PyObject* {
         const at::Tensor& tg = tensor(a[0]);
-        need(tg.dim() == 3, "target_logits must be [B, K+1, V]");
+        need_rank(tg, 3, "target_logits must be [B, K+1, V]");
         const int B = (int)tg.size(0), K = (int)tg.size(1) - 1, V = (int)tg.size(2);
         const bebop_dtype_t dt = dtype_of(tg);
         const int64_t ldt = row_distance(tg, 3);

@@ -85,3 +85,24 @@ def test_an_allocation_that_fails_raises_what_torch_raises(x):
         torch.cuda.set_per_process_memory_fraction(1.0)
         hold.clear()
     assert verify(x)["accept_len"].shape == (5,)
+
+
+def test_what_the_binding_takes_and_refuses(x):
+    t, d = x["target"][:, 0], x["draft"][:, 0]
+    want = P.bebop_tv(t, d, temperature_all=0.5)["tv"]
+    for tau in (0.5, "0.5", torch.tensor(0.5), torch.tensor([0.5], device=DEV)):      # whatever float() takes
+        assert torch.equal(P.bebop_tv(t, d, temperature_all=tau)["tv"], want)
+    assert torch.equal(P.bebop_tv(t, d, temperature_all=1)["tv"], P.bebop_tv(t, d)["tv"])
+    for bad in (lambda: P.bebop_tv(x["target"], x["draft"]), lambda: P.bebop_greedy_verify(t, x["draft_tokens"]), lambda: P.bebop_verify(
+            t, d, x["draft_tokens"], x["u_accept"], x["u_final"])):
+        with pytest.raises(ValueError):
+            bad()
+    for bad in (False, True, 0, "no"):                       # a workspace is a tensor or None
+        with pytest.raises((TypeError, AttributeError)):
+            P.bebop_tv(t, d, workspace=bad)
+    with pytest.raises(P.BebopError) as e:
+        P.bebop_tv(t, d, workspace=torch.empty(256, dtype=torch.uint8, device=DEV))
+    assert e.value.code == 5
+    with pytest.raises(P.BebopError) as e:
+        P.bebop_tv(t.half(), d.half())
+    assert e.value.code == 3
