@@ -53,9 +53,10 @@ struct __align__(16) QRec { double s, ub; int e, bad; double pad; };    // a row
 struct __align__(16) QStat { double inv_s, ub; int e, st; double pad; };
 
 // ------------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() { __syncwarp(); cluster_arrive(); cluster_wait(); }
+// (aligned: all lanes of a warp execute them together, which nothing but a __syncwarp() makes a warp do that has split before)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 // the address of `p` (this CTA's shared memory) in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t at_rank(const void* p, int rank) {
@@ -408,7 +409,6 @@ __global__ void __launch_bounds__(kSeqThreads, 2) k_seq(const __grid_constant__ 
     double* const raux = reinterpret_cast<double*>(tables + a.p.o_raux);
     unsigned long long* const bar = reinterpret_cast<unsigned long long*>(tables + a.p.o_bar);
     auto row_of = [&](int i) { return smem + (size_t)i * sv * 16; };          // row 2k: target k, 2k + 1: draft k, 2L: bonus
-    __syncwarp();
     cluster_arrive();                                       // (waited for before the first store into another CTA)
     if (warp == 0) {
         for (int i = lane; i < a.p.rows; i += 32) mbar_init(&bar[i], 1);
@@ -626,7 +626,6 @@ __global__ void __launch_bounds__(kSeqThreads, 2) k_seq_greedy(const __grid_cons
     const int rank = (int)cluster_rank(), b = (int)(blockIdx.x / (unsigned)a.C), K = R.K;
     QMax* const part = reinterpret_cast<QMax*>(smem);                       // [K + 1][nch]
     QMax* const all = part + (K + 1) * a.nch;                               // [K + 1][C] by rank
-    __syncwarp();
     cluster_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");       // (as in k_seq)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
