@@ -168,7 +168,8 @@ bebop_status_t bebop_greedy_verify(
  * wherever it applies; 3 the fused kernel wherever it applies (the greedy mode has no fused form); 4 the sequence kernel
  * wherever it applies.  All give the same results up to the documented tolerances.  bebop_debug_last_kernel() says
  * what the last of these calls ran: 1 the general kernels, 2 the pipelined kernel, 3 a kernel that reads every logit
- * once, the fused or the sequence kernel (0: no call yet).
+ * once, the fused or the sequence kernel (0: no call yet); bebop_debug_last_kernel_name() says it by the main kernel's name:
+ * "general", "k_pipe", "k_fuse", "k_seq", "k_seq_greedy" ("none": no call yet).
  * bebop_debug_fallback_offset returns the byte offset, inside the workspace of this
  * shape, of an int32 that after a bebop_verify call through the pipelined or the fused kernel holds the number of
  * sequences whose draw was re-done by the fp64 kernels.
@@ -185,6 +186,7 @@ bebop_status_t bebop_greedy_verify(
  */
 void bebop_debug_force_general_path(int on);
 int bebop_debug_last_kernel(void);
+const char* bebop_debug_last_kernel_name(void);
 size_t bebop_debug_fallback_offset(int B, int K, int V, bebop_dtype_t dt);
 void bebop_debug_set_timing_events(void* start, void* stop);
 void bebop_debug_expire_wait(int which);

@@ -56,6 +56,8 @@ def load_library():
     lib.bebop_debug_set_timing_events.argtypes = [vp, vp]
     lib.bebop_debug_last_kernel.restype = C.c_int
     lib.bebop_debug_last_kernel.argtypes = []
+    lib.bebop_debug_last_kernel_name.restype = C.c_char_p
+    lib.bebop_debug_last_kernel_name.argtypes = []
     lib.bebop_debug_set_draw_kappa.restype = None
     lib.bebop_debug_set_draw_kappa.argtypes = [f32]
     lib.bebop_debug_expire_wait.restype = None
@@ -110,8 +112,14 @@ def bebop_debug_force_general_path(on) -> None:
 
 
 def bebop_debug_last_kernel() -> int:
-    """What the last bebop_verify / bebop_tv / bebop_greedy_verify call ran: 1 general kernels, 2 pipelined kernel, 3 fused kernel."""
+    """What the last bebop_verify / bebop_tv / bebop_greedy_verify call ran: 1 general kernels, 2 pipelined kernel,
+    3 a kernel that reads every logit once (fused or sequence kernel)."""
     return int(load_library().bebop_debug_last_kernel())
+
+
+def bebop_debug_last_kernel_name() -> str:
+    """The main kernel of the last of these calls: "general", "k_pipe", "k_fuse", "k_seq" or "k_seq_greedy" ("none": no call yet)."""
+    return load_library().bebop_debug_last_kernel_name().decode()
 
 
 def bebop_debug_set_draw_kappa(kappa) -> None:

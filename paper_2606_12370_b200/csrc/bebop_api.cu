@@ -7,12 +7,12 @@ using namespace bebop;
 
 namespace {
 
-// Test hook: route bebop_verify through the general (split-row) path even where the fused
-// kernel applies, so that both paths are covered by the parity tests.
-int g_last_kernel = 0;   // what the last call ran: 1 general kernels, 2 pipelined kernel, 3 a kernel that reads every logit once
-                         // (fused or sequence kernel)
-int g_path = 0;   // 0: the fastest for the shape; 1: general kernels only; 2: never a one-read kernel; 3: the fused kernel wherever
-                  // it applies; 4: the sequence kernel wherever it applies
+// Test hooks: what the last call ran -- 1 general kernels, 2 pipelined kernel, 3 a kernel that reads every logit once (fused or
+// sequence kernel) -- and the name of its main kernel;
+struct LastKernel { int id; const char* name; } g_last = {0, "none"};
+// and which kernels calls may take: 0 the fastest for the shape; 1 general kernels only; 2 never a one-read kernel; 3 the fused
+// kernel wherever it applies; 4 the sequence kernel wherever it applies.
+int g_path = 0;
 
 int g_expire_wait = 0;   // test hook: which device-side wait the next call lets give up at once
 float g_draw_kappa = -1.f;   // test hook: factor of the fast draw's error bound (negative: the built-in value)
@@ -113,18 +113,18 @@ bebop_status_t bebop_verify(const void* target_logits, int64_t ld_target, const 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     cudaError_t e = cudaSuccess;
     bool launched = false;
-    g_last_kernel = 1;
+    g_last = {1, "general"};
     if ((g_path == 4 && seq_supported(a, false)) || (g_path == 0 && seq_preferred(a, false))) {
         e = seq_verify(a, draft_tokens, u_accept, u_final, o, stream, &launched);
-        if (launched) g_last_kernel = 3;
+        if (launched) g_last = {3, "k_seq"};
     }
     if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, false))) && fuse_supported(a)) {
         e = fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
-        if (launched) g_last_kernel = 3;
+        if (launched) g_last = {3, "k_fuse"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
         e = pipe_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
-        if (launched) g_last_kernel = 2;
+        if (launched) g_last = {2, "k_pipe"};
     }
     if (e == cudaSuccess && !launched) e = general_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream);
     return e == cudaSuccess ? BEBOP_OK : BEBOP_ERR_CUDA;
@@ -150,19 +150,19 @@ bebop_status_t bebop_tv(const void* target_logits, int64_t ld_target, const void
     cudaError_t e = cudaSuccess;
     bool launched = false;
     VerifyOut o{nullptr, nullptr, tv, nullptr, nullptr, row_status};
-    g_last_kernel = 1;
+    g_last = {1, "general"};
     if ((g_path == 4 && seq_supported(a, true)) || (g_path == 0 && seq_preferred(a, true))) {
         e = seq_verify(a, nullptr, nullptr, nullptr, o, stream, &launched, true, s_aux);
-        if (launched) g_last_kernel = 3;
+        if (launched) g_last = {3, "k_seq"};
     }
     if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, true))) && fuse_supported(a)) {
         e = fuse_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
-        if (launched) g_last_kernel = 3;
+        if (launched) g_last = {3, "k_fuse"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
         // the pipelined kernel with row pairs in place of sequences: first sweep, second sweep, no draw
         e = pipe_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
-        if (launched) g_last_kernel = 2;
+        if (launched) g_last = {2, "k_pipe"};
     }
     if (e == cudaSuccess && !launched)
         e = general_tv(a, p, tv, s_aux, row_status, static_cast<char*>(workspace), stream);
@@ -187,14 +187,14 @@ bebop_status_t bebop_greedy_verify(const void* target_logits, int64_t ld_target,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     cudaError_t e = cudaSuccess;
     bool launched = false;
-    g_last_kernel = 1;
+    g_last = {1, "general"};
     if (g_path == 4 || (g_path == 0 && seq_greedy_preferred(a))) {
         e = seq_greedy(a, draft_tokens, accept_len, out_tokens, row_status, stream, &launched);
-        if (launched) g_last_kernel = 3;
+        if (launched) g_last = {3, "k_seq_greedy"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
         e = pipe_greedy(a, p, draft_tokens, accept_len, out_tokens, row_status, static_cast<char*>(workspace), stream, &launched);
-        if (launched) g_last_kernel = 2;
+        if (launched) g_last = {2, "k_pipe"};
     }
     if (e == cudaSuccess && !launched)
         e = general_greedy(a, p, draft_tokens, accept_len, out_tokens, row_status, static_cast<char*>(workspace), stream);
@@ -236,7 +236,9 @@ bebop_status_t bebop_tv_static(const void* target_logits, int64_t ld_target, con
 
 void bebop_debug_force_general_path(int on) { g_path = on; }
 
-int bebop_debug_last_kernel(void) { return g_last_kernel; }
+int bebop_debug_last_kernel(void) { return g_last.id; }
+
+const char* bebop_debug_last_kernel_name(void) { return g_last.name; }
 
 void bebop_debug_expire_wait(int which) { g_expire_wait = which; }
 

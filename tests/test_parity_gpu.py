@@ -15,14 +15,13 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-PATHS = {"pipe": 2, "general": 1, "fuse": 3}
+PATHS = {"pipe": 2, "general": 1, "fuse": 3, "seq": 4}
 
 
-@pytest.fixture(autouse=True, params=["pipe", "general", "fuse"])
+@pytest.fixture(autouse=True, params=["pipe", "general", "fuse", "seq"])
 def kernel_path(request):
-    """Every test runs three times: through the pipelined kernel and through the fused kernel where the shape admits
-    them, and through the general split-row kernels.  (Left alone, the library picks the faster of the first two for
-    the shape: the other GPU test files run that way.)"""
+    """Every test runs four times: through the pipelined, the fused and the sequence kernel where the shape admits
+    them, and through the general split-row kernels.  (Left alone, the library picks the fastest for the shape.)"""
     P.bebop_debug_force_general_path(PATHS[request.param])
     yield request.param
     P.bebop_debug_force_general_path(0)
@@ -122,7 +121,7 @@ def test_every_sequence_goes_to_the_fp64_redraw(dtype, kernel_path):
     got = run_verify(x)
     got = run_verify(x, workspace=got["workspace"])     # the second call finds the first call's records there
     torch.cuda.synchronize()
-    if kernel_path != "general":
+    if kernel_path in ("pipe", "fuse"):                 # (the sequence kernel re-draws on the spot and keeps no count)
         off = P.bebop_debug_fallback_offset(cfg.B, cfg.K, cfg.V, 0 if dtype == "f32" else 1)
         assert int(got["workspace"][off:off + 4].view(torch.int32).item()) == cfg.B
     check_properties(got, x)

@@ -13,7 +13,7 @@ from parity import TOL, compare_verify, oracle_on, to_np
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
-PATHS = {"pipe": 2, "general": 1, "fuse": 3}
+PATHS = {"pipe": 2, "general": 1, "fuse": 3, "seq": 4}
 
 
 def run_verify(x, **kw):
@@ -92,7 +92,7 @@ def _intact(buf, nbytes):
     return bool((buf[:GUARD] == 0xA5).all()) and bool((buf[GUARD + nbytes:] == 0xA5).all())
 
 
-@pytest.mark.parametrize("path", ["pipe", "general", "fuse"])
+@pytest.mark.parametrize("path", ["pipe", "general", "fuse", "seq"])
 @pytest.mark.parametrize("dtype,B,K,V", [("f32", 9, 2, 1000), ("bf16", 9, 2, 8), ("bf16", 5, 32, 4096), ("f32", 3, 1, 70001),
                                           ("bf16", 7, 3, 3 * 151936 // 2), ("bf16", 300, 1, 2040)])
 def test_kernels_stay_inside_the_workspace(path, dtype, B, K, V):
@@ -122,7 +122,7 @@ def test_kernels_stay_inside_the_workspace(path, dtype, B, K, V):
 
 
 # --------------------------------------------------------------------------- greedy, signed zeros
-@pytest.mark.parametrize("path", ["pipe", "general"])
+@pytest.mark.parametrize("path", ["pipe", "general", "seq"])
 def test_greedy_lowest_index_among_signed_zeros(path):
     """A row whose maximum is zero with both signs present: -0.0 at a low index, +0.0 later (in another warp's and
     another slice's range).  The two are equal, so the lowest index wins."""
@@ -145,13 +145,14 @@ def test_greedy_lowest_index_among_signed_zeros(path):
 
 
 # ------------------------------------------------------------- the fast draw's bound over many seeds
-@pytest.mark.parametrize("path", ["pipe", "fuse"])
+@pytest.mark.parametrize("path", ["pipe", "fuse", "seq"])
 def test_fast_draw_bound_over_many_seeds_and_temperatures(path):
     """bebop_verify against the oracle on more than 5,000 sequences at V = 151936: 24 seeds, four temperatures, the
     peaked (rollout) and the flat (high-entropy) recipe, residual and bonus draws.  No unflagged mismatch is allowed,
-    flagged draws stay below 1e-4, and the share of sequences the fp64 re-draw had to decide is reported.  Both
+    flagged draws stay below 1e-4, and the share of sequences the fp64 re-draw had to decide is reported.  All
     kernels that keep fast draws: they bound the error in different ways (the pipelined one from the rows' sums of
-    squares, the fused one from the rows' largest probabilities)."""
+    squares, the fused and the sequence kernel from upper bounds of them per chunk; the sequence kernel re-draws on the spot and
+    does not count)."""
     P.bebop_debug_force_general_path(PATHS[path])
     B, K, V = 224, 3, 151936
     seen = flagged = draws = redrawn = bonus = 0
@@ -165,6 +166,7 @@ def test_fast_draw_bound_over_many_seeds_and_temperatures(path):
         if seed % 3 == 0:                                   # a third of the batches: short drafts, so more bonus draws
             x["draft_len"] = torch.tensor([i % 2 for i in range(B)], dtype=torch.int32, device=DEV)
         got = run_verify(x)
+        assert P.bebop_debug_last_kernel_name() == "k_" + path
         torch.cuda.synchronize()
         off = P.bebop_debug_fallback_offset(B, K, V, 1)
         redrawn += int(got["workspace"][off:off + 4].view(torch.int32).item())
@@ -185,10 +187,11 @@ def test_fast_draw_bound_over_many_seeds_and_temperatures(path):
             wrong[kap] += int(((to_np(g2["out_tokens"]) != ref["out_tokens"]).any(axis=1) & ok).sum())
     P.bebop_debug_force_general_path(0)
     print("\nfast-draw bound (%s kernel): %d sequences (%d bonus draws), %d draws, %d flagged by the oracle (%.2e), "
-          "%d re-drawn in fp64 (%.2f %%), 0 unflagged mismatches"
-          % (path, seen, bonus, draws, flagged, flagged / draws, redrawn, 100.0 * redrawn / seen))
+          "%s re-drawn in fp64, 0 unflagged mismatches"
+          % (path, seen, bonus, draws, flagged, flagged / draws, "not counted" if path == "seq" else "%d (%.2f %%)" % (redrawn, 100.0 * redrawn / seen)))
     for kap in kappas:
-        print("  factor %.2f: %d of %d draws kept in fp32, %d of them differ from the oracle" % (kap, kept[kap], seen, wrong[kap]))
+        print("  factor %.2f: %s of %d draws kept in fp32, %d of them differ from the oracle"
+              % (kap, "not counted" if path == "seq" else kept[kap], seen, wrong[kap]))
     assert seen >= 5000 and flagged <= 1e-4 * draws + 1
     assert wrong[1.0] == 0, "a quarter of the built-in factor already lets a wrong token through"
 
@@ -232,3 +235,31 @@ def test_the_sign_of_p_minus_q_below_fp32_resolution(path, dtype):
         assert np.abs(to_np(got["tv"]) - ref["tv"]).max() <= 1e-9      # TV is 3e-8: sums of 4,096 terms of fp32, about 1e-10 off
     finally:
         P.bebop_debug_force_general_path(0)
+
+
+def test_the_kernel_behind_each_entry_point_by_name():
+    """The choice on both sides of its lines: small calls and short rows, the fused kernel's rows and calls, large vocabularies,
+    rows beyond all of them."""
+    dt = {"f32": torch.float32, "bf16": torch.bfloat16}
+    def call(op, B, K, V, dtype="bf16"):
+        ld = V + (-V) % 8
+        rows = lambda R: torch.zeros((B, R, ld), dtype=dt[dtype], device=DEV)[:, :, :V]
+        tok = torch.zeros((B, K), dtype=torch.int32, device=DEV)
+        if op == "tv":
+            r = P.bebop_tv(rows(1)[:, 0], rows(1)[:, 0])
+            assert (to_np(r["tv"]) == 0).all()
+        elif op == "greedy":
+            r = P.bebop_greedy_verify(rows(K + 1), tok)
+            assert (to_np(r["accept_len"]) == K).all()
+        else:
+            r = P.bebop_verify(rows(K + 1), rows(K), tok, torch.full((B, K), 0.5, device=DEV), torch.full((B,), 0.5, device=DEV))
+            assert (to_np(r["accept_len"]) == K).all()
+        assert (to_np(r["row_status"]) == 0).all()
+        return P.bebop_debug_last_kernel_name()
+    for args, want in ((("verify", 4, 3, 1024, "f32"), "k_seq"), (("verify", 1, 3, 151936), "k_seq"), (("verify", 24, 5, 49999, "f32"), "k_seq"),
+                       (("verify", 400, 3, 8192), "k_seq"), (("verify", 16, 3, 151936), "k_fuse"), (("verify", 64, 3, 151936), "k_fuse"),
+                       (("verify", 192, 7, 32000), "k_fuse"), (("verify", 200, 3, 151936), "k_pipe"), (("verify", 100, 3, 262144), "k_pipe"),
+                       (("verify", 1, 1, 1100000), "general"), (("tv", 100, 1, 32003, "f32"), "k_seq"), (("tv", 1, 1, 1024), "k_seq"),
+                       (("tv", 200, 1, 151936), "k_fuse"), (("tv", 40, 1, 400000), "k_pipe"), (("greedy", 4, 3, 1024), "k_seq_greedy"),
+                       (("greedy", 50, 5, 151936), "k_seq_greedy"), (("greedy", 256, 5, 151936), "k_pipe"), (("greedy", 1, 1, 1100000), "k_seq_greedy")):
+        assert call(*args) == want, args

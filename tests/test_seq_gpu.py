@@ -59,6 +59,7 @@ def test_tv_and_greedy(dtype, B, K, V):
     tau = torch.linspace(0.6, 1.2, B, device=DEV)
     tau[0] = -1.0 if B > 1 else 1.0
     got = P.bebop_tv(tgt, drf, temperature=tau)
+    assert P.bebop_debug_last_kernel_name() == "k_seq"
     ref = oracle.tv(tgt.float().cpu().numpy(), drf.float().cpu().numpy(), temperature=to_np(tau))
     np.testing.assert_array_equal(to_np(got["row_status"]), ref["row_status"])
     assert np.abs(to_np(got["tv"]) - ref["tv"]).max() <= TOL[dtype]
@@ -66,6 +67,7 @@ def test_tv_and_greedy(dtype, B, K, V):
     x["target"][0, 0, V - 1] = float("nan")
     x["target"][B - 1, K, :] = float("-inf")
     g = P.bebop_greedy_verify(x["target"], x["draft_tokens"])
+    assert P.bebop_debug_last_kernel_name() == "k_seq_greedy"
     r = oracle.greedy_verify(x["target"].float().cpu().numpy(), to_np(x["draft_tokens"]))
     for k in ("accept_len", "out_tokens", "row_status"):
         np.testing.assert_array_equal(to_np(g[k]), r[k], err_msg=k)
