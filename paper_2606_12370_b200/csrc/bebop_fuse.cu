@@ -80,9 +80,9 @@ struct __align__(16) FTask {
 struct __align__(16) FScale { double inv_p, inv_q; int ep, eq; float rho_h, rho_l; int stp, stq, pad0, pad1; };
 struct __align__(16) FWarpE { int ep, eq, flags, pad; };               // a consumer warp's exponents of a task
 // Softmax partial of one slice of one row; each 8-byte word is valid by itself once non-zero.  `flags`: bit 0 says
-// that the slice holds a NaN or +inf; the other bits are those of a float u, with which the slice's sum of e^2
-// (around the slice's exponent) is at most sqrt(2) u: u = sum over the warp chunks of 4^(E_w - E_s) times the
-// chunk's sum of e, as the e of a chunk are at most sqrt(2) around the chunk's own exponent.
+// that the slice holds a NaN or +inf; the other bits are those of a float u, an upper bound of the slice's sum of e^2
+// (around the slice's exponent): the sum over the warp chunks of 4^(E_w - E_s) times the chunk's sum of e, as the e of a
+// chunk are at most 1 around the chunk's own exponent.
 struct __align__(16) FRec { double s; int ecode; int flags; };
 __device__ __forceinline__ float rec_ub(const FRec& r) { return __int_as_float(r.flags & ~1); }
 struct __align__(16) FRow { double inv_s; int e; int st; };           // a merged row: 1/S, exponent, status bits
@@ -981,8 +981,8 @@ __device__ __noinline__ void f_finish_seq(const FuseArgs& a, FShared& S, int b, 
     FRow rq = shfl_row(sq, pair ? nn : 0);
     if (!pair) { rq.inv_s = 0.0; rq.e = E_EMPTY; rq.st = 0; }
     // The draw's error bound wants sum p^2 + q^2 over the row pair, for which the records carry an upper bound per slice
-    // (a chunk's e are at most sqrt(2) around its own exponent, so its sum of e^2 is at most sqrt(2) times its sum of e:
-    // chunks far below the row's largest logit count next to nothing, and a peaked row gets a bound close to the sum).
+    // (a chunk's e are at most 1 around its own exponent, so its sum of e^2 is at most its sum of e: chunks far below the row's
+    // largest logit count next to nothing, and a peaked row gets a bound close to the sum).
     double s2 = 0.0;
     if (pair) {
         const FRec* base = a.rec + ((int64_t)du * T) * 2;
@@ -1002,7 +1002,7 @@ __device__ __noinline__ void f_finish_seq(const FuseArgs& a, FShared& S, int b, 
         for (int i = 0; i < SPL; ++i) s2 += bu[i] * rp.inv_s * rp.inv_s;
     }
     s2 = warp_sum(s2);
-    const double bound = draw_bound(1.4142135623730951 * s2, (double)a.kappa);
+    const double bound = draw_bound(s2, (double)a.kappa);
     // the slices' masses (bonus row: sums of e around the row's exponent -> probabilities); the slice that owns u Z
     double sm[SPL];
 #pragma unroll

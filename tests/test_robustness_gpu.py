@@ -193,6 +193,7 @@ def test_fast_draw_bound_over_many_seeds_and_temperatures(path):
         print("  factor %.2f: %s of %d draws kept in fp32, %d of them differ from the oracle"
               % (kap, "not counted" if path == "seq" else kept[kap], seen, wrong[kap]))
     assert seen >= 5000 and flagged <= 1e-4 * draws + 1
+    assert redrawn <= 0.02 * seen, "the bound is wider than the weights (at most 1 around a chunk's exponent) make it"
     assert wrong[1.0] == 0, "a quarter of the built-in factor already lets a wrong token through"
 
 
