@@ -162,7 +162,7 @@ __device__ __forceinline__ double draw_bound(double sumsq, double kappa = kDrawK
 // is a sum of zero-mean terms of the size draw_bound() already allows per token.
 struct TempScale { float hi; };
 __device__ __forceinline__ TempScale temp_scale(float tau) {
-    TempScale r; r.hi = fminf(kLog2e / (tau_ok(tau) ? tau : 1.f), 3e38f);      // (finite: 0 * c is 0)
+    TempScale r; r.hi = kLog2e / (tau_ok(tau) ? tau : 1.f);
     return r;
 }
 struct DrawShared {

@@ -15,9 +15,9 @@
 // grid-wide meeting, no kernel behind it.  What other sequences do does not matter, so nothing can wait on a CTA that
 // has not started (a cluster is placed as a whole).
 //
-// What bounds it: latency.  A call of four sequences of 1,024 fp32 logits (K = 3) takes 11 us (28 through the pipelined
-// kernel with its clearing and its re-draw kernel): start 1.8, pass 1 0.5, the exchange 1.5, scan 0.4, pass 2 1.3, exchange 0.9, draw 2;
-// a re-draw adds 5 to 10 (24 when its exponentials were spread over the chunks' warps only).  One sequence of 151,936 bf16
+// What bounds it: latency.  A call of four sequences of 1,024 fp32 logits (K = 3) takes 7.5 to 7.9 us (28 through the pipelined
+// kernel with its clearing and its re-draw kernel); its parts, timed inside the kernel, are in that order of size: start 1.8, pass 1
+// 0.5, the exchange 1.5, scan 0.4, pass 2 1.3, exchange 0.9, draw 2.  A re-draw adds 5 to 10 (24 when its exponentials were spread over the chunks' warps only).  One sequence of 151,936 bf16
 // logits, sixteen CTAs of 133 KB: 16 us (32), of which the exponentials of the two passes take 7.
 #include "bebop_chunk.cuh"
 
@@ -73,6 +73,8 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b) {
     for (uint32_t i = 0; i < kQSpin; ++i) if (mbar_try(addr, 0)) return true;
     return false;
 }
+// log2(e) / tau, finite whatever tau: 0 * c is 0
+__device__ __forceinline__ float seq_scale(float tau) { return fminf(temp_scale(tau).hi, 3e38f); }
 // vector `vi` of a row slice of nv vectors; what lies beyond the slice or the vocabulary reads as -inf
 template <int DT>
 __device__ __forceinline__ uint4 slice_vec(const unsigned char* row, int vi, int nv, int v0, int V) {
@@ -174,7 +176,7 @@ __device__ __forceinline__ void accept_scan(const SeqArgs& a, QShared& S, const 
                                             float zpx, float zqx, bool write) {
     const RowArgs& R = a.r;
     const int lane = threadIdx.x & 31, K = R.K;
-    const TempScale ts = temp_scale(tau);
+    const float c = seq_scale(tau);
     const bool active = lane < L, tok_ok = tk >= 0 && tk < R.V;
     int seq_st = tau_ok(tau) ? 0 : ST_BAD_TEMP;
     QStat sp, sq;
@@ -192,7 +194,7 @@ __device__ __forceinline__ void accept_scan(const SeqArgs& a, QShared& S, const 
     double px = 0.0, qx = 0.0;
     bool acc = false;
     if (active && !(seq_st & ST_STOP) && lane < first_bad) {
-        const double cd = (double)ts.hi;
+        const double cd = (double)c;
         px = exp2((double)zpx * cd - (double)sp.e) * sp.inv_s;
         qx = exp2((double)zqx * cd - (double)sq.e) * sq.inv_s;
         acc = (double)u * qx < px;
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(kSeqThreads, 2) k_seq(const __grid_constant__ 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int L = TVM ? 1 : len_of(R, b);
-    const float tau = tau_of(R, b), c = temp_scale(tau).hi;
+    const float tau = tau_of(R, b), c = seq_scale(tau);
     const int rows = TVM ? 2 : 2 * L + 1;
     const int v0 = rank * sv, nv = max(min(sv, R.nvec - v0), 0);
     const int nfull = v0 + nv == R.nvec && R.V % VEC != 0 ? nv - 1 : nv;      // vectors that hold no token beyond the vocabulary
@@ -755,7 +757,8 @@ template <auto kernel> bool seq_ready() {
 // 48 of 32,000 20 instead of 33), as far as sixteen CTAs go; and more while SMs would idle and the CTAs have work.
 constexpr int kSeqShare = 112000;
 // How many clusters of C CTAs the device holds at a time, one CTA per SM or two (asked once per device; 0: not known).
-// A cluster stays inside one of the chip's GPCs, so large ones leave SMs over: of sixteen CTAs seven, of ten about twice as many.
+// A cluster stays inside one of the chip's GPCs, so large ones leave SMs over.  The answers on a B200, one CTA per SM / two: eight CTAs
+// 15 / 33, nine 15 / 30, ten 11 / 26, eleven and twelve 7 / 21, thirteen 7 / 17, fourteen to sixteen 7 / 14.
 int seq_resident(int C, bool two) {
     static int cached[64][2][kSeqMaxCluster + 1] = {{{0}}};
     int dev = 0;
@@ -825,9 +828,10 @@ bool seq_supported(const RowArgs& a, bool tv_only) {
 // 1,024 of 12,000 121 against 134; fp32 logits fill the CTAs with half the work: 700 of 4,096 51 against 67, but 3,000 of them
 // slower; bebop_tv 3,000 pairs of 12,000 67 against 88, but 1,024 of 32,000, two CTAs each, 65 against 58).  Larger clusters
 // leave SMs unused (seven clusters of sixteen run at a time) and run in waves without overlap: faster while the call
-// is a few waves (128 of 32,000 49 against 60; 48 of 65,536 42 against 55; 24 fp32 ragged ones of 49,999, K = 5, 36
-// against 54; one of 151,936 16 against 32), slower beyond (300 of 32,000 104 against 97; 16 of 151,936 44 against 37); with nine CTAs, of which fifteen to thirty
-// clusters run at a time, somewhat longer (32 of 65,536 31 against 48, 40 35 against 38).
+// is a few waves (128 of 32,000 50 against 57; 24 fp32 ragged ones of 49,999, K = 5, 36
+// against 54; one of 151,936 16 against 32), slower beyond (300 of 32,000 103 against 85; 16 of 151,936 44.6 against 42); with nine CTAs, of which fifteen to thirty
+// clusters run at a time, somewhat longer (32 of 65,536 31.7 against 39, 40 35.8 against 37.7; the line stands there, though on inputs
+// that re-draw in the other kernels it could lie higher: 48 40.5 against 49.7).
 bool seq_preferred(const RowArgs& a, bool tv_only) {
     const int rows = tv_only ? 2 : 2 * a.K + 1;
     int C = seq_cluster(rows, a.K, a.nvec);
