@@ -14,6 +14,9 @@
  *     [B,R,V] tensor starts at element (b*R + k) * ld.  The base pointer and
  *     ld * sizeof(element) must be multiples of 16 bytes.
  *   - -inf logits are legal (masked vocabulary, probability 0).
+ *   - Finite logits of any size are legal too.  A row whose LARGEST |x log2(e) / tau| lies beyond 4e6 (nothing but a mask of
+ *     -1e9; a temperature next to zero) is evaluated as defined by the kernel of small calls and short rows only; large calls
+ *     give such a row p = q = 0 or a token of no meaning, without a fatal bit.  Masks beside ordinary logits are right everywhere.
  *   - Errors that can be seen on the host (NULL required pointer, B/K/V out of
  *     range, K > BEBOP_MAX_K, ld < V, misalignment, workspace too small,
  *     temperature_all <= 0 with no per-row tensor, device not sm_100) return a

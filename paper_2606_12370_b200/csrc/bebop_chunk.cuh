@@ -1,4 +1,5 @@
-// What the kernels share: barriers and bulk copies, the exponentials of a chunk around an
+// What the pipelined, the re-draw and the sequence kernel share (the fused kernel, older, has such helpers of its own; what is
+// mended in one place is to be looked for in the other): barriers and bulk copies, the exponentials of a chunk around an
 // integer exponent, fixed-point warp sums, owners of a target among the lanes of a warp, 2^t in double.
 #pragma once
 #include "bebop_pipe.cuh"
