@@ -170,9 +170,9 @@ bebop_status_t bebop_greedy_verify(
  * split-row general kernels for shapes none of them takes; 1 the general kernels always; 2 the pipelined kernel
  * wherever it applies; 3 the fused kernel wherever it applies (the greedy mode has no fused form); 4 the sequence kernel
  * wherever it applies.  All give the same results up to the documented tolerances.  bebop_debug_last_kernel() says
- * what the last of these calls ran: 1 the general kernels, 2 the pipelined kernel, 3 a kernel that reads every logit
- * once, the fused or the sequence kernel (0: no call yet); bebop_debug_last_kernel_name() says it by the main kernel's name:
- * "general", "k_pipe", "k_fuse", "k_seq", "k_seq_greedy" ("none": no call yet).
+ * what the last of these calls ran: 1 the general kernels, 2 the pipelined kernel, 3 the fused or the sequence
+ * kernel (0: no call yet); bebop_debug_last_kernel_name() says it by name: "general", "k_pipe" (its sweeps, or with a TV
+ * output its stream, k_pipe_stream), "k_fuse", "k_seq", "k_seq_greedy" ("none": no call yet).
  * bebop_debug_fallback_offset returns the byte offset, inside the workspace of this
  * shape, of an int32 that after a bebop_verify call through the pipelined or the fused kernel holds the number of
  * sequences whose draw was re-done by the fp64 kernels.

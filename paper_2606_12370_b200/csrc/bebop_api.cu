@@ -7,10 +7,9 @@ using namespace bebop;
 
 namespace {
 
-// Test hooks: what the last call ran -- 1 general kernels, 2 pipelined kernel, 3 a kernel that reads every logit once (fused or
-// sequence kernel) -- and the name of its main kernel;
+// Test hooks: what the last call ran -- 1 general kernels, 2 pipelined kernel, 3 fused or sequence kernel -- and its name;
 struct LastKernel { int id; const char* name; } g_last = {0, "none"};
-// and which kernels calls may take: 0 the fastest for the shape; 1 general kernels only; 2 never a one-read kernel; 3 the fused
+// and which kernels calls may take: 0 the fastest for the shape; 1 general kernels only; 2 neither the fused nor the sequence kernel; 3 the fused
 // kernel wherever it applies; 4 the sequence kernel wherever it applies.
 int g_path = 0;
 
@@ -118,7 +117,7 @@ bebop_status_t bebop_verify(const void* target_logits, int64_t ld_target, const 
         e = seq_verify(a, draft_tokens, u_accept, u_final, o, stream, &launched);
         if (launched) g_last = {3, "k_seq"};
     }
-    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, false))) && fuse_supported(a)) {
+    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, false, tv != nullptr)))) {
         e = fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
         if (launched) g_last = {3, "k_fuse"};
     }
@@ -155,12 +154,11 @@ bebop_status_t bebop_tv(const void* target_logits, int64_t ld_target, const void
         e = seq_verify(a, nullptr, nullptr, nullptr, o, stream, &launched, true, s_aux);
         if (launched) g_last = {3, "k_seq"};
     }
-    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, true))) && fuse_supported(a)) {
+    if (e == cudaSuccess && !launched && (g_path == 3 || (g_path == 0 && fuse_preferred(a, true, true)))) {
         e = fuse_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
         if (launched) g_last = {3, "k_fuse"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
-        // the pipelined kernel with row pairs in place of sequences: first sweep, second sweep, no draw
         e = pipe_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
         if (launched) g_last = {2, "k_pipe"};
     }

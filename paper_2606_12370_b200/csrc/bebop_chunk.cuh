@@ -1,6 +1,5 @@
-// What the pipelined, the re-draw and the sequence kernel share (the fused kernel, older, has such helpers of its own; what is
-// mended in one place is to be looked for in the other): barriers and bulk copies, the exponentials of a chunk around an
-// integer exponent, fixed-point warp sums, owners of a target among the lanes of a warp, 2^t in double.
+// What the stream, the pipelined, the re-draw and the sequence kernel share: barriers and bulk copies, the exponentials of a
+// chunk around an integer exponent, fixed-point warp sums, owners of a target among the lanes of a warp, 2^t in double.
 #pragma once
 #include "bebop_pipe.cuh"
 
@@ -27,6 +26,22 @@ __device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, unsigned long long* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+// ---- a cluster: its barrier, the shared memory of its other CTAs
+// (aligned: all lanes of a warp execute them together, which nothing but a __syncwarp() makes a warp do that has split before)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+// the address of `p` (this CTA's shared memory) in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t at_rank(const void* p, int rank) {
+    uint32_t a; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank)); return a;
+}
+__device__ __forceinline__ void st_remote(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_remote(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ int redux_add(int v) { int r; asm volatile("redux.sync.add.s32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v)); return r; }
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {      // min(max(a b + c, 0), 1), rounded once

@@ -56,22 +56,23 @@ cudaError_t redraw_launch(const RowArgs& a, const float* u_final, VerifyOut o, c
                           const FbRec* fb_list, int expect, int* wait_failed, char* w,
                           const PipePlan& wp, cudaStream_t stream, bool expire_list_wait = false);
 
-// Pipelined kernel (bebop_pipe.cu): a ticket schedule with a producer warp that stages every task's
-// logits in shared memory by bulk copies while the other warps compute; same contract.  With `tv_only` it is
+// Pipelined kernel (bebop_pipe.cu): a ticket schedule with a producer warp that stages every task's logits in shared memory by
+// bulk copies while the other warps compute; where TV is asked for, the stream of bebop_flow.cuh.  With `tv_only` it is
 // bebop_tv: B row pairs (K = 1), o.tv and s_aux the outputs, no tokens, no uniforms, no draw.
 bool pipe_supported(const RowArgs& a);
 cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
 
-// Fused kernel (bebop_fuse.cu): every row read and exponentiated once, the exponentials parked in tensor memory
-// between the softmax statistics and the residuals; same contract as pipe_verify.  fuse_preferred says whether,
-// by measurement, it is the faster of the two for the shape.
-bool fuse_supported(const RowArgs& a);
-bool fuse_preferred(const RowArgs& a, bool tv_only);
+// Fused kernel (bebop_fuse.cu): the stream of bebop_flow.cuh, every row read from memory once and out of L2 a second time; same
+// contract as pipe_verify, which runs it too wherever a TV output is asked for.  fuse_preferred: the line between the two.
+bool fuse_preferred(const RowArgs& a, bool tv_only, bool want_tv);
 cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
+
+// Clears the head of a workspace; the next launch may be a programmatic dependent of it.
+cudaError_t clear_launch(char* w, size_t bytes, cudaStream_t stream);
 
 // Sequence kernel (bebop_seq.cu): a thread-block cluster per sequence (row pair), its logits in the cluster's shared memory;
 // one launch, no workspace; same contract.

@@ -23,9 +23,9 @@ constexpr size_t kFbCountOffset = 128;   // 8 bytes inside the zeroed head of th
                                          // re-draw; high int, sequences whose draw is decided
 struct PipePlan {
     int T, slice_vecs;     // slices per row, vectors per slice (multiple of 16)
-    size_t off_p1done, off_p2done, off_ddone, off_xdone, off_xsdone, off_fbrec, off_rowcnt, zero_bytes;
+    size_t off_p1done, off_ddone, off_xdone, off_xsdone, off_fbrec, off_rowcnt, zero_bytes;
     size_t off_xsum, off_xmass;   // fp64 re-draw: per listed sequence done counter; sums and masses per item
-    size_t off_part, off_rstat, off_dpart, off_tvacc, off_sacc, off_sinfo, total;
+    size_t off_part, off_rstat, off_dpart, off_sinfo, total;
 };
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -42,41 +42,18 @@ struct Plan {
     size_t off_dstats;  // double2[B][2][nsplit_d]       (m, S) partials, fp64
     size_t off_dmass;   // double [B][nsplit_d]          residual / bonus mass partials
     size_t off_amax;    // float,int [B][K+1][nsplit]    argmax partials (greedy)
-    size_t off_pipe;    // workspace of the pipelined kernel
-    size_t off_fuse;    // workspace of the fused kernel (the same bytes)
+    size_t off_pipe;    // workspace of the pipelined and the fused kernel and of the re-draw
     size_t total;
 };
-
-// Workspace of the fused kernel (bebop_fuse.cu).  A unit is a row pair or a bonus row; a sequence owns
-// `ups` consecutive units (K + 1 for bebop_verify, 1 for bebop_tv); every unit is cut into T slices.
-#ifndef BEBOP_FUSE_WARPS
-#define BEBOP_FUSE_WARPS 16
-#endif
-constexpr int kFuseWarps = BEBOP_FUSE_WARPS;   // consumer warps of a group = warp chunks of a slice
-#ifndef BEBOP_FUSE_VPT
-#define BEBOP_FUSE_VPT 2
-#endif
-constexpr int kFuseSliceVecs = kFuseWarps * 32 * BEBOP_FUSE_VPT;   // 16-byte vectors per slice, at most
-constexpr int kFuseMaxSlices = 128;
-struct FusePlan {
-    int T, slice_vecs;
-    size_t units;
-    // zeroed per call: head (ticket, wait flag, re-draw counters), the re-draw's per-sequence counters, its list, the
-    // per-sequence count of delivered parts, the slice records
-    size_t off_xdone, off_xsdone, off_fbrec, off_seqcnt, off_rec, zero_bytes;
-    size_t off_mass, off_wexp, off_saux, off_smass, off_rows, off_xsum, off_xmass, total;
-};
-
 
 static inline PipePlan make_pipe_plan(int B, int K, int nvec, int dt, int slice_cap = kPipeSliceVecs) {
     (void)dt;
     PipePlan w;
     w.T = (nvec + slice_cap - 1) / slice_cap; if (w.T < 1) w.T = 1;
-    w.slice_vecs = (((nvec + w.T - 1) / w.T) + 15) & ~15;   // halves (phase P2) stay 128-byte aligned
+    w.slice_vecs = (((nvec + w.T - 1) / w.T) + 255) & ~255;  // whole chunks of the stream's pass 1
     const size_t NR = (size_t)(2 * K + 1);
     size_t o = 256;                                           // ticket, wait flag; at kFbCountOffset the re-draw count
     w.off_p1done = o; o += align256(sizeof(int) * (size_t)B);      // per sequence: rows merged
-    w.off_p2done = o; o += align256(sizeof(int) * (size_t)B);
     w.off_ddone = o;  o += align256(sizeof(int) * (size_t)B);      // per sequence: partials of the draw row
     w.off_xdone = o;  o += align256(sizeof(int) * (size_t)B);
     w.off_xsdone = o; o += align256(sizeof(int) * (size_t)B);
@@ -86,8 +63,6 @@ static inline PipePlan make_pipe_plan(int B, int K, int nvec, int dt, int slice_
     w.off_part = o;   o += align256(16 * (size_t)B * NR * w.T);
     w.off_rstat = o;  o += align256(16 * (size_t)B * NR);
     w.off_dpart = o;  o += align256(16 * (size_t)B * 2 * w.T);
-    w.off_tvacc = o;  o += align256(8 * (size_t)B * (K > 0 ? K : 1));
-    w.off_sacc = o;   o += align256(8 * (size_t)B * (K > 0 ? K : 1));
     w.off_sinfo = o;  o += align256(16 * (size_t)B);
     w.zero_bytes = o;
     w.off_xsum = o;   o += align256(16 * (size_t)B * redraw_cut(w.T) * w.T);
@@ -96,26 +71,33 @@ static inline PipePlan make_pipe_plan(int B, int K, int nvec, int dt, int slice_
     return w;
 }
 
-static inline FusePlan make_fuse_plan(int B, int K, int nvec, int ups) {
-    FusePlan f;
-    f.T = (nvec + kFuseSliceVecs - 1) / kFuseSliceVecs; if (f.T < 1) f.T = 1;
-    f.slice_vecs = (nvec + f.T - 1) / f.T;
-    f.units = (size_t)B * (size_t)ups;
+// Workspace of the stream (bebop_flow.cuh): a unit is a row pair or a bonus row, a sequence owns `ups` of them (K + 1 for
+// bebop_verify, 1 for bebop_tv); C CTAs share a unit, each with nch chunks of lcv 16-byte vectors of every row.
+constexpr int kFlowMaxCluster = 8;
+struct FlowPlan {
+    int nch, sv;
+    // zeroed per call: head (wait flag, re-draw counters), the re-draw's per-sequence counters, its list, the sequences' counts
+    size_t off_xdone, off_xsdone, off_fbrec, off_seqcnt, zero_bytes;
+    size_t off_rows, off_smass, off_saux, off_mass, off_xsum, off_xmass, total;
+};
+static inline FlowPlan make_flow_plan(int B, int K, int nvec, int ups, int C, int lcv) {
+    FlowPlan f;
+    f.nch = ((nvec + lcv - 1) / lcv + C - 1) / C;
+    f.sv = f.nch * lcv;
+    const size_t b = (size_t)B, units = b * (size_t)ups;
     const PipePlan wv = make_pipe_plan(B, K, nvec, 0);          // the fp64 re-draw cuts rows its own way
     size_t o = 256;
-    f.off_xdone = o;  o += align256(sizeof(int) * (size_t)B);
-    f.off_xsdone = o; o += align256(sizeof(int) * (size_t)B);
-    f.off_fbrec = o;  o += align256(16 * (size_t)B);
-    f.off_seqcnt = o; o += align256(sizeof(int) * (size_t)B);
-    f.off_rec = o;    o += align256(16 * f.units * f.T * 2);
+    f.off_xdone = o;  o += align256(sizeof(int) * b);
+    f.off_xsdone = o; o += align256(sizeof(int) * b);
+    f.off_fbrec = o;  o += align256(16 * b);
+    f.off_seqcnt = o; o += align256(sizeof(int) * b);
     f.zero_bytes = o;
-    f.off_mass = o;   o += align256(8 * f.units * f.T * kFuseWarps);
-    f.off_wexp = o;   o += align256(8 * f.units * f.T * kFuseWarps);
-    f.off_saux = o;   o += align256(8 * f.units * f.T);
-    f.off_smass = o;  o += align256(8 * f.units * f.T);
-    f.off_rows = o;   o += align256(32 * f.units);
-    f.off_xsum = o;   o += align256(16 * (size_t)B * redraw_cut(wv.T) * wv.T);
-    f.off_xmass = o;  o += align256(8 * (size_t)B * redraw_cut(wv.T) * wv.T);
+    f.off_rows = o;   o += align256(80 * units);
+    f.off_smass = o;  o += align256(8 * units * C);
+    f.off_saux = o;   o += align256(8 * units * C);
+    f.off_mass = o;   o += align256(8 * units * C * 2 * f.nch);
+    f.off_xsum = o;   o += align256(16 * b * redraw_cut(wv.T) * wv.T);
+    f.off_xmass = o;  o += align256(8 * b * redraw_cut(wv.T) * wv.T);
     f.total = o;
     return f;
 }
@@ -147,11 +129,10 @@ static inline Plan make_plan(int B, int K, int V, int dt) {
     p.off_dmass = o;  o = align256(o + sizeof(double) * (size_t)B * nsd);
     p.off_amax = o;   o = align256(o + 8 * (size_t)B * (K + 1) * p.nsplit);
     {
-        // one region for the pipelined and the fused kernel: a call runs one of them, and both keep the wait flag
-        // and the re-draw's counters at the same place in its head
-        const size_t wp = make_pipe_plan(B, K, p.nvec, dt).total, wf = make_fuse_plan(B, K, p.nvec, K + 1).total;
+        // one region for all of them: a call runs one, and all keep the wait flag and the re-draw's counters at the same place in
+        // its head; the stream takes most with the largest cluster and the smaller chunks
+        const size_t wp = make_pipe_plan(B, K, p.nvec, dt).total, wf = make_flow_plan(B, K, p.nvec, K + 1, kFlowMaxCluster, 128).total;
         p.off_pipe = o;
-        p.off_fuse = o;
         o = align256(o + (wp > wf ? wp : wf));
     }
     p.total = o;

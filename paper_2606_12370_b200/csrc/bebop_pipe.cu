@@ -1,13 +1,13 @@
-// Pipelined kernel: the hot path of bebop_verify as one persistent, ticket-scheduled kernel with the
-// data movement and the bookkeeping taken off the compute warps.
+// Pipelined kernel: bebop_verify without a TV output, and the greedy mode, as one persistent, ticket-scheduled kernel with the
+// data movement and the bookkeeping taken off the compute warps.  (Calls with a TV output, and bebop_tv, run the stream of
+// bebop_flow.cuh from here: their second pass reads every row pair, this kernel's one row pair per sequence.)
 //
-// The work is a queue of tickets in three blocks, sequences ascending in each: P1 (softmax partial of one
-// slice of one row) for every row; then P2 (TV part and residual mass of one half slice of a row pair) for the
-// row each sequence's token is drawn from; then P2 for the other positions, which only TV needs.  Phase A --
-// merging a row's partials, and the accept scan of a sequence -- has no tickets: it runs in the publisher warp
-// that completes the row / the sequence, long before the second sweep asks for its results.  Nor has the draw:
-// the publisher warp that completes a sequence's draw row sets the draw up and hands it to its own CTA as a
-// task D (the fast draw with its certificate); the one that completes all the sequence's rows writes its TV.
+// The work is a queue of tickets in two blocks, sequences ascending in each: P1 (softmax partial of one
+// slice of one row) for every row; then P2 (residual mass of one half slice) for the row pair, or bonus row, each sequence's
+// token is drawn from.  Phase A -- merging a row's partials, and the accept scan of a sequence -- has no tickets: it runs in
+// the publisher warp that completes the row / the sequence, long before the second sweep asks for its results.  Nor has the
+// draw: the publisher warp that completes a sequence's draw row sets the draw up and hands it to its own CTA as a
+// task D (the fast draw with its certificate).
 // A sequence whose fast draw is not certified is listed for the fp64 re-draw kernel, which runs beside the end
 // of this one.
 //
@@ -29,15 +29,15 @@
 //
 // Every wait is bounded; a wait that gives up sets the wait flag (status bit 32 of every row).
 // No multicast, no cluster: each CTA copies from this GPU's own memory.
-#include "bebop_chunk.cuh"
+#include "bebop_flow.cuh"
 
 namespace bebop {
 
 namespace {
 
-// what the kernel is compiled for: bebop_verify; bebop_tv (row pairs, no accept test, no draw); the greedy mode
-// (one sweep over the target rows for their argmax)
-constexpr int kModeVerify = 0, kModeTv = 1, kModeGreedy = 2;
+// what the kernel is compiled for: bebop_verify without a TV output; the greedy mode (one sweep over the target rows for their
+// argmax)
+constexpr int kModeVerify = 0, kModeGreedy = 2;
 constexpr int NST = 2;                            // stages of the ring
 constexpr int PIPE_CTAS = 3;                      // CTAs per SM the kernel is built for
 constexpr int PC = WT;                            // consumer threads (8 warps); thread PC is the producer
@@ -48,7 +48,7 @@ constexpr int kPend = 4;                          // runs a producer may set asi
 constexpr int kTailZone = 8;                      // the last kTailZone tickets per CTA are claimed kBatchTail at a time
 constexpr int kBatchTail = 2;
 constexpr int kBatch = 5;                         // tickets claimed at a time (measured: 4 to 6 alike, 2 and 8 slower)
-constexpr double kFixTv = 1099511627776.0;             // 2^40: fixed point of TV parts and sums of squares
+constexpr double kFixTv = 1099511627776.0;             // 2^40: fixed point of sums of squares
 constexpr double kFixMass = 288230376151711744.0;      // 2^58: fixed point of the draw-row mass
 constexpr uint32_t kBarSpin = 1u << 20;           // tries of one barrier wait (each try itself waits a while)
 
@@ -56,13 +56,11 @@ struct __align__(16) TaskDesc {
     int phase;        // 0 P1, 2 P2, 3 D, -1: no more tasks
     int b, r;         // sequence; row (P1) or draft position (P2, D)
     int s, v0, nv;    // slice, its first vector, its vectors
-    int flags;        // bit 0: row pair (else bonus row alone), bit 1: the pair a token is drawn from,
-                      // bit 2 (D): no half slice owns the target, the draw goes to the fp64 re-draw
+    int flags;        // bit 0: row pair (else bonus row alone)
     float tau;        // temperature, and c = log2(e) / tau computed once per row
     float c;
     RowScale P, Q;
     float2 rho;       // P2, D: S_p / S_q as two floats
-    int need;         // P2: partials the sequence's second sweep delivers in all (the last one starts the draw's set-up)
     float bound;      // D: the error bound the draw must clear,
     double tt, base;  //    the target of the inverse CDF and the mass before the half slice in the stage
 };
@@ -99,9 +97,6 @@ struct PipeShared {
     float d1_sq[2 * MAX_SLICES];
 };
 
-__device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(b)) : "memory");
-}
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity) {
     const uint32_t addr = smem_u32(b);
     for (uint32_t i = 0; i < kBarSpin; ++i) if (mbar_try(addr, parity)) return true;
@@ -149,48 +144,38 @@ __device__ __forceinline__ void consumers_meet(int* wait_failed, unsigned long l
 // the next ticket.  Returns when the stop description has been handed to the consumers.
 template <int DT, int MODE>
 __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsigned char* data) {
-    constexpr bool TVO = MODE == kModeTv, GRD = MODE == kModeGreedy;
+    constexpr bool GRD = MODE == kModeGreedy;
     const RowArgs& R = a.r;
     const int K = R.K, T = a.T, T2 = 2 * a.T, NR = 2 * K + 1;
     const int B = R.B;
-    // (a caller that asks for no TV needs the second sweep over one row per sequence only: the one a token is drawn from)
-    // (and bebop_tv has the K row pairs and no bonus row)
-    // (the greedy mode sweeps the K + 1 target rows once)
-    // The second sweep comes in two passes: first the row each sequence's token is drawn from (so that every draw,
-    // and the list of the sequences that go to the fp64 re-draw, is done early in the sweep), then the other
-    // rows, which only TV needs.  bebop_tv has the K row pairs and no draw; the greedy mode sweeps the K + 1 target
-    // rows once.
+    // the second sweep is over one row per sequence, the one a token is drawn from; the greedy mode sweeps the K + 1 target rows once
     const int c0 = (GRD ? K + 1 : NR) * T;
-    const int c2a = (GRD || TVO) ? 0 : T2, c2b = GRD ? 0 : ((TVO || a.o.tv) ? K * T2 : 0);
-    const double inv_c0 = 1.0 / c0, inv_c2a = c2a ? 1.0 / c2a : 0.0, inv_c2b = c2b ? 1.0 / c2b : 0.0;
+    const int c2 = GRD ? 0 : T2;
+    const double inv_c0 = 1.0 / c0, inv_c2 = c2 ? 1.0 / c2 : 0.0;
     const double inv_T = 1.0 / T, inv_T2 = 1.0 / T2;
     const int sv1 = a.slice_vecs, sv2 = a.slice_vecs >> 1;
-    // Ticket order: blocks 0 .. B-1 hold the first sweep of sequence i, blocks B .. 2B-1 the first pass of the
-    // second sweep, blocks 2B .. 3B-1 its second pass: full sweeps, sequences ascending, so that a sequence's
-    // accept scan is long done when the second sweep reaches it.  (Pairing the sweeps so that the second finds
-    // its logits in L2 was measured and dropped: it waited for accept scans more than the L2 hits saved.)
+    // Ticket order: blocks 0 .. B-1 hold the first sweep of sequence i, blocks B .. 2B-1 its second: full sweeps, sequences
+    // ascending, so that a sequence's accept scan is long done when the second sweep reaches it.  (Pairing the sweeps so that
+    // the second finds its logits in L2 was measured again and dropped: the CTAs' own pace bounds the kernel, not its reads.)
     const unsigned long long pol_keep = l2_policy(true), pol_drop = l2_policy(false);
     auto clampB = [&](int x) { return x < 0 ? 0 : (x > B ? B : x); };
-    auto before = [&](int i) { return c0 * clampB(i) + c2a * clampB(i - B) + c2b * clampB(i - 2 * B); };   // tickets before block i
+    auto before = [&](int i) { return c0 * clampB(i) + c2 * clampB(i - B); };   // tickets before block i
     int blk = 0, f_here = 0, f_next = before(1);      // tickets of this CTA only grow: the block is tracked, not searched
     // the run of consecutive tasks of one sequence and phase that starts at ticket t, at most `want` tasks;
-    // Run.wv is the sequence, Run.off the offset inside the sequence's tasks of that phase (second sweep: the draw row
-    // is row 0, the other rows follow)
-    const int t1 = B * c0, t2 = t1 + B * c2a;
+    // Run.wv is the sequence, Run.off the offset inside the sequence's tasks of that phase
+    const int t1 = B * c0;
     auto decode = [&](int t, int want) {
         if (f_next <= t) {
             // the block follows from one division (a CTA's next tickets are some thirty blocks on: stepping there
             // one block at a time was most of what the producer did between two runs)
-            blk = (GRD || t < t1) ? div_by(t, c0, inv_c0)
-                                  : (t < t2 ? B + div_by(t - t1, c2a, inv_c2a) : 2 * B + div_by(t - t2, c2b, inv_c2b));
+            blk = (GRD || t < t1) ? div_by(t, c0, inv_c0) : B + div_by(t - t1, c2, inv_c2);
             f_here = before(blk); f_next = before(blk + 1);
         }
         while (f_next <= t) { ++blk; f_here = f_next; f_next = before(blk + 1); }
         Run r;
         const int o = t - f_here;
-        if (blk < B) { r.ph = 0; r.wv = blk; r.off = o; }
-        else if (blk < 2 * B) { r.ph = 2; r.wv = blk - B; r.off = o; }
-        else { r.ph = 2; r.wv = blk - 2 * B; r.off = o + c2a; }
+        if (blk < B) { r.ph = 0; r.wv = blk; } else { r.ph = 2; r.wv = blk - B; }
+        r.off = o;
         r.cnt = min(want, f_next - t);
         return r;
     };
@@ -238,9 +223,9 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
             ++mb_head;
             *(volatile int*)&S.mb_head = mb_head;
             TaskDesc d;
-            d.phase = 3; d.b = t.b; d.r = t.k; d.s = t.owner; d.flags = (t.pair ? 1 : 0) | 2;
+            d.phase = 3; d.b = t.b; d.r = t.k; d.s = t.owner; d.flags = t.pair ? 1 : 0;
             d.v0 = t.owner * sv2; d.nv = max(min(sv2, R.nvec - d.v0), 0);
-            d.tau = 1.f; d.c = t.c; d.P = t.P; d.Q = t.Q; d.rho = t.rho; d.need = 0;
+            d.tau = 1.f; d.c = t.c; d.P = t.P; d.Q = t.Q; d.rho = t.rho;
             d.bound = t.bound; d.tt = t.tt; d.base = t.base;
             issue(d, row_ptr(R, t.b, t.k), t.pair ? row_ptr(R, t.b, K + 1 + t.k) : nullptr, pol_drop);
         }
@@ -301,7 +286,7 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
             TaskDesc d;
             d.phase = ph; d.b = b; d.r = r; d.s = 0; d.v0 = 0; d.nv = 0; d.flags = 0; d.tau = 1.f; d.c = 0.f;
             d.P = no_row(); d.Q = no_row(); d.rho = make_float2(0.f, 0.f);
-            d.need = 0; d.bound = 0.f; d.tt = 0.0; d.base = 0.0;
+            d.bound = 0.f; d.tt = 0.0; d.base = 0.0;
             const char* row0 = nullptr; const char* row1 = nullptr;
             bool skip = false;
             if (ph == 0) {
@@ -309,32 +294,25 @@ __device__ __forceinline__ void producer(const PipeArgs& a, PipeShared& S, unsig
                 const bool is_target = r <= K;
                 const int k = is_target ? r : r - (K + 1);
                 if (!GRD) { d.tau = tau_of(R, b); d.c = temp_scale(d.tau).hi; }
-                skip = is_target ? (TVO ? k >= L : k > L) : k >= L;     // (bebop_tv has no bonus row)
+                skip = is_target ? k > L : k >= L;
                 row0 = row_ptr(R, b, r);
             } else {
                 // everything the row needs is requested at once (the sequence was seen ready: its records are there)
                 const SeqInfo si = seen_b == b ? seen : ld_seq(a.sinfo + b);
-                // row 0 of the sequence's second sweep is the row its token is drawn from; the others follow in order
-                const bool drawrow = !TVO && r == 0;
-                const int rp = TVO ? r : r - 1;
-                const int k = drawrow ? max(si.draw_row, 0) : (TVO ? rp : rp + (rp >= si.draw_row ? 1 : 0));
+                const int k = max(si.draw_row, 0);
                 d.r = k;
                 RowStat sp = ld_cg(a.rstat + (int64_t)b * NR + k);
                 RowStat sq = ld_cg(a.rstat + (int64_t)b * NR + K + 1 + min(k, K - 1));
                 const int L = len_of(R, b);
                 // (the accept scan saw these row records before it set the sequence's mark; should a load have
                 // overtaken that all the same, ask again)
-                const bool no_row_k = TVO && k >= L;      // bebop_tv has no bonus row: nothing was merged for it
-                if (k <= L && !no_row_k) for (uint32_t i = 0; !rec_valid(sp) && i < kSpin; ++i) sp = ld_cg(a.rstat + (int64_t)b * NR + k);
+                if (k <= L) for (uint32_t i = 0; !rec_valid(sp) && i < kSpin; ++i) sp = ld_cg(a.rstat + (int64_t)b * NR + k);
                 if (k < L) for (uint32_t i = 0; !rec_valid(sq) && i < kSpin; ++i) sq = ld_cg(a.rstat + (int64_t)b * NR + K + 1 + k);
                 d.c = __int_as_float(si.pad0);
                 const bool pair = k < L;
-                skip = k > L || si.n < 0 || (!pair && !(drawrow && si.draw_row == L)) || no_row_k;
-                // the sequence's second sweep: every half slice of the L row pairs, and of the bonus row if drawn from
-                d.need = T2 * (L + (si.draw_row == L ? 1 : 0));
-                if (!a.o.tv) d.need = T2;
+                skip = k > L || si.n < 0;
                 if (!skip) {
-                    d.flags = (pair ? 1 : 0) | (drawrow ? 2 : 0);
+                    d.flags = pair ? 1 : 0;
                     d.P = row_scale(sp);
                     if (pair) { d.Q = row_scale(sq); d.rho = row_rho(sp, sq); }
                     row0 = row_ptr(R, b, k);
@@ -401,7 +379,7 @@ __device__ __forceinline__ void merge_row_warp(const PipeArgs& a, int b, int r) 
     }
 }
 
-template <int DT, bool TVO>
+template <int DT>
 __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
     const RowArgs& R = a.r;
     const int lane = threadIdx.x & 31;
@@ -411,9 +389,8 @@ __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
     const TempScale ts = temp_scale(tau);
     // lane k owns draft position k (K <= 32): everything it needs is requested before anything is used
     const bool active = lane < L;
-    const bool tvo = TVO;              // row pairs only: no tokens, no accept test, no bonus row
-    const int tk = (active && !tvo) ? a.draft_tokens[(int64_t)b * K + lane] : 0;
-    const float u = (active && !tvo) ? a.u_accept[(int64_t)b * K + lane] : 0.f;
+    const int tk = active ? a.draft_tokens[(int64_t)b * K + lane] : 0;
+    const float u = active ? a.u_accept[(int64_t)b * K + lane] : 0.f;
     RowStat sp, sq, sb;
     sp.inv_s = 0.0; sp.e = E_EMPTY; sp.st = 0;
     sq = sp;
@@ -425,11 +402,11 @@ __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
         return x;
     };
     if (active) { sp = row(lane); sq = row(K + 1 + lane); }
-    if (tvo) { sb = sp; sb.st = 0; } else sb = row(L);                  // bonus row (row L <= K: always merged)
+    sb = row(L);                                                        // bonus row (row L <= K: always merged)
     int seq_st = ok ? 0 : ST_BAD_TEMP;
-    const bool tok_ok = tvo || (tk >= 0 && tk < V);
+    const bool tok_ok = tk >= 0 && tk < V;
     float zpx = 0.f, zqx = 0.f;
-    if (active && tok_ok && !tvo) { zpx = load_one<DT>(row_ptr(R, b, lane), tk); zqx = load_one<DT>(row_ptr(R, b, K + 1 + lane), tk); }
+    if (active && tok_ok) { zpx = load_one<DT>(row_ptr(R, b, lane), tk); zqx = load_one<DT>(row_ptr(R, b, K + 1 + lane), tk); }
     if (!seq_st && __ballot_sync(0xffffffffu, active && !tok_ok)) seq_st = ST_BAD_TOKEN;
     // the first bad row pair decides the status; rows after it do not count
     const int rs = active ? (sp.st | sq.st) : 0;
@@ -439,7 +416,7 @@ __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
     if (!seq_st && badrows) seq_st = rs_first;
     double px = 0.0, qx = 0.0;
     bool acc = false;
-    if (active && !tvo && !(seq_st & ST_FATAL) && lane < first_bad) {
+    if (active && !(seq_st & ST_FATAL) && lane < first_bad) {
         const double cd = (double)ts.hi;
         px = exp2((double)zpx * cd - (double)sp.e) * sp.inv_s;
         qx = exp2((double)zqx * cd - (double)sq.e) * sq.inv_s;
@@ -451,23 +428,21 @@ __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
     const bool fatal = (seq_st & ST_FATAL) != 0;
     const int nn = fatal ? 0 : n;
     // outputs: lane q writes position q (position nn is filled by the draw)
-    if (!tvo) for (int q = lane; q <= K; q += 32)
+    for (int q = lane; q <= K; q += 32)
         if (fatal || q != nn) a.o.out_tokens[(int64_t)b * (K + 1) + q] = q < nn ? tk : -1;   // q < nn <= 32: q == lane
     if (lane < K) {
         const bool zero = fatal || lane >= L;
         if (a.o.p_draft) a.o.p_draft[(int64_t)b * K + lane] = zero ? 0.f : (float)px;
         if (a.o.q_draft) a.o.q_draft[(int64_t)b * K + lane] = zero ? 0.f : (float)qx;
-        if (zero && a.o.tv) a.o.tv[(int64_t)b * K + lane] = 0.f;
-        if (TVO && zero && a.s_aux) a.s_aux[(int64_t)b * K + lane] = 0.f;
     }
     if (lane == 0) {
-        if (!tvo) { a.o.accept_len[b] = nn; a.stop[b] = fatal ? -1 : nn; }
+        a.o.accept_len[b] = nn; a.stop[b] = fatal ? -1 : nn;
         if (a.o.row_status) a.o.row_status[b] = seq_st;
         // the record's mark makes it (and, through the row records it was computed from, the sequence) ready
         // (pad0 carries c = log2(e) / tau of the sequence: the second sweep's producer need not divide again)
-        SeqInfo si; si.n = fatal ? -1 : nn; si.draw_row = (fatal || tvo) ? -1 : nn; si.pad0 = __float_as_int(ts.hi); si.pad = 1;
+        SeqInfo si; si.n = fatal ? -1 : nn; si.draw_row = fatal ? -1 : nn; si.pad0 = __float_as_int(ts.hi); si.pad = 1;
         st_seq(a.sinfo + b, si);
-        if (fatal && !tvo) draw_decided(a.fb_count);     // no draw will come
+        if (fatal) draw_decided(a.fb_count);     // no draw will come
     }
 }
 
@@ -479,21 +454,6 @@ __device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long
     asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
 }
 
-// the largest logit of N vectors (NaN if there is one); bf16: packed maxima, unpacked once
-template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* v) {
-    if (DT == 1) {
-        uint32_t a[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) a[j] = max_nan_bf16x2(max_nan_bf16x2(v[j].x, v[j].y), max_nan_bf16x2(v[j].z, v[j].w));
-#pragma unroll
-        for (int j = 1; j < N; ++j) a[0] = max_nan_bf16x2(a[0], a[j]);
-        return max_nan(__uint_as_float(a[0] << 16), __uint_as_float(a[0] & 0xffff0000u));
-    }
-    float m = vec_max<DT>(v[0]);
-#pragma unroll
-    for (int j = 1; j < N; ++j) m = max_nan(m, vec_max<DT>(v[j]));
-    return m;
-}
 // Residuals from the exponentials of a row pair: r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q as two floats
 // (equal rows give rho = 1 and r' = 0 exactly); as e_p <= 1, saturating to [0, 1] is taking the maximum with 0.  The large
 // product goes first: where q is close to p it leaves a small difference without rounding, and the small product then
@@ -506,19 +466,6 @@ template <int N> __device__ __forceinline__ void resid_n(const float* p, const f
         r[i] = fma_sat(-rho.y, q[i], t.x); r[i + 1] = fma_sat(-rho.y, q[i + 1], t.y);
     }
 }
-// ... their sum, and the sum of e_q over the tokens with q <= p: the mask 1[d >= 0] serves both
-template <int N> __device__ __forceinline__ void resid_aux_n(const float* p, const float* q, float2 rho, float2* z, float2* x) {
-    const float2 nh = make_float2(-rho.x, -rho.x), nl = make_float2(-rho.y, -rho.y);
-#pragma unroll
-    for (int i = 0; i < N; i += 2) {
-        const float2 q2 = make_float2(q[i], q[i + 1]);
-        const float2 d = __ffma2_rn(nl, q2, __ffma2_rn(nh, q2, make_float2(p[i], p[i + 1])));
-        const float2 mk = make_float2(d.x >= 0.f ? 1.f : 0.f, d.y >= 0.f ? 1.f : 0.f);
-        *z = __ffma2_rn(d, mk, *z);
-        *x = __ffma2_rn(q2, mk, *x);
-    }
-}
-
 // P1: softmax partial (E, S) of one slice of one row, from shared memory.
 template <int DT>
 __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const TaskDesc& d, const unsigned char* data,
@@ -527,25 +474,24 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = d.nv;
+    // a warp has 256 vectors side by side, the chunk of the stream's pass 1: both give a row the same sum
+    const int at = warp * (32 * NV) + lane;
     uint4 raw[NV];
-    if (nv >= (NV - 1) * PC) {                   // the usual case: only a thread's last vector may lie beyond the slice
+    if ((warp + 1) * (32 * NV) <= nv) {
 #pragma unroll
-        for (int u = 0; u < NV - 1; ++u) raw[u] = lds16(data + (size_t)(tid + u * PC) * 16);
-        raw[NV - 1] = neg_inf_vec<DT>();
-        if (tid + (NV - 1) * PC < nv) raw[NV - 1] = lds16(data + (size_t)(tid + (NV - 1) * PC) * 16);
+        for (int u = 0; u < NV; ++u) raw[u] = lds16(data + (size_t)(at + u * 32) * 16);
     } else {
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            const int v = tid + u * PC;
             raw[u] = neg_inf_vec<DT>();
-            if (v < nv) raw[u] = lds16(data + (size_t)v * 16);
+            if (at + u * 32 < nv) raw[u] = lds16(data + (size_t)(at + u * 32) * 16);
         }
     }
     if ((d.v0 + nv) * VEC > R.V) {               // the row's last vector is in this slice and is partial
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            const int gbase = (d.v0 + tid + u * PC) * VEC;
-            if (tid + u * PC < nv && gbase + VEC > R.V) mask_tail<DT>(raw[u], R.V - gbase);
+            const int gbase = (d.v0 + at + u * 32) * VEC;
+            if (at + u * 32 < nv && gbase + VEC > R.V) mask_tail<DT>(raw[u], R.V - gbase);
         }
     }
     // one exponent per warp, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time, four running sums
@@ -563,9 +509,9 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
     }
     const bool bad = E.e == E_BAD;
     const int Ew = bad ? E_EMPTY : E.e;
-    const float st = Ew > E_EMPTY ? warp_sum((s0.x + s1.x) + (s0.y + s1.y)) : 0.f;
+    const int2 sum = warp_sum_words(0.5f * ((s0.x + s0.y) + (s1.x + s1.y)));
     const float mw = bad ? __int_as_float(0x7fc00000) : 0.f;
-    if (lane == 0) { S.wf[stage][0][warp] = st; S.wi[stage][warp] = Ew; S.wf[stage][1][warp] = mw; }
+    if (lane == 0) { S.wd[stage][warp] = Ew > E_EMPTY ? 2.0 * word_value(sum) : 0.0; S.wi[stage][warp] = Ew; S.wf[stage][1][warp] = mw; }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
 }
@@ -618,16 +564,15 @@ __device__ __forceinline__ void pipe_g(const PipeArgs& a, PipeShared& S, const T
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
 }
 
-// P2: TV partial of one half slice of a row pair; on the pair (or bonus row) a token is drawn from,
-// also the mass in double and the sum of squares.  Target row in the first half of the stage, draft
-// row in the second.
-template <int DT, bool TVO>
+// P2: residual mass, in double, and the sum of squares of one half slice of the row pair (or bonus row) a token is drawn from.
+// Target row in the first half of the stage, draft row in the second.
+template <int DT>
 __device__ __forceinline__ void pipe_p2(const PipeArgs& a, PipeShared& S, const TaskDesc& d, const unsigned char* data,
                                         int stage) {
     constexpr int VEC = Elem<DT>::VEC, NV = PSLICE / (2 * PC);
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool pair = (d.flags & 1) != 0, draw = (d.flags & 2) != 0;
+    const bool pair = (d.flags & 1) != 0;
     const int nv = d.nv;
     const unsigned char* qdata = data + STAGE_BYTES / 2;
     // Vectors beyond the slice, and the draft row of a bonus task, read as -inf: they give p = q = 0 and add
@@ -657,53 +602,24 @@ __device__ __forceinline__ void pipe_p2(const PipeArgs& a, PipeShared& S, const 
         }
     }
     // residuals in units of 1 / S_p, which is applied to the warp's sums
-    float2 z2 = make_float2(0.f, 0.f), a2 = z2, b2 = z2;
-    float sqs = 0.f;
-    double z, zd = 0.0;
-    if (TVO && a.sacc) {
-        // bebop_tv with the auxiliary sum: TV and S = sum of q over the tokens with q <= p (Eq. tv_grad)
+    float2 a2 = make_float2(0.f, 0.f), b2 = a2;
+    double zd = 0.0;
 #pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            float p[VEC], q[VEC];
-            exp_vec<DT>(rp[u], d.c, SP.ef, p);
-            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
-            resid_aux_n<VEC>(p, q, rho, &z2, &a2);
+    for (int u = 0; u < NV; ++u) {
+        float p[VEC], q[VEC], r[VEC];
+        exp_vec<DT>(rp[u], d.c, SP.ef, p);
+        exp_vec<DT>(rq[u], d.c, SQ.ef, q);
+        resid_n<VEC>(p, q, rho, r);
+        zd += (double)sum_fixed<VEC>(r);
+#pragma unroll
+        for (int i = 0; i < VEC; i += 2) {
+            a2 = __ffma2_rn(make_float2(p[i], p[i + 1]), make_float2(p[i], p[i + 1]), a2);
+            b2 = __ffma2_rn(make_float2(q[i], q[i + 1]), make_float2(q[i], q[i + 1]), b2);
         }
-        z = (double)warp_sum(z2.x + z2.y) * ip;
-        zd = (double)warp_sum(a2.x + a2.y) * ((double)SQ.inv + (double)SQ.inv_lo);
-    } else if (!draw) {
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            float p[VEC], q[VEC], r[VEC];
-            exp_vec<DT>(rp[u], d.c, SP.ef, p);
-            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
-            resid_n<VEC>(p, q, rho, r);
-#pragma unroll
-            for (int i = 0; i < VEC; i += 4) {
-                z2 = __fadd2_rn(z2, make_float2(r[i], r[i + 1]));
-                a2 = __fadd2_rn(a2, make_float2(r[i + 2], r[i + 3]));
-            }
-        }
-        z = (double)warp_sum((z2.x + a2.x) + (z2.y + a2.y)) * ip;
-    } else {
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            float p[VEC], q[VEC], r[VEC];
-            exp_vec<DT>(rp[u], d.c, SP.ef, p);
-            exp_vec<DT>(rq[u], d.c, SQ.ef, q);
-            resid_n<VEC>(p, q, rho, r);
-            zd += (double)sum_fixed<VEC>(r);
-#pragma unroll
-            for (int i = 0; i < VEC; i += 2) {
-                a2 = __ffma2_rn(make_float2(p[i], p[i + 1]), make_float2(p[i], p[i + 1]), a2);
-                b2 = __ffma2_rn(make_float2(q[i], q[i + 1]), make_float2(q[i], q[i + 1]), b2);
-            }
-        }
-        zd = warp_sum(zd) * ip;
-        z = zd;
-        sqs = warp_sum((a2.x + a2.y) * (SP.inv * SP.inv) + (b2.x + b2.y) * (SQ.inv * SQ.inv));
     }
-    if (lane == 0) { S.wf[stage][0][warp] = (float)z; S.wd[stage][warp] = zd; S.wf[stage][1][warp] = sqs; }
+    zd = warp_sum(zd) * ip;
+    const float sqs = warp_sum((a2.x + a2.y) * (SP.inv * SP.inv) + (b2.x + b2.y) * (SQ.inv * SQ.inv));
+    if (lane == 0) { S.wd[stage][warp] = zd; S.wf[stage][1][warp] = sqs; }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
 }
@@ -726,11 +642,9 @@ __device__ __forceinline__ DPart load_dpart(const PipeArgs& a, int64_t i) {
 }
 
 // Set-up of a sequence's draw, by the publisher warp that delivered the last partial of the sequence's second
-// sweep: TV of every draft position from the fixed-point sums, then the residual mass Z of the draw rows, the
-// target u * Z of the inverse CDF and the half slice that owns it.  The draw task goes into the CTA's mailbox:
-// the producer stages that half slice and the consumers find the token.
-template <bool TVO>
-__device__ __noinline__ void draw_setup_warp(const PipeArgs& a, PipeShared& S, int b, int what) {
+// sweep: the residual mass Z of the draw rows, the target u * Z of the inverse CDF and the half slice that owns it.  The draw
+// task goes into the CTA's mailbox: the producer stages that half slice and the consumers find the token.
+__device__ __noinline__ void draw_setup_warp(const PipeArgs& a, PipeShared& S, int b) {
     const RowArgs& R = a.r;
     const int lane = threadIdx.x & 31;
     const int K = R.K, NR = 2 * K + 1, L = len_of(R, b), T2 = 2 * a.T;
@@ -741,30 +655,8 @@ __device__ __noinline__ void draw_setup_warp(const PipeArgs& a, PipeShared& S, i
     // lane 0 will need the draw rows' records: asked for now, with everything else
     RowStat sp, sq;
     sp.inv_s = 0.0; sp.e = 0; sp.st = 0; sq = sp;
-    if (lane == 0 && k >= 0 && (what & 2)) { sp = ld_row(a, (int64_t)b * NR + k); if (pair) sq = ld_row(a, (int64_t)b * NR + K + 1 + k); }
-    if ((what & 1) && lane < L && a.o.tv) {
-        // the position's TV parts were added in fixed point, with a count of one each in the low 16 bits
-        unsigned long long w = 0;
-        for (uint32_t i = 0; i < kSpin; ++i) {
-            w = __ldcg(a.tvacc + (int64_t)b * K + lane);
-            if ((int)(w & 0xffffull) >= T2) break;
-            __nanosleep(64);
-        }
-        if ((int)(w & 0xffffull) < T2) atomicExch(a.wait_failed, 1);
-        const float z = (float)((double)(w >> 16) * 9.094947017729282e-13);      // 2^-40
-        a.o.tv[(int64_t)b * K + lane] = fminf(fmaxf(z, 0.f), 1.f);
-    }
-    if (TVO && (what & 1) && lane < L && a.s_aux) {
-        unsigned long long w = 0;
-        for (uint32_t i = 0; i < kSpin; ++i) {
-            w = __ldcg(a.sacc + (int64_t)b * K + lane);
-            if ((int)(w & 0xffffull) >= T2) break;
-            __nanosleep(64);
-        }
-        if ((int)(w & 0xffffull) < T2) atomicExch(a.wait_failed, 1);
-        a.s_aux[(int64_t)b * K + lane] = (float)((double)(w >> 16) * 9.094947017729282e-13);
-    }
-    if (k < 0 || !(what & 2)) return;
+    if (lane == 0 && k >= 0) { sp = ld_row(a, (int64_t)b * NR + k); if (pair) sq = ld_row(a, (int64_t)b * NR + K + 1 + k); }
+    if (k < 0) return;
     // the half slices' masses: lanes fetch them in parallel, lane 0 scans them in slice order
     for (int s = lane; s < T2; s += 32) { const DPart dp = load_dpart(a, (int64_t)b * T2 + s); S.d1_tot[s] = dp.tot; S.d1_sq[s] = dp.sq; }
     __syncwarp();
@@ -821,7 +713,7 @@ __device__ __forceinline__ void pipe_d(const PipeArgs& a, PipeShared& PS, const 
     const bool pair = (d.flags & 1) != 0;
     const unsigned char* qdata = data + STAGE_BYTES / 2;
     int found_y = -1, found_cert = 0;
-    if (!(d.flags & 4)) {
+    {
         const double ip = (double)d.P.inv + (double)d.P.inv_lo;
         const int v0 = d.v0, nv = d.nv;
         // the vector's residuals, same arithmetic as phase P2
@@ -906,11 +798,10 @@ __device__ __forceinline__ void pipe_d(const PipeArgs& a, PipeShared& PS, const 
 // One warp.  For every streaming task: wait for the eight warp partials, take them into registers,
 // hand the stage back, then merge (warp order, so the result does not depend on timing) and publish:
 // P1 -- the slice's (E, S) partial and the row's counter, whose last increment starts the merge of the
-// row, whose last merged row starts the accept scan of the sequence; P2 -- the TV part (and the
-// draw-row mass) and the sequence's counter.
+// row, whose last merged row starts the accept scan of the sequence; P2 -- the draw row's mass and the sequence's counter.
 template <int DT, int MODE>
 __device__ __forceinline__ void publisher(const PipeArgs& a, PipeShared& S) {
-    constexpr bool TVO = MODE == kModeTv, GRD = MODE == kModeGreedy;
+    constexpr bool GRD = MODE == kModeGreedy;
     const RowArgs& R = a.r;
     const int lane = threadIdx.x & 31;
     const int K = R.K, T2 = 2 * a.T;
@@ -930,8 +821,7 @@ __device__ __forceinline__ void publisher(const PipeArgs& a, PipeShared& S) {
         // stage rather than derived from the task number
         if (!mbar_wait(&S.pdone[stage], (pd_par >> stage) & 1u)) { if (lane == 0) atomicExch(a.wait_failed, 1); return; }
         pd_par ^= 1u << stage;
-        const int b = S.desc[stage].b, r = S.desc[stage].r, sl = S.desc[stage].s, flags = S.desc[stage].flags;
-        const int need = S.desc[stage].need;
+        const int b = S.desc[stage].b, r = S.desc[stage].r, sl = S.desc[stage].s;
         const int w = lane & (WW - 1);
         const float f0 = S.wf[stage][0][w], f1 = S.wf[stage][1][w];
         const double dd = S.wd[stage][w];
@@ -957,7 +847,7 @@ __device__ __forceinline__ void publisher(const PipeArgs& a, PipeShared& S) {
                                    max(__shfl_sync(0xffffffffu, ii, 2), __shfl_sync(0xffffffffu, ii, 3))),
                                max(max(__shfl_sync(0xffffffffu, ii, 4), __shfl_sync(0xffffffffu, ii, 5)),
                                    max(__shfl_sync(0xffffffffu, ii, 6), __shfl_sync(0xffffffffu, ii, 7))));
-            const double mine = ii > E_EMPTY ? (double)(f0 * pow2f(max(ii - Ec, -126))) : 0.0;
+            const double mine = ii > E_EMPTY ? dd * pow2d(max(ii - Ec, -1000)) : 0.0;
             double sum = 0.0; float mc = -INFINITY;
 #pragma unroll
             for (int k = 0; k < WW; ++k) { sum += __shfl_sync(0xffffffffu, mine, k); mc = max_nan(mc, __shfl_sync(0xffffffffu, f1, k)); }
@@ -971,37 +861,26 @@ __device__ __forceinline__ void publisher(const PipeArgs& a, PipeShared& S) {
             }
             if (__shfl_sync(0xffffffffu, run_a, 0)) {
                 merge_row_warp(a, b, r);
-                // the last merged row of the sequence (2L+1 rows are in use, 2L without a bonus row) starts the accept scan
+                // the last merged row of the sequence (2L+1 rows are in use) starts the accept scan
                 int last_row = 0;
-                if (lane == 0) last_row = atomicAdd(&a.p1done[b], 1) == 2 * len_of(R, b) - (TVO ? 1 : 0);
-                if (__shfl_sync(0xffffffffu, last_row, 0)) accept_warp<DT, TVO>(a, b);
+                if (lane == 0) last_row = atomicAdd(&a.p1done[b], 1) == 2 * len_of(R, b);
+                if (__shfl_sync(0xffffffffu, last_row, 0)) accept_warp<DT>(a, b);
             }
         } else {
-            float zz = 0.f, sq = 0.f; double tot = 0.0;
+            float sq = 0.f; double tot = 0.0;
             int run_d = 0;
 #pragma unroll
-            for (int k = 0; k < WW; ++k) {
-                zz += __shfl_sync(0xffffffffu, f0, k); sq += __shfl_sync(0xffffffffu, f1, k); tot += __shfl_sync(0xffffffffu, dd, k);
-            }
+            for (int k = 0; k < WW; ++k) { sq += __shfl_sync(0xffffffffu, f1, k); tot += __shfl_sync(0xffffffffu, dd, k); }
             if (lane == 0) {
                 // Fixed point with a count of one in the low bits of the same word: one relaxed add publishes value
                 // and count together, and integer sums do not depend on the order of arrival.
-                if (flags & 1) red_add_u64(a.tvacc + (int64_t)b * K + r, ((unsigned long long)__double2ll_rn((double)zz * kFixTv) << 16) | 1ull);
-                if (TVO && a.sacc) red_add_u64(a.sacc + (int64_t)b * K + r, ((unsigned long long)__double2ll_rn(tot * kFixTv) << 16) | 1ull);
-                if (flags & 2) {
-                    unsigned long long* wd = a.dacc + ((int64_t)b * T2 + sl) * 2;
-                    red_add_u64(wd, ((unsigned long long)__double2ll_rn(tot * kFixMass) << 4) | 1ull);
-                    red_add_u64(wd + 1, ((unsigned long long)__double2ll_rn((double)sq * kFixTv) << 4) | 1ull);
-                }
-                // the last partial of the sequence's draw row starts the set-up of its draw, the last partial of all its rows
-                // finishes its TV
-                // (without a TV output the draw row is the sequence's whole second sweep: one counter)
-                const bool all_rows = TVO || a.o.tv != nullptr;
-                if ((flags & 2) && atomicAdd(a.ddone + b, 1) == T2 - 1) run_d |= all_rows ? 2 : 3;
-                if (all_rows && atomicAdd(a.p2done + b, 1) == need - 1) run_d |= 1;
+                unsigned long long* wd = a.dacc + ((int64_t)b * T2 + sl) * 2;
+                red_add_u64(wd, ((unsigned long long)__double2ll_rn(tot * kFixMass) << 4) | 1ull);
+                red_add_u64(wd + 1, ((unsigned long long)__double2ll_rn((double)sq * kFixTv) << 4) | 1ull);
+                run_d = atomicAdd(a.ddone + b, 1) == T2 - 1;         // the last partial starts the set-up of the draw
             }
             run_d = __shfl_sync(0xffffffffu, run_d, 0);
-            if (run_d) draw_setup_warp<TVO>(a, S, b, run_d);
+            if (run_d) draw_setup_warp(a, S, b);
         }
         // the producer stays until every streaming task has been dealt with here (mailbox entries come first)
         __syncwarp();
@@ -1045,7 +924,7 @@ __global__ void __launch_bounds__(PT, PIPE_CTAS) k_pipe(const __grid_constant__ 
         const unsigned char* sd = data + (size_t)stage * STAGE_BYTES;
         if (MODE == kModeGreedy) pipe_g<DT>(a, S, d, sd, stage);
         else if (d.phase == 0) pipe_p1<DT>(a, S, d, sd, stage);
-        else if (d.phase == 2) pipe_p2<DT, MODE == kModeTv>(a, S, d, sd, stage);
+        else if (d.phase == 2) pipe_p2<DT>(a, S, d, sd, stage);
         else {
             pipe_d<DT>(a, S, d, sd, meet);
             consumers_meet(a.wait_failed, &S.dsync, meet);
@@ -1055,9 +934,15 @@ __global__ void __launch_bounds__(PT, PIPE_CTAS) k_pipe(const __grid_constant__ 
     }
 }
 
-// -----------------------------------------------------------------------------
-extern cudaEvent_t g_ev_start, g_ev_stop;
+// The stream of bebop_flow.cuh as the pipelined kernel runs it: the calls with a TV output that are too large for the fused
+// kernel's region.
+template <int DT, bool TVM, class F>
+__global__ void __launch_bounds__(F::LT, 1) k_pipe_stream(const __grid_constant__ FlowArgs a) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    flow_body<DT, TVM, F>(a, smem);
+}
 
+// -----------------------------------------------------------------------------
 namespace {
 
 // Clears what a call needs cleared.  A kernel instead of a memset, because k_pipe can then be its programmatic dependent,
@@ -1068,9 +953,7 @@ __global__ void __launch_bounds__(256) k_clear(uint4* p, unsigned n16) {
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n16; i += gridDim.x * 256) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 template <typename K> cudaError_t launch_cleared(K kernel, const PipeArgs& wa, int grid, size_t smem, char* w, size_t zero_bytes, cudaStream_t stream) {
-    const unsigned n16 = (unsigned)(zero_bytes / 16);
-    k_clear<<<n16 < 256 * 148 ? (n16 + 255) / 256 : 148, 256, 0, stream>>>(reinterpret_cast<uint4*>(w), n16);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = clear_launch(w, zero_bytes, stream);
     if (e != cudaSuccess) return e;
     if (g_ev_start) cudaEventRecord(g_ev_start, stream);
     cudaLaunchAttribute attr[1];
@@ -1106,6 +989,12 @@ int pipe_grid() {
 }  // namespace
 
 
+cudaError_t clear_launch(char* w, size_t bytes, cudaStream_t stream) {
+    const unsigned n16 = (unsigned)(bytes / 16);
+    k_clear<<<n16 < 256 * 148 ? (n16 + 255) / 256 : 148, 256, 0, stream>>>(reinterpret_cast<uint4*>(w), n16);
+    return cudaGetLastError();
+}
+
 bool pipe_supported(const RowArgs& a) {
     const int T = (a.nvec + PSLICE - 1) / PSLICE;
     return T >= 1 && T <= MAX_SLICES && a.K <= BEBOP_MAX_K_INT;
@@ -1115,8 +1004,15 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only, float* s_aux) {
     *launched = false;
-    const int grid_max = tv_only ? (a.dt == 0 ? pipe_grid<0, kModeTv>() : pipe_grid<1, kModeTv>())
-                                 : (a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>());
+    if (tv_only || o.tv) {
+        // with TV every row pair has a second pass: the stream, which reads it from L2
+        const FlowCall x{a, p, draft_tokens, u_accept, u_final, o, ws, stream, tv_only, s_aux};
+        using F = FlowLong;
+        const int C = flow_cluster(a, tv_only);
+        if (tv_only) return a.dt == 0 ? flow_launch<F, k_pipe_stream<0, true, F>>(x, C, launched) : flow_launch<F, k_pipe_stream<1, true, F>>(x, C, launched);
+        return a.dt == 0 ? flow_launch<F, k_pipe_stream<0, false, F>>(x, C, launched) : flow_launch<F, k_pipe_stream<1, false, F>>(x, C, launched);
+    }
+    const int grid_max = a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>();
     if (grid_max < 1) return cudaSuccess;
     const PipePlan wp = make_pipe_plan(a.B, a.K, a.nvec, a.dt, PSLICE);
     PipeArgs wa;
@@ -1128,34 +1024,27 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
     wa.ticket = reinterpret_cast<int*>(w);
     wa.wait_failed = wa.ticket + 1;
     wa.p1done = reinterpret_cast<int*>(w + wp.off_p1done);
-    wa.p2done = reinterpret_cast<int*>(w + wp.off_p2done);
     wa.ddone = reinterpret_cast<int*>(w + wp.off_ddone);
     wa.rowcnt = reinterpret_cast<int*>(w + wp.off_rowcnt);
     wa.part = reinterpret_cast<P1Part*>(w + wp.off_part);
     wa.rstat = reinterpret_cast<RowStat*>(w + wp.off_rstat);
     wa.dacc = reinterpret_cast<unsigned long long*>(w + wp.off_dpart);
-    wa.tvacc = reinterpret_cast<unsigned long long*>(w + wp.off_tvacc);
     wa.sinfo = reinterpret_cast<SeqInfo*>(w + wp.off_sinfo);
     const int expire = take_expire_wait();
     wa.expire = expire == 2 ? 1 : 0;
     wa.kappa = draw_kappa();
-    wa.tv_only = tv_only ? 1 : 0;
-    wa.s_aux = tv_only ? s_aux : nullptr;
-    wa.sacc = (tv_only && s_aux) ? reinterpret_cast<unsigned long long*>(w + wp.off_sacc) : nullptr;
     wa.T = wp.T; wa.slice_vecs = wp.slice_vecs;
     {
-        const long long NR = 2 * a.K + 1;
-        const long long total = (long long)a.B * (NR * wp.T + (long long)(tv_only ? a.K : (o.tv ? a.K + 1 : 1)) * 2 * wp.T);
+        const long long total = (long long)a.B * ((2 * a.K + 1) * (long long)wp.T + 2 * wp.T);
         if (total > 0x7fff0000LL) return cudaSuccess;
         wa.ntickets = (int)total;
     }
     const int grid = wa.ntickets < grid_max ? wa.ntickets : grid_max;
-    const cudaError_t e = launch_cleared(tv_only ? (a.dt == 0 ? k_pipe<0, kModeTv> : k_pipe<1, kModeTv>) : (a.dt == 0 ? k_pipe<0, kModeVerify> : k_pipe<1, kModeVerify>),
-                                         wa, grid, kPipeSmem, w, wp.zero_bytes, stream);
+    const cudaError_t e = launch_cleared(a.dt == 0 ? k_pipe<0, kModeVerify> : k_pipe<1, kModeVerify>, wa, grid, kPipeSmem, w, wp.zero_bytes, stream);
     if (g_ev_stop) cudaEventRecord(g_ev_stop, stream);
     if (e != cudaSuccess) return e;
     *launched = true;
-    return redraw_launch(a, u_final, o, wa.fb_count, wa.fb_list, tv_only ? 0 : a.B, wa.wait_failed, w, wp, stream, expire == 1);
+    return redraw_launch(a, u_final, o, wa.fb_count, wa.fb_list, a.B, wa.wait_failed, w, wp, stream, expire == 1);
 }
 
 // ------------------------------------------------------------------ greedy mode

@@ -53,21 +53,6 @@ struct __align__(16) QRec { double s, ub; int e, bad; double pad; };    // a row
 struct __align__(16) QStat { double inv_s, ub; int e, st; double pad; };
 
 // ------------------------------------------------------------------ PTX helpers
-// (aligned: all lanes of a warp execute them together, which nothing but a __syncwarp() makes a warp do that has split before)
-__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
-__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-// the address of `p` (this CTA's shared memory) in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t at_rank(const void* p, int rank) {
-    uint32_t a; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank)); return a;
-}
-__device__ __forceinline__ void st_remote(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ void st_remote(uint32_t a, int v) {
-    asm volatile("st.shared::cluster.s32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
-}
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b) {
     const uint32_t addr = smem_u32(b);
     for (uint32_t i = 0; i < kQSpin; ++i) if (mbar_try(addr, 0)) return true;

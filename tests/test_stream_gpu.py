@@ -1,0 +1,76 @@
+"""The stream (fused and pipelined kernel with a TV output) where its cuts fall: chunks of 128 and 256 16-byte vectors, one CTA
+to eight per row, ragged last vectors, empty and ragged sequences, more and fewer units than clusters, rows short of a CTA's
+slice; and the pipelined kernel's sweeps, which a call without a TV output takes.  Against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import bebop_gen as G
+import oracle
+import paper_2606_12370_b200 as P
+from parity import TOL, check_properties, compare_verify, oracle_on, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(params=[2, 3])
+def path(request):
+    P.bebop_debug_force_general_path(request.param)
+    yield request.param
+    P.bebop_debug_force_general_path(0)
+
+
+def vocab(dtype, vectors, tail):
+    return (4 if dtype == "f32" else 8) * vectors - tail
+
+
+# vectors per row: a chunk and its neighbours, two stages' worth, the limits of one, two and four CTAs per row, a last CTA without
+# a vector of its own (129 chunks of 256 over eight CTAs: 17 each for seven of them)
+# (V = 1 is left out: p = q = 1 there, and whether q <= p, by which S jumps from 1 to 0, is a matter of the last bit)
+SIZES = [("bf16", 1, 3), ("f32", 128, 0), ("bf16", 129, 3), ("bf16", 257, 0), ("f32", 3073, 1), ("bf16", 7499, 5), ("f32", 7500, 2),
+         ("bf16", 10240, 0), ("bf16", 10241, 1), ("f32", 15001, 3), ("bf16", 40960, 0), ("bf16", 40961, 7), ("f32", 81921, 1)]
+
+
+@pytest.mark.parametrize("dtype,vectors,tail", SIZES)
+def test_verify(path, dtype, vectors, tail):
+    V = vocab(dtype, vectors, tail)
+    cfg = G.Config("stream", 5 if vectors > 20000 else 11, 3, V, dtype, 2.0, V >= 64, 0.8, (0.6, 1.2), ragged=True, seed=vectors)
+    x = G.make_inputs(cfg, "cuda", pad_ld=(-V) % 8)
+    x["draft_len"][1] = 0                                   # a sequence that is its bonus row
+    got = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
+                         temperature=x["temperature"], temperature_all=x["temperature_all"])
+    assert P.bebop_debug_last_kernel_name() == ("k_pipe" if path == 2 else "k_fuse")
+    ref = oracle_on(x)
+    compare_verify(got, ref, dtype, context=str(cfg))
+    check_properties(got, x)
+    if path == 2:                                           # the same call without a TV output: the sweeps
+        again = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
+                               temperature=x["temperature"], temperature_all=x["temperature_all"], want_tv=False)
+        compare_verify({k: v for k, v in again.items() if k != "tv"}, ref, dtype, context=str(cfg) + " without tv")
+
+
+@pytest.mark.parametrize("dtype,vectors,tail", SIZES)
+def test_tv(path, dtype, vectors, tail):
+    V, N = vocab(dtype, vectors, tail), 4 if vectors > 20000 else 300 if vectors < 200 else 9
+    g = torch.Generator(device="cuda").manual_seed(vectors)
+    store = torch.zeros((2, N, V + (-V) % 8), device="cuda")
+    store[0, :, :V] = 2.0 * torch.randn((N, V), generator=g, device="cuda")
+    store[1, :, :V] = store[0, :, :V] + torch.randn((N, V), generator=g, device="cuda")
+    store = store.to(torch.float32 if dtype == "f32" else torch.bfloat16)
+    got = P.bebop_tv(store[0, :, :V], store[1, :, :V])
+    ref = oracle.tv(store[0, :, :V].float().cpu().numpy(), store[1, :, :V].float().cpu().numpy())
+    assert np.abs(to_np(got["tv"]) - ref["tv"]).max() <= TOL[dtype]
+    assert np.abs(to_np(got["s_aux"]) - ref["s_aux"]).max() <= TOL[dtype]
+    assert (to_np(got["row_status"]) == 0).all()
+
+
+@pytest.mark.parametrize("B,K", [(1, 1), (2, 32), (900, 1), (2000, 4)])
+def test_shares(path, B, K):
+    """Fewer units than clusters, a sequence cut by many of them, more sequences than threads of a CTA."""
+    cfg = G.Config("shares", B, K, 1030, "bf16", 2.0, True, 0.8, 1.0, ragged=K > 1, seed=B + K)
+    x = G.make_inputs(cfg, "cuda", pad_ld=2)
+    got = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
+                         temperature=x["temperature"], temperature_all=x["temperature_all"])
+    check_properties(got, x)
+    idx = np.unique(np.linspace(0, B - 1, 200).astype(np.int64))
+    compare_verify(got, oracle_on(x, idx), "bf16", idx=idx, context=str(cfg))
