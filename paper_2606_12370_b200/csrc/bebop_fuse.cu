@@ -30,8 +30,9 @@ cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
 // run the stream, and the line only says under which name: bebop_tv up to 32 slices of 1024 vectors per row, bebop_verify up to eight
 // slices (fp32: six), with one draft position, or up to 40 (row, slice) tasks per SM.  Without TV the sweeps read one row
 // per sequence twice and the stream all of them: calls of up to 40 tasks per SM go through the stream (64 of 151,936 logits 73
-// against 77, 24 47 against 53), larger ones through the sweeps (192 of 32,000, K = 7, 74 against 95; 300 of 65,536 97 against
-// 106; 256 of 151,936, K = 1, 97 both).
+// against 77, 24 47 against 53), and rows of two or three slices with up to four positions (1,000 of 16,000, K = 2, 89 against 108; 400 of
+// 24,000, K = 4, 79 against 85); the others through the sweeps (192 of 32,000, K = 7, 74 against 95; 300 of 65,536 97 against 106;
+// 1,000 of 8,000, K = 8, 143 against 175).
 bool fuse_preferred(const RowArgs& a, bool tv_only, bool want_tv) {
     const int T = (a.nvec + 1023) / 1024;
     int sms = 0, dev = 0;
@@ -40,7 +41,7 @@ bool fuse_preferred(const RowArgs& a, bool tv_only, bool want_tv) {
     if (T > 32 || tasks < 2LL * sms) return false;
     if (tv_only) return true;
     if (want_tv && (T <= (a.dt == 0 ? 6 : 8) || a.K == 1)) return true;
-    return tasks <= 40LL * sms;
+    return tasks <= 40LL * sms || (!want_tv && a.K <= 4 && (T == 2 || T == 3));
 }
 
 }  // namespace bebop
