@@ -126,19 +126,33 @@ template <class F> __device__ __forceinline__ void flow_give_up(const FlowArgs& 
     atomicExch(a.wait_failed, 1);
     *(volatile int*)&S.abort = 1;
 }
-// bounded; gives up at once when the CTA has given up somewhere
-template <bool CL, class F> __device__ __noinline__ bool flow_wait_slow(const FlowArgs& a, FlowShared<F>& S, uint32_t addr, uint32_t parity) {
+// bounded; gives up at once when the CTA has given up somewhere; the answer is the lane's own
+template <class F> __device__ __noinline__ bool flow_wait_slow(const FlowArgs& a, FlowShared<F>& S, uint32_t addr, uint32_t parity) {
     for (uint32_t i = 0; i < kLSpin; ++i) {
-        if (CL ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity)) return true;
+        if (mbar_try(addr, parity)) return true;
         if (*(volatile int*)&S.abort) return false;
+    }
+    flow_give_up(a, S);
+    return false;
+}
+template <class F> __device__ __forceinline__ bool flow_wait_one(const FlowArgs& a, FlowShared<F>& S, unsigned long long* b, uint32_t parity) {
+    const uint32_t addr = smem_u32(b);
+    return mbar_try(addr, parity) || flow_wait_slow(a, S, addr, parity);
+}
+// The same for a whole warp, with one answer for all of its lanes: a lane that gave up alone would leave the others in warp-wide
+// reductions that it never comes to.
+template <bool CL, class F> __device__ __noinline__ bool flow_wait_slow_warp(const FlowArgs& a, FlowShared<F>& S, uint32_t addr, uint32_t parity) {
+    for (uint32_t i = 0; i < kLSpin; ++i) {
+        if (__all_sync(0xffffffffu, CL ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity))) return true;
+        if (__any_sync(0xffffffffu, *(volatile int*)&S.abort)) return false;
     }
     flow_give_up(a, S);
     return false;
 }
 template <bool CL = false, class F> __device__ __forceinline__ bool flow_wait(const FlowArgs& a, FlowShared<F>& S, unsigned long long* b, uint32_t parity) {
     const uint32_t addr = smem_u32(b);
-    if (CL ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity)) return true;
-    return flow_wait_slow<CL>(a, S, addr, parity);
+    if (__all_sync(0xffffffffu, CL ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity))) return true;
+    return flow_wait_slow_warp<CL>(a, S, addr, parity);
 }
 
 // ------------------------------------------------------------------ the cluster's run of units
@@ -214,7 +228,7 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
     // task: x = kind (0 pass 1, 1 pass 2, 3 stop) | row << 2 | last << 3 | first warp << 4 | chunks << 10 | first chunk << 16;
     // y = vectors of the task (of one row) | ragged << 16, z = c, w = unit's number
     auto issue = [&](int kind, int row, bool last, int c0, int chunks, int vecs, bool rag, float c, uint32_t u, const char* src0, const char* src1, unsigned long long pol) {
-        if (!flow_wait(a, S, &S.empty[st], ph)) { ok = false; return; }
+        if (!flow_wait_one(a, S, &S.empty[st], ph)) { ok = false; return; }
         S.task[st] = make_int4(kind | row << 2 | (last ? 8 : 0) | rot << 4 | chunks << 10 | c0 << 16, vecs | (rag ? 1 << 16 : 0), __float_as_int(c), (int)u);
         const uint32_t bytes = (uint32_t)vecs * 16u, dst = smem_u32(ring + (size_t)st * F::LSTAGE);
         if (bytes) {
@@ -334,8 +348,10 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
 #pragma unroll 1
     for (int st = -1, ph = 0;;) {
         if (++st == F::LNS) { st = 0; ph ^= 1; }
-        if (!flow_wait(a, S, &S.full[st], (uint32_t)ph)) break;
+        const bool there = flow_wait_one(a, S, &S.full[st], (uint32_t)ph);
         const int4 d = S.task[st];
+        // (one answer for the warp, as in flow_wait; voted here and not in front of the load: 1 per cent of a call)
+        if (!__all_sync(0xffffffffu, there)) break;
         if ((d.x & 3) == 3) break;
         int j = warp - ((d.x >> 4) & 63);
         if (j < 0) j += F::LW;
@@ -365,10 +381,10 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 // The lane's sum of e^2 is at most its sum of e, and at most that sum's square: the smaller, rounded up to 2^-15.
                 const int sq = redux_add(__float_as_int(__fmaf_ru(__fmul_ru(sum, fminf(sum, 1.f)), 32768.f, kMagic)));
                 if (lane == 0) { const int row = (d.x >> 2) & 1; S.psum[par][row][c0] = w; S.pexp[par][row][c0] = E.e; S.psq[par][row][c0] = sq; }
-            } else if (lane == 0) mbar_arrive(&S.empty[st]);
+            } else { __syncwarp(); if (lane == 0) mbar_arrive(&S.empty[st]); }          // (every lane has read the description)
             if (lane == 0 && (d.x & 8)) mbar_arrive(&S.p1[par]);
         } else {
-            if (!flow_wait(a, S, &S.stat[par], ((uint32_t)d.w / F::LSL) & 1u)) break;
+            const bool merged = flow_wait_one(a, S, &S.stat[par], ((uint32_t)d.w / F::LSL) & 1u);
             if (has) {
                 const unsigned char* src = ring + (size_t)st * F::LSTAGE + (size_t)(j * (F::LCV / 2) + lane) * 16;
                 constexpr int H = F::LQV / 2;
@@ -376,6 +392,7 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
 #pragma unroll
                 for (int i = 0; i < H; ++i) { xp[i] = *reinterpret_cast<const uint4*>(src + i * 512); xq[i] = *reinterpret_cast<const uint4*>(src + F::LSTAGE / 2 + i * 512); }
                 const float4 sc = S.scale[par];
+                if (!__all_sync(0xffffffffu, merged)) break;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[st]);
                 if ((j + 1) * (F::LCV / 2) > nv - (d.y >> 16)) {
@@ -393,7 +410,11 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 const int2 w = warp_sum_words(z.x + z.y);
                 if (lane == 0) S.cm[par][c0] = w;
                 if (TVM) { const int2 v = warp_sum_words(x.x + x.y); if (lane == 0) S.ca[par][c0] = v; }
-            } else if (lane == 0) mbar_arrive(&S.empty[st]);
+            } else {
+                if (!__all_sync(0xffffffffu, merged)) break;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.empty[st]);
+            }
             if (lane == 0 && (d.x & 8)) mbar_arrive(&S.p2[par]);
         }
         __syncwarp();
