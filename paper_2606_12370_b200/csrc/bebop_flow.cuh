@@ -762,18 +762,27 @@ __device__ __forceinline__ void flow_finisher(const FlowArgs& a, FlowShared<F>& 
     }
 }
 
-// A CTA that gave up: the sequences that nobody has completed and nobody will say so in their outputs.
+// A CTA that gave up: the sequences that nobody has completed and nobody will say so in their outputs.  The count decides, in the one
+// access that marks it: whoever delivers a last part afterwards finds the mark and completes nothing.
 template <bool TVM, class F>
 __device__ __noinline__ void flow_failed(const FlowArgs& a) {
     const RowArgs& R = a.r;
     const int K = R.K;
     for (int b = threadIdx.x; b < R.B; b += F::LT) {
         const int need = a.C * (TVM ? 1 : len_of(R, b) + 1);
-        if (ld_acquire(a.seqcnt + b) >= need || (atomicAdd(a.seqcnt + b, kFailed) & kFailed)) continue;
+        if (ld_acquire(a.seqcnt + b) >= need) continue;
+        const int old = atomicOr(a.seqcnt + b, kFailed);         // (added, two marks would overflow into a count that looks open)
+        if ((old & kFailed) || old >= need) continue;
         if (TVM) { a.o.tv[b] = 0.f; if (a.s_aux) a.s_aux[b] = 0.f; }
         else {
             a.o.accept_len[b] = 0;
             for (int q = 0; q <= K; ++q) a.o.out_tokens[(int64_t)b * (K + 1) + q] = -1;
+            for (int k = 0; k < K; ++k) {
+                const int64_t i = (int64_t)b * K + k;
+                if (a.o.tv) a.o.tv[i] = 0.f;
+                if (a.o.p_draft) a.o.p_draft[i] = 0.f;
+                if (a.o.q_draft) a.o.q_draft[i] = 0.f;
+            }
             draw_decided(a.fb_count);
         }
         if (a.o.row_status) a.o.row_status[b] = ST_WAIT;

@@ -74,3 +74,19 @@ def test_shares(path, B, K):
     check_properties(got, x)
     idx = np.unique(np.linspace(0, B - 1, 200).astype(np.int64))
     compare_verify(got, oracle_on(x, idx), "bf16", idx=idx, context=str(cfg))
+
+
+@pytest.mark.parametrize("B,K,V", [(6, 2, 1030), (300, 3, 20000)])
+def test_a_wait_that_runs_out_leaves_no_output_unwritten(path, B, K, V):
+    """Every CTA gives up on its first unit (test hook), so no sequence is completed: all outputs say so, and none keeps what
+    the caller's buffer held."""
+    x = G.make_inputs(G.Config("failed", B, K, V, "bf16", 2.0, True, 0.8, 1.0, seed=B), "cuda", pad_ld=(-V) % 8)
+    P.bebop_debug_expire_wait(2)
+    got = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"])
+    assert (to_np(got["row_status"]) & 32 == 32).all()
+    assert (to_np(got["accept_len"]) == 0).all() and (to_np(got["out_tokens"]) == -1).all()
+    for k in ("tv", "p_draft", "q_draft"):
+        assert (to_np(got[k]) == 0).all(), k
+    P.bebop_debug_expire_wait(2)
+    tv = P.bebop_tv(x["target"][:, 0], x["draft"][:, 0])
+    assert (to_np(tv["row_status"]) & 32 == 32).all() and (to_np(tv["tv"]) == 0).all() and (to_np(tv["s_aux"]) == 0).all()
