@@ -105,6 +105,57 @@ template <int N> __device__ __forceinline__ float sum_fixed(const float* e) {
     for (int i = 2; i < N; i += 2) acc = __fadd2_rn(acc, make_float2(e[i], e[i + 1]));
     return acc.x + acc.y;
 }
+// The warp's sum of the lanes' N vector sums, at most 32 times 2^SC a lane, as warp_sum_words of its 2^-SC, without further rounding
+// above 2^-38: each is split into a multiple of 2^-17 and the rest, two at a time.  The masses a token is drawn from are such sums:
+// added up in fp32, a lane's 64 tokens put a prefix of a flat row (151,936 logits N(0, 1), 20 rows on the host) off by up to 1.8 times
+// 2^-22 sqrt(sum p^2), the unit of the draw's bound; eight of them, a vector's, by 0.8.
+template <int N, int SC> __device__ __forceinline__ int2 vector_sum_words(const float* v) {
+    constexpr unsigned kBase = kSumBits0 + ((unsigned)SC << 23), kRest = 0x38C00000u + ((unsigned)SC << 23);          // 64 and 1.5 * 2^-14 (ulp 2^-37), times 2^SC
+    const float b = __int_as_float((int)kBase);
+    const float2 base = make_float2(b, b), below = make_float2(-b, -b), minus = make_float2(-1.f, -1.f);
+    unsigned hi = kSumBits0 - (unsigned)N * kBase;
+    float2 r = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        const float2 x = make_float2(v[i], v[i + 1]), y = __fadd2_rn(x, base), z = __ffma2_rn(__fadd2_rn(y, below), minus, x);
+        hi += (unsigned)__float_as_int(y.x) + (unsigned)__float_as_int(y.y);
+        r = i == 0 ? z : __fadd2_rn(r, z);
+    }
+    const int lo = redux_add(__float_as_int(__fadd_rn(r.x + r.y, __int_as_float((int)kRest))));
+    return make_int2(redux_add((int)hi), (int)(((unsigned)lo - 32u * kRest) * 8u + (unsigned)kNoSum1));
+}
+// Pass 1 of a chunk of Q vectors a lane around exponent Ef: half its sum of exponentials, in words, and the lane's sum.  EXACT (a
+// sequence's rows, the bonus row among them): the vectors' sums are added exactly; bebop_tv, which draws nothing, adds a lane's
+// tokens in fp32 (256 x 151,936 178.1 us with fp32 sums for both, 181.4 with exact ones; as a branch for bonus rows alone 181.8 and up).
+template <int DT, int Q, bool EXACT>
+__device__ __forceinline__ int2 chunk_sum(const uint4* x, float c, float Ef, float* sum) {
+    constexpr int VEC = Elem<DT>::VEC;
+    if constexpr (EXACT) {
+        float v[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            float e[VEC];
+            exp_vec<DT>(x[i], c, Ef, e);
+            v[i] = sum_fixed<VEC>(e);
+        }
+        float2 t = make_float2(v[0], v[1]);
+#pragma unroll
+        for (int i = 2; i < Q; i += 2) t = __fadd2_rn(t, make_float2(v[i], v[i + 1]));
+        *sum = t.x + t.y;
+        return vector_sum_words<Q, 1>(v);
+    } else {
+        float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            float e[VEC];
+            exp_vec<DT>(x[i], c, Ef, e);
+#pragma unroll
+            for (int q = 0; q < VEC; q += 4) { s0 = __fadd2_rn(s0, make_float2(e[q], e[q + 1])); s1 = __fadd2_rn(s1, make_float2(e[q + 2], e[q + 3])); }
+        }
+        *sum = (s0.x + s0.y) + (s1.x + s1.y);
+        return warp_sum_words(0.5f * *sum);
+    }
+}
 // Owner of the target t of an inverse CDF among values that the lanes hold in order (`below` lies before lane 0): its
 // lane (-1: none), the running sum before it in *base, the total in *total.
 __device__ __forceinline__ int owner_lane(double v, double below, double t, double* base, double* total) {

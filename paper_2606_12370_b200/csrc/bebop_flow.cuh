@@ -227,9 +227,9 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
     bool ok = true;
     // task: x = kind (0 pass 1, 1 pass 2, 3 stop) | row << 2 | last << 3 | first warp << 4 | chunks << 10 | first chunk << 16;
     // y = vectors of the task (of one row) | ragged << 16, z = c, w = unit's number
-    auto issue = [&](int kind, int row, bool last, int c0, int chunks, int vecs, bool rag, float c, uint32_t u, const char* src0, const char* src1, unsigned long long pol) {
+    auto issue = [&](int kind, int row, bool last, int c0, int chunks, int vecs, int flags, float c, uint32_t u, const char* src0, const char* src1, unsigned long long pol) {
         if (!flow_wait_one(a, S, &S.empty[st], ph)) { ok = false; return; }
-        S.task[st] = make_int4(kind | row << 2 | (last ? 8 : 0) | rot << 4 | chunks << 10 | c0 << 16, vecs | (rag ? 1 << 16 : 0), __float_as_int(c), (int)u);
+        S.task[st] = make_int4(kind | row << 2 | (last ? 8 : 0) | rot << 4 | chunks << 10 | c0 << 16, vecs | flags << 16, __float_as_int(c), (int)u);
         const uint32_t bytes = (uint32_t)vecs * 16u, dst = smem_u32(ring + (size_t)st * F::LSTAGE);
         if (bytes) {
             mbar_arrive_expect(&S.full[st], src1 ? 2u * bytes : bytes);
@@ -245,21 +245,21 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
         do {
             const int left = nv - c0 * F::LCV, vecs = min(left, F::LW * F::LCV), chunks = (vecs + F::LCV - 1) / F::LCV;
             const bool fin = vecs == left;
-            issue(0, which, end && fin, c0, chunks, vecs, fin && ragged, c, u, row + (int64_t)(v0 + c0 * F::LCV) * 16, nullptr, pol);
+            issue(0, which, end && fin, c0, chunks, vecs, fin ? ragged : 0, c, u, row + (int64_t)(v0 + c0 * F::LCV) * 16, nullptr, pol);
             c0 += F::LW;
         } while (ok && c0 * F::LCV < nv);
     };
     auto pass2 = [&](uint32_t u) {
         const FlowUnit x = S.unit[u % LUD];
         const float c = S.uc[u % LUD];
-        if (!x.pair || nv == 0) { issue(1, 0, true, 0, 0, 0, false, c, u, nullptr, nullptr, drop); return; }
+        if (!x.pair || nv == 0) { issue(1, 0, true, 0, 0, 0, 0, c, u, nullptr, nullptr, drop); return; }
         constexpr int CV = F::LCV / 2;
         const char* p = row_ptr(R, x.b, x.k) + (int64_t)v0 * 16; const char* q = row_ptr(R, x.b, R.K + 1 + x.k) + (int64_t)v0 * 16;
         int c0 = 0;
         do {
             const int left = nv - c0 * CV, vecs = min(left, F::LW * CV), chunks = (vecs + CV - 1) / CV;
             const bool fin = vecs == left;
-            issue(1, 0, fin, c0, chunks, vecs, fin && ragged, c, u, p + (int64_t)c0 * CV * 16, q + (int64_t)c0 * CV * 16, drop);
+            issue(1, 0, fin, c0, chunks, vecs, fin ? ragged : 0, c, u, p + (int64_t)c0 * CV * 16, q + (int64_t)c0 * CV * 16, drop);
             c0 += F::LW;
         } while (ok && c0 * CV < nv);
     };
@@ -291,7 +291,7 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
     for (uint32_t i = u < (uint32_t)a.lag ? 0u : u - a.lag; ok && i < u; ++i) pass2(i);
     S.unit[u % LUD].b = -1;
     mbar_arrive(&S.ud[u % LUD]);
-    if (ok) issue(3, 0, false, 0, 0, 0, false, 0.f, u, nullptr, nullptr, drop);
+    if (ok) issue(3, 0, false, 0, 0, 0, 0, 0.f, u, nullptr, nullptr, drop);
     // no copy of this CTA is under way when it leaves: the last ones have arrived (bounded)
     for (int i = 0; i < F::LNS && i < n; ++i) {
         if (--st < 0) { st = F::LNS - 1; ph ^= 1u; }
@@ -325,22 +325,32 @@ __device__ __forceinline__ void mask_vecs(uint4* x, int vi, int nv, bool ragged,
     }
 }
 // Residuals of one vector pair: r' = max(0, e_p - rho e_q), rho as two floats, the large product first; as e_p <= 1, saturating
-// to [0, 1] is the maximum with 0.  Their sum goes to *z; with AUX the sum of e_q over the tokens with q <= p to *x.
-template <int N, bool AUX>
-__device__ __forceinline__ void resid_sum(const float* p, const float* q, float2 rho, float2* z, float2* x) {
+// to [0, 1] is the maximum with 0.  Their sum (the one that the finisher forms, sum_fixed).
+template <int N>
+__device__ __forceinline__ float resid_sum(const float* p, const float* q, float2 rho) {
+    const float2 nh = make_float2(-rho.x, -rho.x);
+    float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        const float2 t = __ffma2_rn(nh, make_float2(q[i], q[i + 1]), make_float2(p[i], p[i + 1]));
+        const float2 r = make_float2(fma_sat(-rho.y, q[i], t.x), fma_sat(-rho.y, q[i + 1], t.y));
+        z = i == 0 ? r : __fadd2_rn(z, r);
+    }
+    return z.x + z.y;
+}
+// bebop_tv: adds the residuals to *z and the e_q of the tokens with q <= p to *x.
+template <int N>
+__device__ __forceinline__ void resid_aux(const float* p, const float* q, float2 rho, float2* z, float2* x) {
     const float2 nh = make_float2(-rho.x, -rho.x), nl = make_float2(-rho.y, -rho.y);
 #pragma unroll
     for (int i = 0; i < N; i += 2) {
-        const float2 q2 = make_float2(q[i], q[i + 1]), t = __ffma2_rn(nh, q2, make_float2(p[i], p[i + 1]));
-        if (AUX) {
-            const float2 d = __ffma2_rn(nl, q2, t);
-            const float2 mk = make_float2(d.x >= 0.f ? 1.f : 0.f, d.y >= 0.f ? 1.f : 0.f);
-            *z = __ffma2_rn(d, mk, *z);
-            *x = __ffma2_rn(q2, mk, *x);
-        } else *z = __fadd2_rn(*z, make_float2(fma_sat(nl.x, q[i], t.x), fma_sat(nl.x, q[i + 1], t.y)));
+        const float2 q2 = make_float2(q[i], q[i + 1]);
+        const float2 d = __ffma2_rn(nl, q2, __ffma2_rn(nh, q2, make_float2(p[i], p[i + 1])));
+        const float2 mk = make_float2(d.x >= 0.f ? 1.f : 0.f, d.y >= 0.f ? 1.f : 0.f);
+        *z = __ffma2_rn(d, mk, *z);
+        *x = __ffma2_rn(q2, mk, *x);
     }
 }
-
 template <int DT, bool TVM, class F>
 __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& S, const unsigned char* ring, int warp, int lane) {
     constexpr int VEC = Elem<DT>::VEC;
@@ -357,6 +367,7 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
         if (j < 0) j += F::LW;
         const int c0 = (d.x >> 16) + j, par = d.w & (F::LSL - 1), nv = d.y & 0xffff;
         const bool has = j < ((d.x >> 10) & 63);
+        const int ragged = d.y >> 16;
         const float c = __int_as_float(d.z);
         if ((d.x & 3) == 0) {
             if (has) {
@@ -366,18 +377,10 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 for (int i = 0; i < F::LQV; ++i) x[i] = *reinterpret_cast<const uint4*>(src + i * 512);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[st]);
-                if ((j + 1) * F::LCV > nv - (d.y >> 16)) mask_vecs<DT, F::LQV>(x, j * F::LCV + lane, nv, d.y >> 16, keep);
+                if ((j + 1) * F::LCV > nv - ragged) mask_vecs<DT, F::LQV>(x, j * F::LCV + lane, nv, ragged, keep);
                 const QExp E = chunk_exponent(vecs_max<DT, F::LQV>(x), c);
-                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
-#pragma unroll
-                for (int i = 0; i < F::LQV; ++i) {
-                    float e[VEC];
-                    exp_vec<DT>(x[i], c, E.ef, e);
-#pragma unroll
-                    for (int q = 0; q < VEC; q += 4) { s0 = __fadd2_rn(s0, make_float2(e[q], e[q + 1])); s1 = __fadd2_rn(s1, make_float2(e[q + 2], e[q + 3])); }
-                }
-                const float sum = (s0.x + s0.y) + (s1.x + s1.y);
-                const int2 w = warp_sum_words(0.5f * sum);
+                float sum;
+                const int2 w = chunk_sum<DT, F::LQV, !TVM>(x, c, E.ef, &sum);
                 // The lane's sum of e^2 is at most its sum of e, and at most that sum's square: the smaller, rounded up to 2^-15.
                 const int sq = redux_add(__float_as_int(__fmaf_ru(__fmul_ru(sum, fminf(sum, 1.f)), 32768.f, kMagic)));
                 if (lane == 0) { const int row = (d.x >> 2) & 1; S.psum[par][row][c0] = w; S.pexp[par][row][c0] = E.e; S.psq[par][row][c0] = sq; }
@@ -395,21 +398,34 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 if (!__all_sync(0xffffffffu, merged)) break;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[st]);
-                if ((j + 1) * (F::LCV / 2) > nv - (d.y >> 16)) {
-                    mask_vecs<DT, H>(xp, j * (F::LCV / 2) + lane, nv, d.y >> 16, keep);
-                    mask_vecs<DT, H>(xq, j * (F::LCV / 2) + lane, nv, d.y >> 16, keep);
+                if ((j + 1) * (F::LCV / 2) > nv - ragged) {
+                    mask_vecs<DT, H>(xp, j * (F::LCV / 2) + lane, nv, ragged, keep);
+                    mask_vecs<DT, H>(xq, j * (F::LCV / 2) + lane, nv, ragged, keep);
                 }
-                float2 z = make_float2(0.f, 0.f), x = z;
+                const float2 rho = make_float2(sc.z, sc.w);
+                if (TVM) {
+                    float2 z = make_float2(0.f, 0.f), x = z;
 #pragma unroll
-                for (int i = 0; i < H; ++i) {
-                    float p[VEC], q[VEC];
-                    exp_vec<DT>(xp[i], c, sc.x, p);
-                    exp_vec<DT>(xq[i], c, sc.y, q);
-                    resid_sum<VEC, TVM>(p, q, make_float2(sc.z, sc.w), &z, &x);
+                    for (int i = 0; i < H; ++i) {
+                        float p[VEC], q[VEC];
+                        exp_vec<DT>(xp[i], c, sc.x, p);
+                        exp_vec<DT>(xq[i], c, sc.y, q);
+                        resid_aux<VEC>(p, q, rho, &z, &x);
+                    }
+                    const int2 w = warp_sum_words(z.x + z.y), v = warp_sum_words(x.x + x.y);
+                    if (lane == 0) { S.cm[par][c0] = w; S.ca[par][c0] = v; }
+                } else {
+                    float v[H];
+#pragma unroll
+                    for (int i = 0; i < H; ++i) {
+                        float p[VEC], q[VEC];
+                        exp_vec<DT>(xp[i], c, sc.x, p);
+                        exp_vec<DT>(xq[i], c, sc.y, q);
+                        v[i] = resid_sum<VEC>(p, q, rho);
+                    }
+                    const int2 w = vector_sum_words<H, 0>(v);
+                    if (lane == 0) S.cm[par][c0] = w;
                 }
-                const int2 w = warp_sum_words(z.x + z.y);
-                if (lane == 0) S.cm[par][c0] = w;
-                if (TVM) { const int2 v = warp_sum_words(x.x + x.y); if (lane == 0) S.ca[par][c0] = v; }
             } else {
                 if (!__all_sync(0xffffffffu, merged)) break;
                 __syncwarp();

@@ -494,22 +494,12 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
             if (at + u * 32 < nv && gbase + VEC > R.V) mask_tail<DT>(raw[u], R.V - gbase);
         }
     }
-    // one exponent per warp, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time, four running sums
+    // one exponent per warp, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time
     const QExp E = chunk_exponent(vecs_max<DT, NV>(raw), d.c);
-    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-        float e[VEC];
-        exp_vec<DT>(raw[u], d.c, E.ef, e);
-#pragma unroll
-        for (int i = 0; i < VEC; i += 4) {
-            s0 = __fadd2_rn(s0, make_float2(e[i], e[i + 1]));
-            s1 = __fadd2_rn(s1, make_float2(e[i + 2], e[i + 3]));
-        }
-    }
+    float lane_sum;
+    const int2 sum = chunk_sum<DT, NV, true>(raw, d.c, E.ef, &lane_sum);
     const bool bad = E.e == E_BAD;
     const int Ew = bad ? E_EMPTY : E.e;
-    const int2 sum = warp_sum_words(0.5f * ((s0.x + s0.y) + (s1.x + s1.y)));
     const float mw = bad ? __int_as_float(0x7fc00000) : 0.f;
     if (lane == 0) { S.wd[stage][warp] = Ew > E_EMPTY ? 2.0 * word_value(sum) : 0.0; S.wi[stage][warp] = Ew; S.wf[stage][1][warp] = mw; }
     __syncwarp();
