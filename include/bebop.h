@@ -172,7 +172,7 @@ bebop_status_t bebop_greedy_verify(
  * wherever it applies.  All give the same results up to the documented tolerances.  bebop_debug_last_kernel() says
  * what the last of these calls ran: 1 the general kernels, 2 the pipelined kernel, 3 the fused or the sequence
  * kernel (0: no call yet); bebop_debug_last_kernel_name() says it by name: "general", "k_pipe" (its sweeps, or with a TV
- * output its stream, k_pipe_stream), "k_fuse", "k_seq", "k_seq_greedy" ("none": no call yet).
+ * output the stream, k_fuse, under this name), "k_fuse", "k_seq", "k_seq_greedy" ("none": no call yet).
  * bebop_debug_fallback_offset returns the byte offset, inside the workspace of this
  * shape, of an int32 that after a bebop_verify call through the pipelined or the fused kernel holds the number of
  * sequences whose draw was re-done by the fp64 kernels.

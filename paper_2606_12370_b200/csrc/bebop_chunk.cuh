@@ -17,6 +17,9 @@ __device__ __forceinline__ void mbar_init(unsigned long long* b, int count) {
 __device__ __forceinline__ void mbar_arrive_expect(unsigned long long* b, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(b)), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(b)) : "memory");
+}
 __device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
     uint32_t ok;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -80,9 +83,22 @@ __device__ __forceinline__ int2 warp_sum_words(float x) {
 __device__ __forceinline__ long long words_sum(int hi, int lo) {
     return ((long long)(int)((unsigned)hi - (unsigned)kNoSum0) << 23) + (int)((unsigned)lo - (unsigned)kNoSum1);
 }
-__device__ __forceinline__ double warp_sum_fixed(float x) {
-    const int2 w = warp_sum_words(x);
-    return (double)words_sum(w.x, w.y) * 9.094947017729282e-13;            // 2^-40
+__device__ __forceinline__ double word_value(int2 w) { return (double)words_sum(w.x, w.y) * 9.094947017729282e-13; }      // 2^-40
+__device__ __forceinline__ double warp_sum_fixed(float x) { return word_value(warp_sum_words(x)); }
+// the largest logit of a lane's N vectors (NaN if there is one); bf16: packed maxima, unpacked once
+template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* v) {
+    if (DT == 1) {
+        uint32_t m[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) m[j] = max_nan_bf16x2(max_nan_bf16x2(v[j].x, v[j].y), max_nan_bf16x2(v[j].z, v[j].w));
+#pragma unroll
+        for (int j = 1; j < N; ++j) m[0] = max_nan_bf16x2(m[0], m[j]);
+        return max_nan(__uint_as_float(m[0] << 16), __uint_as_float(m[0] & 0xffff0000u));
+    }
+    float m = vec_max<DT>(v[0]);
+#pragma unroll
+    for (int j = 1; j < N; ++j) m = max_nan(m, vec_max<DT>(v[j]));
+    return m;
 }
 // the exponentials of one vector around exponent Ef, two at a time
 template <int DT>

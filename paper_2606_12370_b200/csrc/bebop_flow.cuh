@@ -106,9 +106,6 @@ template <class F> struct FlowShared {
 };
 
 // ------------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(b)) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_cluster(uint32_t addr, uint32_t parity) {
     uint32_t ok;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -300,20 +297,6 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
 }
 
 // ------------------------------------------------------------------ consumers
-template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* v) {
-    if (DT == 1) {
-        uint32_t m[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) m[j] = max_nan_bf16x2(max_nan_bf16x2(v[j].x, v[j].y), max_nan_bf16x2(v[j].z, v[j].w));
-#pragma unroll
-        for (int j = 1; j < N; ++j) m[0] = max_nan_bf16x2(m[0], m[j]);
-        return max_nan(__uint_as_float(m[0] << 16), __uint_as_float(m[0] & 0xffff0000u));
-    }
-    float m = vec_max<DT>(v[0]);
-#pragma unroll
-    for (int j = 1; j < N; ++j) m = max_nan(m, vec_max<DT>(v[j]));
-    return m;
-}
 // what a chunk does not have in full: vectors beyond the task read as -inf, the row's ragged last vector loses the lanes
 // beyond the vocabulary
 template <int DT, int N>
@@ -438,9 +421,6 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
 }
 
 // ------------------------------------------------------------------ helper
-constexpr double kWordUnit = 9.094947017729282e-13;            // 2^-40
-__device__ __forceinline__ double word_value(int2 w) { return (double)words_sum(w.x, w.y) * kWordUnit; }
-
 // over the 16 lanes of a half warp, every lane gets the result (one fixed tree)
 __device__ __forceinline__ int half_max(int v) {
 #pragma unroll

@@ -26,9 +26,9 @@ cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
     return a.dt == 0 ? go(F32{}, std::false_type{}) : go(BF16{}, std::false_type{});
 }
 
-// The lines between the two, and to the sweeps without TV (us per call on a B200, bf16 and K = 3 unless said).  With TV both
-// run the stream, and the line only says under which name: bebop_tv up to 32 slices of 1024 vectors per row, bebop_verify up to eight
-// slices (fp32: six), with one draft position, or up to 40 (row, slice) tasks per SM.  Without TV the sweeps read one row
+// With TV both names run the stream, by the same rules for clusters and chunks, and the line only says under which name a call
+// goes: bebop_tv up to 32 slices of 1024 vectors per row, bebop_verify up to eight slices (fp32: six), with one draft position, or up to 40
+// (row, slice) tasks per SM.  Without TV (us per call on a B200, bf16) the sweeps read one row
 // per sequence twice and the stream all of them: calls of up to 40 tasks per SM go through the stream (64 of 151,936 logits 73
 // against 77, 24 47 against 53), and rows of two or three slices with up to four positions (1,000 of 16,000, K = 2, 89 against 108; 400 of
 // 24,000, K = 4, 79 against 85); the others through the sweeps (192 of 32,000, K = 7, 74 against 95; 300 of 65,536 97 against 106;

@@ -57,8 +57,8 @@ cudaError_t redraw_launch(const RowArgs& a, const float* u_final, VerifyOut o, c
                           const PipePlan& wp, cudaStream_t stream, bool expire_list_wait = false);
 
 // Pipelined kernel (bebop_pipe.cu): a ticket schedule with a producer warp that stages every task's logits in shared memory by
-// bulk copies while the other warps compute; where TV is asked for, the stream of bebop_flow.cuh.  With `tv_only` it is
-// bebop_tv: B row pairs (K = 1), o.tv and s_aux the outputs, no tokens, no uniforms, no draw.
+// bulk copies while the other warps compute.  Where TV is asked for, and with `tv_only` (bebop_tv: B row pairs, K = 1, o.tv and
+// s_aux the outputs, no tokens, no uniforms, no draw), it passes the call on to fuse_verify.
 bool pipe_supported(const RowArgs& a);
 cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,

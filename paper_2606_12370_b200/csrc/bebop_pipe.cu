@@ -1,6 +1,6 @@
 // Pipelined kernel: bebop_verify without a TV output, and the greedy mode, as one persistent, ticket-scheduled kernel with the
-// data movement and the bookkeeping taken off the compute warps.  (Calls with a TV output, and bebop_tv, run the stream of
-// bebop_flow.cuh from here: their second pass reads every row pair, this kernel's one row pair per sequence.)
+// data movement and the bookkeeping taken off the compute warps.  (Calls with a TV output, and bebop_tv, are passed on to the
+// stream, bebop_fuse.cu: their second pass reads every row pair, this kernel's one row pair per sequence.)
 //
 // The work is a queue of tickets in two blocks, sequences ascending in each: P1 (softmax partial of one
 // slice of one row) for every row; then P2 (residual mass of one half slice) for the row pair, or bonus row, each sequence's
@@ -29,7 +29,7 @@
 //
 // Every wait is bounded; a wait that gives up sets the wait flag (status bit 32 of every row).
 // No multicast, no cluster: each CTA copies from this GPU's own memory.
-#include "bebop_flow.cuh"
+#include "bebop_chunk.cuh"
 
 namespace bebop {
 
@@ -924,15 +924,9 @@ __global__ void __launch_bounds__(PT, PIPE_CTAS) k_pipe(const __grid_constant__ 
     }
 }
 
-// The stream of bebop_flow.cuh as the pipelined kernel runs it: the calls with a TV output that are too large for the fused
-// kernel's region.
-template <int DT, bool TVM, class F>
-__global__ void __launch_bounds__(F::LT, 1) k_pipe_stream(const __grid_constant__ FlowArgs a) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    flow_body<DT, TVM, F>(a, smem);
-}
-
 // -----------------------------------------------------------------------------
+extern cudaEvent_t g_ev_start, g_ev_stop;
+
 namespace {
 
 // Clears what a call needs cleared.  A kernel instead of a memset, because k_pipe can then be its programmatic dependent,
@@ -994,14 +988,8 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only, float* s_aux) {
     *launched = false;
-    if (tv_only || o.tv) {
-        // with TV every row pair has a second pass: the stream, which reads it from L2
-        const FlowCall x{a, p, draft_tokens, u_accept, u_final, o, ws, stream, tv_only, s_aux};
-        using F = FlowLong;
-        const int C = flow_cluster(a, tv_only);
-        if (tv_only) return a.dt == 0 ? flow_launch<F, k_pipe_stream<0, true, F>>(x, C, launched) : flow_launch<F, k_pipe_stream<1, true, F>>(x, C, launched);
-        return a.dt == 0 ? flow_launch<F, k_pipe_stream<0, false, F>>(x, C, launched) : flow_launch<F, k_pipe_stream<1, false, F>>(x, C, launched);
-    }
+    // with TV every row pair has a second pass: the stream, which reads it from L2
+    if (tv_only || o.tv) return fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, launched, tv_only, s_aux);
     const int grid_max = a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>();
     if (grid_max < 1) return cudaSuccess;
     const PipePlan wp = make_pipe_plan(a.B, a.K, a.nvec, a.dt, PSLICE);
