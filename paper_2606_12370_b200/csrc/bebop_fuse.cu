@@ -26,8 +26,6 @@ cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
     return a.dt == 0 ? go(F32{}, std::false_type{}) : go(BF16{}, std::false_type{});
 }
 
-bool fuse_small_chunks(const RowArgs& a) { return !flow_long(a, false, flow_cluster(a, false)); }
-
 // With TV both names run the stream, by the same rules for clusters and chunks, and the line only says under which name a call
 // goes: bebop_tv up to 32 slices of 1024 vectors per row, bebop_verify up to eight slices (fp32: six), with one draft position, or up to 40
 // (row, slice) tasks per SM.  Without TV (us per call on a B200, bf16) the sweeps read one row

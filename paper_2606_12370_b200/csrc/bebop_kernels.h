@@ -67,8 +67,6 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
 // Fused kernel (bebop_fuse.cu): the stream of bebop_flow.cuh, every row read from memory once and out of L2 a second time; same
 // contract as pipe_verify, which runs it too wherever a TV output is asked for.  fuse_preferred: the line between the two.
 bool fuse_preferred(const RowArgs& a, bool tv_only, bool want_tv);
-// Whether bebop_verify's rows go through the stream in chunks of 128 vectors (else 256): the sweeps follow it.
-bool fuse_small_chunks(const RowArgs& a);
 cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
                         cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);

@@ -467,16 +467,14 @@ template <int N> __device__ __forceinline__ void resid_n(const float* p, const f
     }
 }
 // P1: softmax partial (E, S) of one slice of one row, from shared memory.
-// HALF: in two chunks of 128 vectors a warp, the stream's chunks of short rows.
-template <int DT, bool HALF>
+template <int DT>
 __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const TaskDesc& d, const unsigned char* data,
                                         int stage) {
     constexpr int VEC = Elem<DT>::VEC, NV = PSLICE / PC;
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = d.nv;
-    // a warp has 256 vectors side by side, one or two chunks of the stream's pass 1: both give a row the same sum, so that p and q of the
-    // drafts do not depend on whether TV is asked for
+    // a warp has 256 vectors side by side, the chunk of the stream's pass 1: both give a row the same sum
     const int at = warp * (32 * NV) + lane;
     uint4 raw[NV];
     if ((warp + 1) * (32 * NV) <= nv) {
@@ -496,26 +494,14 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
             if (at + u * 32 < nv && gbase + VEC > R.V) mask_tail<DT>(raw[u], R.V - gbase);
         }
     }
-    // one exponent per chunk, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time
-    constexpr int NC = HALF ? 2 : 1, Q = NV / NC;
-    int Ec[NC], E = E_EMPTY;
-    int2 sum[NC];
-#pragma unroll
-    for (int h = 0; h < NC; ++h) {
-        const QExp x = chunk_exponent(vecs_max<DT, Q>(raw + h * Q), d.c);
-        float lane_sum;
-        sum[h] = chunk_sum<DT, Q, true>(raw + h * Q, d.c, x.ef, &lane_sum);
-        Ec[h] = x.e;
-        E = max(E, x.e);
-    }
-    const bool bad = E == E_BAD;
-    if (bad) E = E_EMPTY;
-    if (lane == 0) {
-        double s = 0.0;
-#pragma unroll
-        for (int h = 0; h < NC; ++h) if (!bad && Ec[h] > E_EMPTY) s += 2.0 * word_value(sum[h]) * pow2d(max(Ec[h] - E, -1000));
-        S.wd[stage][warp] = s; S.wi[stage][warp] = E; S.wf[stage][1][warp] = bad ? __int_as_float(0x7fc00000) : 0.f;
-    }
+    // one exponent per warp, which bounds every e = 2^(x c - E) by 1; the exponentials two at a time
+    const QExp E = chunk_exponent(vecs_max<DT, NV>(raw), d.c);
+    float lane_sum;
+    const int2 sum = chunk_sum<DT, NV, true>(raw, d.c, E.ef, &lane_sum);
+    const bool bad = E.e == E_BAD;
+    const int Ew = bad ? E_EMPTY : E.e;
+    const float mw = bad ? __int_as_float(0x7fc00000) : 0.f;
+    if (lane == 0) { S.wd[stage][warp] = Ew > E_EMPTY ? 2.0 * word_value(sum) : 0.0; S.wi[stage][warp] = Ew; S.wf[stage][1][warp] = mw; }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.pdone[stage]);
 }
@@ -894,7 +880,7 @@ __device__ __forceinline__ void publisher(const PipeArgs& a, PipeShared& S) {
 
 }  // namespace
 
-template <int DT, int MODE, bool HALF = false>
+template <int DT, int MODE>
 __global__ void __launch_bounds__(PT, PIPE_CTAS) k_pipe(const __grid_constant__ PipeArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* data = smem;
@@ -927,7 +913,7 @@ __global__ void __launch_bounds__(PT, PIPE_CTAS) k_pipe(const __grid_constant__ 
         if (d.phase < 0) break;
         const unsigned char* sd = data + (size_t)stage * STAGE_BYTES;
         if (MODE == kModeGreedy) pipe_g<DT>(a, S, d, sd, stage);
-        else if (d.phase == 0) pipe_p1<DT, HALF>(a, S, d, sd, stage);
+        else if (d.phase == 0) pipe_p1<DT>(a, S, d, sd, stage);
         else if (d.phase == 2) pipe_p2<DT>(a, S, d, sd, stage);
         else {
             pipe_d<DT>(a, S, d, sd, meet);
@@ -965,18 +951,18 @@ template <typename K> cudaError_t launch_cleared(K kernel, const PipeArgs& wa, i
 
 constexpr size_t kPipeSmem = (size_t)NST * STAGE_BYTES + sizeof(PipeShared);
 
-template <int DT, int MODE, bool HALF = false>
+template <int DT, int MODE>
 int pipe_grid() {
     static int cached[64] = {0};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (dev >= 0 && dev < 64 && cached[dev]) return cached[dev];
-    if (cudaFuncSetAttribute(k_pipe<DT, MODE, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_pipe<DT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pipe<DT, MODE, HALF>, PT, kPipeSmem) != cudaSuccess) per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pipe<DT, MODE>, PT, kPipeSmem) != cudaSuccess) per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaGetLastError();
     const int n = per_sm * sms;
@@ -1004,9 +990,7 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
     *launched = false;
     // with TV every row pair has a second pass: the stream, which reads it from L2
     if (tv_only || o.tv) return fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, launched, tv_only, s_aux);
-    const bool half = fuse_small_chunks(a);
-    const int grid_max = half ? (a.dt == 0 ? pipe_grid<0, kModeVerify, true>() : pipe_grid<1, kModeVerify, true>())
-                              : (a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>());
+    const int grid_max = a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>();
     if (grid_max < 1) return cudaSuccess;
     const PipePlan wp = make_pipe_plan(a.B, a.K, a.nvec, a.dt, PSLICE);
     PipeArgs wa;
@@ -1034,8 +1018,7 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
         wa.ntickets = (int)total;
     }
     const int grid = wa.ntickets < grid_max ? wa.ntickets : grid_max;
-    const cudaError_t e = launch_cleared(half ? (a.dt == 0 ? k_pipe<0, kModeVerify, true> : k_pipe<1, kModeVerify, true>)
-                                            : (a.dt == 0 ? k_pipe<0, kModeVerify> : k_pipe<1, kModeVerify>), wa, grid, kPipeSmem, w, wp.zero_bytes, stream);
+    const cudaError_t e = launch_cleared(a.dt == 0 ? k_pipe<0, kModeVerify> : k_pipe<1, kModeVerify>, wa, grid, kPipeSmem, w, wp.zero_bytes, stream);
     if (g_ev_stop) cudaEventRecord(g_ev_stop, stream);
     if (e != cudaSuccess) return e;
     *launched = true;

@@ -103,13 +103,3 @@ def test_one_rule_for_the_chunks_whatever_the_name(dtype, B, K, V):
     P.bebop_debug_force_general_path(0)
     for k in ("accept_len", "out_tokens", "tv", "p_draft", "q_draft", "row_status"):
         assert torch.equal(got[2][k], got[3][k]), k
-
-
-@pytest.mark.parametrize("dtype,B,K,V", [("bf16", 192, 7, 32000), ("f32", 96, 8, 30001), ("bf16", 220, 2, 100001), ("bf16", 700, 6, 9999)])
-def test_probabilities_do_not_depend_on_the_tv_output(dtype, B, K, V):
-    """Left to choose, a call with TV streams in small or large chunks, one without goes through the sweeps or the stream: the
-    same p and q of every draft, so the same accept tests."""
-    x = G.make_inputs(G.Config("bits", B, K, V, dtype, 2.0, True, 0.8, 0.9, seed=B), "cuda", pad_ld=(-V) % 8)
-    a, b = (P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], temperature_all=0.9, want_tv=w) for w in (True, False))
-    for k in ("accept_len", "p_draft", "q_draft", "row_status"):
-        assert torch.equal(a[k], b[k]), k
