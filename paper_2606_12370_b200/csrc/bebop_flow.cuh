@@ -119,7 +119,11 @@ __device__ __forceinline__ void bulk_load_hint(uint32_t dst, const void* src, ui
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy) : "memory");
 }
+// What the call clears (the sequences' counts, the re-draw's list and counters, the wait flag) is clear from here on.  Everything
+// else goes ahead of it: the clearing kernel in front has waited for what came before the call.
+__device__ __forceinline__ void flow_cleared() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class F> __device__ __forceinline__ void flow_give_up(const FlowArgs& a, FlowShared<F>& S) {
+    flow_cleared();
     atomicExch(a.wait_failed, 1);
     *(volatile int*)&S.abort = 1;
 }
@@ -520,6 +524,8 @@ __device__ __forceinline__ void flow_publish(const FlowArgs& a, FlowShared<F>& S
     const int lane = threadIdx.x & 31, C = a.C;
     const int v0 = rank * a.sv, nv = max(min(a.sv, R.nvec - v0), 0), n2 = (nv + F::LCV / 2 - 1) / (F::LCV / 2);
     int parts = 0, b = 0, need = 0;
+    flow_cleared();
+    if (lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");          // (the re-draw kernel reads what was cleared)
     auto deliver = [&](int b, int parts, int need) {
         __syncwarp();
         if (lane == 0) {
@@ -798,9 +804,6 @@ __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem
         S.start_b = a.r.B; S.start_k = 0; S.start_w = 0; S.end_w = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // the start of this grid overlaps the clearing of its workspace, which is through from here on
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
     flow_share<TVM>(a, S, g);
     __syncthreads();

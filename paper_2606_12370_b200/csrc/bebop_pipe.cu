@@ -931,8 +931,11 @@ namespace {
 
 // Clears what a call needs cleared.  A kernel instead of a memset, because k_pipe can then be its programmatic dependent,
 // with its start off the call's path: 256 sequences of 151,936 bf16 logits, K = 5 without TV, 190.5 -> 188.4 us, K = 3
-// 196.2 -> 195.3.
+// 196.2 -> 195.3.  It is one itself, of whatever came before the call, and lets its dependent start when that is through: the stream
+// then reads logits while this kernel clears, and waits for it only where it counts (flow_cleared): 2 to 3 us of every call (64 of
+// 151,936 70.8 -> 68.3, 4 of 262,144 28.7 -> 26.4, 100 row pairs of 151,936 39.0 -> 37.0; tokens only 183.0 -> 179.9).
 __global__ void __launch_bounds__(256) k_clear(uint4* p, unsigned n16) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n16; i += gridDim.x * 256) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
@@ -975,8 +978,13 @@ int pipe_grid() {
 
 cudaError_t clear_launch(char* w, size_t bytes, cudaStream_t stream) {
     const unsigned n16 = (unsigned)(bytes / 16);
-    k_clear<<<n16 < 256 * 148 ? (n16 + 255) / 256 : 148, 256, 0, stream>>>(reinterpret_cast<uint4*>(w), n16);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n16 < 256 * 148 ? (n16 + 255) / 256 : 148); cfg.blockDim = dim3(256); cfg.stream = stream;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_clear, reinterpret_cast<uint4*>(w), n16);
 }
 
 bool pipe_supported(const RowArgs& a) {
