@@ -122,7 +122,7 @@ bebop_status_t bebop_verify(const void* target_logits, int64_t ld_target, const 
         if (launched) g_last = {3, "k_fuse"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
-        e = pipe_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched);
+        e = pipe_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, &launched, false, nullptr, g_path == 2);
         if (launched) g_last = {2, "k_pipe"};
     }
     if (e == cudaSuccess && !launched) e = general_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream);
@@ -159,7 +159,7 @@ bebop_status_t bebop_tv(const void* target_logits, int64_t ld_target, const void
         if (launched) g_last = {3, "k_fuse"};
     }
     if (e == cudaSuccess && !launched && g_path != 1 && pipe_supported(a)) {
-        e = pipe_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux);
+        e = pipe_verify(a, p, nullptr, nullptr, nullptr, o, static_cast<char*>(workspace), stream, &launched, true, s_aux, g_path == 2);
         if (launched) g_last = {2, "k_pipe"};
     }
     if (e == cudaSuccess && !launched)

@@ -12,10 +12,10 @@ __global__ void __launch_bounds__(F::LT, 1) k_fuse(const __grid_constant__ FlowA
 
 cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens, const float* u_accept,
                         const float* u_final, VerifyOut o, char* ws, cudaStream_t stream, bool* launched, bool tv_only,
-                        float* s_aux) {
+                        float* s_aux, bool large_chunks) {
     const FlowCall x{a, p, draft_tokens, u_accept, u_final, o, ws, stream, tv_only, s_aux};
     const int C = flow_cluster(a, tv_only);
-    const bool big = flow_long(a, tv_only, C);
+    const bool big = large_chunks || flow_long(a, tv_only, C);
     const auto go = [&](auto dt, auto tvm) {
         return big ? flow_launch<FlowLong, k_fuse<dt.value, tvm.value, FlowLong>>(x, C, launched)
                    : flow_launch<FlowShort, k_fuse<dt.value, tvm.value, FlowShort>>(x, C, launched);

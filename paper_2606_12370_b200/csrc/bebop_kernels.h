@@ -58,18 +58,19 @@ cudaError_t redraw_launch(const RowArgs& a, const float* u_final, VerifyOut o, c
 
 // Pipelined kernel (bebop_pipe.cu): a ticket schedule with a producer warp that stages every task's logits in shared memory by
 // bulk copies while the other warps compute.  Where TV is asked for, and with `tv_only` (bebop_tv: B row pairs, K = 1, o.tv and
-// s_aux the outputs, no tokens, no uniforms, no draw), it passes the call on to fuse_verify.
+// s_aux the outputs, no tokens, no uniforms, no draw), it passes the call on to fuse_verify.  `large_chunks`: with the sweeps' chunks
+// of 256 vectors whatever the shape, so that both give a row the same sums (the hook that asks for this kernel by name).
 bool pipe_supported(const RowArgs& a);
 cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
-                        cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
+                        cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr, bool large_chunks = false);
 
 // Fused kernel (bebop_fuse.cu): the stream of bebop_flow.cuh, every row read from memory once and out of L2 a second time; same
 // contract as pipe_verify, which runs it too wherever a TV output is asked for.  fuse_preferred: the line between the two.
 bool fuse_preferred(const RowArgs& a, bool tv_only, bool want_tv);
 cudaError_t fuse_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
-                        cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr);
+                        cudaStream_t stream, bool* launched, bool tv_only = false, float* s_aux = nullptr, bool large_chunks = false);
 
 // Clears the head of a workspace; the next launch may be a programmatic dependent of it.
 cudaError_t clear_launch(char* w, size_t bytes, cudaStream_t stream);

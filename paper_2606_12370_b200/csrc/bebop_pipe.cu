@@ -994,10 +994,10 @@ bool pipe_supported(const RowArgs& a) {
 
 cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_tokens,
                         const float* u_accept, const float* u_final, VerifyOut o, char* ws,
-                        cudaStream_t stream, bool* launched, bool tv_only, float* s_aux) {
+                        cudaStream_t stream, bool* launched, bool tv_only, float* s_aux, bool large_chunks) {
     *launched = false;
     // with TV every row pair has a second pass: the stream, which reads it from L2
-    if (tv_only || o.tv) return fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, launched, tv_only, s_aux);
+    if (tv_only || o.tv) return fuse_verify(a, p, draft_tokens, u_accept, u_final, o, ws, stream, launched, tv_only, s_aux, large_chunks);
     const int grid_max = a.dt == 0 ? pipe_grid<0, kModeVerify>() : pipe_grid<1, kModeVerify>();
     if (grid_max < 1) return cudaSuccess;
     const PipePlan wp = make_pipe_plan(a.B, a.K, a.nvec, a.dt, PSLICE);
