@@ -80,10 +80,11 @@ __device__ __forceinline__ int2 warp_sum_words(float x) {
     const float y = __fadd_rn(x, 64.f), r = __fsub_rn(x, __fsub_rn(y, 64.f)), z = __fadd_rn(r, __int_as_float((int)kSumBits1));
     return make_int2(redux_add(__float_as_int(y)), redux_add(__float_as_int(z)));
 }
-__device__ __forceinline__ long long words_sum(int hi, int lo) {
-    return ((long long)(int)((unsigned)hi - (unsigned)kNoSum0) << 23) + (int)((unsigned)lo - (unsigned)kNoSum1);
+// (an integer as a double by its bits: a conversion waits behind the exponentials of the other warps, whose unit it shares)
+__device__ __forceinline__ double int_value(int v) { return __hiloint2double(0x43300000, (int)((unsigned)v ^ 0x80000000u)) - 4503601774854144.0; }      // 2^52 + 2^31
+__device__ __forceinline__ double word_value(int2 w) {                 // exact
+    return fma(int_value((int)((unsigned)w.x - (unsigned)kNoSum0)), 7.62939453125e-06, int_value((int)((unsigned)w.y - (unsigned)kNoSum1)) * 9.094947017729282e-13);      // 2^-17, 2^-40
 }
-__device__ __forceinline__ double word_value(int2 w) { return (double)words_sum(w.x, w.y) * 9.094947017729282e-13; }      // 2^-40
 __device__ __forceinline__ double warp_sum_fixed(float x) { return word_value(warp_sum_words(x)); }
 // the largest logit of a lane's N vectors (NaN if there is one); bf16: packed maxima, unpacked once
 template <int DT, int N> __device__ __forceinline__ float vecs_max(const uint4* v) {

@@ -42,23 +42,27 @@ extern cudaEvent_t g_ev_start, g_ev_stop;
 namespace {
 
 // Consumer warps and vectors per lane of a chunk.
-template <int W, int Q, int SL> struct FlowDims {
-    static constexpr int LW = W, LQV = Q, LSL = SL;           // LSL: units under way, at most: tables by the unit's number mod LSL
+template <int W, int Q, int SL, int X> struct FlowDims {
+    static constexpr int LW = W, LQV = Q, LSL = SL, LNX = X;  // LSL: units under way, at most: tables by the unit's number mod LSL; LNX: exchange warps
     static constexpr int LCV = 32 * Q;                       // vectors of a chunk of pass 1; a chunk of pass 2 has half as many of each row
     static constexpr int LSTAGE = W * LCV * 16, LNS = 196608 / LSTAGE;
-    static constexpr int W_FPROD = W, W_EXCH = W + 1, W_PUB = W + 2, W_FIN = W + 3, LT = (W + 4) * 32;
+    static constexpr int W_FPROD = W, W_PUB = W + 1, W_FIN = W + 2, W_EXCH = W + 3, LT = (W + 3 + X) * 32;
     static constexpr int MAXCH = (Q == 8 ? 20480 : 12288) / LCV;         // chunks of a row slice, at most
 };
 constexpr int LUD = 16, LMB = 256;              // unit descriptions in flight, entries of the finisher's mailbox
 // Long: rows of which a CTA's slice is long enough for large chunks, which cost less per logit; Short: finer pieces for short rows.
-using FlowLong = FlowDims<16, 8, 2>;
-using FlowShort = FlowDims<24, 4, 4>;
+using FlowLong = FlowDims<16, 8, 2, 1>;
+using FlowShort = FlowDims<24, 4, 4, 1>;
 constexpr uint32_t kLSpin = 1u << 20;
 constexpr int kFailed = 1 << 30;              // mark in a sequence's count: given up, its outputs say so
 
 struct FlowRow { double inv_s, ub; int e, st; double pad; };         // a merged row: 1/S, bound of sum p^2, exponent, status
 struct FlowRec { double s, ub; int e, bad; double pad; };              // a CTA's part of a row
-struct __align__(16) FlowUnit { int b, k, pair, unit; };               // b < 0: no more units
+struct __align__(16) FlowUnit {
+    int b, k, kind, unit;                      // b < 0: no more units; kind: bit 0 a row pair (else the bonus row), above it the sequence's length
+    __device__ __forceinline__ bool pair() const { return kind & 1; }
+};
+struct __align__(16) FlowSrc { const char *p, *q; };                   // the CTA's slices of a unit's rows (no q: a bonus row)
 
 struct FlowArgs {
     RowArgs r;
@@ -91,13 +95,12 @@ template <class F> struct FlowShared {
     unsigned long long pub[F::LSL];                // ... the sums of its pass 2 have been read
     int4 task[F::LNS];
     FlowUnit unit[LUD];
+    FlowSrc src[LUD];
     float uc[LUD];                            // log2(e) / tau of the unit's sequence
     float4 scale[F::LSL];                          // exponents of both rows, rho as two floats
     double inv[F::LSL][2];                         // 1/S of both rows
     FlowRec rrec[F::LSL][kFlowMaxCluster][2];
-    int2 psum[F::LSL][2][F::MAXCH];          // warp_sum_words of the chunks' sums
-    int pexp[F::LSL][2][F::MAXCH];
-    int psq[F::LSL][2][F::MAXCH];            // upper bounds of the chunks' sums of e^2, in 2^-15
+    int4 part[F::LSL][2][F::MAXCH];          // chunks of pass 1: warp_sum_words, exponent, upper bound of the sum of e^2 in 2^-15
     int2 cm[F::LSL][2 * F::MAXCH], ca[F::LSL][2 * F::MAXCH];
     int wsum[F::LT / 32];
     int start_b, start_k, end_w, start_w;     // the cluster's run of units: the first one, weights of its begin and end
@@ -214,12 +217,14 @@ __device__ __forceinline__ void flow_share(const FlowArgs& a, FlowShared<F>& S, 
 }
 
 // ------------------------------------------------------------------ producer
+// One thread, whose instructions are its time (some ten cycles each beside the consumers): what does not change from unit to unit is
+// worked out once, rows are found by adding strides, and pass 2 finds its rows where pass 1 left them.
 template <int DT, bool TVM, class F>
 __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& S, unsigned char* ring, int rank) {
-    constexpr int VEC = Elem<DT>::VEC;
+    constexpr int VEC = Elem<DT>::VEC, CV = F::LCV / 2;
     const RowArgs& R = a.r;
     const int v0 = rank * a.sv, nv = max(min(a.sv, R.nvec - v0), 0);
-    const int ragged = (R.V % VEC != 0 && nv > 0 && v0 + nv == R.nvec) ? 1 : 0;
+    const int ragged = (R.V % VEC != 0 && nv > 0 && v0 + nv == R.nvec) ? 1 << 16 : 0;
     unsigned long long keep, drop;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(drop));
@@ -228,10 +233,10 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
     bool ok = true;
     // task: x = kind (0 pass 1, 1 pass 2, 3 stop) | row << 2 | last << 3 | first warp << 4 | chunks << 10 | first chunk << 16;
     // y = vectors of the task (of one row) | ragged << 16, z = c, w = unit's number
-    auto issue = [&](int kind, int row, bool last, int c0, int chunks, int vecs, int flags, float c, uint32_t u, const char* src0, const char* src1, unsigned long long pol) {
+    auto issue = [&](int x, int chunks, int y, float c, uint32_t u, const char* src0, const char* src1, unsigned long long pol) {
         if (!flow_wait_one(a, S, &S.empty[st], ph)) { ok = false; return; }
-        S.task[st] = make_int4(kind | row << 2 | (last ? 8 : 0) | rot << 4 | chunks << 10 | c0 << 16, vecs | flags << 16, __float_as_int(c), (int)u);
-        const uint32_t bytes = (uint32_t)vecs * 16u, dst = smem_u32(ring + (size_t)st * F::LSTAGE);
+        S.task[st] = make_int4(x | rot << 4 | chunks << 10, y, __float_as_int(c), (int)u);
+        const uint32_t bytes = (uint32_t)(y & 0xffff) * 16u, dst = smem_u32(ring + (size_t)st * F::LSTAGE);
         if (bytes) {
             mbar_arrive_expect(&S.full[st], src1 ? 2u * bytes : bytes);
             bulk_load_hint(dst, src0, bytes, &S.full[st], pol);
@@ -242,57 +247,66 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
         if (++st == F::LNS) { st = 0; ph ^= 1u; }
     };
     auto pass1 = [&](const char* row, int which, bool end, float c, uint32_t u, unsigned long long pol) {
-        int c0 = 0;
+        int c0 = 0, left = nv;
         do {
-            const int left = nv - c0 * F::LCV, vecs = min(left, F::LW * F::LCV), chunks = (vecs + F::LCV - 1) / F::LCV;
-            const bool fin = vecs == left;
-            issue(0, which, end && fin, c0, chunks, vecs, fin ? ragged : 0, c, u, row + (int64_t)(v0 + c0 * F::LCV) * 16, nullptr, pol);
-            c0 += F::LW;
-        } while (ok && c0 * F::LCV < nv);
+            const int vecs = min(left, F::LW * F::LCV);
+            left -= vecs;
+            issue(which << 2 | (end && left == 0 ? 8 : 0) | c0 << 16, (vecs + F::LCV - 1) / F::LCV, vecs | (left == 0 ? ragged : 0), c, u, row, nullptr, pol);
+            c0 += F::LW; row += F::LW * F::LCV * 16;
+        } while (ok && left > 0);
     };
     auto pass2 = [&](uint32_t u) {
-        const FlowUnit x = S.unit[u % LUD];
+        const FlowSrc x = S.src[u % LUD];
         const float c = S.uc[u % LUD];
-        if (!x.pair || nv == 0) { issue(1, 0, true, 0, 0, 0, 0, c, u, nullptr, nullptr, drop); return; }
-        constexpr int CV = F::LCV / 2;
-        const char* p = row_ptr(R, x.b, x.k) + (int64_t)v0 * 16; const char* q = row_ptr(R, x.b, R.K + 1 + x.k) + (int64_t)v0 * 16;
-        int c0 = 0;
+        if (!x.q || nv == 0) { issue(1 | 8, 0, 0, c, u, nullptr, nullptr, drop); return; }
+        const char *p = x.p, *q = x.q;
+        int c0 = 0, left = nv;
         do {
-            const int left = nv - c0 * CV, vecs = min(left, F::LW * CV), chunks = (vecs + CV - 1) / CV;
-            const bool fin = vecs == left;
-            issue(1, 0, fin, c0, chunks, vecs, fin ? ragged : 0, c, u, p + (int64_t)c0 * CV * 16, q + (int64_t)c0 * CV * 16, drop);
-            c0 += F::LW;
-        } while (ok && c0 * CV < nv);
+            const int vecs = min(left, F::LW * CV);
+            left -= vecs;
+            issue(1 | (left == 0 ? 8 : 0) | c0 << 16, (vecs + CV - 1) / CV, vecs | (left == 0 ? ragged : 0), c, u, p, q, drop);
+            c0 += F::LW; p += F::LW * CV * 16; q += F::LW * CV * 16;
+        } while (ok && left > 0);
     };
     int b = S.start_b, k = S.start_k, w = S.start_w;
     uint32_t u = 0;
+    const char* seq_p = R.target + (int64_t)b * R.t_seq_rows * R.t_row_bytes + (int64_t)v0 * 16;          // the sequence's first rows, at this CTA's slice
+    const char* seq_q = R.draft + (int64_t)b * R.d_seq_rows * R.d_row_bytes + (int64_t)v0 * 16;
+    const char *p = seq_p + k * R.t_row_bytes, *q = seq_q + k * R.d_row_bytes;
+    const int64_t seq_p_bytes = R.t_seq_rows * R.t_row_bytes, seq_q_bytes = R.d_seq_rows * R.d_row_bytes;
     // a sequence's length and temperature are asked for one sequence ahead
     auto len = [&](int i) { return TVM ? 1 : len_of(R, min(i, R.B - 1)); };
     int L = len(b), L1 = len(b + 1);
     float tau1 = tau_of(R, min(b + 1, R.B - 1)), c = temp_scale(tau_of(R, min(b, R.B - 1))).hi;
     while (ok && w < S.end_w && b < R.B) {
+        const bool pair = k < L;
         FlowUnit x;
-        x.b = b; x.k = k; x.pair = k < L ? 1 : 0; x.unit = TVM ? b : b * (R.K + 1) + k;
+        x.b = b; x.k = k; x.kind = 2 * L + (pair ? 1 : 0); x.unit = TVM ? b : b * (R.K + 1) + k;
         S.unit[u % LUD] = x;
         S.uc[u % LUD] = c;
         mbar_arrive(&S.ud[u % LUD]);
-        if (x.pair) {
-            pass1(row_ptr(R, b, k), 0, false, c, u, keep);
-            if (ok) pass1(row_ptr(R, b, R.K + 1 + k), 1, true, c, u, keep);
-        } else pass1(row_ptr(R, b, k), 0, true, c, u, drop);
+        FlowSrc y; y.p = p; y.q = pair ? q : nullptr;
+        S.src[u % LUD] = y;
+        if (!pair) pass1(p, 0, true, c, u, drop);
+        else {
+            pass1(p, 0, false, c, u, keep);
+            if (ok) pass1(q, 1, true, c, u, keep);
+        }
         if (ok && u >= (uint32_t)a.lag) pass2(u - a.lag);
         ++u;
-        w += x.pair ? 2 : 1;
+        w += pair ? 2 : 1;
+        p += R.t_row_bytes; q += R.d_row_bytes;
         if (++k > (TVM ? 0 : L)) {
             ++b; k = 0;
+            seq_p += seq_p_bytes; seq_q += seq_q_bytes;
+            p = seq_p; q = seq_q;
             L = L1; c = temp_scale(tau1).hi;
             L1 = len(b + 1); tau1 = tau_of(R, min(b + 1, R.B - 1));
         }
     }
     for (uint32_t i = u < (uint32_t)a.lag ? 0u : u - a.lag; ok && i < u; ++i) pass2(i);
-    S.unit[u % LUD].b = -1;
-    mbar_arrive(&S.ud[u % LUD]);
-    if (ok) issue(3, 0, false, 0, 0, 0, 0, 0.f, u, nullptr, nullptr, drop);
+    for (int i = 0; i < F::LNX; ++i) { S.unit[(u + i) % LUD].b = -1; mbar_arrive(&S.ud[(u + i) % LUD]); }          // (an end for each exchange warp)
+    if (ok) issue(3, 0, 0, 0.f, u, nullptr, nullptr, drop);
     // no copy of this CTA is under way when it leaves: the last ones have arrived (bounded)
     for (int i = 0; i < F::LNS && i < n; ++i) {
         if (--st < 0) { st = F::LNS - 1; ph ^= 1u; }
@@ -370,7 +384,7 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 const int2 w = chunk_sum<DT, F::LQV, !TVM>(x, c, E.ef, &sum);
                 // The lane's sum of e^2 is at most its sum of e, and at most that sum's square: the smaller, rounded up to 2^-15.
                 const int sq = redux_add(__float_as_int(__fmaf_ru(__fmul_ru(sum, fminf(sum, 1.f)), 32768.f, kMagic)));
-                if (lane == 0) { const int row = (d.x >> 2) & 1; S.psum[par][row][c0] = w; S.pexp[par][row][c0] = E.e; S.psq[par][row][c0] = sq; }
+                if (lane == 0) S.part[par][(d.x >> 2) & 1][c0] = make_int4(w.x, w.y, E.e, sq);
             } else { __syncwarp(); if (lane == 0) mbar_arrive(&S.empty[st]); }          // (every lane has read the description)
             if (lane == 0 && (d.x & 8)) mbar_arrive(&S.p1[par]);
         } else {
@@ -427,9 +441,9 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
 // ------------------------------------------------------------------ helper
 // over the 16 lanes of a half warp, every lane gets the result (one fixed tree)
 __device__ __forceinline__ int half_max(int v) {
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    const bool low = (threadIdx.x & 16) == 0;
+    const int a = redux_max(low ? v : INT_MIN), b = redux_max(low ? INT_MIN : v);
+    return low ? a : b;
 }
 __device__ __forceinline__ double half_sum(double v) {
 #pragma unroll
@@ -439,29 +453,33 @@ __device__ __forceinline__ double half_sum(double v) {
 
 // The sums of pass 1, exchanged and merged.  Half a warp per row: lanes 0 to 15 the target row, 16 to 31 the draft row.
 template <class F>
-__device__ __forceinline__ void flow_exchange(const FlowArgs& a, FlowShared<F>& S, int rank) {
+__device__ __forceinline__ void flow_exchange(const FlowArgs& a, FlowShared<F>& S, int rank, uint32_t first) {
     const RowArgs& R = a.r;
     const int lane = threadIdx.x & 31, C = a.C, row = lane >> 4, l = lane & 15;
     const int v0 = rank * a.sv, nv = max(min(a.sv, R.nvec - v0), 0), n1 = (nv + F::LCV - 1) / F::LCV;
 #pragma unroll 1
-    for (uint32_t u = 0;; ++u) {
+    for (uint32_t u = first;; u += F::LNX) {
         if (!flow_wait(a, S, &S.ud[u % LUD], (u / LUD) & 1u)) return;
         const FlowUnit x = S.unit[u % LUD];
         const int par = u & (F::LSL - 1);
         if (x.b < 0) return;
         if (!flow_wait(a, S, &S.p1[par], (u / F::LSL) & 1u)) return;
         // ---- the CTA's sum of the row, sent to all CTAs of the cluster (a bonus row has an empty one beside it)
-        const int n = row == 0 || x.pair ? n1 : 0;
-        int em = E_EMPTY;
-        for (int q = l; q < n; q += 16) em = max(em, S.pexp[par][row][q]);
+        const int n = row == 0 || x.pair() ? n1 : 0;
+        const int4 none = make_int4(kNoSum0, kNoSum1, E_EMPTY, 0);
+        const int4 v = l < n ? S.part[par][row][l] : none;
+        int em = v.z;
+        for (int q = l + 16; q < n; q += 16) em = max(em, S.part[par][row][q].z);
         em = half_max(em);
         const int bad = em == E_BAD;
         double s = 0.0, ub = 0.0;
-        for (int q = l; q < n; q += 16) {
-            const int e = S.pexp[par][row][q];
-            const double f = e > E_EMPTY && e != E_BAD ? pow2d(max(e - em, -500)) : 0.0;
-            if (f > 0.0) { s += 2.0 * word_value(S.psum[par][row][q]) * f; ub += (double)(int)((unsigned)S.psq[par][row][q] - 32u * (unsigned)kMagicBits) * (f * f); }
-        }
+        auto add = [&](const int4& v) {
+            const double f = v.z > E_EMPTY && v.z != E_BAD ? pow2d(max(v.z - em, -500)) : 0.0;
+            s = fma(2.0 * word_value(make_int2(v.x, v.y)), f, s);
+            ub = fma(int_value((int)((unsigned)v.w - 32u * (unsigned)kMagicBits)), f * f, ub);
+        };
+        add(v);
+        for (int q = l + 16; q < n; q += 16) add(S.part[par][row][q]);
         s = half_sum(s); ub = half_sum(ub);
         FlowRow m;
         int anybad = bad;
@@ -489,15 +507,14 @@ __device__ __forceinline__ void flow_exchange(const FlowArgs& a, FlowShared<F>& 
         m.inv_s = !m.st && s > 0.0 ? 1.0 / s : 0.0; m.ub = ub * 3.0517578125e-05 * m.inv_s * m.inv_s; m.pad = 0.0;
         const double inv_q = __shfl_sync(0xffffffffu, m.inv_s, 16);
         const int eq = __shfl_sync(0xffffffffu, m.e, 16);
-        if (rank == 0 && l == 0 && (row == 0 || x.pair)) a.rows[2 * (int64_t)x.unit + row] = m;
-        if (!x.pair) {
+        if (!x.pair()) {
             // a bonus row has no pass 2: its chunks' masses are written now, before the consumers may use their places again
             const double inv_p = __shfl_sync(0xffffffffu, m.inv_s, 0);
             const int ep = __shfl_sync(0xffffffffu, m.e, 0);
             double t = 0.0;
             for (int q = lane; q < n1; q += 32) {
-                const int e = S.pexp[par][0][q];
-                const double v = e > E_EMPTY && e != E_BAD ? 2.0 * word_value(S.psum[par][0][q]) * pow2d(max(e - ep, -1000)) * inv_p : 0.0;
+                const int4 w = S.part[par][0][q];
+                const double v = w.z > E_EMPTY && w.z != E_BAD ? 2.0 * word_value(make_int2(w.x, w.y)) * pow2d(max(w.z - ep, -1000)) * inv_p : 0.0;
                 a.mass[((int64_t)x.unit * C + rank) * (2 * a.nch) + q] = v;
                 t += v;
             }
@@ -506,11 +523,13 @@ __device__ __forceinline__ void flow_exchange(const FlowArgs& a, FlowShared<F>& 
         }
         if (u >= F::LSL && !flow_wait(a, S, &S.pub[par], ((u - F::LSL) / F::LSL) & 1u)) return;
         if (lane == 0) {
-            const double rh = m.inv_s > 0.0 ? inv_q / m.inv_s : 0.0;
+            // (S_p / S_q; rows of equal sums have exactly 1)
+            const double rh = !(m.inv_s > 0.0) ? 0.0 : inv_q == m.inv_s ? 1.0 : s * inv_q;
             const float h = (float)rh;
             S.scale[par] = make_float4((float)m.e, (float)eq, h, (float)(rh - (double)h));
             S.inv[par][0] = m.inv_s; S.inv[par][1] = inv_q;
         }
+        if (rank == 0 && l == 0 && (row == 0 || x.pair())) a.rows[2 * (int64_t)x.unit + row] = m;
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.stat[par]);
         __syncwarp();
@@ -554,9 +573,8 @@ __device__ __forceinline__ void flow_publish(const FlowArgs& a, FlowShared<F>& S
         const FlowUnit x = S.unit[u % LUD];
         const int par = u & (F::LSL - 1);
         if (x.b < 0) { if (parts) deliver(b, parts, need); break; }
-        const int L = TVM ? 1 : len_of(R, x.b);
         if (!flow_wait(a, S, &S.p2[par], (u / F::LSL) & 1u)) break;
-        if (x.pair) {
+        if (x.pair()) {
             const double ip = S.inv[par][0];
             double s = 0.0, sx = 0.0;
             for (int q = lane; q < n2; q += 32) {
@@ -574,8 +592,8 @@ __device__ __forceinline__ void flow_publish(const FlowArgs& a, FlowShared<F>& S
         // the sequence's count takes the parts of a run of its units at once, with its last unit or this cluster's (the fence and
         // the atomic once per unit took as long as a short unit itself, and a cluster of one CTA sends itself nothing: 600
         // sequences of 8,000 bf16 logits, K = 7, 120.2 -> 101.4 us, 600 of 4,000 fp32, K = 8, 118.0 -> 89.7)
-        ++parts; b = x.b; need = C * (TVM ? 1 : L + 1);
-        if (TVM || !x.pair) { deliver(b, parts, need); parts = 0; }
+        ++parts; b = x.b; need = C * (TVM ? 1 : (x.kind >> 1) + 1);
+        if (TVM || !x.pair()) { deliver(b, parts, need); parts = 0; }
         __syncwarp();
     }
     __syncwarp();
@@ -810,9 +828,9 @@ __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem
     if (a.C > 1) cluster_sync();                            // every CTA of the cluster has its barriers
     if (warp < F::LW) { flow_consumer<DT, TVM>(a, S, smem, warp, lane); flow_finisher<DT, TVM>(a, S); }
     else if (warp == F::W_FPROD) { if (lane == 0) flow_producer<DT, TVM>(a, S, smem, rank); __syncwarp(); }
-    else if (warp == F::W_EXCH) flow_exchange(a, S, rank);
     else if (warp == F::W_PUB) flow_publish<TVM>(a, S, rank);
-    else flow_finisher<DT, TVM>(a, S);
+    else if (warp == F::W_FIN) flow_finisher<DT, TVM>(a, S);
+    else flow_exchange(a, S, rank, (uint32_t)(warp - F::W_EXCH));
     __syncthreads();
     if (a.C > 1) cluster_sync();                            // nothing is sent to a CTA that has left
     if (*(volatile int*)&S.abort) flow_failed<TVM, F>(a);
