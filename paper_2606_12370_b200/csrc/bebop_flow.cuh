@@ -41,18 +41,26 @@ extern cudaEvent_t g_ev_start, g_ev_stop;
 
 namespace {
 
-// Consumer warps and vectors per lane of a chunk.
-template <int W, int Q, int SL, int X> struct FlowDims {
-    static constexpr int LW = W, LQV = Q, LSL = SL, LNX = X;  // LSL: units under way, at most: tables by the unit's number mod LSL; LNX: exchange warps
+// Consumer warps; vectors per lane of a chunk; units under way at most (tables by the unit's number mod LSL); exchange warps; RES: a
+// unit's logits stay in their stage until pass 2, which then needs no second copy.
+template <int W, int Q, int SL, int X, bool RES> struct FlowDims {
+    static constexpr int LW = W, LQV = Q, LSL = SL, LNX = X;
+    static constexpr bool LRES = RES;
     static constexpr int LCV = 32 * Q;                       // vectors of a chunk of pass 1; a chunk of pass 2 has half as many of each row
-    static constexpr int LSTAGE = W * LCV * 16, LNS = 196608 / LSTAGE;
+    static constexpr int LRING = 196608, LSTAGE = W * LCV * 16, LNS = RES ? 8 : LRING / LSTAGE;      // (RES: so many stages at most, of the size of a unit)
     static constexpr int W_FPROD = W, W_PUB = W + 1, W_FIN = W + 2, W_EXCH = W + 3, LT = (W + 3 + X) * 32;
-    static constexpr int MAXCH = (Q == 8 ? 20480 : 12288) / LCV;         // chunks of a row slice, at most
+    static constexpr int MAXCH = RES ? W / 2 : (Q == 8 ? 20480 : 12288) / LCV;         // chunks of a row slice, at most
 };
 constexpr int LUD = 16, LMB = 256;              // unit descriptions in flight, entries of the finisher's mailbox
 // Long: rows of which a CTA's slice is long enough for large chunks, which cost less per logit; Short: finer pieces for short rows.
-using FlowLong = FlowDims<16, 8, 2, 1>;
-using FlowShort = FlowDims<24, 4, 4, 1>;
+// Resident: rows so short that four units or more fit the ring.  Their units are over sooner than one producer thread hands out
+// three tasks, or one warp exchanges their sums: 1,000 sequences of 8,000 bf16 logits, K = 8, 178 us as Short (whose producer was busy for 324 of
+// 349 us of 2,000 such, its exchange warp for 271), 159 with both rows' pass 1 in one task, 145 with the logits kept, 131 with two
+// exchange warps; 2,000 of 11,000, K = 3, 194 -> 134, 1,000 of 5,000 fp32, K = 8, 149 -> 107.
+using FlowLong = FlowDims<16, 8, 2, 1, false>;
+using FlowShort = FlowDims<24, 4, 4, 1, false>;
+using FlowResident = FlowDims<24, 4, 4, 2, true>;
+constexpr int kResidentVecs = FlowResident::MAXCH * FlowResident::LCV;     // of a row, at most
 constexpr uint32_t kLSpin = 1u << 20;
 constexpr int kFailed = 1 << 30;              // mark in a sequence's count: given up, its outputs say so
 
@@ -73,6 +81,7 @@ struct FlowArgs {
     float* s_aux;
     int share;                                // rows of a cluster, at most; 0: even shares; -1: even shares of ragged sequences
     int lag;                                  // units between a unit's passes, below LSL
+    int ns, pitch;                            // resident form: stages, bytes of one
     int C, G, nch, sv;                        // CTAs per cluster, clusters, chunks and vectors of a row slice
     int expire;                               // test hook: the helper's wait for the cluster's sums counts as run out
     float kappa;
@@ -314,6 +323,70 @@ __device__ __forceinline__ void flow_producer(const FlowArgs& a, FlowShared<F>& 
     }
 }
 
+// The producer of the resident form: a unit is one task and stays in its stage through both passes.
+template <int DT, bool TVM, class F>
+__device__ __forceinline__ void flow_producer_res(const FlowArgs& a, FlowShared<F>& S, unsigned char* ring, int rank) {
+    constexpr int VEC = Elem<DT>::VEC, CV = F::LCV / 2;
+    const RowArgs& R = a.r;
+    const int v0 = rank * a.sv, nv = max(min(a.sv, R.nvec - v0), 0), n1 = (nv + F::LCV - 1) / F::LCV, n2 = (nv + CV - 1) / CV;
+    const int y = nv | (R.V % VEC != 0 && nv > 0 && v0 + nv == R.nvec ? 1 << 16 : 0);
+    int st = 0, n = 0, rot = 0;
+    uint32_t ph = 1, u = 0;
+    int b = S.start_b, k = S.start_k, w = S.start_w;
+    const char* p = R.target + ((int64_t)b * R.t_seq_rows + k) * R.t_row_bytes + (int64_t)v0 * 16;
+    const char* q = R.draft + ((int64_t)b * R.d_seq_rows + k) * R.d_row_bytes + (int64_t)v0 * 16;
+    auto len = [&](int i) { return TVM ? 1 : len_of(R, min(i, R.B - 1)); };
+    int L = len(b), L1 = len(b + 1);
+    float tau1 = tau_of(R, min(b + 1, R.B - 1)), c = temp_scale(tau_of(R, min(b, R.B - 1))).hi;
+    bool ok = true;
+    for (;;) {
+        // task: x = stop (3) | row pair << 2 | first warp of pass 1 << 4 | its chunks << 10 | first warp of pass 2 << 16 | its chunks << 22;
+        // y = vectors of a row | ragged << 16, z = c, w = unit's number
+        const bool more = w < S.end_w && b < R.B, pair = more && k < L;
+        if (!flow_wait_one(a, S, &S.empty[st], ph)) { ok = false; break; }
+        if (!more) break;
+        FlowUnit x;
+        x.b = b; x.k = k; x.kind = 2 * L + (pair ? 1 : 0); x.unit = TVM ? b : b * (R.K + 1) + k;
+        S.unit[u % LUD] = x;
+        mbar_arrive(&S.ud[u % LUD]);
+        int t = rot << 4;
+        const int chunks = pair ? 2 * n1 : n1;
+        rot += chunks; if (rot >= F::LW) rot -= F::LW;
+        t |= chunks << 10 | rot << 16;
+        if (pair) { t |= 4 | n2 << 22; rot += n2; if (rot >= F::LW) rot -= F::LW; }
+        S.task[st] = make_int4(t, y, __float_as_int(c), (int)u);
+        const uint32_t bytes = (uint32_t)nv * 16u, dst = smem_u32(ring) + (uint32_t)(st * a.pitch);
+        if (bytes) {
+            mbar_arrive_expect(&S.full[st], pair ? 2u * bytes : bytes);
+            bulk_load(dst, p, bytes, &S.full[st]);
+            if (pair) bulk_load(dst + a.pitch / 2, q, bytes, &S.full[st]);
+        } else mbar_arrive(&S.full[st]);
+        ++n; ++u;
+        if (++st == a.ns) { st = 0; ph ^= 1u; }
+        w += pair ? 2 : 1;
+        p += R.t_row_bytes; q += R.d_row_bytes;
+        if (++k > (TVM ? 0 : L)) {
+            ++b; k = 0;
+            p = R.target + (int64_t)b * R.t_seq_rows * R.t_row_bytes + (int64_t)v0 * 16;
+            q = R.draft + (int64_t)b * R.d_seq_rows * R.d_row_bytes + (int64_t)v0 * 16;
+            L = L1; c = temp_scale(tau1).hi;
+            L1 = len(b + 1); tau1 = tau_of(R, min(b + 1, R.B - 1));
+        }
+    }
+    for (int i = 0; i < F::LNX; ++i) { S.unit[(u + i) % LUD].b = -1; mbar_arrive(&S.ud[(u + i) % LUD]); }          // (an end for each exchange warp)
+    if (ok) {
+        S.task[st] = make_int4(3, 0, 0, (int)u);
+        mbar_arrive(&S.full[st]);
+        ++n;
+        if (++st == a.ns) { st = 0; ph ^= 1u; }
+    }
+    // no copy of this CTA is under way when it leaves: the last ones have arrived (bounded)
+    for (int i = 0; i < a.ns && i < n; ++i) {
+        if (--st < 0) { st = a.ns - 1; ph ^= 1u; }
+        for (uint32_t t = 0; t < kLSpin && !mbar_try(smem_u32(&S.full[st]), ph ^ 1u); ++t) {}
+    }
+}
+
 // ------------------------------------------------------------------ consumers
 // what a chunk does not have in full: vectors beyond the task read as -inf, the row's ragged last vector loses the lanes
 // beyond the vocabulary
@@ -352,6 +425,46 @@ __device__ __forceinline__ void resid_aux(const float* p, const float* q, float2
         *x = __ffma2_rn(q2, mk, *x);
     }
 }
+// A warp's chunk of pass 1, from registers: its exponent, its sum and a bound of its sum of squares into the table.
+template <int DT, bool TVM, class F>
+__device__ __forceinline__ void flow_chunk1(FlowShared<F>& S, const uint4* x, float c, int par, int row, int at, int lane) {
+    const QExp E = chunk_exponent(vecs_max<DT, F::LQV>(x), c);
+    float sum;
+    const int2 w = chunk_sum<DT, F::LQV, !TVM>(x, c, E.ef, &sum);
+    // The lane's sum of e^2 is at most its sum of e, and at most that sum's square: the smaller, rounded up to 2^-15.
+    const int sq = redux_add(__float_as_int(__fmaf_ru(__fmul_ru(sum, fminf(sum, 1.f)), 32768.f, kMagic)));
+    if (lane == 0) S.part[par][row][at] = make_int4(w.x, w.y, E.e, sq);
+}
+// ... of pass 2: its mass (bebop_tv: and its part of S).
+template <int DT, bool TVM, class F>
+__device__ __forceinline__ void flow_chunk2(FlowShared<F>& S, const uint4* xp, const uint4* xq, float c, const float4& sc, int par, int at, int lane) {
+    constexpr int VEC = Elem<DT>::VEC, H = F::LQV / 2;
+    const float2 rho = make_float2(sc.z, sc.w);
+    if (TVM) {
+        float2 z = make_float2(0.f, 0.f), x = z;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            float p[VEC], q[VEC];
+            exp_vec<DT>(xp[i], c, sc.x, p);
+            exp_vec<DT>(xq[i], c, sc.y, q);
+            resid_aux<VEC>(p, q, rho, &z, &x);
+        }
+        const int2 w = warp_sum_words(z.x + z.y), v = warp_sum_words(x.x + x.y);
+        if (lane == 0) { S.cm[par][at] = w; S.ca[par][at] = v; }
+    } else {
+        float v[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            float p[VEC], q[VEC];
+            exp_vec<DT>(xp[i], c, sc.x, p);
+            exp_vec<DT>(xq[i], c, sc.y, q);
+            v[i] = resid_sum<VEC>(p, q, rho);
+        }
+        const int2 w = vector_sum_words<H, 0>(v);
+        if (lane == 0) S.cm[par][at] = w;
+    }
+}
+
 template <int DT, bool TVM, class F>
 __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& S, const unsigned char* ring, int warp, int lane) {
     constexpr int VEC = Elem<DT>::VEC;
@@ -379,12 +492,7 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[st]);
                 if ((j + 1) * F::LCV > nv - ragged) mask_vecs<DT, F::LQV>(x, j * F::LCV + lane, nv, ragged, keep);
-                const QExp E = chunk_exponent(vecs_max<DT, F::LQV>(x), c);
-                float sum;
-                const int2 w = chunk_sum<DT, F::LQV, !TVM>(x, c, E.ef, &sum);
-                // The lane's sum of e^2 is at most its sum of e, and at most that sum's square: the smaller, rounded up to 2^-15.
-                const int sq = redux_add(__float_as_int(__fmaf_ru(__fmul_ru(sum, fminf(sum, 1.f)), 32768.f, kMagic)));
-                if (lane == 0) S.part[par][(d.x >> 2) & 1][c0] = make_int4(w.x, w.y, E.e, sq);
+                flow_chunk1<DT, TVM>(S, x, c, par, (d.x >> 2) & 1, c0, lane);
             } else { __syncwarp(); if (lane == 0) mbar_arrive(&S.empty[st]); }          // (every lane has read the description)
             if (lane == 0 && (d.x & 8)) mbar_arrive(&S.p1[par]);
         } else {
@@ -403,36 +511,76 @@ __device__ __forceinline__ void flow_consumer(const FlowArgs& a, FlowShared<F>& 
                     mask_vecs<DT, H>(xp, j * (F::LCV / 2) + lane, nv, ragged, keep);
                     mask_vecs<DT, H>(xq, j * (F::LCV / 2) + lane, nv, ragged, keep);
                 }
-                const float2 rho = make_float2(sc.z, sc.w);
-                if (TVM) {
-                    float2 z = make_float2(0.f, 0.f), x = z;
-#pragma unroll
-                    for (int i = 0; i < H; ++i) {
-                        float p[VEC], q[VEC];
-                        exp_vec<DT>(xp[i], c, sc.x, p);
-                        exp_vec<DT>(xq[i], c, sc.y, q);
-                        resid_aux<VEC>(p, q, rho, &z, &x);
-                    }
-                    const int2 w = warp_sum_words(z.x + z.y), v = warp_sum_words(x.x + x.y);
-                    if (lane == 0) { S.cm[par][c0] = w; S.ca[par][c0] = v; }
-                } else {
-                    float v[H];
-#pragma unroll
-                    for (int i = 0; i < H; ++i) {
-                        float p[VEC], q[VEC];
-                        exp_vec<DT>(xp[i], c, sc.x, p);
-                        exp_vec<DT>(xq[i], c, sc.y, q);
-                        v[i] = resid_sum<VEC>(p, q, rho);
-                    }
-                    const int2 w = vector_sum_words<H, 0>(v);
-                    if (lane == 0) S.cm[par][c0] = w;
-                }
+                flow_chunk2<DT, TVM>(S, xp, xq, c, sc, par, c0, lane);
             } else {
                 if (!__all_sync(0xffffffffu, merged)) break;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[st]);
             }
             if (lane == 0 && (d.x & 8)) mbar_arrive(&S.p2[par]);
+        }
+        __syncwarp();
+    }
+}
+
+// The consumers of the resident form: pass 1 of the unit that has arrived, pass 2 of the one `lag` before it, and its stage is free.
+template <int DT, bool TVM, class F>
+__device__ __forceinline__ void flow_consumer_res(const FlowArgs& a, FlowShared<F>& S, const unsigned char* ring, int warp, int lane) {
+    constexpr int VEC = Elem<DT>::VEC, H = F::LQV / 2;
+    const int keep = a.r.V - (a.r.nvec - 1) * VEC, lag = a.lag;
+    int st = 0, st2 = 0, ph = 0;
+    uint32_t end = 0xffffffffu;
+#pragma unroll 1
+    for (uint32_t u = 0;; ++u) {
+        if (u < end) {
+            const bool there = flow_wait_one(a, S, &S.full[st], (uint32_t)ph);
+            const int4 d = S.task[st];
+            if (!__all_sync(0xffffffffu, there)) return;
+            if (d.x == 3) end = u;
+            else {
+                const int n1 = ((d.x >> 10) & 63) >> ((d.x >> 2) & 1), nv = d.y & 0xffff, par = u & (F::LSL - 1);      // chunks of a row
+                int j = warp - ((d.x >> 4) & 63);
+                if (j < 0) j += F::LW;
+                if (j < ((d.x >> 10) & 63)) {
+                    const int row = j >= n1 ? 1 : 0, jr = row ? j - n1 : j;
+                    const unsigned char* src = ring + (size_t)st * a.pitch + (row ? a.pitch / 2 : 0) + (size_t)(jr * F::LCV + lane) * 16;
+                    uint4 x[F::LQV];
+#pragma unroll
+                    for (int i = 0; i < F::LQV; ++i) x[i] = *reinterpret_cast<const uint4*>(src + i * 512);
+                    if ((jr + 1) * F::LCV > nv - (d.y >> 16)) mask_vecs<DT, F::LQV>(x, jr * F::LCV + lane, nv, d.y >> 16, keep);
+                    flow_chunk1<DT, TVM>(S, x, __int_as_float(d.z), par, row, jr, lane);
+                }
+                if (lane == 0) mbar_arrive(&S.p1[par]);
+                if (++st == a.ns) { st = 0; ph ^= 1; }
+            }
+        }
+        if (u >= (uint32_t)lag) {
+            const uint32_t v = u - (uint32_t)lag;
+            if (v >= end) return;
+            const int par = v & (F::LSL - 1);
+            const int4 d = S.task[st2];                      // (there since the unit's pass 1)
+            const bool merged = flow_wait_one(a, S, &S.stat[par], (v / F::LSL) & 1u);
+            int j = warp - ((d.x >> 16) & 63);
+            if (j < 0) j += F::LW;
+            const int nv = d.y & 0xffff;
+            const bool has = j < ((d.x >> 22) & 63);
+            if (!__all_sync(0xffffffffu, merged)) return;
+            if (has) {
+                const unsigned char* src = ring + (size_t)st2 * a.pitch + (size_t)(j * (F::LCV / 2) + lane) * 16;
+                uint4 xp[H], xq[H];
+#pragma unroll
+                for (int i = 0; i < H; ++i) { xp[i] = *reinterpret_cast<const uint4*>(src + i * 512); xq[i] = *reinterpret_cast<const uint4*>(src + a.pitch / 2 + i * 512); }
+                const float4 sc = S.scale[par];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.empty[st2]);
+                if ((j + 1) * (F::LCV / 2) > nv - (d.y >> 16)) {
+                    mask_vecs<DT, H>(xp, j * (F::LCV / 2) + lane, nv, d.y >> 16, keep);
+                    mask_vecs<DT, H>(xq, j * (F::LCV / 2) + lane, nv, d.y >> 16, keep);
+                }
+                flow_chunk2<DT, TVM>(S, xp, xq, __int_as_float(d.z), sc, par, j, lane);
+            } else { __syncwarp(); if (lane == 0) mbar_arrive(&S.empty[st2]); }
+            if (lane == 0) mbar_arrive(&S.p2[par]);
+            if (++st2 == a.ns) st2 = 0;
         }
         __syncwarp();
     }
@@ -811,7 +959,7 @@ __device__ __noinline__ void flow_failed(const FlowArgs& a) {
 
 template <int DT, bool TVM, class F>
 __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem) {
-    FlowShared<F>& S = *reinterpret_cast<FlowShared<F>*>(smem + (size_t)F::LNS * F::LSTAGE);
+    FlowShared<F>& S = *reinterpret_cast<FlowShared<F>*>(smem + F::LRING);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = a.C > 1 ? (int)cluster_rank() : 0, g = (int)blockIdx.x / a.C;
     if (tid == 0) {
@@ -826,9 +974,13 @@ __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem
     flow_share<TVM>(a, S, g);
     __syncthreads();
     if (a.C > 1) cluster_sync();                            // every CTA of the cluster has its barriers
-    if (warp < F::LW) { flow_consumer<DT, TVM>(a, S, smem, warp, lane); flow_finisher<DT, TVM>(a, S); }
-    else if (warp == F::W_FPROD) { if (lane == 0) flow_producer<DT, TVM>(a, S, smem, rank); __syncwarp(); }
-    else if (warp == F::W_PUB) flow_publish<TVM>(a, S, rank);
+    if (warp < F::LW) {
+        if constexpr (F::LRES) flow_consumer_res<DT, TVM>(a, S, smem, warp, lane); else flow_consumer<DT, TVM>(a, S, smem, warp, lane);
+        flow_finisher<DT, TVM>(a, S);
+    } else if (warp == F::W_FPROD) {
+        if (lane == 0) { if constexpr (F::LRES) flow_producer_res<DT, TVM>(a, S, smem, rank); else flow_producer<DT, TVM>(a, S, smem, rank); }
+        __syncwarp();
+    } else if (warp == F::W_PUB) flow_publish<TVM>(a, S, rank);
     else if (warp == F::W_FIN) flow_finisher<DT, TVM>(a, S);
     else flow_exchange(a, S, rank, (uint32_t)(warp - F::W_EXCH));
     __syncthreads();
@@ -837,7 +989,7 @@ __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem
 }
 
 // ------------------------------------------------------------------ host side
-template <class F> constexpr size_t flow_smem() { return (size_t)F::LNS * F::LSTAGE + sizeof(FlowShared<F>); }
+template <class F> constexpr size_t flow_smem() { return F::LRING + sizeof(FlowShared<F>); }
 
 // Clusters of so many CTAs for a call.  A CTA's slice of a row should be long (every unit costs an exchange and some short
 // stages), but two units of every cluster have to stay in L2, and the tables hold 20,480 vectors: one CTA up to
@@ -852,6 +1004,7 @@ inline int flow_cluster(const RowArgs& a, bool tv_only) {
     while (C < kFlowMaxCluster && rows * C < 3.15 * 148.0 && a.nvec > 4 * 256 * C) C *= 2;
     return C;
 }
+inline bool flow_resident_rows(const RowArgs& a, int C) { return C == 1 && a.nvec <= kResidentVecs; }
 // Large chunks for long slices (row pairs of 151,936 over two CTAs 152.7 against 164.7 us for 768 of them; 192 sequences of 32,000,
 // K = 7, over one CTA 79.7 against 70.0; 24 of 151,936 over four 45.0 against 42.3).
 inline bool flow_long(const RowArgs& a, bool tv_only, int C) { return a.nvec > (tv_only ? 4000 : 7500) * C; }
@@ -918,6 +1071,12 @@ template <class F, auto kernel> cudaError_t flow_launch(const FlowCall& x, int C
     // short rows: an exchange takes longer than a unit's work, so more units go between (600 sequences of 8,000 bf16 logits, K = 7:
     // one 101.4, two 98.7, three 96.7 us; 192 of 32,000 68.8, 68.1, 69.6); longer ones have no use for it, and L2 has to hold them
     fa.lag = F::LSL > 3 && a.nvec <= 2560 ? 3 : 1;
+    fa.ns = 0; fa.pitch = 0;
+    if (F::LRES) {
+        fa.pitch = 2 * ((min(f.sv, a.nvec) * 16 + 127) & ~127);
+        fa.ns = min(F::LNS, F::LRING / fa.pitch);
+        fa.lag = min(3, fa.ns - 2);
+    }
     const long long units = (long long)a.B * (x.tv_only ? 1 : a.K + 1);
     fa.G = (int)(units < G ? units : G);
     fa.share = x.tv_only || !a.draft_len ? flow_share_of(a, x.tv_only, fa.G) : -1;

@@ -824,10 +824,11 @@ bool seq_preferred(const RowArgs& a, bool tv_only) {
     while (C < kSeqMaxCluster && seq_plan(rows, a.K, a.nvec, C).bytes > kSeqShare) ++C;
     const double logits = (double)a.B * rows * a.V;
     if (C == 1) return true;
-    // (short rows leave the stream little to do between two exchanges, us against it: 2,000 sequences of 8,000 158 against 193, 1,000 of
-    // 2,000 fp32, K = 8, 85 against 149, 600 of 3,000 fp32 72 against 91.  Longer rows would be faster streamed from about 20 million logits
-    // on -- 250 of 16,000 57.0 against 41.4, 128 of 32,000 50.6 against 44.7 -- but stay here, where rows far from zero are right.)
-    if (C == 2 && !tv_only && a.nvec < 1200) return true;
+    // (Longer rows would be faster streamed from about 20 million logits on -- 250 of 16,000 57.0 against 41.4, 128 of 32,000 50.6 against
+    // 44.7, 1,000 of 8,000 90 against 70 -- but stay here, where rows far from zero are right.  Beyond the line the stream: 2,000 of 8,000 118
+    // against 158, 2,000 of 5,000, K = 8, 192 against 252, 1,000 of 2,000 fp32, K = 8, 80 against 86; of rows below 400 vectors a unit is too
+    // little between two exchanges.)
+    if (C == 2 && !tv_only && a.nvec < 400) return true;
     if (C == 2) return logits <= (tv_only || a.dt == 0 ? 30e6 : 100e6);
     if (C <= 8) return logits <= (tv_only ? 15e6 : 30e6);
     if (C == 9 && !tv_only) return logits <= 20e6;

@@ -100,3 +100,53 @@ def test_one_rule_for_the_chunks_whatever_the_name(dtype, B, K, V, n):
     a, b = (P.bebop_verify(y["target"], y["draft"], y["draft_tokens"], y["u_accept"], y["u_final"], temperature_all=0.9) for y in (x, part))
     for k in ("accept_len", "out_tokens", "tv", "p_draft", "q_draft", "row_status"):
         assert torch.equal(a[k][:n], b[k]), k
+
+
+def sampled(cfg, x, got, n, context=""):
+    idx = np.unique(np.linspace(0, cfg.B - 1, n).astype(np.int64))
+    compare_verify(got, oracle_on(x, idx), cfg.dtype, idx=idx, context=str(cfg) + context)
+    check_properties(got, x)
+
+
+# the resident form: rows of one chunk, of a chunk and a vector, around half and all of what fits (1,536 vectors: four stages), and the
+# first row beyond it; sequences of no drafts, cut by clusters, temperatures of their own; with and without a TV output
+@pytest.mark.parametrize("dtype,vectors,tail,B,K", [("bf16", 1, 3, 400, 5), ("f32", 128, 0, 500, 3), ("bf16", 129, 5, 900, 4), ("bf16", 769, 7, 400, 8),
+                                                     ("f32", 1024, 1, 300, 2), ("bf16", 1535, 7, 300, 2), ("bf16", 1536, 0, 200, 4), ("f32", 1536, 3, 160, 32),
+                                                     ("bf16", 1537, 0, 300, 3)])
+def test_resident_rows(dtype, vectors, tail, B, K):
+    V = vocab(dtype, vectors, tail)
+    cfg = G.Config("resident", B, K, V, dtype, 2.0, V >= 64, 0.8, (0.6, 1.2), ragged=True, seed=vectors)
+    x = G.make_inputs(cfg, "cuda", pad_ld=(-V) % 8)
+    x["draft_len"][::7] = 0
+    P.bebop_debug_force_general_path(3)
+    try:
+        for tv in (True, False):
+            got = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
+                                 temperature=x["temperature"], temperature_all=x["temperature_all"], want_tv=tv)
+            assert P.bebop_debug_last_kernel_name() == "k_fuse"
+            sampled(cfg, x, got, 96)
+    finally:
+        P.bebop_debug_force_general_path(0)
+
+
+def test_resident_rows_masked_and_broken():
+    """What the chunks of the resident form meet besides ordinary logits: masks, NaN, empty rows, bad tokens and temperatures."""
+    cfg = G.Config("res", 40, 3, 9000, "bf16", 2.0, True, 0.8, 1.0, seed=9)
+    x = G.make_inputs(cfg, "cuda")
+    t, d = x["target"], x["draft"]
+    t[1, :, 3000:] = float("-inf"); d[1, :, 3000:] = float("-inf")
+    t[2, 0, :8192] = -1e9; d[3, 1, 64:] = -1e4
+    t[4, 1, 8999] = float("nan"); d[5, 0, 0] = float("inf"); d[6, 2] = float("-inf"); t[7, 3] = float("-inf")
+    x["draft_tokens"][1:4] = 5
+    x["draft_tokens"][8, 1] = 9000
+    x["temperature"] = torch.ones(40, device="cuda"); x["temperature"][9] = -1.0; x["temperature"][10] = float("nan")
+    d[11] = t[11, :3]                                       # p = q: everything is accepted
+    P.bebop_debug_force_general_path(3)
+    try:
+        got = P.bebop_verify(t, d, x["draft_tokens"], x["u_accept"], x["u_final"], temperature=x["temperature"])
+        compare_verify(got, oracle_on(x), "bf16")
+        P.bebop_debug_set_draw_kappa(1e9)                   # no fp32 draw clears its bound: the re-draw kernel does them all
+        compare_verify(P.bebop_verify(t, d, x["draft_tokens"], x["u_accept"], x["u_final"], temperature=x["temperature"]), oracle_on(x), "bf16")
+    finally:
+        P.bebop_debug_set_draw_kappa(-1.0)
+        P.bebop_debug_force_general_path(0)
