@@ -991,23 +991,6 @@ __device__ __forceinline__ void flow_body(const FlowArgs& a, unsigned char* smem
 // ------------------------------------------------------------------ host side
 template <class F> constexpr size_t flow_smem() { return F::LRING + sizeof(FlowShared<F>); }
 
-// Clusters of so many CTAs for a call.  A CTA's slice of a row should be long (every unit costs an exchange and some short
-// stages), but two units of every cluster have to stay in L2, and the tables hold 20,480 vectors: one CTA up to
-// 10,240 vectors per row, two up to 40,960 (us per call on a B200 with one, two, four CTAs, bf16, K = 3: 300 sequences of 80,000
-// logits 126, 129, 157; 200 of 100,000 120, 116, 128; 200 of 151,936 158, 149, 170; 512 of 262,144 two 537, four 546).  Calls of few
-// rows want more and smaller shares, until a cluster has three (24 of 151,936: two CTAs 47.1, four 41.8; 40 row pairs of
-// 262,144: two 35.1, four 31.7, eight 28.6; but 120 of 151,936: two 38.7, four 41.1).
-inline int flow_cluster(const RowArgs& a, bool tv_only) {
-    int C = 1;
-    while (C < kFlowMaxCluster && a.nvec > (C == 1 ? 10240 : 20480 * C)) C *= 2;
-    const double rows = (double)a.B * (tv_only ? 2 : 2 * a.K + 1);
-    while (C < kFlowMaxCluster && rows * C < 3.15 * 148.0 && a.nvec > 4 * 256 * C) C *= 2;
-    return C;
-}
-inline bool flow_resident_rows(const RowArgs& a, int C) { return C == 1 && a.nvec <= kResidentVecs; }
-// Large chunks for long slices (row pairs of 151,936 over two CTAs 152.7 against 164.7 us for 768 of them; 192 sequences of 32,000,
-// K = 7, over one CTA 79.7 against 70.0; 24 of 151,936 over four 45.0 against 42.3).
-inline bool flow_long(const RowArgs& a, bool tv_only, int C) { return a.nvec > (tv_only ? 4000 : 7500) * C; }
 // The smallest share, in rows, that G clusters of at most that many take all units with (a row pair is not cut), for calls of a few
 // rows per cluster, where even shares leave some clusters a row more (48 sequences of 151,936, K = 3, 65.1 -> 61.0 us, 30 of 200,000,
 // K = 2, 50.3 -> 47.7).  From five rows on the even shares stay (0): they leave some clusters a row less, and are done
@@ -1021,6 +1004,43 @@ inline int flow_share_of(const RowArgs& a, bool tv_only, int G) {
         if (at >= total) return share;
     }
 }
+// Multiprocessors of the device (asked once per device).
+inline int flow_sms() {
+    static int cached[64] = {0};
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 148; }
+    if (!cached[dev]) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); return 148; }
+        cached[dev] = n;
+    }
+    return cached[dev];
+}
+// Clusters of so many CTAs for a call.  Two units of every cluster have to stay in L2, and the tables hold 20,480 vectors of a slice:
+// one CTA up to 10,240 vectors per row, two up to 40,960, and so on.  Above that the least work of the busiest cluster decides: the
+// rows of its share, each a slice and what a unit costs beside it, in vectors -- exchanges of two CTAs hide under 130, of four and
+// eight they cost 1,300 and 800 where few units come between (us per call on a B200 with one, two, four, eight CTAs, bf16; fitted to 110
+// such calls: bebop_tv of 300 row pairs of 65,536 40, 36, 43, 59; 100 of 100,000 -, 27, 29, 31; 100 of 262,144 -, 50, 49, 46;
+// K = 3: 200 sequences of 65,536 77, 85, 92, 136; 24 of 151,936 -, 37, 39, 41; 12 of 151,936 -, 35, 32, 30; 4 of 151,936, K = 8, -,
+// 33, 27.5, 27.6; 512 of 262,144 -, 537, 546, -).
+inline int flow_cluster(const RowArgs& a, bool tv_only) {
+    constexpr int kUnit[kFlowMaxCluster + 1] = {0, 0, 130, 0, 1300, 0, 0, 0, 800};
+    int C = 1, best = 0;
+    while (C < kFlowMaxCluster && a.nvec > (C == 1 ? 10240 : 20480 * C)) C *= 2;
+    const double rows = (double)a.B * (tv_only ? 2 : 2 * a.K + 1);
+    double least = 0.0;
+    for (; C <= kFlowMaxCluster; C *= 2) {
+        const int G = flow_sms() / C > 0 ? flow_sms() / C : 1, share = flow_share_of(a, tv_only, G);
+        const double t = (share ? (double)share : rows / G) * ((double)a.nvec / C + kUnit[C]);
+        if (!best || t < least) { best = C; least = t; }
+        if (a.nvec <= 4 * 256 * C) break;
+    }
+    return best;
+}
+inline bool flow_resident_rows(const RowArgs& a, int C) { return C == 1 && a.nvec <= kResidentVecs; }
+// Large chunks for long slices (row pairs of 151,936 over two CTAs 152.7 against 164.7 us for 768 of them; 192 sequences of 32,000,
+// K = 7, over one CTA 79.7 against 70.0; 24 of 151,936 over four 45.0 against 42.3; 500 of 50,000 over one 155 against 133; 500 of 90,000 over
+// two, slices of 5,600 vectors, 235 against 208, 200 of 100,000, K = 8, slices of 6,300, 226 against 231).
+inline bool flow_long(const RowArgs& a, bool tv_only, int C) { return a.nvec > (tv_only ? 4000 : C == 1 ? 7500 : 6000) * C; }
 template <class F, auto kernel> bool flow_ready() {
     static bool done[64] = {false};
     int dev = 0;
@@ -1068,9 +1088,10 @@ template <class F, auto kernel> cudaError_t flow_launch(const FlowCall& x, int C
     FlowArgs fa;
     fa.r = a; fa.draft_tokens = x.draft_tokens; fa.u_accept = x.u_accept; fa.u_final = x.u_final; fa.o = x.o; fa.s_aux = x.tv_only ? x.s_aux : nullptr;
     fa.C = C; fa.nch = f.nch; fa.sv = f.sv;
-    // short rows: an exchange takes longer than a unit's work, so more units go between (600 sequences of 8,000 bf16 logits, K = 7:
-    // one 101.4, two 98.7, three 96.7 us; 192 of 32,000 68.8, 68.1, 69.6); longer ones have no use for it, and L2 has to hold them
-    fa.lag = F::LSL > 3 && a.nvec <= 2560 ? 3 : 1;
+    // small chunks: an exchange may take longer than a unit's work, so more units go between (600 sequences of 8,000 bf16 logits, K = 7:
+    // one 101.4, two 98.7, three 96.7 us; 96 of 65,536, K = 1, over two CTAs 38.1, 35.6, 35.6; 12 of 151,936 over eight 30.7, 29.6, 29.5);
+    // longer slices have no use for it, and L2 has to hold them
+    fa.lag = F::LSL > 3 ? (a.nvec <= 2560 ? 3 : 2) : 1;
     fa.ns = 0; fa.pitch = 0;
     if (F::LRES) {
         fa.pitch = 2 * ((min(f.sv, a.nvec) * 16 + 127) & ~127);
