@@ -24,8 +24,9 @@ def vocab(dtype, vectors, tail):
     return (4 if dtype == "f32" else 8) * vectors - tail
 
 
-# vectors per row: a chunk and its neighbours, two stages' worth, the limits of one, two and four CTAs per row, a last CTA without
-# a vector of its own (129 chunks of 256 over eight CTAs: 17 each for seven of them)
+# vectors per row: a chunk and its neighbours, one and more stages, ragged ends.  The calls are small, so rows of more than 3,072 vectors
+# go over four or eight CTAs; 10,241 vectors over eight in chunks of 256 (path 2) leave the last of them one vector.  The limits of
+# one, two and eight CTAs and of their chunk tables are test_the_limits_of_a_slice's.
 # (V = 1 is left out: p = q = 1 there, and whether q <= p, by which S jumps from 1 to 0, is a matter of the last bit)
 SIZES = [("bf16", 1, 3), ("f32", 128, 0), ("bf16", 129, 3), ("bf16", 257, 0), ("f32", 3073, 1), ("bf16", 7499, 5), ("f32", 7500, 2),
          ("bf16", 10240, 0), ("bf16", 10241, 1), ("f32", 15001, 3), ("bf16", 40960, 0), ("bf16", 40961, 7), ("f32", 81921, 1)]
@@ -150,3 +151,111 @@ def test_resident_rows_masked_and_broken():
     finally:
         P.bebop_debug_set_draw_kappa(-1.0)
         P.bebop_debug_force_general_path(0)
+
+
+# rows at the limits of a CTA's slice, in batches for which one, two and eight CTAs share a row: 10,240 vectors over one (40 large chunks) and
+# one more, over two; 7,500 over one in small chunks (59); 40,960 over two, whose tables of 80 large chunks they fill; 163,840 over eight,
+# the longest rows of the stream
+@pytest.mark.parametrize("dtype,vectors,tail,B,K", [("bf16", 10240, 0, 120, 3), ("bf16", 10241, 1, 120, 3), ("f32", 7500, 0, 300, 3),
+                                                     ("bf16", 40960, 3, 60, 3), ("f32", 163840, 0, 6, 2)])
+def test_the_limits_of_a_slice(dtype, vectors, tail, B, K):
+    V = vocab(dtype, vectors, tail)
+    cfg = G.Config("limits", B, K, V, dtype, 2.0, True, 0.8, 0.9, seed=vectors)
+    x = G.make_inputs(cfg, "cuda", pad_ld=(-V) % 8)
+    P.bebop_debug_force_general_path(3)
+    try:
+        got = P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], temperature_all=0.9)
+        assert P.bebop_debug_last_kernel_name() == "k_fuse"
+        sampled(cfg, x, got, 6 if vectors > 20000 else 24)
+    finally:
+        P.bebop_debug_force_general_path(0)
+
+
+def test_the_limits_of_a_slice_tv():
+    N, V = 100, 8 * 40960
+    g = torch.Generator(device="cuda").manual_seed(3)
+    tgt = (2.0 * torch.randn((N, V), generator=g, device="cuda")).to(torch.bfloat16)
+    drf = (tgt.float() + torch.randn((N, V), generator=g, device="cuda")).to(torch.bfloat16)
+    P.bebop_debug_force_general_path(3)
+    got = P.bebop_tv(tgt, drf)
+    P.bebop_debug_force_general_path(0)
+    sel = [0, 1, 50, 98, 99]
+    ref = oracle.tv(tgt[sel].float().cpu().numpy(), drf[sel].float().cpu().numpy())
+    assert np.abs(to_np(got["tv"])[sel] - ref["tv"]).max() <= TOL["bf16"] and np.abs(to_np(got["s_aux"])[sel] - ref["s_aux"]).max() <= TOL["bf16"]
+
+
+# ---- the sweeps (path 2 without a TV output), which the suites of the other files reach through calls with TV no longer
+@pytest.fixture
+def sweeps():
+    P.bebop_debug_force_general_path(2)
+    yield lambda x, **kw: P.bebop_verify(x["target"], x["draft"], x["draft_tokens"], x["u_accept"], x["u_final"], draft_len=x["draft_len"],
+                                         temperature=x["temperature"], temperature_all=x["temperature_all"], want_tv=False, **kw)
+    P.bebop_debug_set_draw_kappa(-1.0)
+    P.bebop_debug_force_general_path(0)
+
+
+def test_sweeps_fast_draw_bound_over_many_seeds(sweeps):
+    """As the calibration of the other kernels: no unflagged mismatch, and none with a quarter of the factor either."""
+    B, K, V = 224, 3, 151936
+    off = P.bebop_debug_fallback_offset(B, K, V, 1)
+    redrawn = seen = wrong = 0
+    for seed in range(8):
+        flat = seed % 2 == 1
+        cfg = G.Config("cert", B, K, V, "bf16", 1.0 if flat else 3.0, not flat, 1.5 if flat else 1.0, (0.6, 0.7, 1.0, 1.2)[seed % 4], seed=2000 + seed)
+        x = G.make_inputs(cfg, "cuda")
+        if seed % 3 == 0:
+            x["draft_len"] = torch.tensor([i % 2 for i in range(B)], dtype=torch.int32, device="cuda")
+        got = sweeps(x)
+        assert P.bebop_debug_last_kernel_name() == "k_pipe"
+        redrawn += int(got["workspace"][off:off + 4].view(torch.int32).item())
+        ref = oracle_on(x)
+        compare_verify(got, ref, "bf16", context=str(cfg))
+        P.bebop_debug_set_draw_kappa(1.0)
+        again = sweeps(x, workspace=got["workspace"])
+        P.bebop_debug_set_draw_kappa(-1.0)
+        wrong += int(((to_np(again["out_tokens"]) != ref["out_tokens"]).any(axis=1) & ~ref["flagged"]).sum())
+        seen += B
+    print("\nfast-draw bound (sweeps): %d sequences, %d (%.2f %%) re-drawn in fp64" % (seen, redrawn, 100.0 * redrawn / seen))
+    assert wrong == 0 and redrawn <= 0.06 * seen
+
+
+@pytest.mark.parametrize("which", [1, 2])
+def test_sweeps_a_wait_that_runs_out_returns_with_the_status_bit(sweeps, which):
+    cfg = G.Config("wait", 64, 3, 8192, "bf16", 2.0, True, 1.0, 1.0, seed=63)
+    x = G.make_inputs(cfg, "cuda")
+    ok = sweeps(x)
+    P.bebop_debug_expire_wait(which)
+    bad = sweeps(x, workspace=ok["workspace"])
+    torch.cuda.synchronize()                                # returns: nothing hangs
+    assert (to_np(bad["row_status"]) & 32 == 32).all()
+    again = sweeps(x, workspace=ok["workspace"])
+    for k in ("accept_len", "out_tokens", "row_status"):
+        assert torch.equal(again[k], ok[k]), k
+    compare_verify(again, oracle_on(x), cfg.dtype)
+
+
+def test_sweeps_status_bits_and_masks(sweeps):
+    cfg = G.Config("st", 12, 2, 20000, "f32", 1.0, False, 0.5, 1.0, seed=4)
+    x = G.make_inputs(cfg, "cuda")
+    t, d = x["target"], x["draft"]
+    x["temperature"] = torch.ones(12, device="cuda"); x["temperature"][4] = 0.0
+    t[1, 0, 17] = float("nan"); d[2, 1, :] = float("-inf"); x["draft_tokens"][3, 1] = 20000; t[5, 1, 5] = float("inf")
+    d[6] = t[6, :2]; t[6, 0, 9] = float("-inf"); d[6, 0, 9] = float("-inf"); x["draft_tokens"][6, 0] = 9        # p = q: no residual at the reject
+    d[7] = t[7, :2]; t[7, 2, 100] = float("nan")                                                                  # a bad bonus row
+    t[8, :, :10000] = float("-inf"); d[8, :, 10000:] = float("-inf"); x["draft_tokens"][8] = 11                  # supports that do not meet
+    t[9, :, : 5000] = -1e9; t[10, 1, 300:] = -1e4
+    got = sweeps(x)
+    compare_verify(got, oracle_on(x), "f32")
+    st = to_np(got["row_status"])
+    assert st[1] & 1 and st[2] & 2 and st[3] & 4 and st[4] & 16 and st[5] & 1 and st[6] == 8 and st[7] & 1 and st[0] == 0
+
+
+@pytest.mark.parametrize("dtype,B,K,V", [("bf16", 600, 2, 20000), ("f32", 600, 2, 20000), ("bf16", 5, 2, 16383), ("bf16", 3, 1, 131072), ("f32", 3, 1, 65537)])
+def test_sweeps_every_sequence_goes_to_the_fp64_redraw(sweeps, dtype, B, K, V):
+    cfg = G.Config("redraw", B, K, V, dtype, 2.0, True, 0.8, (0.6, 1.2), ragged=True, seed=B + K)
+    x = G.make_inputs(cfg, "cuda", pad_ld=(-V) % 8)
+    P.bebop_debug_set_draw_kappa(1e9)
+    got = sweeps(x)
+    off = P.bebop_debug_fallback_offset(B, K, V, 0 if dtype == "f32" else 1)
+    assert int(got["workspace"][off:off + 4].view(torch.int32).item()) == B
+    sampled(cfg, x, {k: v for k, v in got.items() if k != "tv"}, 64)
