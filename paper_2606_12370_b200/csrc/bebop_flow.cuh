@@ -6,12 +6,13 @@
 //   pass 1  per chunk of 256 (short rows: 128) 16-byte vectors, a warp each: the reference exponent E (an integer) and the sum of
 //           e = 2^(x c - E);
 //   pass 2  per half as many vectors of both rows: the residuals r' = max(0, e_p - rho e_q) = (p - q) S_p, rho = S_p / S_q,
-// and the stream interleaves them, pass 1 of unit u before pass 2 of unit u - 1 (of very short rows: u - 3): between the passes of a unit lies another
-// unit's work, under which the exchange of the sums within the cluster disappears, and the second pass finds its logits in L2
-// (two units of every cluster are under way, 90 MB in all at 151,936 bf16 logits; DRAM reads 1.01 times the logits).
+// and the stream interleaves them, pass 1 of unit u before pass 2 of unit u - 1 (small chunks: u - 2 or u - 3): between the passes of a unit lies
+// another unit's work, under which the exchange of the sums within the cluster disappears, and the second pass finds its logits in L2
+// (two units of every cluster are under way, 90 MB in all at 151,936 bf16 logits; DRAM reads 1.07 times the logits of 256 such sequences, K = 3, 1.01
+// of 64), or, if the rows are short, in the stage where pass 1 left them (FlowResident).
 //
-// Warps: the consumers; a producer (one thread: bulk copies into a ring of 192 KB in three or four stages, with a description
-// each); one warp that exchanges and merges the sums of pass 1, one that writes out the masses of pass 2, and a finisher.  The
+// Warps: the consumers; a producer (one thread: bulk copies into a ring of 192 KB in three to eight stages, with a description
+// each); one or two warps that exchange and merge the sums of pass 1, one that writes out the masses of pass 2, and a finisher.  The
 // consumers do not meet: a warp takes the chunk of a stage that falls to it (the first chunk's warp moves on from
 // stage to stage, so that short stages load the warps evenly), leaves its sums in a table and moves on.  The exchange warp adds
 // the chunks up, half a warp per row, sends the CTA's sums to the cluster through distributed shared memory, merges what it is
@@ -19,15 +20,18 @@
 // delivers the last part of a sequence has its finisher complete it -- accept scan (Algorithm 3), TV, the fast draw with its
 // certificate or a place in the list for the fp64 re-draw -- while the stream goes on.
 //
-// What bounds it: the exponential unit, 16 lanes per SM and clock, which two passes keep for 104 us of the 152 that 768 row pairs of
+// What bounds it: the exponential unit, 16 lanes per SM and clock, which two passes keep for 104 us of the 150 that 768 row pairs of
 // 151,936 bf16 logits take; 69 per cent busy while an SM works (6.2 instructions per logit and pass), the rest are the chains at
 // both ends of a warp's chunk (barrier, maximum, reduction) and the ends of the clusters' runs.  Neither DRAM nor L2 does (the
 // bulk copies reach 19 TB/s out of L2).  What a task costs beyond its exponentials, 0.3 to 0.4 us, hardly depends on its size:
 // 768 row pairs in stages of 32, 48, 64 KB 182, 164, 152 us; sixteen warps of eight vectors a lane are better than twelve (172) or than
 // 24 of four (164), except on short rows, whose units those pieces fit better.  The same calls through the kernels in
 // whose place the stream stands (exponentials parked in tensor memory; two full sweeps over DRAM): 768 row pairs 168 us, 256
-// sequences of 151,936, K = 3, 198 (178), 1,024 of them, K = 4 ragged, 686 (525), 192 of 32,000, K = 7 ragged, 83 (68).
-// Tried and left out: warps in two or four groups on alternate stages (179 us and 196 for the 256 sequences), two or three units
+// sequences of 151,936, K = 3, 198 (178), 1,024 of them, K = 4 ragged, 686 (531), 192 of 32,000, K = 7 ragged, 83 (60.5).
+// The size of the consumers' loop counts: a branch in it for the bonus row's masses cost 2 to 7 per cent, a call in its place 6 (their sums
+// are exact for all rows instead), a vote in front of the load of a task's description 1.  Tried and left out: more and smaller stages for
+// short rows (1,000 of 8,000, K = 8, 174 us in four stages of 48 KB, 191 in twelve of 16), one place in the producer that hands out all tasks
+// (256 of 151,936 178 -> 183 us), the finisher's loads all asked for at once (no change, and short rows 5 per cent slower), warps in two or four groups on alternate stages (179 us and 196 for the 256 sequences), two or three units
 // between the passes (184), four CTAs a cluster (209 to 222).
 //
 // Every wait is bounded; one that gives up sets the wait flag and the CTA's abort flag, under which all warps run out.  No

@@ -22,7 +22,7 @@ constexpr size_t kRedrawTicketOffset = 192;   // unsigned: next work item of the
 constexpr size_t kFbCountOffset = 128;   // 8 bytes inside the zeroed head of the workspace: low int, sequences listed for the fp64
                                          // re-draw; high int, sequences whose draw is decided
 struct PipePlan {
-    int T, slice_vecs;     // slices per row, vectors per slice (multiple of 16)
+    int T, slice_vecs;     // slices per row, vectors per slice (multiple of 256)
     size_t off_p1done, off_ddone, off_xdone, off_xsdone, off_fbrec, off_rowcnt, zero_bytes;
     size_t off_xsum, off_xmass;   // fp64 re-draw: per listed sequence done counter; sums and masses per item
     size_t off_part, off_rstat, off_dpart, off_sinfo, total;
@@ -50,7 +50,7 @@ static inline PipePlan make_pipe_plan(int B, int K, int nvec, int dt, int slice_
     (void)dt;
     PipePlan w;
     w.T = (nvec + slice_cap - 1) / slice_cap; if (w.T < 1) w.T = 1;
-    w.slice_vecs = (((nvec + w.T - 1) / w.T) + 255) & ~255;  // whole chunks of the stream's pass 1
+    w.slice_vecs = (((nvec + w.T - 1) / w.T) + 255) & ~255;  // whole chunks of the stream's pass 1 (dealt evenly, 7 or 8 a slice: no faster)
     const size_t NR = (size_t)(2 * K + 1);
     size_t o = 256;                                           // ticket, wait flag; at kFbCountOffset the re-draw count
     w.off_p1done = o; o += align256(sizeof(int) * (size_t)B);      // per sequence: rows merged

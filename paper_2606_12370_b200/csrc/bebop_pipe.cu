@@ -436,7 +436,7 @@ __device__ __noinline__ void accept_warp(const PipeArgs& a, int b) {
         if (a.o.q_draft) a.o.q_draft[(int64_t)b * K + lane] = zero ? 0.f : (float)qx;
     }
     if (lane == 0) {
-        a.o.accept_len[b] = nn; a.stop[b] = fatal ? -1 : nn;
+        a.o.accept_len[b] = nn;
         if (a.o.row_status) a.o.row_status[b] = seq_st;
         // the record's mark makes it (and, through the row records it was computed from, the sequence) ready
         // (pad0 carries c = log2(e) / tau of the sequence: the second sweep's producer need not divide again)
@@ -474,7 +474,7 @@ __device__ __forceinline__ void pipe_p1(const PipeArgs& a, PipeShared& S, const 
     const RowArgs& R = a.r;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = d.nv;
-    // a warp has 256 vectors side by side, the chunk of the stream's pass 1: both give a row the same sum
+    // a warp has 256 vectors side by side, a large chunk of the stream's pass 1: with those both give a row the same sum
     const int at = warp * (32 * NV) + lane;
     uint4 raw[NV];
     if ((warp + 1) * (32 * NV) <= nv) {
@@ -1003,7 +1003,6 @@ cudaError_t pipe_verify(const RowArgs& a, const Plan& p, const int32_t* draft_to
     const PipePlan wp = make_pipe_plan(a.B, a.K, a.nvec, a.dt, PSLICE);
     PipeArgs wa;
     wa.r = a; wa.draft_tokens = draft_tokens; wa.u_accept = u_accept; wa.u_final = u_final; wa.o = o;
-    wa.stop = reinterpret_cast<int*>(ws + p.off_stop);
     char* w = ws + p.off_pipe;
     wa.fb_count = reinterpret_cast<unsigned long long*>(w + kFbCountOffset);
     wa.fb_list = reinterpret_cast<FbRec*>(w + wp.off_fbrec);

@@ -60,7 +60,6 @@ struct PipeArgs {
     const float* u_accept;
     const float* u_final;
     VerifyOut o;
-    int* stop;
     unsigned long long* fb_count;   // [1] low half: sequences listed for the fp64 re-draw; high half: sequences whose
                                     // draw is decided (token written, listed, or none to come); zeroed with the workspace
     FbRec* fb_list;       // [B] (zeroed with the workspace: a record is valid once its b1 is non-zero)

@@ -20,8 +20,6 @@ __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i ^ ((i >>
 
 // 2^k as a double for k in [-1022, 1023], else 0 (k below) -- exact
 __device__ __forceinline__ double pow2d(int k) { return k < -1022 ? 0.0 : __hiloint2double((1023 + k) << 20, 0); }
-// 2^k as a float for k in [-126, 127] (0 below): exact
-__device__ __forceinline__ float pow2f(int k) { return k < -126 ? 0.f : __int_as_float((127 + k) << 23); }
 __device__ __forceinline__ double shfl_xor_d(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 __device__ __forceinline__ double shfl_up_d(double v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
 
